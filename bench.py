@@ -826,7 +826,7 @@ def run_prefill(args):
         "data": "synthetic: seeded N(0,1) bf16 q/k/v of the long_32k video's whole sequence",
         "config": {"workload": "prefill_long_32k", "prefix_tokens": S, "branches": int(lens.size),
                    "branch_tokens": int(lens.sum()), "tokens": N, "h_q": H, "h_kv": Hkv, "head_dim": D,
-                   "kernel": "prefix_tc_kernel (tcgen05, prefill mode)"},
+                   "kernel": "prefill_tc_kernel (tcgen05)"},
         "ms": ms,
         "roofline": {"bound": "tensor", "achieved": flops / (ms * 1e-3) / 1e12, "peak": peak, "unit": "TFLOP/s",
                      "frac": flops / (ms * 1e-3) / 1e12 / peak, "peak_kind": peak_kind,

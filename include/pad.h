@@ -456,16 +456,16 @@ pad_status pad_attn_aggregate(const void* x, int64_t n_tokens, int32_t d_model, 
  * attends causally within the prefix; a branch token attends to the whole prefix and
  * causally to its own branch; never to another branch.  Block-sparse: each query tile reads
  * only the key ranges its rows can see.
- *   prob        h_q, h_kv, head_dim (64 or 128), scale, out_dtype (num_sms, flags, page_size
+ *   prob        h_q, h_kv, head_dim (64 or 128), scale, out_dtype, flags (num_sms, page_size
  *               unused)
  *   branch_len  [n_branches] HOST, each >= 0; n_branches <= 1024
  *   q           [N, h_q, head_dim] bf16, k / v [N, h_kv, head_dim] bf16, N = prefix_len +
  *               sum(branch_len), token-major; out [N, h_q, head_dim] fp32 or bf16; lse [N, h_q]
  *               fp32 (natural log) or NULL; all device, 16-byte aligned (lse 4-byte)
- * One video per call; the work is asynchronous on `stream`.  head_dim 128 runs on the
- * tensor-core kernel (a CTA: 128 / G tokens x the G heads of one kv-head against its visible
- * key ranges, output normalised in place); head_dim 64, or flags PAD_FLAG_PREFIX_MMA, on the
- * warp-level kernel (64 tokens x one head). */
+ * One video per call; the work is asynchronous on `stream`.  It runs on the tensor-core
+ * kernel (a CTA: two groups of 128 / G tokens x the G heads of one kv-head against their
+ * visible key ranges, output normalised in place); with flags PAD_FLAG_PREFIX_MMA or
+ * PAD_FLAG_PREFIX_SIMT on the warp-level kernel (64 tokens x one head). */
 pad_status pad_prefill_attn(const pad_problem* prob, int32_t prefix_len, int32_t n_branches,
                             const int32_t* branch_len, const void* q, const void* k, const void* v, void* out,
                             float* lse, pad_stream_t stream);

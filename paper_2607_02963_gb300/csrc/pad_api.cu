@@ -1888,11 +1888,12 @@ pad_status pad_prefill_attn(const pad_problem* prob, int32_t prefix_len, int32_t
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out) || (lse && (reinterpret_cast<uintptr_t>(lse) & 3u)))
     return fail(PAD_ERR_INVALID_ARG, "tensors must be 16-byte aligned (lse 4-byte)");
   cudaError_t e;
-  if (prob->head_dim == 128 && !(prob->flags & (PAD_FLAG_PREFIX_MMA | PAD_FLAG_PREFIX_SIMT))) {
+  if (!(prob->flags & (PAD_FLAG_PREFIX_MMA | PAD_FLAG_PREFIX_SIMT))) {
     const uint64_t gen = next_generation();
     g_prefill_gen.store(gen);
-    e = launch_prefill_tc((int32_t)n, prefix_len, n_branches, branch_len, prob->h_q, prob->h_kv, prob->scale,
-                          prob->out_dtype == 1, gen, q, k, v, out, lse, reinterpret_cast<cudaStream_t>(stream));
+    e = launch_prefill_tc((int32_t)n, prefix_len, n_branches, branch_len, prob->h_q, prob->h_kv, prob->head_dim,
+                          prob->scale, prob->out_dtype == 1, gen, q, k, v, out, lse,
+                          reinterpret_cast<cudaStream_t>(stream));
   } else {
     e = launch_prefill((int32_t)n, prefix_len, n_branches, branch_len, prob->h_q, prob->h_kv, prob->head_dim,
                        prob->scale, prob->out_dtype == 1, q, k, v, out, lse, reinterpret_cast<cudaStream_t>(stream));

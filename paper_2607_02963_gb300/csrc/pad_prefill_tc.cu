@@ -1,0 +1,675 @@
+// Whole-sequence forward attention under the event-factorized mask (Sec. 3.4, Fig. 3) on the
+// 5th-generation tensor cores: the sequence of one video is [prefix of S tokens ; branch 0 ;
+// ... ; branch E-1]; a prefix token attends causally within the prefix, a branch token to the
+// prefix and causally to its own branch.
+//
+// One CTA per (query tile, kv-head).  A query tile is two slots of 128 rows: slot g holds
+// 128 / G consecutive tokens x the G query heads of the kv-head (126 rows at G = 7), slot 1
+// the tokens right after slot 0's.  The CTA walks the 128-key tiles its rows can see (the
+// prefix up to its last token, then the keys from the start of its first branch token's
+// branch to its last token) and masks per row only where a tile needs it.  Query tiles start
+// in descending order, so that the longest key ranges go first.
+//
+//   warps 0, 3  TMA producers of K and V tiles (64-column boxes, 128-byte swizzle)
+//   warp 1      S issuer: S_g(k) = Q_g K(k)^T
+//   warp 2      TMEM allocation (512 columns) and deallocation, and P.V issuer: O_g += P_g(k)
+//               V(k), P read back from TMEM, 96 keys and then the last 32
+//   warps 4-7   softmax of slot 0, warps 8-11 of slot 1: one query row per thread, all 128
+//               scores of a tile in registers (setmaxnreg moves registers from warps 0-3 to
+//               these); online sum in base 2 on a maximum that follows lazily.  At the end each
+//               warp normalises its own 32 rows and writes them through its part of the
+//               slot's (idle) Q stage.
+//
+// What bounds it, and why it looks like this (sequence of 34.7 k tokens, 28/4 heads, D 128: 7.08
+// ms with one 128-row group per CTA, 5.36 ms = 1.60 PFLOP/s of visible pairs, 0.86 of cuBLAS's
+// rate, as it is; 8.7 k tokens, 14/2 heads, D 64: 724 us on the mma.sync kernel, 140 us here):
+//   - Two slots share each K/V tile: with one 128-row group the MMAs' shared-memory operand
+//     reads (S: 8 KB per K = 16 step, P.V: 4 KB) and the 64 KB that a tile brings in exceed 128
+//     B per clock by a fifth; and one slot's softmax runs under the other's MMAs.
+//   - What is left is the chain S -> softmax -> P.V of a slot, ~2900 cycles per tile against
+//     2 x 1036 of MMAs.  So the softmax makes no pass for the maximum (the row sum tells
+//     whether the running one still bounds the scores), tiles that need no mask run a loop
+//     without mask code, and P is released in two unequal parts, so that little of P.V is
+//     left to do once the last of P is written (halves: 5.67 ms).
+//   - The issuer warps run their loops with all lanes and elect the issuing one (elect_one),
+//     and the TMEM addresses are immediates: 6.34 -> 6.02 ms.
+//
+// TMEM columns: S_0 at 0, S_1 at 128.  head_dim 128: O_0 at 256, O_1 at 384, and P_g goes over
+// the first half of S_g (all of a row's scores are in registers by then), so S_g(k + 1) waits
+// for P.V of tile k.  head_dim 64: P_0 at 256, P_1 at 320, O_0 at 384, O_1 at 448; S_g(k + 1)
+// only waits until the scores of tile k have been read.
+//
+// Barrier phases: every barrier is per slot or per stage, so that the completion a thread
+// waits for by parity cannot be overtaken by the next one before the thread moves on.  Every
+// wait is bounded (about one second of %globaltimer); one that runs out records
+// PAD_ERR_DEVICE_TIMEOUT in the prefill status word, raises a CTA-wide abort flag, lets the
+// producers and issuers drain what they started, frees TMEM and returns.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+#include <cuda_bf16.h>
+#include <cstdint>
+#include <type_traits>
+
+#include "pad_internal.h"
+#include "pad_tc_common.cuh"
+
+namespace pad {
+
+namespace {
+
+using namespace tc;
+
+constexpr int kMaxBranches = 1024;
+constexpr int kBN = 128;        // keys per tile
+constexpr int kThreads = 384;
+constexpr int kLoGroups = 3;          // 32-key groups of a tile whose P is released first
+constexpr float kRescaleSum = 256.0f; // a part of a row whose P sum to more is redone on a new maximum
+constexpr float kNegInf = -__builtin_huge_valf();
+// Registers per thread after setmaxnreg: the launch gives 384 x 168 = 64512, and
+// 128 x 80 + 256 x 208 = 63488.
+constexpr int kRegsIssue = 80, kRegsSoftmax = 208;
+
+template <int D>
+struct Cfg {
+  static constexpr int kHalves = D / 64;                      // 64-column boxes of a row
+  static constexpr uint32_t kBoxBytes = kBN * 128;            // 128 rows x 64 bf16
+  static constexpr uint32_t kTileBytes = kHalves * kBoxBytes; // a K or V tile, or Q of a slot
+  static constexpr int kKS = D == 128 ? 3 : 4;                // K stages
+  static constexpr int kVS = D == 128 ? 2 : 4;                // V stages
+  static constexpr uint32_t kOffK = 2 * kTileBytes;           // Q_0, Q_1 first
+  static constexpr uint32_t kOffV = kOffK + kKS * kTileBytes;
+  static constexpr uint32_t kOffBar = kOffV + kVS * kTileBytes;
+  static constexpr uint32_t kSmemBytes = kOffBar + 512;
+  static constexpr bool kOwnP = D == 64;                      // P has TMEM columns of its own
+  static constexpr uint32_t kColP = 256;                      // + 64 g   (kOwnP)
+  static constexpr uint32_t kColO = D == 128 ? 256 : 384;     // + D g
+  static constexpr uint32_t kIdescS = make_idesc(128, kBN, false);  // B = K tile, K-major
+  static constexpr uint32_t kIdescPV = make_idesc(128, D, true);    // B = V tile, N(=d)-major
+  static_assert(kSmemBytes <= 232448, "fits the 227 KB opt-in shared memory");
+};
+
+struct PrefillTcParams {
+  int32_t n_tokens, prefix_len, n_branches;
+  int32_t h_q, h_kv, group, tps;        // tps: query tokens per slot (128 / group)
+  float scale_log2;
+  int32_t out_bf16;
+  uint64_t gen;
+  PadDevHeader* header;
+  void* out;
+  float* lse;
+  int32_t bstart[kMaxBranches + 1];     // branch b occupies [bstart[b], bstart[b + 1]); bstart[0] = prefix_len
+};
+
+struct Bars {
+  uint64_t kfull[4], kfree[4];
+  uint64_t vfull[4], vfree[4];
+  uint64_t qfull[2];
+  uint64_t sfull[2];          // S of the slot's current tile has completed
+  uint64_t sread[2];          // its scores have been read (4 warp arrivals; kOwnP)
+  uint64_t plo[2], phi[2];    // P of its first 32 kLoGroups keys / of the rest is written (4 warp arrivals)
+  uint64_t pvlo[2];           // P.V of its first part has completed
+  uint64_t pvdone[2];         // its P.V has completed
+  uint64_t drain_s, drain_pv; // every MMA of the S / P.V issuer has completed
+  uint64_t tdone;             // the softmax warps are done with TMEM (8 warp arrivals)
+  uint32_t tmem_base;
+  int32_t abort;
+};
+static_assert(sizeof(Bars) <= 512, "barrier block fits its slot");
+
+// Bounded wait, inlined (setmaxnreg leaves no room for calls).
+__device__ __forceinline__ bool pwait(uint64_t* bar, uint32_t parity, Bars* bars, const PrefillTcParams& p, int where) {
+  unsigned long long t0 = 0;
+  for (uint32_t i = 1;; ++i) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((i & 255u) == 0) {
+      if (*reinterpret_cast<volatile int32_t*>(&bars->abort)) return false;
+      const unsigned long long now = globaltimer();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > kWaitNs) {
+        pad_set_error(p.header, p.gen, PAD_ERR_DEVICE_TIMEOUT, (int)blockIdx.x, where, (int)threadIdx.x);
+        *reinterpret_cast<volatile int32_t*>(&bars->abort) = 1;
+        return false;
+      }
+    }
+  }
+}
+
+// The same for a whole warp (warp-uniform result).
+__device__ __forceinline__ bool pwait_warp(uint64_t* bar, uint32_t parity, Bars* bars, const PrefillTcParams& p, int where) {
+  return __all_sync(0xffffffffu, pwait(bar, parity, bars, p, where)) != 0;
+}
+
+// First token of the branch that holds token t (t >= prefix_len).
+__device__ __forceinline__ int branch_start(const PrefillTcParams& p, int t) {
+  int lo = 0, hi = p.n_branches - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (p.bstart[mid] <= t) lo = mid; else hi = mid - 1;
+  }
+  return p.bstart[lo];
+}
+
+// Maximum of a row's 128 raw scores (eight chains of three-input max).
+__device__ __forceinline__ float row_max(const uint32_t (&s)[4][32]) {
+  float m[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) m[u] = kNegInf;
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+#pragma unroll
+    for (int i = 0; i < 32; i += 2) {
+      const int u = (i >> 1) & 7;
+      m[u] = max3f(m[u], __uint_as_float(s[c][i]), __uint_as_float(s[c][i + 1]));
+    }
+  return fmaxf(max3f(m[0], m[1], m[2]), max3f(max3f(m[3], m[4], m[5]), m[6], m[7]));
+}
+
+// P = 2^(s * sl2 - m) of the 32-score groups [C0, C1) of a row, written as packed bf16 (two
+// keys per column) to TMEM columns taddr + 16 C0 ..; returns their fp32 sums as four pairs.
+template <int C0, int C1>
+__device__ __forceinline__ void part_exp(const uint32_t (&s)[4][32], uint64_t sc2, float m, uint32_t taddr,
+                                         uint64_t (&sum)[4]) {
+  const uint64_t nm2 = f2pack(-m, -m);
+#pragma unroll
+  for (int u = 0; u < 4; ++u) sum[u] = 0ull;
+#pragma unroll
+  for (int c = C0; c < C1; ++c) {
+    uint32_t pk[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const uint64_t x = ffma2(f2pack(__uint_as_float(s[c][2 * i]), __uint_as_float(s[c][2 * i + 1])), sc2, nm2);
+      const float a = ex2(f2lo(x)), b = ex2(f2hi(x));
+      sum[i & 3] = fadd2(sum[i & 3], f2pack(a, b));
+      pk[i] = pack_bf16(a, b);
+    }
+    tmem_st16(taddr + 16 * c, pk);
+  }
+}
+
+template <int D>
+__global__ void __launch_bounds__(kThreads, 1)
+    prefill_tc_kernel(const __grid_constant__ PrefillTcParams p, const __grid_constant__ CUtensorMap tmQ,
+                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
+  using C = Cfg<D>;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  const uint32_t sbase = smem_u32(smem);
+  if (sbase & 1023u) {  // the 128-byte swizzle atoms need 1024-byte alignment (never expected)
+    if (threadIdx.x == 0) pad_set_error(p.header, p.gen, PAD_ERR_UNSUPPORTED, (int)blockIdx.x, (int)sbase, 0);
+    return;
+  }
+  Bars* bars = reinterpret_cast<Bars*>(smem + C::kOffBar);
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+
+  const int N = p.n_tokens, S = p.prefix_len, G = p.group;
+  const int tpc = 2 * p.tps;                              // query tokens per CTA
+  const int n_qt = (N + tpc - 1) / tpc;
+  const int qt = n_qt - 1 - (int)blockIdx.x / p.h_kv;
+  const int kvh = (int)blockIdx.x % p.h_kv;
+  const int tok0 = qt * tpc;
+  const int last = min(tok0 + tpc, N) - 1;
+  // key tiles: [0, a_end) of the prefix, then [b_lo, last] of the branches
+  const int a_tiles = (min(S, last + 1) + kBN - 1) / kBN;
+  int b_lo = 0, b_tiles = 0;
+  if (last >= S) {
+    b_lo = branch_start(p, max(tok0, S));
+    b_tiles = (last + 1 - b_lo + kBN - 1) / kBN;
+  }
+  const int n_tiles = a_tiles + b_tiles;                  // >= 1
+  auto tile_tok = [&](int t) { return t < a_tiles ? t * kBN : b_lo + (t - a_tiles) * kBN; };
+  auto load_tile = [&](const CUtensorMap* map, uint32_t off, int t, uint64_t* full) {
+    mbar_expect_tx(full, C::kTileBytes);
+#pragma unroll
+    for (int h = 0; h < C::kHalves; ++h)
+      tma_load_3d(sbase + off + h * C::kBoxBytes, map, 64 * h, kvh, tile_tok(t), full);
+  };
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < 4; ++s) {
+      mbar_init(&bars->kfull[s], 1);
+      mbar_init(&bars->kfree[s], 1);
+      mbar_init(&bars->vfull[s], 1);
+      mbar_init(&bars->vfree[s], 1);
+    }
+    for (int g = 0; g < 2; ++g) {
+      mbar_init(&bars->qfull[g], 1);
+      mbar_init(&bars->sfull[g], 1);
+      mbar_init(&bars->sread[g], 4);
+      mbar_init(&bars->plo[g], 4);
+      mbar_init(&bars->phi[g], 4);
+      mbar_init(&bars->pvlo[g], 1);
+      mbar_init(&bars->pvdone[g], 1);
+    }
+    mbar_init(&bars->drain_s, 1);
+    mbar_init(&bars->drain_pv, 1);
+    mbar_init(&bars->tdone, 8);
+    bars->abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // Q of both slots (box: 64 columns x G heads x tps tokens, so that smem row = token * G +
+    // head; tokens past N are zero-filled) and the first K tile go out from here
+    const uint32_t q_bytes = (uint32_t)C::kHalves * 128u * (uint32_t)(G * p.tps);
+    for (int g = 0; g < 2; ++g) {
+      mbar_expect_tx(&bars->qfull[g], q_bytes);
+#pragma unroll
+      for (int h = 0; h < C::kHalves; ++h)
+        tma_load_3d(sbase + g * C::kTileBytes + h * C::kBoxBytes, &tmQ, 64 * h, kvh * G, tok0 + g * p.tps,
+                    &bars->qfull[g]);
+      if (g == 0) load_tile(&tmK, C::kOffK, 0, &bars->kfull[0]);
+    }
+    load_tile(&tmV, C::kOffV, 0, &bars->vfull[0]);
+  }
+  if (warp == 2) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem_base)),
+                 "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  // an allocation of all 512 columns starts at TMEM address 0: known at compile time, so that
+  // the MMAs' TMEM operands are immediates (a word read back from shared memory is not)
+  constexpr uint32_t tmem = 0;
+
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
+    bool ok = true;
+    if (warp == 0 || warp == 3) {
+      // ------------------------------------------------------------ TMA producers
+      if (lane == 0) {
+        const bool isK = warp == 0;
+        const CUtensorMap* map = isK ? &tmK : &tmV;
+        const int ns = isK ? C::kKS : C::kVS;
+        uint64_t* full = isK ? bars->kfull : bars->vfull;
+        uint64_t* freed = isK ? bars->kfree : bars->vfree;
+        const uint32_t base = isK ? C::kOffK : C::kOffV;
+        int s = 1, ph = 0, issued = 1;  // tile 0 went out in the prologue; ph: uses of stage s
+        for (int t = 1; t < n_tiles; ++t) {
+          if (s == ns) {
+            s = 0;
+            ++ph;
+          }
+          if (ph > 0) ok = pwait(&freed[s], (uint32_t)((ph - 1) & 1), bars, p, isK ? 1 : 2);
+          if (!ok) break;
+          load_tile(map, base + (uint32_t)s * C::kTileBytes, t, &full[s]);
+          issued = t + 1;
+          ++s;
+        }
+        if (!ok) {
+          // the loads already issued must land before the CTA leaves
+          for (int t = max(0, issued - ns); t < issued; ++t) drain_wait(&full[t % ns], (uint32_t)((t / ns) & 1));
+        }
+      }
+    } else if (warp == 1) {
+      // ------------------------------------------------------------ S issuer
+      const bool el = elect_one();
+      const uint64_t dK = sdesc(sbase + C::kOffK, 16, 1024);
+      int s = 0, ph = 0;
+      for (int t = 0; t < n_tiles && ok; ++t) {
+        ok = pwait_warp(&bars->kfull[s], (uint32_t)ph, bars, p, 3);
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          if (!ok) break;
+          if (t == 0)
+            ok = pwait_warp(&bars->qfull[g], 0u, bars, p, 11);
+          else  // S_g is free: its scores are read (and, where P lies over them, P.V is done)
+            ok = pwait_warp(C::kOwnP ? &bars->sread[g] : &bars->pvdone[g], (uint32_t)((t - 1) & 1), bars, p, 6);
+          if (!ok) break;
+          fence_after();
+          const uint64_t qd = sdesc(sbase + (uint32_t)g * C::kTileBytes, 16, 1024);
+          const uint64_t kd = dK + ((uint32_t)s * C::kTileBytes >> 4);
+          if (el) {
+#pragma unroll
+            for (int kk = 0; kk < D / 16; ++kk) {
+              const uint32_t off = (uint32_t)(kk >> 2) * C::kBoxBytes + (uint32_t)(kk & 3) * 32;
+              mma_ss(tmem + 128u * g, qd + (off >> 4), kd + (off >> 4), C::kIdescS, kk > 0 ? 1u : 0u);
+            }
+            mma_commit(&bars->sfull[g]);
+            if (g == 1) mma_commit(&bars->kfree[s]);
+          }
+          __syncwarp();
+        }
+        if (++s == C::kKS) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+      if (el) mma_commit(&bars->drain_s);
+      __syncwarp();
+      drain_wait(&bars->drain_s, 0u);
+    } else {
+      // ------------------------------------------------------------ P.V issuer
+      // V tile, N(=head-dim)-major: 16 keys per K-step (2048 bytes), a second 64-column box
+      // at + kBoxBytes (leading byte offset), 8-row groups 1024 apart.
+      const bool el = elect_one();
+      const uint64_t dV = sdesc(sbase + C::kOffV, C::kBoxBytes, 1024);
+      int s = 0, ph = 0;
+      for (int t = 0; t < n_tiles && ok; ++t) {
+        ok = pwait_warp(&bars->vfull[s], (uint32_t)ph, bars, p, 4);
+        const uint64_t vd = dV + ((uint32_t)s * C::kTileBytes >> 4);
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          const uint32_t a = tmem + (C::kOwnP ? C::kColP + 64u * g : 128u * g);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (ok) ok = pwait_warp(h ? &bars->phi[g] : &bars->plo[g], (uint32_t)(t & 1), bars, p, 5);
+            if (!ok) break;
+            fence_after();
+            if (el) {
+#pragma unroll
+              for (int kk = h ? 2 * kLoGroups : 0; kk < (h ? 8 : 2 * kLoGroups); ++kk)
+                mma_ts(tmem + C::kColO + (uint32_t)D * g, a + kk * 8, vd + ((uint32_t)kk * 2048 >> 4), C::kIdescPV,
+                       (t > 0 || kk > 0) ? 1u : 0u);
+              if (h == 0) mma_commit(&bars->pvlo[g]);
+              if (h == 1) {
+                mma_commit(&bars->pvdone[g]);
+                if (g == 1) mma_commit(&bars->vfree[s]);
+              }
+            }
+            __syncwarp();
+          }
+        }
+        if (++s == C::kVS) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+      if (el) mma_commit(&bars->drain_pv);
+      __syncwarp();
+      drain_wait(&bars->drain_pv, 0u);
+    }
+    __syncwarp();
+    if (warp == 2) {
+      // TMEM is freed only after every softmax warp has arrived
+      drain_wait(&bars->tdone, 0u);
+      __syncwarp();
+      fence_after();
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+    }
+  } else {
+    // ------------------------------------------------------------ softmax
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
+    const int g = (warp - 4) >> 2;             // slot
+    const int wrow = 32 * (warp & 3);          // TMEM lanes wrow .. wrow + 31
+    const int row = wrow + lane;               // row of the slot: token row / G, head row % G
+    const int tl = row / G;
+    const int tok = tok0 + g * p.tps + tl;
+    const bool active = tl < p.tps && tok < N;
+    const int bs = active && tok >= S ? branch_start(p, tok) : -1;
+    const uint32_t tb = tmem + ((uint32_t)wrow << 16);
+    const uint32_t tS = tb + 128u * g, tP = C::kOwnP ? tb + C::kColP + 64u * g : tS;
+    const uint32_t tO = tb + C::kColO + (uint32_t)D * g;
+    const float sl2 = p.scale_log2;
+    const uint64_t sc2 = f2pack(sl2, sl2);
+    // an inactive row (past the slot's rows or the sequence) takes no part in any decision
+    float m_run = active ? kNegInf : 0.f;
+    uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+    bool ok = true;
+
+    // One tile, in its two parts (h): P is computed on the running maximum m, and its sum,
+    // which the row sum needs anyway, shows whether m still bounds the scores: a sum of at most
+    // 2^8 means that every P is.  Only a part that exceeds it (and the first of all, which has
+    // no m yet) finds the row's maximum, rescales O and l to it and is redone.
+    auto tile = [&](int t, auto masked) -> bool {
+      if (!__all_sync(0xffffffffu, pwait(&bars->sfull[g], (uint32_t)(t & 1), bars, p, 8))) return false;
+      fence_after();
+      uint32_t s[4][32];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) tmem_ld32(tS + 32 * c, s[c]);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) tmem_wait_ld_dep(s[c]);
+      if (C::kOwnP) {
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->sread[g]);
+      }
+      if (decltype(masked)::value) {
+        // the tile's columns this row sees: [lo, hi)
+        int lo = 0, hi = kBN;
+        if (active) {
+          const int t0 = tile_tok(t);
+          if (t < a_tiles) {
+            hi = (bs < 0 ? tok + 1 : S) - t0;
+          } else {
+            lo = bs < 0 ? kBN : bs - t0;
+            hi = tok + 1 - t0;
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const int col = 32 * c + i;
+            if (col < lo || col >= hi) s[c][i] = 0xff800000u;  // -inf
+          }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (C::kOwnP && h == 0 && t > 0) {
+          // P's own columns are free once P.V of tile t - 1 has completed
+          if (!__all_sync(0xffffffffu, pwait(&bars->pvdone[g], (uint32_t)((t - 1) & 1), bars, p, 9))) return false;
+          fence_after();
+        }
+        uint64_t sum[4];
+        if (h == 0) part_exp<0, kLoGroups>(s, sc2, m_run == kNegInf ? 0.f : m_run, tP, sum);
+        else part_exp<kLoGroups, 4>(s, sc2, m_run == kNegInf ? 0.f : m_run, tP, sum);
+        const uint64_t s2 = fadd2(fadd2(sum[0], sum[1]), fadd2(sum[2], sum[3]));
+        const bool grow = active && (m_run == kNegInf || f2lo(s2) + f2hi(s2) > kRescaleSum);
+        if (__any_sync(0xffffffffu, grow)) {
+          if (t > 0 || h == 1) {
+            // every P.V issued on O so far has completed: O may be rescaled
+            if (!__all_sync(0xffffffffu, h == 1 ? pwait(&bars->pvlo[g], (uint32_t)(t & 1), bars, p, 9)
+                                                : pwait(&bars->pvdone[g], (uint32_t)((t - 1) & 1), bars, p, 9)))
+              return false;
+            fence_after();
+          }
+          const float m_new = fmaxf(m_run, row_max(s) * sl2);
+          const bool need = grow && m_new > m_run;
+          const float alpha = need ? ex2(m_run - m_new) : 1.f;
+          if (t > 0 || h == 1) {
+#pragma unroll 1
+            for (int c = 0; c < D / 32; ++c) {
+              uint32_t r[32];
+              tmem_ld32(tO + 32 * c, r);
+              tmem_wait_ld_dep(r);
+#pragma unroll
+              for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
+              tmem_st32(tO + 32 * c, r);
+            }
+          }
+          const uint64_t al2 = f2pack(alpha, alpha);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) acc[u] = fmul2(acc[u], al2);
+          if (need) m_run = m_new;
+          // (a row that has seen no visible key keeps m = -inf; its exponent base is 0)
+          if (h == 0) part_exp<0, kLoGroups>(s, sc2, m_run == kNegInf ? 0.f : m_run, tP, sum);
+          else part_exp<kLoGroups, 4>(s, sc2, m_run == kNegInf ? 0.f : m_run, tP, sum);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] = fadd2(acc[u], sum[u]);
+        tmem_wait_st();
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(h ? &bars->phi[g] : &bars->plo[g]);
+      }
+      return true;
+    };
+    // the leading prefix tiles that every row of the warp sees in full need no mask
+    int lim = active ? (bs < 0 ? tok + 1 : S) : 0x7fffffff;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) lim = min(lim, __shfl_xor_sync(0xffffffffu, lim, o));
+    const int n_full = min(a_tiles, lim / kBN);
+    int t = 0;
+    for (; t < n_full && ok; ++t) ok = tile(t, std::false_type{});
+    for (; t < n_tiles && ok; ++t) ok = tile(t, std::true_type{});
+    // O is final once the last P.V has completed; the slot's Q is idle by then too (its last S
+    // completed before that P could be written)
+    if (ok) ok = pwait(&bars->pvdone[g], (uint32_t)((n_tiles - 1) & 1), bars, p, 10);
+    ok = __all_sync(0xffffffffu, ok);
+    if (ok) {
+      fence_after();
+      const uint64_t a2 = fadd2(fadd2(acc[0], acc[1]), fadd2(acc[2], acc[3]));
+      const float l = f2lo(a2) + f2hi(a2);
+      const float inv = 1.0f / l;
+      if (active && p.lse != nullptr)
+        p.lse[(int64_t)tok * p.h_q + kvh * G + row % G] = (m_run + log2f(l)) * 0.69314718055994531f;
+      // Rows out through this warp's 32 rows of the slot's Q stage (2 D bytes per row: all
+      // columns in bf16, half of them in fp32): row r's 16-byte chunk c at chunk position
+      // c ^ (r % chunks), so that both sides touch distinct banks; then coalesced rows.
+      constexpr int kCh = 2 * D / 16;           // chunks per staged row
+      uint8_t* stg = smem + (uint32_t)g * C::kTileBytes + (uint32_t)wrow * (2 * D);
+      const int passes = p.out_bf16 ? 1 : 2;
+      const int esz = p.out_bf16 ? 2 : 4;
+#pragma unroll 1
+      for (int ps = 0; ps < passes; ++ps) {
+        if (p.out_bf16) {
+#pragma unroll 1
+          for (int c = 0; c < D / 32; ++c) {
+            uint32_t r[32];
+            tmem_ld32(tO + 32 * c, r);
+            tmem_wait_ld_dep(r);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              uint32_t w[4];
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                w[u] = pack_bf16(__uint_as_float(r[8 * j + 2 * u]) * inv, __uint_as_float(r[8 * j + 2 * u + 1]) * inv);
+              *reinterpret_cast<uint4*>(stg + lane * (2 * D) + (((4 * c + j) ^ (lane & (kCh - 1))) << 4)) =
+                  make_uint4(w[0], w[1], w[2], w[3]);
+            }
+          }
+        } else {
+#pragma unroll 1
+          for (int c = 0; c < D / 64; ++c) {
+            uint32_t r[32];
+            tmem_ld32(tO + (D / 2) * ps + 32 * c, r);
+            tmem_wait_ld_dep(r);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              uint32_t w[4];
+#pragma unroll
+              for (int u = 0; u < 4; ++u) w[u] = __float_as_uint(__uint_as_float(r[4 * j + u]) * inv);
+              *reinterpret_cast<uint4*>(stg + lane * (2 * D) + (((8 * c + j) ^ (lane & (kCh - 1))) << 4)) =
+                  make_uint4(w[0], w[1], w[2], w[3]);
+            }
+          }
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int i = lane; i < 32 * kCh; i += 32) {
+          const int r = i / kCh, c = i % kCh;
+          const int rr = wrow + r, rt = rr / G, rtok = tok0 + g * p.tps + rt;
+          if (rt < p.tps && rtok < N) {
+            const uint4 v = *reinterpret_cast<const uint4*>(stg + r * (2 * D) + ((c ^ (r & (kCh - 1))) << 4));
+            const int64_t o = ((int64_t)rtok * p.h_q + kvh * G + (rr - rt * G)) * D * esz + (int64_t)ps * (2 * D) + 16 * c;
+            *reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.out) + o) = v;
+          }
+        }
+        __syncwarp();
+      }
+    }
+    fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&bars->tdone);
+  }
+}
+
+PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
+  static const PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
+    void* ptr = nullptr;
+    cudaDriverEntryPointQueryResult qres;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000, cudaEnableDefault, &qres) != cudaSuccess ||
+        qres != cudaDriverEntryPointSuccess)
+      ptr = nullptr;
+    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
+  }();
+  return fn;
+}
+
+// Token-major [tokens, heads, D] bf16 as a 3-D tensor (d, head, token); one box is 64 columns
+// x box_heads x box_tokens with the 128-byte swizzle.
+bool make_map(CUtensorMap* map, const void* base, int D, int heads, int64_t tokens, int box_heads, int box_tokens) {
+  auto enc = get_encode();
+  if (!enc) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)heads, (cuuint64_t)tokens};
+  cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)heads * D * 2};
+  cuuint32_t box[3] = {64, (cuuint32_t)box_heads, (cuuint32_t)box_tokens};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int D>
+cudaError_t launch(const PrefillTcParams& p, const void* q, const void* k, const void* v, cudaStream_t s) {
+  CUtensorMap mq, mk, mv;
+  if (!make_map(&mq, q, D, p.h_q, p.n_tokens, p.group, p.tps) || !make_map(&mk, k, D, p.h_kv, p.n_tokens, 1, kBN) ||
+      !make_map(&mv, v, D, p.h_kv, p.n_tokens, 1, kBN))
+    return cudaErrorInvalidValue;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  static bool configured[64] = {};
+  if (dev >= 0 && dev < 64 && !configured[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(prefill_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)Cfg<D>::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    configured[dev] = true;
+  }
+  const int64_t n_qt = ((int64_t)p.n_tokens + 2 * p.tps - 1) / (2 * p.tps);
+  if (n_qt * p.h_kv > INT32_MAX) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n_qt * p.h_kv));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = Cfg<D>::kSmemBytes;
+  cfg.stream = s;
+  return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D>, p, mq, mk, mv);
+}
+
+}  // namespace
+
+// Device status word of the whole-sequence prefill (no plan or workspace is involved).
+__device__ PadDevHeader g_prefill_header;
+
+cudaError_t prefill_header(PadDevHeader** out) {
+  static PadDevHeader* ptr[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!ptr[dev]) {
+    void* a = nullptr;
+    e = cudaGetSymbolAddress(&a, g_prefill_header);
+    if (e != cudaSuccess) return e;
+    ptr[dev] = static_cast<PadDevHeader*>(a);
+  }
+  *out = ptr[dev];
+  return cudaSuccess;
+}
+
+cudaError_t launch_prefill_tc(int32_t n_tokens, int32_t prefix_len, int32_t n_branches, const int32_t* branch_len,
+                              int32_t h_q, int32_t h_kv, int32_t head_dim, float scale, int32_t out_bf16, uint64_t gen,
+                              const void* q, const void* k, const void* v, void* out, float* lse, cudaStream_t s) {
+  const int G = h_q / h_kv;
+  if (G < 1 || G > 128 || n_tokens <= 0 || n_branches < 0 || n_branches > kMaxBranches) return cudaErrorInvalidValue;
+  PrefillTcParams p;
+  p.n_tokens = n_tokens;
+  p.prefix_len = prefix_len;
+  p.n_branches = n_branches;
+  p.h_q = h_q;
+  p.h_kv = h_kv;
+  p.group = G;
+  p.tps = 128 / G;
+  p.scale_log2 = (float)((double)scale * 1.4426950408889634);
+  p.out_bf16 = out_bf16;
+  p.gen = gen;
+  cudaError_t e = prefill_header(&p.header);
+  if (e != cudaSuccess) return e;
+  p.out = out;
+  p.lse = lse;
+  p.bstart[0] = prefix_len;
+  for (int b = 0; b < n_branches; ++b) p.bstart[b + 1] = p.bstart[b] + branch_len[b];
+  if (head_dim == 128) return launch<128>(p, q, k, v, s);
+  if (head_dim == 64) return launch<64>(p, q, k, v, s);
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace pad

@@ -16,12 +16,9 @@
 //   warp 2      TMEM allocator (512 columns) and deallocator; its lane 0 issues
 //               O += P V with P read back from TMEM
 //   warp 3      TMA producer of V tiles (refilled once the P.V of the tile completed)
-//   warps 4-11  softmax: two warps per 32-row lane quarter.  Decode: each warp takes 16
+//   warps 4-11  softmax: two warps per 32-row lane quarter, each with 16
 //               of the quarter's rows and all 128 columns of a tile (two rows per
-//               thread, a row shared by a quad of lanes), so the warps never meet.
-//               Whole-sequence prefill: each takes 64 of the columns for one row per
-//               thread, and the two meet once per tile to combine their partial row
-//               maxima (an mbarrier, so the wait is bounded).  Online max and sum in
+//               thread, a row shared by a quad of lanes), so the warps never meet.  Online max and sum in
 //               base 2, P written as packed bf16 over the S columns already read, lazy
 //               rescaling of O (only when a row maximum grows by more than 2^8)
 //
@@ -76,10 +73,7 @@ constexpr uint32_t kOffQ = 0;
 constexpr uint32_t kOffK = kOffQ + kQTileBytes;
 constexpr uint32_t kOffV = kOffK + kStages * kTileBytes;
 constexpr uint32_t kOffBar = kOffV + kStages * kTileBytes;
-constexpr uint32_t kOffX = kOffBar + 256;               // prefill: partial row maxima [2][2][128] fp32
-constexpr uint32_t kSmemBytes = kOffX + 2 * 2 * 128 * 4;
-constexpr int kOStage = kD + 4;                       // fp32 row stride of the O staging rows
-static_assert((128 * kOStage + 128) * 4 <= kStages * kTileBytes, "O staging (and 1 / l) fits the K stages");
+constexpr uint32_t kSmemBytes = kOffBar + 256;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColO = 384;
 constexpr float kLazyRescale = 8.0f;                  // log2 units
@@ -95,7 +89,6 @@ struct TcBars {
   uint64_t drain_pv;          // every P.V MMA has completed (P.V issuer)
   uint64_t qready;            // Q staged in shared memory (8 warp arrivals)
   uint64_t tdone;             // the softmax warps are done with TMEM (8 warp arrivals)
-  uint64_t xchg[4];           // prefill: the two softmax warps of a lane quarter met (64 arrivals)
   uint64_t gen;               // the plan's generation, for the status word
   uint32_t tmem_base;
   int32_t abort;
@@ -104,72 +97,6 @@ static_assert(sizeof(TcBars) <= 256, "barrier block fits its slot");
 
 constexpr uint32_t kIdescS = make_idesc(128, kBN, false);   // S = Q K^T: B = K tile, K-major
 constexpr uint32_t kIdescPV = make_idesc(128, kD, true);    // O += P V: B = V tile, N(=d)-major
-
-// The prefill path splits a 128-row group by columns: the two warps of a lane quarter take
-// 64 columns each of its 32 rows (one row per thread) and meet on every tile to share their
-// row maxima; one causal mask per thread keeps it below the register limit, where two rows'
-// masks per thread spilled.
-// Visible columns of a warp's 64 (used on the MASK path only): the set bits of `keep`.
-struct HalfBits {
-  uint64_t keep;
-  __device__ bool vis(int c) const { return (keep >> c) & 1ull; }
-};
-// Maximum of the raw scores of one softmax warp's 64 columns (eight chains of three-input
-// max); with MASK, columns the row does not see are left out.
-template <bool MASK, class Cols>
-__device__ __forceinline__ float half_row_max(const uint32_t (&sr)[2][32], Cols cols) {
-  float mxa[8];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) mxa[u] = -__builtin_huge_valf();
-#pragma unroll
-  for (int c = 0; c < 2; ++c)
-#pragma unroll
-    for (int i = 0; i < 32; i += 2) {
-      float a = __uint_as_float(sr[c][i]), b = __uint_as_float(sr[c][i + 1]);
-      if (MASK) {
-        if (!cols.vis(32 * c + i)) a = -__builtin_huge_valf();
-        if (!cols.vis(32 * c + i + 1)) b = -__builtin_huge_valf();
-      }
-      const int u = (16 * c + i / 2) & 7;
-      mxa[u] = max3f(mxa[u], a, b);
-    }
-  return fmaxf(max3f(mxa[0], mxa[1], mxa[2]), max3f(max3f(mxa[3], mxa[4], mxa[5]), mxa[6], mxa[7]));
-}
-
-// P = 2^(s * scale_log2 - m) for one softmax warp's 64 columns, written as packed bf16
-// over the S columns already read; returns the fp32 sum of the P values.
-template <bool MASK, class Cols>
-__device__ __forceinline__ float half_row_exp(const uint32_t (&sr)[2][32], Cols cols, float sl2,
-                                              float m, uint32_t taddr_p);
-
-template <bool MASK, class Cols>
-__device__ __forceinline__ float half_row_exp(const uint32_t (&sr)[2][32], Cols cols, float sl2,
-                                              float m, uint32_t taddr_p) {
-  const uint64_t sc2 = f2pack(sl2, sl2), nm2 = f2pack(-m, -m);
-  uint64_t lacc[4] = {0ull, 0ull, 0ull, 0ull};
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    uint32_t pk[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const int col = 32 * c + 2 * i;
-      const uint64_t x =
-          ffma2(f2pack(__uint_as_float(sr[c][2 * i]), __uint_as_float(sr[c][2 * i + 1])), sc2, nm2);
-      float p0 = ex2(f2lo(x)), p1 = ex2(f2hi(x));
-      if (MASK) {
-        if (!cols.vis(col)) p0 = 0.f;
-        if (!cols.vis(col + 1)) p1 = 0.f;
-      }
-      lacc[i & 3] = fadd2(lacc[i & 3], f2pack(p0, p1));
-      pk[i] = pack_bf16(p0, p1);
-    }
-    // P of tokens 32c .. 32c+31 of this half, two per column
-    tmem_st16(taddr_p + 16 * c, pk);
-  }
-  const uint64_t ls = fadd2(fadd2(lacc[0], lacc[1]), fadd2(lacc[2], lacc[3]));
-  return f2lo(ls) + f2hi(ls);
-}
-
 
 // The softmax warps split a 128-row group by rows: warp w of lane quarter q takes the 16
 // rows 32q + 16h .. +15 (h = (w-4)/4) and every column of a tile, through the 16-lane TMEM
@@ -314,27 +241,7 @@ __device__ __forceinline__ bool tail_partials_ready(const KParams& p, const PadV
   return bm::SyncNamed{1}.all(good);
 }
 
-// Whole-sequence prefill (PREFILL): branch start of token p >= pf_S, from the branch
-// offsets carried in the parameters.
-__device__ __forceinline__ int pf_branch_start(const KParams& p, int t) {
-  const int32_t* bs = reinterpret_cast<const int32_t*>(p.img);
-  int lo = 0, hi = p.pf_nb - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (bs[mid] <= t) lo = mid; else hi = mid - 1;
-  }
-  return bs[lo];
-}
-// Bits c of [0, 64) with lo <= c < hi (clamped).
-__device__ __forceinline__ uint64_t range_bits(int lo, int hi) {
-  lo = max(lo, 0);
-  hi = min(hi, 64);
-  if (lo >= hi) return 0ull;
-  const uint64_t up = hi >= 64 ? ~0ull : ((1ull << hi) - 1ull);
-  return up & ~((1ull << lo) - 1ull);
-}
-
-template <bool ROPE, bool GSELF, bool PREFILL>
+template <bool ROPE, bool GSELF>
 __global__ void __launch_bounds__(kThreads, 1)
     prefix_tc_kernel(const __grid_constant__ KParams p, const __nv_bfloat16* __restrict__ q, const int n_groups,
                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
@@ -366,35 +273,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     item = blockIdx.x / n_groups;
     group = blockIdx.x - item * n_groups;
   }
-  PadWorkItem it;
-  // PREFILL: the CTA's query tokens [it.first_event, +n_events) of kv-head it.kvh (query
-  // tiles in descending order, so that the longest key ranges start first) see the keys
-  // [0, pf_a_end) of the prefix and [pf_b_lo, pf_b_end) of the branches
-  int pf_a_tiles = 0, pf_b_lo = 0, pf_a_end = 0, pf_last = 0;
-  if (PREFILL) {
-    const int n_qt = (p.pf_N + p.pf_tpc - 1) / p.pf_tpc;
-    const int qt = n_qt - 1 - (int)blockIdx.x / p.h_kv;
-    it.first_event = qt * p.pf_tpc;
-    it.n_events = min(p.pf_tpc, p.pf_N - it.first_event);
-    it.kvh = (int16_t)(blockIdx.x % p.h_kv);
-    it.split = 0;
-    it.tok0 = 0;
-    it.tok_begin = 0;
-    it.part_row0 = 0;
-    const int last = it.first_event + it.n_events - 1;
-    const int a_end = min(p.pf_S, last + 1);
-    pf_a_end = a_end;
-    pf_last = last;
-    pf_a_tiles = (a_end + kBN - 1) / kBN;
-    int b_tiles = 0;
-    if (last >= p.pf_S) {
-      pf_b_lo = pf_branch_start(p, max(it.first_event, p.pf_S));
-      b_tiles = (last + 1 - pf_b_lo + kBN - 1) / kBN;
-    }
-    it.tok_end = (pf_a_tiles + b_tiles) * kBN;  // tile count; columns are masked per tile
-  } else {
-    it = plan_items(p)[item];
-  }
+  const PadWorkItem it = plan_items(p)[item];
   const int R = it.n_events * p.group;
   const int row0 = group * 128;
   if (row0 >= R) return;  // uniform over the CTA, before any barrier or allocation
@@ -403,10 +282,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int kvh = it.kvh;
   const int tok0 = (int)it.tok0;
   // first token of K/V tile t
-  auto tile_tok = [&](int t) -> int {
-    if (PREFILL) return t < pf_a_tiles ? t * kBN : pf_b_lo + (t - pf_a_tiles) * kBN;
-    return tok0 + t * kBN;
-  };
+  auto tile_tok = [&](int t) -> int { return tok0 + t * kBN; };
 
   // The softmax warps load their Q rows now, so that the loads overlap barrier set-up
   // and TMEM allocation; they are stored to shared memory after the block barrier.
@@ -468,7 +344,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(&bars->drain_pv, 1);
     mbar_init(&bars->qready, 8);
     mbar_init(&bars->tdone, 8);
-    for (int qq = 0; qq < 4; ++qq) mbar_init(&bars->xchg[qq], 64);
     bars->abort = 0;
     bars->gen = p.gen;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -525,7 +400,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     __syncwarp();
-    if (!PREFILL && warp == 0 && !p.causal) prefetch_branch_tasks(p, q, kpool, vpool, lane);
+    if (warp == 0 && !p.causal) prefetch_branch_tasks(p, q, kpool, vpool, lane);
   } else if (warp == 1 || warp == 2) {
     // ------------------------------------------------------------ MMA issuers
     // Two threads feed the tensor pipe so that one's waits and commits overlap the
@@ -649,119 +524,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) mbar_arrive(&bars->qready);
     const float sl2 = p.scale_log2;
     bool ok = true;
-    // Prefill: O leaves through shared memory, its rows staged in the K stages (idle once
-    // every MMA has completed) at a padded stride, then normalised and written one 512-byte
-    // row per warp instruction.  (One row per thread stored straight to global memory would
-    // touch 32 lines per instruction; the decode layout stores straight, eight rows of 32
-    // contiguous bytes per instruction.)
-    float* ostage = reinterpret_cast<float*>(smem + kOffK);
-    float* inv_row = ostage + 128 * kOStage;  // PREFILL: 1 / l of each row for the write-out
-    if constexpr (PREFILL) {
-      // columns 64*half .. +63 of every tile, one query row per thread
-      const int row = lane_base + lane;
-      const int grow = row0 + row;
-      const bool warp_active = (row0 + lane_base) < R;  // same for both warps of the quarter
-      const uint32_t tl = tmem + ((uint32_t)lane_base << 16);
-      const uint32_t col0 = 64u * (uint32_t)half;
-      float* xmax = reinterpret_cast<float*>(smem + kOffX);  // [tile parity][half][row]
-      uint64_t* xbar = &bars->xchg[quarter];
-      float m_run = -__builtin_huge_valf(), l_run = 0.f;
-      uint32_t r[32];
-      // this row's token and the first token of its branch (-1 in the prefix)
-      int pf_p = 0, pf_bs = -1;
-      if (grow < R) {
-        pf_p = it.first_event + grow / p.group;
-        pf_bs = pf_p >= p.pf_S ? pf_branch_start(p, pf_p) : -1;
-      }
-      for (int j = 0; j < n_tiles; ++j) {
-        const uint32_t cS = 128u * (uint32_t)(j % kSBuf);
-        ok = mbar_wait(&bars->sfull[j % kSBuf], (uint32_t)((j / kSBuf) & 1), bars, p.header, 8);
-        ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld/st below are warp-collective
-        if (!ok) break;
-        fence_after();
-        if (warp_active) {
-          uint32_t sr[2][32];
-          tmem_ld32(tl + cS + col0, sr[0]);
-          tmem_ld32(tl + cS + col0 + 32, sr[1]);
-          tmem_wait_ld_dep(sr[0]);
-          tmem_wait_ld_dep(sr[1]);
-          // the tile's range end, then this row's rule: a prefix token sees keys up to
-          // itself, a branch token the prefix and its own branch up to itself
-          const int tb = tile_tok(j);
-          const int t0 = tb + (int)col0;
-          uint64_t keep = range_bits(0, min(kBN, (j < pf_a_tiles ? pf_a_end : pf_last + 1) - tb) - (int)col0);
-          if (grow < R)
-            keep &= pf_bs < 0 ? range_bits(0, pf_p - t0 + 1)
-                              : (range_bits(0, p.pf_S - t0) | range_bits(pf_bs - t0, pf_p - t0 + 1));
-          const bool masked = __any_sync(0xffffffffu, keep != ~0ull);
-          const float pmax = masked ? half_row_max<true>(sr, HalfBits{keep}) : half_row_max<false>(sr, HalfBits{keep});
-          // meet the other half: this also orders both warps' S reads before either
-          // writes P over columns the other one read
-          xmax[(j & 1) * 256 + half * 128 + row] = pmax;
-          mbar_arrive(xbar);
-          ok = mbar_wait(xbar, (uint32_t)(j & 1), bars, p.header, 12);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
-          const float mx = fmaxf(pmax, xmax[(j & 1) * 256 + (1 - half) * 128 + row]) * sl2;
-          const float m_new = fmaxf(m_run, mx);
-          const bool need = m_new > m_run + kLazyRescale;
-          if (__any_sync(0xffffffffu, need && j > 0)) {
-            // O must hold P.V of tile j-1 before it is rescaled (each half rescales its
-            // own 64 head-dim columns; both halves take the same decision per row)
-            ok = mbar_wait(&bars->pvfree[(j - 1) % kStages], (uint32_t)(((j - 1) / kStages) & 1), bars,
-                           p.header, 9);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            fence_after();
-            const float alpha = need ? ex2(m_run - m_new) : 1.f;
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-              tmem_ld32(tl + kColO + col0 + 32 * c, r);
-              tmem_wait_ld_dep(r);
-#pragma unroll
-              for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
-              tmem_st32(tl + kColO + col0 + 32 * c, r);
-            }
-            tmem_wait_st();
-            if (need) l_run *= alpha;
-          }
-          if (need) m_run = m_new;
-          l_run += masked ? half_row_exp<true>(sr, HalfBits{keep}, sl2, m_run, tl + cS + col0 / 2)
-                          : half_row_exp<false>(sr, HalfBits{keep}, sl2, m_run, tl + cS + col0 / 2);
-          tmem_wait_st();
-        }
-        fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->pfull[j % kSBuf]);
-      }
-      // the P.V issuer commits `drain_pv` after its last MMA: O is final once it lands
-      if (ok) ok = mbar_wait(&bars->drain_pv, 0u, bars, p.header, 10);
-      ok = __all_sync(0xffffffffu, ok);
-      if (ok && warp_active) {
-        fence_after();
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          tmem_ld32(tl + kColO + col0 + 32 * c, r);
-          tmem_wait_ld_dep(r);
-          float4* dst = reinterpret_cast<float4*>(ostage + row * kOStage + col0 + 32 * c);
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            dst[i] = make_float4(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]),
-                                 __uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3]));
-        }
-        // row sum = both halves' partial sums (slot n_tiles & 1 was last read two tiles ago)
-        xmax[(n_tiles & 1) * 256 + half * 128 + row] = l_run;
-        mbar_arrive(xbar);
-        ok = mbar_wait(xbar, (uint32_t)(n_tiles & 1), bars, p.header, 13);
-        if (ok && half == 0 && grow < R) {
-          // normalised output: 1 / l for the write-out below, the LSE now
-          const float l_tot = l_run + xmax[(n_tiles & 1) * 256 + 128 + row];
-          inv_row[row] = 1.0f / l_tot;
-          const int64_t orow = (int64_t)pf_p * p.h_q + kvh * p.group + grow % p.group;
-          if (p.pf_lse != nullptr) p.pf_lse[orow] = (m_run + log2f(l_tot)) * 0.69314718055994531f;
-        }
-      }
-    } else {
+    {
       // this warp's 16 rows (TMEM lanes), this thread's two of them and its first column of
       // every 8-column chunk
       const int wrow = lane_base + 16 * half;
@@ -892,25 +655,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
     if (lane == 0) mbar_arrive(&bars->tdone);
     // every softmax warp reaches this barrier exactly once (the loop above only breaks);
-    // it orders the staged rows (prefill) and the partial rows before the fused tail
-    if (PREFILL || p.fused) asm volatile("bar.sync 1, 256;" ::: "memory");
-    const int nrows = PREFILL ? min(128, R - row0) : 0;  // prefill: normalised rows out
-    for (int rr = warp - 4; rr < nrows; rr += 8) {
-      float4 v = *reinterpret_cast<const float4*>(ostage + rr * kOStage + 4 * lane);
-      const float inv = inv_row[rr];
-      v.x *= inv;
-      v.y *= inv;
-      v.z *= inv;
-      v.w *= inv;
-      const int gr = row0 + rr;
-      const size_t oi = ((size_t)(it.first_event + gr / p.group) * p.h_q + kvh * p.group + gr % p.group) * kD + 4 * lane;
-      if (p.out_bf16)
-        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.pf_out) + oi) =
-            make_uint2(bm::pack_bf16(v.x, v.y), bm::pack_bf16(v.z, v.w));
-      else
-        *reinterpret_cast<float4*>(static_cast<float*>(p.pf_out) + oi) = v;
-    }
-    if (!PREFILL && p.fused) {
+    // it orders the partial rows before the fused tail
+    if (p.fused) asm volatile("bar.sync 1, 256;" ::: "memory");
+    if (p.fused) {
       // ---------------------------------------------------------- fused a4 + a5
       // Publish this split's rows (every softmax thread's partial stores are ordered
       // before the counter by the barrier and the fence), then run this CTA's (event,
@@ -1046,8 +793,8 @@ cudaError_t launch_prefix_tc(const KParams& p, int max_rows, const void* q, cons
   if (!prefix_tensor_maps(kp, vp, p.h_kv, total_prefix_tokens, dev, &mk, &mv)) return cudaErrorInvalidValue;
   static bool configured[64] = {};
   if (dev >= 0 && dev < 64 && !configured[dev]) {
-    for (auto fn : {prefix_tc_kernel<false, false, false>, prefix_tc_kernel<true, false, false>,
-                    prefix_tc_kernel<false, true, false>, prefix_tc_kernel<true, true, false>}) {
+    for (auto fn : {prefix_tc_kernel<false, false>, prefix_tc_kernel<true, false>,
+                    prefix_tc_kernel<false, true>, prefix_tc_kernel<true, true>}) {
       cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
       if (e != cudaSuccess) return e;
     }
@@ -1066,80 +813,11 @@ cudaError_t launch_prefix_tc(const KParams& p, int max_rows, const void* q, cons
   cfg.numAttrs = 1;
   if (p.fused && bm::smem_bytes<kD>(p.branch_rows, p.group, p.tail_chunk) > kOffBar) return cudaErrorInvalidValue;
   auto fn = p.rope_cs != nullptr
-                ? (p.g_self ? prefix_tc_kernel<true, true, false> : prefix_tc_kernel<true, false, false>)
-                : (p.g_self ? prefix_tc_kernel<false, true, false> : prefix_tc_kernel<false, false, false>);
+                ? (p.g_self ? prefix_tc_kernel<true, true> : prefix_tc_kernel<true, false>)
+                : (p.g_self ? prefix_tc_kernel<false, true> : prefix_tc_kernel<false, false>);
   return cudaLaunchKernelEx(&cfg, fn, p, static_cast<const __nv_bfloat16*>(q), n_groups, mk, mv,
                             static_cast<const __nv_bfloat16*>(k_pool), static_cast<const __nv_bfloat16*>(v_pool),
                             out, lse);
-}
-
-// Device status word of the whole-sequence prefill (no plan or workspace is involved).
-__device__ PadDevHeader g_prefill_header;
-
-cudaError_t prefill_header(PadDevHeader** out) {
-  static PadDevHeader* ptr[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (!ptr[dev]) {
-    void* a = nullptr;
-    e = cudaGetSymbolAddress(&a, g_prefill_header);
-    if (e != cudaSuccess) return e;
-    ptr[dev] = static_cast<PadDevHeader*>(a);
-  }
-  *out = ptr[dev];
-  return cudaSuccess;
-}
-
-cudaError_t launch_prefill_tc(int32_t n_tokens, int32_t prefix_len, int32_t n_branches, const int32_t* branch_len,
-                              int32_t h_q, int32_t h_kv, float scale, int32_t out_bf16, uint64_t gen, const void* q,
-                              const void* k, const void* v, void* out, float* lse, cudaStream_t s) {
-  const int G = h_q / h_kv;
-  if (G < 1 || G > 128 || n_tokens <= 0) return cudaErrorInvalidValue;
-  if ((size_t)(n_branches + 1) * sizeof(int32_t) > sizeof(KParams::img)) return cudaErrorInvalidValue;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  CUtensorMap mk, mv;
-  if (!prefix_tensor_maps(k, v, h_kv, n_tokens, dev, &mk, &mv)) return cudaErrorInvalidValue;
-  static bool configured[64] = {};
-  if (dev >= 0 && dev < 64 && !configured[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(prefix_tc_kernel<false, false, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-    if (e != cudaSuccess) return e;
-    configured[dev] = true;
-  }
-  KParams p;
-  std::memset(&p, 0, offsetof(KParams, img));
-  p.h_q = h_q;
-  p.h_kv = h_kv;
-  p.group = G;
-  p.head_dim = kD;
-  p.out_bf16 = out_bf16;
-  p.scale_log2 = (float)((double)scale * 1.4426950408889634);
-  p.gen = gen;
-  cudaError_t e = prefill_header(&p.header);
-  if (e != cudaSuccess) return e;
-  p.pf_N = n_tokens;
-  p.pf_S = prefix_len;
-  p.pf_nb = n_branches;
-  p.pf_tpc = 128 / G;
-  p.pf_out = out;
-  p.pf_lse = lse;
-  int32_t* bs = reinterpret_cast<int32_t*>(p.img);
-  bs[0] = prefix_len;
-  for (int b = 0; b < n_branches; ++b) bs[b + 1] = bs[b] + branch_len[b];
-  const int n_qt = (n_tokens + p.pf_tpc - 1) / p.pf_tpc;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n_qt * h_kv);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmemBytes;
-  cfg.stream = s;
-  cfg.numAttrs = 0;
-  return cudaLaunchKernelEx(&cfg, prefix_tc_kernel<false, false, true>, p, static_cast<const __nv_bfloat16*>(q), 1,
-                            mk, mv, static_cast<const __nv_bfloat16*>(nullptr),
-                            static_cast<const __nv_bfloat16*>(nullptr), static_cast<void*>(nullptr),
-                            static_cast<float*>(nullptr));
 }
 
 }  // namespace pad

@@ -76,3 +76,52 @@ def test_prefill_tc_group_sizes_and_bf16():
     _run(500, [30, 2, 77], 8, 2, 128, seed=8)            # G = 4: 32 tokens per CTA
     _run(500, [30, 2, 77], 16, 1, 128, seed=9)           # G = 16: 8 tokens per CTA
     _run(500, [30, 2, 77], 28, 4, 128, seed=10, out_dtype=1)
+
+
+@pytest.mark.parametrize("D,h_q,h_kv,prefix,lens", [
+    (64, 14, 2, 36, [1]),                 # one query tile (36 tokens at G = 7) and one token over
+    (64, 14, 2, 127, [1, 127, 2]),        # key tiles one short of full, a branch across a tile edge
+    (64, 4, 1, 129, []),                  # a key tile of one token; tail slot with no rows
+    (64, 16, 1, 0, [1]),                  # one token in all
+    (64, 3, 3, 300, [60, 0, 200]),        # G = 1: 128 tokens per slot
+    (128, 3, 3, 300, [60, 0, 200]),
+    (128, 28, 4, 18, [17, 19, 36]),       # branches that begin and end inside a slot
+    (128, 32, 2, 640, [128] * 3),         # G = 16: 8 tokens per slot
+])
+@pytest.mark.parametrize("out_dtype", [0, 1])
+def test_prefill_tc_edges(D, h_q, h_kv, prefix, lens, out_dtype):
+    """Tile, slot and branch edges of the tensor-core kernel at both head sizes."""
+    _run(prefix, lens, h_q, h_kv, D, seed=prefix + D, out_dtype=out_dtype)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_prefill_warp_level_kernel_still_forced(D):
+    _run(200, [3, 17, 66], 8, 2, D, seed=D, flags=B.FLAG_PREFIX_MMA)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("at", [100, 130, 230, 255, 600])
+def test_prefill_growing_maximum(D, at):
+    """Scores that outgrow the running maximum by far more than 2^8 at one key, in the first or
+    the last part of a tile, so that O, l and the part's P are redone there.  The bar stays
+    the usual one: P's rounding (2^-9 per weight) enters as it does elsewhere."""
+    prefix, lens, h_q, h_kv = 700, [40, 50], 14, 2
+    qb, kb, vb = synth.prefill_inputs(at, prefix, lens, h_q, h_kv, D)
+    q, k = oracle.bf16_to_f64(qb), oracle.bf16_to_f64(kb)
+    q[:, :, 0] = 4.0                      # exact in bf16
+    k[:, :, 0] = 0.0
+    k[at, :, 0] = 32.0                    # score +128 / sqrt(D): 16 at D 64, 11.3 at D 128 (nats)
+    qb, kb = synth.f32_to_bf16_bits(q.astype(np.float32)), synth.f32_to_bf16_bits(k.astype(np.float32))
+    N = qb.shape[0]
+    out = torch.empty((N, h_q, D), device="cuda")
+    lse = torch.empty((N, h_q), device="cuda")
+    B.pad_prefill_attn(B.make_problem(h_q, h_kv, D, 16, 1.0 / math.sqrt(D)), prefix, lens, _dev(qb), _dev(kb),
+                       _dev(vb), out, lse)
+    torch.cuda.synchronize()
+    B.pad_prefill_status()
+    ro, rl = oracle.prefill_attention(oracle.bf16_to_f64(qb), oracle.bf16_to_f64(kb), oracle.bf16_to_f64(vb),
+                                      prefix, lens, 1.0 / math.sqrt(D))
+    go = out.cpu().numpy()
+    assert np.abs(go - ro).max() <= MAX_ABS
+    assert np.linalg.norm(go - ro) / np.linalg.norm(ro) <= REL_L2
+    assert np.abs(lse.cpu().numpy() - rl).max() <= LSE_ABS
