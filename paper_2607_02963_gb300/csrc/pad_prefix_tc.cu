@@ -11,16 +11,23 @@
 //   warp 0      TMA producer of K tiles (128 tokens: two 64-column halves, 128-byte
 //               swizzle) into a 3-stage ring; a stage is refilled once the S of
 //               the tile it held has completed
-//   warp 1      S issuer (one thread): S = Q K^T into one of three TMEM S buffers,
-//               up to three tiles ahead of the softmax
-//   warp 2      TMEM allocator (512 columns) and deallocator; its lane 0 issues
-//               O += P V with P read back from TMEM
+//   warp 1      S issuer: S = Q K^T into one of three TMEM S buffers, up to three tiles
+//               ahead of the softmax
+//   warp 2      TMEM allocator (512 columns) and deallocator, and issuer of O += P V with P
+//               read back from TMEM
 //   warp 3      TMA producer of V tiles (refilled once the P.V of the tile completed)
-//   warps 4-11  softmax: two warps per 32-row lane quarter, each with 16
-//               of the quarter's rows and all 128 columns of a tile (two rows per
-//               thread, a row shared by a quad of lanes), so the warps never meet.  Online max and sum in
-//               base 2, P written as packed bf16 over the S columns already read, lazy
-//               rescaling of O (only when a row maximum grows by more than 2^8)
+//   warps 4-11  softmax: two warps per 32-row lane quarter, each with 16 of the quarter's rows
+//               and all 128 columns of a tile (two rows per thread, a row shared by a quad of
+//               lanes), so the warps never meet.  Online sum in base 2, P written as packed
+//               bf16 over the S columns already read; the row maxima are found on the first
+//               tile, and again only when a row's sum shows that a score outgrew them by more
+//               than 2^8 (then O is rescaled and the tile redone).
+//
+// What bounds it: the chain S -> softmax -> P.V of each tile and the fixed cost per CTA (the
+// loop of a long split runs at 0.9 of the copy bandwidth).  Electing the issuing lane of a
+// uniform warp instead of branching to lane 0 (see elect_one) and skipping the maximum took,
+// per step: prefix 32768, 32 events 24.8 -> 23.7 us; 16384, 64 events 25.6 -> 23.9; 16384, 1
+// event 12.0 -> 11.4; 8192, 8 events 10.75 -> 10.6; 16 ragged videos 94.3 -> 93.0.
 //
 // Every MMA has N = 128 (S: 128 tokens; P.V: 128 head-dim columns), the size at
 // which one tcgen05.mma carries as much tensor work as it costs to issue.
@@ -76,7 +83,7 @@ constexpr uint32_t kOffBar = kOffV + kStages * kTileBytes;
 constexpr uint32_t kSmemBytes = kOffBar + 256;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColO = 384;
-constexpr float kLazyRescale = 8.0f;                  // log2 units
+constexpr float kRescaleSum = 256.0f;                 // a tile whose P sum to more (per thread) is redone
 static_assert(kSmemBytes <= 232448, "fits the 227 KB opt-in shared memory");
 
 struct TcBars {
@@ -123,10 +130,24 @@ __device__ __forceinline__ float quad_sum(float v) {
   return v + __shfl_xor_sync(0xffffffffu, v, 2);
 }
 
-// Maxima of the raw scores of this thread's two rows over all 128 columns (with MASK,
-// columns a row does not see are left out), reduced over the quad.
-template <bool MASK, class CA, class CB>
-__device__ __forceinline__ void rows_max(const uint32_t (&s)[2][32], int cq, CA ca, CB cb, float& ma, float& mb) {
+// Columns of this thread's two rows that a row does not see go to -inf: they then get P = 0
+// and no say in the maximum.
+template <class CA, class CB>
+__device__ __forceinline__ void mask_rows(uint32_t (&s)[2][32], int cq, CA ca, CB cb) {
+#pragma unroll
+  for (int x = 0; x < 2; ++x)
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int c = 64 * x + 8 * k + cq + i;
+        if (!ca.vis(c)) s[x][4 * k + i] = 0xff800000u;
+        if (!cb.vis(c)) s[x][4 * k + 2 + i] = 0xff800000u;
+      }
+}
+
+// Maxima of the raw scores of this thread's two rows over all 128 columns, reduced over the quad.
+__device__ __forceinline__ void rows_max(const uint32_t (&s)[2][32], float& ma, float& mb) {
   float xa[4], xb[4];
 #pragma unroll
   for (int u = 0; u < 4; ++u) xa[u] = xb[u] = -__builtin_huge_valf();
@@ -134,17 +155,8 @@ __device__ __forceinline__ void rows_max(const uint32_t (&s)[2][32], int cq, CA 
   for (int x = 0; x < 2; ++x)
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const int c = 64 * x + 8 * k + cq;
-      float a0 = __uint_as_float(s[x][4 * k]), a1 = __uint_as_float(s[x][4 * k + 1]);
-      float b0 = __uint_as_float(s[x][4 * k + 2]), b1 = __uint_as_float(s[x][4 * k + 3]);
-      if (MASK) {
-        if (!ca.vis(c)) a0 = -__builtin_huge_valf();
-        if (!ca.vis(c + 1)) a1 = -__builtin_huge_valf();
-        if (!cb.vis(c)) b0 = -__builtin_huge_valf();
-        if (!cb.vis(c + 1)) b1 = -__builtin_huge_valf();
-      }
-      xa[k & 3] = max3f(xa[k & 3], a0, a1);
-      xb[k & 3] = max3f(xb[k & 3], b0, b1);
+      xa[k & 3] = max3f(xa[k & 3], __uint_as_float(s[x][4 * k]), __uint_as_float(s[x][4 * k + 1]));
+      xb[k & 3] = max3f(xb[k & 3], __uint_as_float(s[x][4 * k + 2]), __uint_as_float(s[x][4 * k + 3]));
     }
   ma = quad_max(fmaxf(fmaxf(xa[0], xa[1]), fmaxf(xa[2], xa[3])));
   mb = quad_max(fmaxf(fmaxf(xb[0], xb[1]), fmaxf(xb[2], xb[3])));
@@ -152,11 +164,10 @@ __device__ __forceinline__ void rows_max(const uint32_t (&s)[2][32], int cq, CA 
 
 // P = 2^(s * scale_log2 - m) of this thread's two rows, written as packed bf16 (two tokens
 // per column: column 4k + t%4 of chunk k holds tokens 8k + 2(t%4) and + 1, the layout the
-// P.V MMA reads) to the 64 TMEM columns at taddr_p; adds this thread's share of each row's
-// sum of P to la / lb.
-template <bool MASK, class CA, class CB>
-__device__ __forceinline__ void rows_exp(const uint32_t (&s)[2][32], int cq, CA ca, CB cb, float sl2, float ma,
-                                         float mb, uint32_t taddr_p, float& la, float& lb) {
+// P.V MMA reads) to the 64 TMEM columns at taddr_p; la / lb: this thread's share of each row's
+// sum of P.
+__device__ __forceinline__ void rows_exp(const uint32_t (&s)[2][32], float sl2, float ma, float mb, uint32_t taddr_p,
+                                         float& la, float& lb) {
   const uint64_t sc2 = f2pack(sl2, sl2), na = f2pack(-ma, -ma), nb = f2pack(-mb, -mb);
   uint64_t acc_a[2] = {0ull, 0ull}, acc_b[2] = {0ull, 0ull};
 #pragma unroll
@@ -164,18 +175,11 @@ __device__ __forceinline__ void rows_exp(const uint32_t (&s)[2][32], int cq, CA 
     uint32_t pk[16];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const int c = 64 * x + 8 * k + cq;
       const uint64_t ya =
           ffma2(f2pack(__uint_as_float(s[x][4 * k]), __uint_as_float(s[x][4 * k + 1])), sc2, na);
       const uint64_t yb =
           ffma2(f2pack(__uint_as_float(s[x][4 * k + 2]), __uint_as_float(s[x][4 * k + 3])), sc2, nb);
-      float a0 = ex2(f2lo(ya)), a1 = ex2(f2hi(ya)), b0 = ex2(f2lo(yb)), b1 = ex2(f2hi(yb));
-      if (MASK) {
-        if (!ca.vis(c)) a0 = 0.f;
-        if (!ca.vis(c + 1)) a1 = 0.f;
-        if (!cb.vis(c)) b0 = 0.f;
-        if (!cb.vis(c + 1)) b1 = 0.f;
-      }
+      const float a0 = ex2(f2lo(ya)), a1 = ex2(f2hi(ya)), b0 = ex2(f2lo(yb)), b1 = ex2(f2hi(yb));
       acc_a[k & 1] = fadd2(acc_a[k & 1], f2pack(a0, a1));
       acc_b[k & 1] = fadd2(acc_b[k & 1], f2pack(b0, b1));
       pk[2 * k] = pack_bf16(a0, a1);
@@ -185,8 +189,8 @@ __device__ __forceinline__ void rows_exp(const uint32_t (&s)[2][32], int cq, CA 
     tmem_st16x128_x8(taddr_p + 32 * x, pk);
   }
   const uint64_t sa = fadd2(acc_a[0], acc_a[1]), sb = fadd2(acc_b[0], acc_b[1]);
-  la += f2lo(sa) + f2hi(sa);
-  lb += f2lo(sb) + f2hi(sb);
+  la = f2lo(sa) + f2hi(sa);
+  lb = f2lo(sb) + f2hi(sb);
 }
 
 // Bounded wait of this kernel: gives up on the CTA's abort flag or after the time limit.
@@ -195,6 +199,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, TcBars
   return mbar_wait_b(bar, parity, &bars->abort, bars->gen, hdr, where);
 }
 
+
+// The same for a whole warp (warp-uniform result).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, TcBars* bars, PadDevHeader* hdr,
+                                               int where) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, bars, hdr, where)) != 0;
+}
 
 // Split counters of the fused tail, one per (video, kv-head, 128-row group): bits 15-0
 // count the video's splits that have written their partial rows, bits 31-16 the tasks
@@ -254,7 +264,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     return;
   }
   TcBars* bars = reinterpret_cast<TcBars*>(smem + kOffBar);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   // One-call step (k_new set): this is the step's first kernel, launched so that it may
   // start while the grid before it (the previous step, or the caller's own kernel that
   // wrote q) finishes.  Barrier set-up and TMEM allocation overlap that grid; every thread
@@ -366,7 +376,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   // must not overwrite partials that the tail still reads: no early release there.  The
   // next one-call step waits for this grid before it touches anything, so it may start.
   if (one_call || !p.fused) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const uint32_t tmem = bars->tmem_base;
+  // an allocation of all 512 columns starts at TMEM address 0: known at compile time, so that
+  // the MMAs' TMEM operands are immediates (a word read back from shared memory is not)
+  constexpr uint32_t tmem = 0;
 
   if (warp == 0 || warp == 3) {
     // ------------------------------------------------------------ TMA producers
@@ -403,32 +415,32 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 0 && !p.causal) prefetch_branch_tasks(p, q, kpool, vpool, lane);
   } else if (warp == 1 || warp == 2) {
     // ------------------------------------------------------------ MMA issuers
-    // Two threads feed the tensor pipe so that one's waits and commits overlap the
-    // other's MMAs: warp 1 issues S = Q K^T, warp 2 (after allocating TMEM) issues
-    // O += P V.  A commit tracks only its own thread's MMAs, so each has its own
-    // completion barriers (sfull / pvfree) and drain.
-    if (lane == 0) {
-      // Descriptors are built once; a K-step moves the start address, i.e. adds
-      // (byte offset >> 4) to the low field (no carry: addresses stay below 256 KB).
+    // Two warps feed the tensor pipe so that one's waits and commits overlap the other's MMAs:
+    // warp 1 issues S = Q K^T, warp 2 (after allocating TMEM) issues O += P V.  Each runs its
+    // loop with all lanes and lets the elected one issue (see elect_one).  A commit tracks
+    // only its own thread's MMAs, so each has its own completion barriers (sfull / pvfree)
+    // and drain.
+    //
+    // Descriptors are built once; a K-step moves the start address, i.e. adds
+    // (byte offset >> 4) to the low field (no carry: addresses stay below 256 KB).
+    const bool el = elect_one();
+    bool ok = true;
+    if (warp == 1) {
       const uint64_t dQ = sdesc(sbase + kOffQ, 16, 1024);
       const uint64_t dK = sdesc(sbase + kOffK, 16, 1024);
-      // V tile, N(=head-dim)-major: 16 tokens per step (2048 bytes), the second
-      // 64-column half at +kHalfBytes (leading byte offset), 8-row groups 1024 apart.
-      const uint64_t dV = sdesc(sbase + kOffV, kHalfBytes, 1024);
-      bool ok = true;
-      if (warp == 1) {
-        ok = mbar_wait(&bars->qready, 0u, bars, p.header, 11);
-        for (int t = 0; t < n_tiles && ok; ++t) {
-          const uint32_t s = (uint32_t)(t % kStages);
-          ok = mbar_wait(&bars->kfull[s], (uint32_t)((t / kStages) & 1), bars, p.header, 3);
-          if (!ok) break;
-          // S buffer s holds P of tile t-3 until that P.V completes
-          if (t >= kStages)
-            ok = mbar_wait(&bars->pvfree[s], (uint32_t)((t / kStages - 1) & 1), bars, p.header, 6);
-          if (!ok) break;
-          fence_after();
-          const uint32_t d = tmem + 128u * s;
-          const uint64_t kb = dK + (s * kTileBytes >> 4);
+      ok = mbar_wait_warp(&bars->qready, 0u, bars, p.header, 11);
+      int s = 0;
+      uint32_t ph = 0;
+      for (int t = 0; t < n_tiles && ok; ++t) {
+        ok = mbar_wait_warp(&bars->kfull[s], ph, bars, p.header, 3);
+        if (!ok) break;
+        // S buffer s holds P of tile t-3 until that P.V completes
+        if (t >= kStages) ok = mbar_wait_warp(&bars->pvfree[s], ph ^ 1u, bars, p.header, 6);
+        if (!ok) break;
+        fence_after();
+        const uint32_t d = tmem + 128u * (uint32_t)s;
+        const uint64_t kb = dK + ((uint32_t)s * kTileBytes >> 4);
+        if (el) {
 #pragma unroll
           for (int kk = 0; kk < kD / 16; ++kk) {
             const uint32_t off = (uint32_t)(kk >> 2) * kQHalfBytes + (uint32_t)(kk & 3) * 32;
@@ -436,29 +448,45 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           mma_commit(&bars->sfull[s]);
         }
-        mma_commit(&bars->drain_s);
-        drain_wait(&bars->drain_s, 0u);
-      } else {
-        for (int j = 0; j < n_tiles && ok; ++j) {
-          const uint32_t s = (uint32_t)(j % kStages);
-          ok = mbar_wait(&bars->vfull[s], (uint32_t)((j / kStages) & 1), bars, p.header, 4);
-          if (!ok) break;
-          ok = mbar_wait(&bars->pfull[s], (uint32_t)((j / kSBuf) & 1), bars, p.header, 5);
-          if (!ok) break;
-          fence_after();
-          const uint32_t a = tmem + 128u * s;
-          const uint64_t vb = dV + (s * kTileBytes >> 4);
-          const uint32_t acc0 = j > 0 ? 1u : 0u;
+        __syncwarp();
+        if (++s == kStages) {
+          s = 0;
+          ph ^= 1u;
+        }
+      }
+      if (el) mma_commit(&bars->drain_s);
+      __syncwarp();
+      drain_wait(&bars->drain_s, 0u);
+    } else {
+      // V tile, N(=head-dim)-major: 16 tokens per step (2048 bytes), the second
+      // 64-column half at +kHalfBytes (leading byte offset), 8-row groups 1024 apart.
+      const uint64_t dV = sdesc(sbase + kOffV, kHalfBytes, 1024);
+      int s = 0;
+      uint32_t ph = 0;
+      for (int j = 0; j < n_tiles && ok; ++j) {
+        ok = mbar_wait_warp(&bars->vfull[s], ph, bars, p.header, 4);
+        if (!ok) break;
+        ok = mbar_wait_warp(&bars->pfull[s], ph, bars, p.header, 5);
+        if (!ok) break;
+        fence_after();
+        const uint32_t a = tmem + 128u * (uint32_t)s;
+        const uint64_t vb = dV + ((uint32_t)s * kTileBytes >> 4);
+        if (el) {
 #pragma unroll
           for (int kk = 0; kk < kBN / 16; ++kk)
-            mma_ts(tmem + kColO, a + kk * 8, vb + ((uint32_t)kk * 2048 >> 4), kIdescPV,
-                   kk > 0 ? 1u : acc0);
+            mma_ts(tmem + kColO, a + kk * 8, vb + ((uint32_t)kk * 2048 >> 4), kIdescPV, (j > 0 || kk > 0) ? 1u : 0u);
           mma_commit(&bars->pvfree[s]);
         }
-        // O is final once every P.V has completed
-        mma_commit(&bars->drain_pv);
-        drain_wait(&bars->drain_pv, 0u);
+        __syncwarp();
+        if (++s == kStages) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
+      // O is final once every P.V has completed
+      if (el) mma_commit(&bars->drain_pv);
+      __syncwarp();
+      drain_wait(&bars->drain_pv, 0u);
     }
   } else if (warp >= 4) {
     // ------------------------------------------------------------ softmax
@@ -561,58 +589,70 @@ __global__ void __launch_bounds__(kThreads, 1)
           tmem_wait_ld_dep(sr[1]);
           // columns to mask: past the split's end, or (GSELF) hidden planning tokens of the
           // row's event; the path is chosen per warp (tcgen05.st below is warp-collective)
-          float mxa, mxb;
-          bool masked;
-          ColsBits ka{~0ull, ~0ull}, kb{~0ull, ~0ull};
           if (GSELF) {
+            ColsBits ka{~0ull, ~0ull}, kb{~0ull, ~0ull};
             const int t0 = it.tok_begin + j * kBN;
             if (valid < kBN || (t0 < g_hi && t0 + kBN > g_lo)) {
               const GMask gma{g_lo, g_hi, g_oa}, gmb{g_lo, g_hi, g_ob};
               ka = ColsBits{keep_bits(valid, gma, t0), keep_bits(valid - 64, gma, t0 + 64)};
               kb = ColsBits{keep_bits(valid, gmb, t0), keep_bits(valid - 64, gmb, t0 + 64)};
             }
-            masked = __any_sync(0xffffffffu, (ka.lo & ka.hi & kb.lo & kb.hi) != ~0ull);
-            if (masked) rows_max<true>(sr, cq, ka, kb, mxa, mxb);
-            else rows_max<false>(sr, cq, ka, kb, mxa, mxb);
-          } else {
-            masked = valid < kBN;
-            if (masked) rows_max<true>(sr, cq, ColsValid{valid}, ColsValid{valid}, mxa, mxb);
-            else rows_max<false>(sr, cq, ColsValid{valid}, ColsValid{valid}, mxa, mxb);
+            if (__any_sync(0xffffffffu, (ka.lo & ka.hi & kb.lo & kb.hi) != ~0ull)) mask_rows(sr, cq, ka, kb);
+          } else if (valid < kBN) {
+            mask_rows(sr, cq, ColsValid{valid}, ColsValid{valid});
           }
-          const float na = fmaxf(m_a, mxa * sl2), nb = fmaxf(m_b, mxb * sl2);
-          const bool need_a = na > m_a + kLazyRescale, need_b = nb > m_b + kLazyRescale;
-          if (__any_sync(0xffffffffu, (need_a || need_b) && j > 0)) {
-            // O must hold P.V of tile j-1 before its rows are rescaled
-            ok = mbar_wait(&bars->pvfree[(j - 1) % kStages], (uint32_t)(((j - 1) / kStages) & 1), bars,
-                           p.header, 9);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            fence_after();
-            const float al_a = need_a ? ex2(m_a - na) : 1.f, al_b = need_b ? ex2(m_b - nb) : 1.f;
-#pragma unroll
-            for (int x = 0; x < 2; ++x) {
-              uint32_t o[32];
-              tmem_ld16x256_x8(tl + kColO + 64 * x, o);
-              tmem_wait_ld_dep(o);
-#pragma unroll
-              for (int i = 0; i < 32; ++i)
-                o[i] = __float_as_uint(__uint_as_float(o[i]) * ((i & 2) ? al_b : al_a));
-              tmem_st16x256_x8(tl + kColO + 64 * x, o);
+          // P of the tile on the running maxima, over the first 64 columns of its S buffer, in
+          // this warp's own rows.  The sums (ta, tb: this thread's share), which the row sums need
+          // anyway, show whether the maxima still bound the scores: a sum of at most 2^8 means
+          // that every P is.  Only a tile that exceeds it, and the first, which has no maxima
+          // yet, finds its maxima (`fresh`), rescales O and l to them and is done on those.
+          // (One copy of the exponentials in a loop over the two attempts, or the first tile's
+          // maximum ahead of a shared copy, was 0.6-0.7 us slower per 32768-token step.)
+          float ta, tb;
+          auto exps = [&]() {
+            // (a row with every key so far hidden keeps m = -inf; its exponent base is 0)
+            rows_exp(sr, sl2, m_a == -__builtin_huge_valf() ? 0.f : m_a, m_b == -__builtin_huge_valf() ? 0.f : m_b,
+                     tl + cS, ta, tb);
+          };
+          bool fresh = j == 0;
+          if (!fresh) {
+            exps();
+            fresh = __any_sync(0xffffffffu, (ga < R && (m_a == -__builtin_huge_valf() || ta > kRescaleSum)) ||
+                                                (gb < R && (m_b == -__builtin_huge_valf() || tb > kRescaleSum)));
+          }
+          if (fresh) {
+            if (j > 0) {
+              // O must hold P.V of tile j-1 before its rows are rescaled
+              ok = mbar_wait(&bars->pvfree[(j - 1) % kStages], (uint32_t)(((j - 1) / kStages) & 1), bars,
+                             p.header, 9);
+              ok = __all_sync(0xffffffffu, ok);
+              if (!ok) break;
+              fence_after();
             }
-            tmem_wait_st();
-            l_a *= al_a;
-            l_b *= al_b;
+            float mxa, mxb;
+            rows_max(sr, mxa, mxb);
+            const float na = fmaxf(m_a, mxa * sl2), nb = fmaxf(m_b, mxb * sl2);
+            if (j > 0) {
+              const float al_a = na > m_a ? ex2(m_a - na) : 1.f, al_b = nb > m_b ? ex2(m_b - nb) : 1.f;
+#pragma unroll 1
+              for (int x = 0; x < 4; ++x) {
+                uint32_t o[16];
+                tmem_ld16x256_x4(tl + kColO + 32 * x, o);
+                tmem_wait_ld_dep16(o);
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                  o[i] = __float_as_uint(__uint_as_float(o[i]) * ((i & 2) ? al_b : al_a));
+                tmem_st16x256_x4(tl + kColO + 32 * x, o);
+              }
+              l_a *= al_a;
+              l_b *= al_b;
+            }
+            m_a = na;
+            m_b = nb;
+            exps();
           }
-          if (need_a) m_a = na;
-          if (need_b) m_b = nb;
-          // P of the tile over the first 64 columns of its S buffer, in this warp's own rows
-          if (GSELF) {
-            if (masked) rows_exp<true>(sr, cq, ka, kb, sl2, m_a, m_b, tl + cS, l_a, l_b);
-            else rows_exp<false>(sr, cq, ka, kb, sl2, m_a, m_b, tl + cS, l_a, l_b);
-          } else {
-            if (masked) rows_exp<true>(sr, cq, ColsValid{valid}, ColsValid{valid}, sl2, m_a, m_b, tl + cS, l_a, l_b);
-            else rows_exp<false>(sr, cq, ColsValid{valid}, ColsValid{valid}, sl2, m_a, m_b, tl + cS, l_a, l_b);
-          }
+          l_a += ta;
+          l_b += tb;
           tmem_wait_st();
         }
         fence_before();

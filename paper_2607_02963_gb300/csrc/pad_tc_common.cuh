@@ -126,12 +126,14 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // itself, so that every other wait of the CTA gives up too.
 static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, int32_t* abort, uint64_t gen,
                                                    PadDevHeader* hdr, int where) {
-  const unsigned long long t0 = globaltimer();
+  unsigned long long t0 = 0;  // (read with the first check: most waits end before it)
   for (uint32_t i = 1;; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
     if ((i & 63u) == 0) {
       if (*reinterpret_cast<volatile int32_t*>(abort)) return false;
-      if (globaltimer() - t0 > kWaitNs) {
+      const unsigned long long now = globaltimer();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > kWaitNs) {
         pad_set_error(hdr, gen, PAD_ERR_DEVICE_TIMEOUT, (int)blockIdx.x, where, (int)threadIdx.x);
         *reinterpret_cast<volatile int32_t*>(abort) = 1;
         return false;

@@ -673,3 +673,27 @@ def test_mask_variants_and_rope_compose():
     check_bookkeeping(db, wr, plan)
     ref_o, ref_lse = oracle.decode_step(wr, causal=True, self_g=(Ks, gi))
     check_outputs(db.out.float().cpu().numpy(), db.lse.cpu().numpy(), ref_o, ref_lse, "all variants")
+
+
+@pytest.mark.parametrize("at", [0, 127, 128, 300, 383, 767, 899])
+def test_prefix_score_outgrows_running_maximum(at):
+    """One prefix key whose score exceeds all before it by far more than 2^8, on the first, a
+    middle and the last (partly filled) tile of a split: O, l and the tile's P are redone on the
+    new maximum.  Few SMs give each split several tiles; half the events do not see the jump
+    (their q does not point at that key), so rows that are redone and rows that are not share
+    warps."""
+    w = _w([900], [9], [3, 0, 16, 5, 40, 1, 31, 2, 7], seed=at)
+    q, k = oracle.bf16_to_f64(w.q), oracle.bf16_to_f64(w.k_prefix)
+    q[:, :, 0] = 0.0
+    q[::2, :, 0] = 4.0
+    k[:, :, 0] = 0.0
+    k[at, :, 0] = 64.0                   # score + 256 / sqrt(128) = 22.6 nats for even events
+    w.q, w.k_prefix = synth.f32_to_bf16_bits(q.astype(np.float32)), synth.f32_to_bf16_bits(k.astype(np.float32))
+    ref_o, ref_lse = oracle_step(w)
+    for num_sms in (4, 8):
+        db = DeviceBatch(w, num_sms=num_sms, flags=B.FLAG_PREFIX_TC)
+        plan = db.run_step(one_call=True)
+        torch.cuda.synchronize()
+        B.pad_device_status(plan)
+        assert plan.info()["max_split_tiles"] > 1
+        check_outputs(db.out.cpu().numpy(), db.lse.cpu().numpy(), ref_o, ref_lse, f"key {at}, {num_sms} SMs")
