@@ -22,7 +22,7 @@
 //
 // What bounds it, and why it looks like this (sequence of 34.7 k tokens, 28/4 heads, D 128: 7.08
 // ms with one 128-row group per CTA, 5.36 ms = 1.60 PFLOP/s of visible pairs, 0.86 of cuBLAS's
-// rate, as it is; 8.7 k tokens, 14/2 heads, D 64: 724 us on the mma.sync kernel, 140 us here):
+// rate, as it is; 8.7 k tokens, 14/2 heads, D 64: 724 us on the mma.sync kernel, 203 us here):
 //   - Two slots share each K/V tile: with one 128-row group the MMAs' shared-memory operand
 //     reads (S: 8 KB per K = 16 step, P.V: 4 KB) and the 64 KB that a tile brings in exceed 128
 //     B per clock by a fifth; and one slot's softmax runs under the other's MMAs.
@@ -34,10 +34,14 @@
 //   - The issuer warps run their loops with all lanes and elect the issuing one (elect_one),
 //     and the TMEM addresses are immediates: 6.34 -> 6.02 ms.
 //
-// TMEM columns: S_0 at 0, S_1 at 128.  head_dim 128: O_0 at 256, O_1 at 384, and P_g goes over
-// the first half of S_g (all of a row's scores are in registers by then), so S_g(k + 1) waits
-// for P.V of tile k.  head_dim 64: P_0 at 256, P_1 at 320, O_0 at 384, O_1 at 448; S_g(k + 1)
-// only waits until the scores of tile k have been read.
+// TMEM columns: S_0 at 0, S_1 at 128, O_g at 256 + D g.  P_g goes over S_g (all of a row's
+// scores are in registers by then), so S_g(k + 1) waits for P.V of tile k.
+//
+// head_dim 64 holds P as the sum of two bf16 numbers (columns 0-63 and 64-127 of S_g), each with
+// its own P.V: one bf16 on the lazily followed maximum was 5-7 % less exact than the mma.sync
+// kernel's, which follows it every 64 keys (relative error of the fp32 output against 64 bits
+// 1.24e-3 to 1.40e-3 against 1.18e-3 to 1.32e-3; 140 us for the call above).  Two give 2e-6 to
+// 4e-6.
 //
 // Barrier phases: every barrier is per slot or per stage, so that the completion a thread
 // waits for by parity cannot be overtaken by the next one before the thread moves on.  Every
@@ -65,9 +69,6 @@ constexpr int kThreads = 384;
 constexpr int kLoGroups = 3;          // 32-key groups of a tile whose P is released first
 constexpr float kRescaleSum = 256.0f; // a part of a row whose P sum to more is redone on a new maximum
 constexpr float kNegInf = -__builtin_huge_valf();
-// Registers per thread after setmaxnreg: the launch gives 384 x 168 = 64512, and
-// 128 x 80 + 256 x 208 = 63488.
-constexpr int kRegsIssue = 80, kRegsSoftmax = 208;
 
 template <int D>
 struct Cfg {
@@ -80,9 +81,11 @@ struct Cfg {
   static constexpr uint32_t kOffV = kOffK + kKS * kTileBytes;
   static constexpr uint32_t kOffBar = kOffV + kVS * kTileBytes;
   static constexpr uint32_t kSmemBytes = kOffBar + 512;
-  static constexpr bool kOwnP = D == 64;                      // P has TMEM columns of its own
-  static constexpr uint32_t kColP = 256;                      // + 64 g   (kOwnP)
-  static constexpr uint32_t kColO = D == 128 ? 256 : 384;     // + D g
+  static constexpr bool kSplitP = D == 64;                    // P as two bf16 numbers
+  static constexpr uint32_t kColO = 256;                      // + D g
+  // Registers per thread after setmaxnreg: the launch gives 384 x 168 = 64512; 128 x 80 + 256 x
+  // 208 = 63488, and 128 x 56 + 256 x 224 = 64512 where the softmax keeps both parts of P.
+  static constexpr int kRegsIssue = kSplitP ? 56 : 80, kRegsSoftmax = kSplitP ? 224 : 208;
   static constexpr uint32_t kIdescS = make_idesc(128, kBN, false);  // B = K tile, K-major
   static constexpr uint32_t kIdescPV = make_idesc(128, D, true);    // B = V tile, N(=d)-major
   static_assert(kSmemBytes <= 232448, "fits the 227 KB opt-in shared memory");
@@ -105,7 +108,6 @@ struct Bars {
   uint64_t vfull[4], vfree[4];
   uint64_t qfull[2];
   uint64_t sfull[2];          // S of the slot's current tile has completed
-  uint64_t sread[2];          // its scores have been read (4 warp arrivals; kOwnP)
   uint64_t plo[2], phi[2];    // P of its first 32 kLoGroups keys / of the rest is written (4 warp arrivals)
   uint64_t pvlo[2];           // P.V of its first part has completed
   uint64_t pvdone[2];         // its P.V has completed
@@ -166,7 +168,8 @@ __device__ __forceinline__ float row_max(const uint32_t (&s)[4][32]) {
 
 // P = 2^(s * sl2 - m) of the 32-score groups [C0, C1) of a row, written as packed bf16 (two
 // keys per column) to TMEM columns taddr + 16 C0 ..; returns their fp32 sums as four pairs.
-template <int C0, int C1>
+// SPLIT: what the rounding leaves of P goes, rounded to bf16 too, 64 columns further on.
+template <int C0, int C1, bool SPLIT>
 __device__ __forceinline__ void part_exp(const uint32_t (&s)[4][32], uint64_t sc2, float m, uint32_t taddr,
                                          uint64_t (&sum)[4]) {
   const uint64_t nm2 = f2pack(-m, -m);
@@ -174,15 +177,37 @@ __device__ __forceinline__ void part_exp(const uint32_t (&s)[4][32], uint64_t sc
   for (int u = 0; u < 4; ++u) sum[u] = 0ull;
 #pragma unroll
   for (int c = C0; c < C1; ++c) {
-    uint32_t pk[16];
+    if constexpr (SPLIT) {
+      // (half the columns at a time: both parts of all sixteen did not fit the registers)
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const uint64_t x = ffma2(f2pack(__uint_as_float(s[c][2 * i]), __uint_as_float(s[c][2 * i + 1])), sc2, nm2);
-      const float a = ex2(f2lo(x)), b = ex2(f2hi(x));
-      sum[i & 3] = fadd2(sum[i & 3], f2pack(a, b));
-      pk[i] = pack_bf16(a, b);
+      for (int q = 0; q < 2; ++q) {
+        uint32_t pk[8], rest[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int k = 2 * (8 * q + i);
+          const uint64_t x = ffma2(f2pack(__uint_as_float(s[c][k]), __uint_as_float(s[c][k + 1])), sc2, nm2);
+          const float a = ex2(f2lo(x)), b = ex2(f2hi(x));
+          const uint64_t e = f2pack(a, b);
+          sum[i & 3] = fadd2(sum[i & 3], e);
+          pk[i] = pack_bf16(a, b);
+          const uint64_t r = ffma2(f2pack(__uint_as_float(pk[i] << 16), __uint_as_float(pk[i] & 0xffff0000u)),
+                                   f2pack(-1.f, -1.f), e);
+          rest[i] = pack_bf16(f2lo(r), f2hi(r));
+        }
+        tmem_st8(taddr + 16 * c + 8 * q, pk);
+        tmem_st8(taddr + 64 + 16 * c + 8 * q, rest);
+      }
+    } else {
+      uint32_t pk[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const uint64_t x = ffma2(f2pack(__uint_as_float(s[c][2 * i]), __uint_as_float(s[c][2 * i + 1])), sc2, nm2);
+        const float a = ex2(f2lo(x)), b = ex2(f2hi(x));
+        sum[i & 3] = fadd2(sum[i & 3], f2pack(a, b));
+        pk[i] = pack_bf16(a, b);
+      }
+      tmem_st16(taddr + 16 * c, pk);
     }
-    tmem_st16(taddr + 16 * c, pk);
   }
 }
 
@@ -233,7 +258,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int g = 0; g < 2; ++g) {
       mbar_init(&bars->qfull[g], 1);
       mbar_init(&bars->sfull[g], 1);
-      mbar_init(&bars->sread[g], 4);
       mbar_init(&bars->plo[g], 4);
       mbar_init(&bars->phi[g], 4);
       mbar_init(&bars->pvlo[g], 1);
@@ -271,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr uint32_t tmem = 0;
 
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsIssue));
     bool ok = true;
     if (warp == 0 || warp == 3) {
       // ------------------------------------------------------------ TMA producers
@@ -311,8 +335,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (!ok) break;
           if (t == 0)
             ok = pwait_warp(&bars->qfull[g], 0u, bars, p, 11);
-          else  // S_g is free: its scores are read (and, where P lies over them, P.V is done)
-            ok = pwait_warp(C::kOwnP ? &bars->sread[g] : &bars->pvdone[g], (uint32_t)((t - 1) & 1), bars, p, 6);
+          else  // S_g holds P of tile t - 1 until its P.V has completed
+            ok = pwait_warp(&bars->pvdone[g], (uint32_t)((t - 1) & 1), bars, p, 6);
           if (!ok) break;
           fence_after();
           const uint64_t qd = sdesc(sbase + (uint32_t)g * C::kTileBytes, 16, 1024);
@@ -348,7 +372,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint64_t vd = dV + ((uint32_t)s * C::kTileBytes >> 4);
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
-          const uint32_t a = tmem + (C::kOwnP ? C::kColP + 64u * g : 128u * g);
+          const uint32_t a = tmem + 128u * g;
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             if (ok) ok = pwait_warp(h ? &bars->phi[g] : &bars->plo[g], (uint32_t)(t & 1), bars, p, 5);
@@ -359,6 +383,12 @@ __global__ void __launch_bounds__(kThreads, 1)
               for (int kk = h ? 2 * kLoGroups : 0; kk < (h ? 8 : 2 * kLoGroups); ++kk)
                 mma_ts(tmem + C::kColO + (uint32_t)D * g, a + kk * 8, vd + ((uint32_t)kk * 2048 >> 4), C::kIdescPV,
                        (t > 0 || kk > 0) ? 1u : 0u);
+              if (C::kSplitP) {
+#pragma unroll
+                for (int kk = h ? 2 * kLoGroups : 0; kk < (h ? 8 : 2 * kLoGroups); ++kk)
+                  mma_ts(tmem + C::kColO + (uint32_t)D * g, a + 64 + kk * 8, vd + ((uint32_t)kk * 2048 >> 4),
+                         C::kIdescPV, 1u);
+              }
               if (h == 0) mma_commit(&bars->pvlo[g]);
               if (h == 1) {
                 mma_commit(&bars->pvdone[g]);
@@ -387,7 +417,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else {
     // ------------------------------------------------------------ softmax
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::kRegsSoftmax));
     const int g = (warp - 4) >> 2;             // slot
     const int wrow = 32 * (warp & 3);          // TMEM lanes wrow .. wrow + 31
     const int row = wrow + lane;               // row of the slot: token row / G, head row % G
@@ -396,7 +426,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const bool active = tl < p.tps && tok < N;
     const int bs = active && tok >= S ? branch_start(p, tok) : -1;
     const uint32_t tb = tmem + ((uint32_t)wrow << 16);
-    const uint32_t tS = tb + 128u * g, tP = C::kOwnP ? tb + C::kColP + 64u * g : tS;
+    const uint32_t tS = tb + 128u * g;
     const uint32_t tO = tb + C::kColO + (uint32_t)D * g;
     const float sl2 = p.scale_log2;
     const uint64_t sc2 = f2pack(sl2, sl2);
@@ -417,11 +447,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int c = 0; c < 4; ++c) tmem_ld32(tS + 32 * c, s[c]);
 #pragma unroll
       for (int c = 0; c < 4; ++c) tmem_wait_ld_dep(s[c]);
-      if (C::kOwnP) {
-        fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->sread[g]);
-      }
       if (decltype(masked)::value) {
         // the tile's columns this row sees: [lo, hi)
         int lo = 0, hi = kBN;
@@ -444,14 +469,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        if (C::kOwnP && h == 0 && t > 0) {
-          // P's own columns are free once P.V of tile t - 1 has completed
-          if (!__all_sync(0xffffffffu, pwait(&bars->pvdone[g], (uint32_t)((t - 1) & 1), bars, p, 9))) return false;
-          fence_after();
-        }
         uint64_t sum[4];
-        if (h == 0) part_exp<0, kLoGroups>(s, sc2, m_run == kNegInf ? 0.f : m_run, tP, sum);
-        else part_exp<kLoGroups, 4>(s, sc2, m_run == kNegInf ? 0.f : m_run, tP, sum);
+        if (h == 0) part_exp<0, kLoGroups, C::kSplitP>(s, sc2, m_run == kNegInf ? 0.f : m_run, tS, sum);
+        else part_exp<kLoGroups, 4, C::kSplitP>(s, sc2, m_run == kNegInf ? 0.f : m_run, tS, sum);
         const uint64_t s2 = fadd2(fadd2(sum[0], sum[1]), fadd2(sum[2], sum[3]));
         const bool grow = active && (m_run == kNegInf || f2lo(s2) + f2hi(s2) > kRescaleSum);
         if (__any_sync(0xffffffffu, grow)) {
@@ -481,8 +501,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int u = 0; u < 4; ++u) acc[u] = fmul2(acc[u], al2);
           if (need) m_run = m_new;
           // (a row that has seen no visible key keeps m = -inf; its exponent base is 0)
-          if (h == 0) part_exp<0, kLoGroups>(s, sc2, m_run == kNegInf ? 0.f : m_run, tP, sum);
-          else part_exp<kLoGroups, 4>(s, sc2, m_run == kNegInf ? 0.f : m_run, tP, sum);
+          if (h == 0) part_exp<0, kLoGroups, C::kSplitP>(s, sc2, m_run == kNegInf ? 0.f : m_run, tS, sum);
+          else part_exp<kLoGroups, 4, C::kSplitP>(s, sc2, m_run == kNegInf ? 0.f : m_run, tS, sum);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) acc[u] = fadd2(acc[u], sum[u]);

@@ -257,6 +257,11 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
       "r"(r[15])
       : "memory");
 }
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
 // 16-lane shapes (a warp's 16 lanes from the address's lane, which stays in its quarter).
 // 16x256b: thread t holds, for each repetition k (8 columns), lanes L + t/4 and L + 8 + t/4 at
 // columns C + 8k + 2(t%4) and + 1, in the order (row, c), (row, c+1), (row+8, c), (row+8, c+1).
