@@ -127,8 +127,14 @@ struct Layout {
   size_t off_ml = 0, off_o = 0, off_cnt = 0, total_bytes = 0;
 };
 
-pad_status compute_layout(const pad_problem* prob, int32_t n_videos, const int32_t* prefix_len,
-                          int32_t n_events, const int32_t* event_video, int n_sms, Layout* L) {
+// Device scratch inside the library for callers that have none to give (see
+// pad_event_decode_attn_static).
+constexpr size_t kStaticScratchBytes = 16u << 20;  // 16 MiB
+
+// The layout for one choice of the prefix kernel (kern; 0 = the rule below), with a split
+// length per video (per_video) or one for the batch.
+pad_status layout_for(const pad_problem* prob, int32_t n_videos, const int32_t* prefix_len, int32_t n_events,
+                      const int32_t* event_video, int n_sms, int kern, bool per_video, Layout* L) {
   if (n_videos < 0 || n_events < 0) return fail(PAD_ERR_INVALID_ARG, "negative batch size");
   if (n_videos > 0 && !prefix_len) return fail(PAD_ERR_INVALID_ARG, "prefix_len is NULL");
   if (n_events > 0 && !event_video) return fail(PAD_ERR_INVALID_ARG, "event_video is NULL");
@@ -160,9 +166,10 @@ pad_status compute_layout(const pad_problem* prob, int32_t n_videos, const int32
   }
   L->max_rows = max_rows;
 
-  // Prefix kernel: forced by a flag, else the tensor-core path for head_dim 128 and the
-  // warp-level paths for head_dim 64 (mma.sync above 8 rows, warp-shuffle below).
-  int kern = prob->flags & kPrefixFlags;
+  // Prefix kernel: forced by a flag, else the caller's choice, else the tensor-core path for
+  // head_dim 128 and the warp-level paths for head_dim 64 (mma.sync above 8 rows, warp-shuffle
+  // below).
+  if (prob->flags & kPrefixFlags) kern = prob->flags & kPrefixFlags;
   if (kern == 0) {
     if (prob->head_dim == 128)
       kern = PAD_FLAG_PREFIX_TC;
@@ -172,7 +179,7 @@ pad_status compute_layout(const pad_problem* prob, int32_t n_videos, const int32
   if (kern == PAD_FLAG_PREFIX_SIMT && max_rows > 16)
     return fail(PAD_ERR_UNSUPPORTED, "SIMT prefix path takes at most 16 rows per (video, kv-head); got %d",
                 max_rows);
-  if ((kern == PAD_FLAG_PREFIX_TC || kern == PAD_FLAG_PREFIX_DUAL) && prob->head_dim != 128)
+  if ((prob->flags & (PAD_FLAG_PREFIX_TC | PAD_FLAG_PREFIX_DUAL)) && prob->head_dim != 128)
     return fail(PAD_ERR_UNSUPPORTED, "tcgen05 prefix path takes head_dim 128; got %d", prob->head_dim);
   L->prefix_kernel = kern;
 
@@ -246,7 +253,7 @@ pad_status compute_layout(const pad_problem* prob, int32_t n_videos, const int32
   // The decision depends only on the batch's shape, so the last one is reused.
   L->vsplit.assign(n_videos, chunk);
   L->longest_first = false;
-  if ((kern == PAD_FLAG_PREFIX_TC || kern == PAD_FLAG_PREFIX_DUAL) && !want_fused && n_videos > 1) {
+  if ((kern == PAD_FLAG_PREFIX_TC || kern == PAD_FLAG_PREFIX_DUAL) && !want_fused && n_videos > 1 && per_video) {
     constexpr double kTileUs = 0.85, kCtaUs = 4.0;
     std::vector<int64_t> tiles(n_videos, 0), units(n_videos, 0);
     int64_t base_ctas = 0;
@@ -261,7 +268,7 @@ pad_status compute_layout(const pad_problem* prob, int32_t n_videos, const int32
     key.reserve(2 * (size_t)n_videos + 3);
     key.push_back(target);
     key.push_back(chunk);
-    key.push_back(prob->flags);
+    key.push_back(kern);
     for (int b = 0; b < n_videos; ++b) {
       key.push_back(tiles[b]);
       key.push_back(units[b]);
@@ -451,6 +458,32 @@ pad_status compute_layout(const pad_problem* prob, int32_t n_videos, const int32
   off = align_up(off + (size_t)L->n_counters * sizeof(unsigned int), 256);
   L->total_bytes = off;
   return PAD_OK;
+}
+
+// head_dim 64 without a forced kernel (or the fused tail, which that head size does not have):
+// a plan on a workspace takes the tensor-core kernel.  It is the faster one at every size
+// measured, from 4 rows over 512 tokens (6.3 us per step against 14 on mma.sync and 20 on warp
+// shuffles) to 128 rows over 16384 tokens x 8 kv-heads (14.9 against 44) and 16 ragged videos
+// (38 against 113).  A plan without a workspace runs in the static array, where the scratch of
+// up to three waves of splits could exceed what the warp-level kernels need: it keeps those.
+// So does a plan on a workspace that would no longer fit that array (its calls may go there
+// too), after one split length for all videos has been tried.
+pad_status compute_layout(const pad_problem* prob, int32_t n_videos, const int32_t* prefix_len, int32_t n_events,
+                          const int32_t* event_video, int n_sms, bool on_workspace, Layout* L) {
+  auto attempt = [&](int kern, bool per_video) {
+    *L = Layout();
+    return layout_for(prob, n_videos, prefix_len, n_events, event_video, n_sms, kern, per_video, L);
+  };
+  pad_status st = attempt(0, true);
+  if (st != PAD_OK || !on_workspace || prob->head_dim != 64 || (prob->flags & (kPrefixFlags | PAD_FLAG_FUSED_MERGE)) ||
+      L->max_rows > 64 * 128)  // (the CTA list holds a row group in six bits)
+    return st;
+  const bool fits = L->total_bytes <= kStaticScratchBytes;
+  for (bool per_video : {true, false}) {
+    st = attempt(PAD_FLAG_PREFIX_TC, per_video);
+    if (st == PAD_OK && (!fits || L->total_bytes <= kStaticScratchBytes)) return st;
+  }
+  return attempt(0, true);
 }
 
 // Plan images in pinned, device-mapped host memory.  The kernels read a plan's video and
@@ -698,7 +731,7 @@ size_t pad_workspace_size(const pad_problem* prob, int32_t n_videos, const int32
   if (check_problem(prob) != PAD_OK) return 0;
   Layout L;
   const int sms = prob->num_sms > 0 ? prob->num_sms : query_num_sms();
-  if (compute_layout(prob, n_videos, prefix_len, n_events, event_video, sms, &L) != PAD_OK) return 0;
+  if (compute_layout(prob, n_videos, prefix_len, n_events, event_video, sms, true, &L) != PAD_OK) return 0;
   return L.total_bytes;
 }
 
@@ -723,7 +756,7 @@ pad_status pad_plan(const pad_problem* prob, pad_cache_state* cache, int32_t n_v
   const int sms = prob->num_sms > 0 ? prob->num_sms : (workspace ? query_num_sms() : kDefaultSms);
   auto* plan = new pad_plan_t();
   Layout& L = plan->lay;
-  st = compute_layout(prob, n_videos, prefix_len, n_events, event_video, sms, &L);
+  st = compute_layout(prob, n_videos, prefix_len, n_events, event_video, sms, workspace != nullptr, &L);
   if (st != PAD_OK) {
     delete plan;
     return st;
@@ -1635,7 +1668,6 @@ pad_status pad_timing_read(float* total_ms, int32_t* n_launches) {
 // ---------------------------------------------------------------------------
 namespace {
 
-constexpr size_t kStaticScratchBytes = 16u << 20;  // 16 MiB
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 
 std::mutex g_static_mu;

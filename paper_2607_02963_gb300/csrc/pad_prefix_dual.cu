@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       __syncwarp();
-      if (!p.causal) prefetch_branch_tasks(p, q, kpool, vpool, lane);
+      if (!p.causal) prefetch_branch_tasks<kD>(p, q, kpool, vpool, lane);
     } else if (warp == 1 || warp == 2) {
       // ------------------------------------------------------------ MMA issuers
       // Two threads feed the tensor pipe, so that one's waits do not hold back the other's
@@ -704,7 +704,7 @@ cudaError_t launch_prefix_dual(const KParams& p, int max_rows, const void* q, co
   int dev = 0;
   cudaGetDevice(&dev);
   CUtensorMap mk, mv;
-  if (!prefix_tensor_maps(kp, vp, p.h_kv, total_prefix_tokens, dev, &mk, &mv)) return cudaErrorInvalidValue;
+  if (!prefix_tensor_maps(kp, vp, kD, p.h_kv, total_prefix_tokens, dev, &mk, &mv)) return cudaErrorInvalidValue;
   static bool configured[64] = {};
   if (dev >= 0 && dev < 64 && !configured[dev]) {
     for (auto fn : {prefix_dual_kernel<false, false>, prefix_dual_kernel<true, false>, prefix_dual_kernel<false, true>,

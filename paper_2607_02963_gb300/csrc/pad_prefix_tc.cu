@@ -29,6 +29,11 @@
 // per step: prefix 32768, 32 events 24.8 -> 23.7 us; 16384, 64 events 25.6 -> 23.9; 16384, 1
 // event 12.0 -> 11.4; 8192, 8 events 10.75 -> 10.6; 16 ragged videos 94.3 -> 93.0.
 //
+// head_dim 64 (one 64-column box per tile, P.V with N = 64) takes the same pipeline: 14/2 heads,
+// prefix 16384, 16 events 24.0 us per step on the mma.sync kernel, 9.7 here; 4/1 heads, 512
+// tokens, 4 events 14.3 -> 6.2 (latency: programmatic dependent launch and the one-call order
+// come with this path).
+//
 // Every MMA has N = 128 (S: 128 tokens; P.V: 128 head-dim columns), the size at
 // which one tcgen05.mma carries as much tensor work as it costs to issue.
 // TMEM columns: S[b] at 128*b (b = 0, 1, 2), O at 384.  Output: the partial
@@ -67,24 +72,33 @@ namespace {
 
 using namespace tc;
 
-constexpr int kD = 128;
 constexpr int kBN = 128;       // prefix tokens per K/V tile
 constexpr int kStages = 3;
 constexpr int kSBuf = 3;       // S buffers in TMEM
 constexpr int kThreads = 384;
 constexpr uint32_t kHalfBytes = kBN * 128;         // 128 tokens x 64 bf16 = 16 KB
-constexpr uint32_t kTileBytes = 2 * kHalfBytes;    // one K (or V) tile: 32 KB
 constexpr uint32_t kQHalfBytes = 128 * 128;        // 128 rows x 64 bf16 = 16 KB
-constexpr uint32_t kQTileBytes = 2 * kQHalfBytes;  // Q of one 128-row group: 32 KB
-constexpr uint32_t kOffQ = 0;
-constexpr uint32_t kOffK = kOffQ + kQTileBytes;
-constexpr uint32_t kOffV = kOffK + kStages * kTileBytes;
-constexpr uint32_t kOffBar = kOffV + kStages * kTileBytes;
-constexpr uint32_t kSmemBytes = kOffBar + 256;
+template <int D>
+struct Cfg {
+  static constexpr int kHalves = D / 64;                        // 64-column boxes of a row
+  static constexpr uint32_t kTileBytes = kHalves * kHalfBytes;  // one K (or V) tile
+  static constexpr uint32_t kOffQ = 0;                          // Q of the 128-row group
+  static constexpr uint32_t kOffK = kHalves * kQHalfBytes;
+  static constexpr uint32_t kOffV = kOffK + kStages * kTileBytes;
+  static constexpr uint32_t kOffBar = kOffV + kStages * kTileBytes;
+  static constexpr uint32_t kSmemBytes = kOffBar + 256;
+  // head_dim 64: P as the sum of two bf16 numbers, each with its own P.V.  The warp-level
+  // kernels of this head size hold P in 32 bits (up to 8 rows) or in bf16 on maxima of 64 tokens;
+  // one bf16 on the lazily followed maxima here is less exact than either (relative error of
+  // the output 1.6e-3 against 4.5e-5 and 1.4e-3), two are as exact as the former.
+  static constexpr bool kSplitP = D == 64;
+  static constexpr uint32_t kIdescS = make_idesc(128, kBN, false);  // S = Q K^T: B = K tile, K-major
+  static constexpr uint32_t kIdescPV = make_idesc(128, D, true);    // O += P V: B = V tile, N(=d)-major
+  static_assert(kSmemBytes <= 232448, "fits the 227 KB opt-in shared memory");
+};
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColO = 384;
 constexpr float kRescaleSum = 256.0f;                 // a tile whose P sum to more (per thread) is redone
-static_assert(kSmemBytes <= 232448, "fits the 227 KB opt-in shared memory");
 
 struct TcBars {
   uint64_t kfull[kStages];
@@ -101,9 +115,6 @@ struct TcBars {
   int32_t abort;
 };
 static_assert(sizeof(TcBars) <= 256, "barrier block fits its slot");
-
-constexpr uint32_t kIdescS = make_idesc(128, kBN, false);   // S = Q K^T: B = K tile, K-major
-constexpr uint32_t kIdescPV = make_idesc(128, kD, true);    // O += P V: B = V tile, N(=d)-major
 
 // The softmax warps split a 128-row group by rows: warp w of lane quarter q takes the 16
 // rows 32q + 16h .. +15 (h = (w-4)/4) and every column of a tile, through the 16-lane TMEM
@@ -166,13 +177,15 @@ __device__ __forceinline__ void rows_max(const uint32_t (&s)[2][32], float& ma, 
 // per column: column 4k + t%4 of chunk k holds tokens 8k + 2(t%4) and + 1, the layout the
 // P.V MMA reads) to the 64 TMEM columns at taddr_p; la / lb: this thread's share of each row's
 // sum of P.
+// SPLIT: what the rounding to bf16 leaves of P goes, rounded to bf16 too, to the next 64 columns.
+template <bool SPLIT>
 __device__ __forceinline__ void rows_exp(const uint32_t (&s)[2][32], float sl2, float ma, float mb, uint32_t taddr_p,
                                          float& la, float& lb) {
   const uint64_t sc2 = f2pack(sl2, sl2), na = f2pack(-ma, -ma), nb = f2pack(-mb, -mb);
   uint64_t acc_a[2] = {0ull, 0ull}, acc_b[2] = {0ull, 0ull};
 #pragma unroll
   for (int x = 0; x < 2; ++x) {
-    uint32_t pk[16];
+    uint32_t pk[16], rest[16];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const uint64_t ya =
@@ -184,9 +197,15 @@ __device__ __forceinline__ void rows_exp(const uint32_t (&s)[2][32], float sl2, 
       acc_b[k & 1] = fadd2(acc_b[k & 1], f2pack(b0, b1));
       pk[2 * k] = pack_bf16(a0, a1);
       pk[2 * k + 1] = pack_bf16(b0, b1);
+      if (SPLIT) {
+        rest[2 * k] = pack_bf16(a0 - __uint_as_float(pk[2 * k] << 16), a1 - __uint_as_float(pk[2 * k] & 0xffff0000u));
+        rest[2 * k + 1] =
+            pack_bf16(b0 - __uint_as_float(pk[2 * k + 1] << 16), b1 - __uint_as_float(pk[2 * k + 1] & 0xffff0000u));
+      }
     }
     // P columns 32x + 4k + t%4 (tokens 64x + 8k + 2(t%4), + 1)
     tmem_st16x128_x8(taddr_p + 32 * x, pk);
+    if (SPLIT) tmem_st16x128_x8(taddr_p + 64 + 32 * x, rest);
   }
   const uint64_t sa = fadd2(acc_a[0], acc_a[1]), sb = fadd2(acc_b[0], acc_b[1]);
   la = f2lo(sa) + f2hi(sa);
@@ -251,27 +270,26 @@ __device__ __forceinline__ bool tail_partials_ready(const KParams& p, const PadV
   return bm::SyncNamed{1}.all(good);
 }
 
-template <bool ROPE, bool GSELF>
+template <int D, bool ROPE, bool GSELF>
 __global__ void __launch_bounds__(kThreads, 1)
     prefix_tc_kernel(const __grid_constant__ KParams p, const __nv_bfloat16* __restrict__ q, const int n_groups,
                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                      const __nv_bfloat16* __restrict__ kpool, const __nv_bfloat16* __restrict__ vpool,
                      void* __restrict__ out, float* __restrict__ lse) {
+  using C = Cfg<D>;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
   if (sbase & 1023u) {  // the 128-byte swizzle atoms need 1024-byte alignment (never expected)
     if (threadIdx.x == 0) pad_set_error(p.header, p.gen, PAD_ERR_UNSUPPORTED, (int)blockIdx.x, (int)sbase, 0);
     return;
   }
-  TcBars* bars = reinterpret_cast<TcBars*>(smem + kOffBar);
+  TcBars* bars = reinterpret_cast<TcBars*>(smem + C::kOffBar);
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-  // One-call step (k_new set): this is the step's first kernel, launched so that it may
-  // start while the grid before it (the previous step, or the caller's own kernel that
-  // wrote q) finishes.  Barrier set-up and TMEM allocation overlap that grid; every thread
-  // that touches global memory waits for it first (the Q loads, the first TMA issue),
-  // and the block barrier after them orders everything else, including the release of
-  // the grid behind this one.
-  const bool one_call = p.k_new != nullptr;
+  // Launched so that it may start while the grid before it (the previous step, this step's
+  // append, or the caller's own kernel that wrote q) finishes.  Barrier set-up, TMEM
+  // allocation and the first K/V tile overlap that grid; every thread that touches other
+  // global memory waits for it first (the Q loads), and the block barrier after them orders
+  // everything else, including the release of the grid behind this one.
 
   // the CTA's work item and 128-row group: from the plan's CTA list, or the dense grid
   int item, group;
@@ -291,27 +309,33 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int n_tiles = (ntok + kBN - 1) / kBN;
   const int kvh = it.kvh;
   const int tok0 = (int)it.tok0;
-  // first token of K/V tile t
-  auto tile_tok = [&](int t) -> int { return tok0 + t * kBN; };
+  auto load_tile = [&](const CUtensorMap* map, uint32_t off, int t, uint64_t* full) {
+    mbar_expect_tx(full, C::kTileBytes);
+#pragma unroll
+    for (int h = 0; h < C::kHalves; ++h)
+      tma_load_3d(sbase + off + h * kHalfBytes, map, 64 * h, kvh, tok0 + t * kBN, full);
+  };
 
   // The softmax warps load their Q rows now, so that the loads overlap barrier set-up
   // and TMEM allocation; they are stored to shared memory after the block barrier.
-  // Lane `lane` of warp w holds row 32*(w&3) + (lane+32i)/8, 16-byte chunk (lane+32i)%8
-  // of head-dim half (w-4)/4.  Rows past R are zero.
-  uint4 qv[8];
+  // Lane `lane` of warp w holds rows 32*(w&3) + (lane+32i)/8, 16-byte chunk (lane+32i)%8: of
+  // head-dim half (w-4)/4 for i = 0 .. 7 (head_dim 128), or of the one half there is for the
+  // four i from 4 ((w-4)/4) on (head_dim 64).  Rows past R are zero.
+  constexpr int kQi = 4 * C::kHalves;
+  uint4 qv[kQi];
   if (warp >= 4) {
-    if (one_call) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int lane_base = 32 * (warp & 3), half = (warp - 4) >> 2;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int idx = lane + 32 * i;
+    for (int i = 0; i < kQi; ++i) {
+      const int idx = lane + 32 * (D == 128 ? i : i + 4 * half);
       const int qrow = row0 + lane_base + (idx >> 3);
       qv[i] = make_uint4(0u, 0u, 0u, 0u);
       if (qrow < R) {
         const int el = qrow / p.group;
         const int gh = qrow - el * p.group;
-        const __nv_bfloat16* qr = q + ((size_t)(it.first_event + el) * p.h_q + kvh * p.group + gh) * kD;
-        const int d0 = half * 64 + (idx & 7) * 8;
+        const __nv_bfloat16* qr = q + ((size_t)(it.first_event + el) * p.h_q + kvh * p.group + gh) * D;
+        const int d0 = (D == 128 ? half * 64 : 0) + (idx & 7) * 8;
         qv[i] = __ldg(reinterpret_cast<const uint4*>(qr + d0));
       }
     }
@@ -331,14 +355,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmK)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
     if (n_tiles > 0) {
-      mbar_expect_tx(&bars->kfull[0], kTileBytes);
-      tma_load_3d(sbase + kOffK, &tmK, 0, kvh, tile_tok(0), &bars->kfull[0]);
-      tma_load_3d(sbase + kOffK + kHalfBytes, &tmK, 64, kvh, tile_tok(0), &bars->kfull[0]);
-      mbar_expect_tx(&bars->vfull[0], kTileBytes);
-      tma_load_3d(sbase + kOffV, &tmV, 0, kvh, tile_tok(0), &bars->vfull[0]);
-      tma_load_3d(sbase + kOffV + kHalfBytes, &tmV, 64, kvh, tile_tok(0), &bars->vfull[0]);
+      load_tile(&tmK, C::kOffK, 0, &bars->kfull[0]);
+      load_tile(&tmV, C::kOffV, 0, &bars->vfull[0]);
     }
-    if (one_call) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int s = 0; s < kStages; ++s) {
       if (s > 0) {
         mbar_init(&bars->kfull[s], 1);
@@ -375,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // the fused tail of a two-call step the next grid is the next step's append, which
   // must not overwrite partials that the tail still reads: no early release there.  The
   // next one-call step waits for this grid before it touches anything, so it may start.
-  if (one_call || !p.fused) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (p.k_new != nullptr || !p.fused) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // an allocation of all 512 columns starts at TMEM address 0: known at compile time, so that
   // the MMAs' TMEM operands are immediates (a word read back from shared memory is not)
   constexpr uint32_t tmem = 0;
@@ -397,10 +417,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (!ok) break;
         }
         uint64_t* full = isK ? &bars->kfull[s] : &bars->vfull[s];
-        mbar_expect_tx(full, kTileBytes);
-        const uint32_t dst = sbase + (isK ? kOffK : kOffV) + s * kTileBytes;
-        tma_load_3d(dst, map, 0, kvh, tile_tok(t), full);
-        tma_load_3d(dst + kHalfBytes, map, 64, kvh, tile_tok(t), full);
+        load_tile(map, (isK ? C::kOffK : C::kOffV) + s * C::kTileBytes, t, full);
         issued = t + 1;
       }
       if (!ok) {
@@ -412,7 +429,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     __syncwarp();
-    if (warp == 0 && !p.causal) prefetch_branch_tasks(p, q, kpool, vpool, lane);
+    if (warp == 0 && !p.causal) prefetch_branch_tasks<D>(p, q, kpool, vpool, lane);
   } else if (warp == 1 || warp == 2) {
     // ------------------------------------------------------------ MMA issuers
     // Two warps feed the tensor pipe so that one's waits and commits overlap the other's MMAs:
@@ -426,8 +443,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     const bool el = elect_one();
     bool ok = true;
     if (warp == 1) {
-      const uint64_t dQ = sdesc(sbase + kOffQ, 16, 1024);
-      const uint64_t dK = sdesc(sbase + kOffK, 16, 1024);
+      const uint64_t dQ = sdesc(sbase + C::kOffQ, 16, 1024);
+      const uint64_t dK = sdesc(sbase + C::kOffK, 16, 1024);
       ok = mbar_wait_warp(&bars->qready, 0u, bars, p.header, 11);
       int s = 0;
       uint32_t ph = 0;
@@ -439,12 +456,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!ok) break;
         fence_after();
         const uint32_t d = tmem + 128u * (uint32_t)s;
-        const uint64_t kb = dK + ((uint32_t)s * kTileBytes >> 4);
+        const uint64_t kb = dK + ((uint32_t)s * C::kTileBytes >> 4);
         if (el) {
 #pragma unroll
-          for (int kk = 0; kk < kD / 16; ++kk) {
+          for (int kk = 0; kk < D / 16; ++kk) {
             const uint32_t off = (uint32_t)(kk >> 2) * kQHalfBytes + (uint32_t)(kk & 3) * 32;
-            mma_ss(d, dQ + (off >> 4), kb + (off >> 4), kIdescS, kk > 0 ? 1u : 0u);
+            mma_ss(d, dQ + (off >> 4), kb + (off >> 4), C::kIdescS, kk > 0 ? 1u : 0u);
           }
           mma_commit(&bars->sfull[s]);
         }
@@ -460,7 +477,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else {
       // V tile, N(=head-dim)-major: 16 tokens per step (2048 bytes), the second
       // 64-column half at +kHalfBytes (leading byte offset), 8-row groups 1024 apart.
-      const uint64_t dV = sdesc(sbase + kOffV, kHalfBytes, 1024);
+      const uint64_t dV = sdesc(sbase + C::kOffV, kHalfBytes, 1024);
       int s = 0;
       uint32_t ph = 0;
       for (int j = 0; j < n_tiles && ok; ++j) {
@@ -470,11 +487,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!ok) break;
         fence_after();
         const uint32_t a = tmem + 128u * (uint32_t)s;
-        const uint64_t vb = dV + ((uint32_t)s * kTileBytes >> 4);
+        const uint64_t vb = dV + ((uint32_t)s * C::kTileBytes >> 4);
         if (el) {
 #pragma unroll
           for (int kk = 0; kk < kBN / 16; ++kk)
-            mma_ts(tmem + kColO, a + kk * 8, vb + ((uint32_t)kk * 2048 >> 4), kIdescPV, (j > 0 || kk > 0) ? 1u : 0u);
+            mma_ts(tmem + kColO, a + kk * 8, vb + ((uint32_t)kk * 2048 >> 4), C::kIdescPV, (j > 0 || kk > 0) ? 1u : 0u);
+          if (C::kSplitP) {
+#pragma unroll
+            for (int kk = 0; kk < kBN / 16; ++kk)
+              mma_ts(tmem + kColO, a + 64 + kk * 8, vb + ((uint32_t)kk * 2048 >> 4), C::kIdescPV, 1u);
+          }
           mma_commit(&bars->pvfree[s]);
         }
         __syncwarp();
@@ -496,38 +518,42 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Q rows (loaded in the prologue) into the 128-byte-swizzled K-major layout the
     // MMA reads: row r, 16-byte chunk cc of half h at h*16K + r*128 + ((cc ^ (r & 7)) << 4).
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int idx = lane + 32 * i;
+    for (int i = 0; i < kQi; ++i) {
+      const int idx = lane + 32 * (D == 128 ? i : i + 4 * half);
       const int r = lane_base + (idx >> 3), cc = idx & 7;
-      *reinterpret_cast<uint4*>(smem + kOffQ + half * kQHalfBytes + r * 128 + ((cc ^ (r & 7)) << 4)) = qv[i];
+      *reinterpret_cast<uint4*>(smem + C::kOffQ + (D == 128 ? half * kQHalfBytes : 0) + r * 128 + ((cc ^ (r & 7)) << 4)) =
+          qv[i];
     }
     if (ROPE) {
-      // Rotation in place: element d < 64 pairs with d + 64, i.e. chunk cc of half 0 with
-      // chunk cc of half 1 of the same row, which the other warp of this lane quarter
-      // stored.  The two warps meet (named barrier 2 + quarter) and split the quarter's
-      // 32 rows x 8 chunk pairs; every table row is fetched once all four are addressed.
+      // Rotation in place: element d < D/2 pairs with d + D/2.  At head_dim 128 that is chunk
+      // cc of half 0 with chunk cc of half 1 of the same row, at 64 chunk cc with chunk cc + 4;
+      // either way the other warp of this lane quarter may have stored it.  The two warps meet
+      // (named barrier 2 + quarter) and split the quarter's 32 rows x D / 16 chunk pairs;
+      // every table row is fetched once all are addressed.
       asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");
+      constexpr int kPairs = D / 16, kRi = 32 * kPairs / 64;
       const int t = half * 32 + lane;
-      const float* cs[4];
+      const float* cs[kRi];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = lane_base + ((t + 64 * i) >> 3);
+      for (int i = 0; i < kRi; ++i) {
+        const int r = lane_base + (t + 64 * i) / kPairs;
         cs[i] = row0 + r < R
-                    ? p.rope_cs + (size_t)plan_events(p)[it.first_event + (row0 + r) / p.group].pos * kD
+                    ? p.rope_cs + (size_t)plan_events(p)[it.first_event + (row0 + r) / p.group].pos * D
                     : nullptr;
       }
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < kRi; ++i) {
         if (cs[i] == nullptr) continue;
         const int k = t + 64 * i;
-        const int r = lane_base + (k >> 3), cc = k & 7;
-        uint4* lo = reinterpret_cast<uint4*>(smem + kOffQ + r * 128 + ((cc ^ (r & 7)) << 4));
-        uint4* hi = reinterpret_cast<uint4*>(smem + kOffQ + kQHalfBytes + r * 128 + ((cc ^ (r & 7)) << 4));
+        const int r = lane_base + k / kPairs, cc = k % kPairs;
+        const uint32_t hi_off = D == 128 ? kQHalfBytes + ((cc ^ (r & 7)) << 4) : (((cc + 4) ^ (r & 7)) << 4);
+        uint4* lo = reinterpret_cast<uint4*>(smem + C::kOffQ + r * 128 + ((cc ^ (r & 7)) << 4));
+        uint4* hi = reinterpret_cast<uint4*>(smem + C::kOffQ + r * 128 + hi_off);
         const uint4 a = *lo, b = *hi;
         const float4 c0 = *reinterpret_cast<const float4*>(cs[i] + 8 * cc);
         const float4 c1 = *reinterpret_cast<const float4*>(cs[i] + 8 * cc + 4);
-        const float4 s0 = *reinterpret_cast<const float4*>(cs[i] + 64 + 8 * cc);
-        const float4 s1 = *reinterpret_cast<const float4*>(cs[i] + 64 + 8 * cc + 4);
+        const float4 s0 = *reinterpret_cast<const float4*>(cs[i] + D / 2 + 8 * cc);
+        const float4 s1 = *reinterpret_cast<const float4*>(cs[i] + D / 2 + 8 * cc + 4);
         const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
         const float s[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
         const uint32_t av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
@@ -611,7 +637,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           float ta, tb;
           auto exps = [&]() {
             // (a row with every key so far hidden keeps m = -inf; its exponent base is 0)
-            rows_exp(sr, sl2, m_a == -__builtin_huge_valf() ? 0.f : m_a, m_b == -__builtin_huge_valf() ? 0.f : m_b,
+            rows_exp<C::kSplitP>(sr, sl2, m_a == -__builtin_huge_valf() ? 0.f : m_a, m_b == -__builtin_huge_valf() ? 0.f : m_b,
                      tl + cS, ta, tb);
           };
           bool fresh = j == 0;
@@ -635,7 +661,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (j > 0) {
               const float al_a = na > m_a ? ex2(m_a - na) : 1.f, al_b = nb > m_b ? ex2(m_b - nb) : 1.f;
 #pragma unroll 1
-              for (int x = 0; x < 4; ++x) {
+              for (int x = 0; x < D / 32; ++x) {
                 uint32_t o[16];
                 tmem_ld16x256_x4(tl + kColO + 32 * x, o);
                 tmem_wait_ld_dep16(o);
@@ -666,10 +692,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         fence_after();
         // O rows straight from the 16-lane layout: a quad writes 32 contiguous bytes of a
         // row, a warp instruction eight such segments
-        float* po_a = p.part_o + ((int64_t)it.part_row0 + ga) * kD;
-        float* po_b = po_a + 8 * kD;
+        float* po_a = p.part_o + ((int64_t)it.part_row0 + ga) * D;
+        float* po_b = po_a + 8 * D;
 #pragma unroll
-        for (int x = 0; x < 2; ++x) {
+        for (int x = 0; x < C::kHalves; ++x) {
           uint32_t o[32];
           tmem_ld16x256_x8(tl + kColO + 64 * x, o);
           tmem_wait_ld_dep(o);
@@ -696,8 +722,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) mbar_arrive(&bars->tdone);
     // every softmax warp reaches this barrier exactly once (the loop above only breaks);
     // it orders the partial rows before the fused tail
-    if (p.fused) asm volatile("bar.sync 1, 256;" ::: "memory");
-    if (p.fused) {
+    if (D == 128 && p.fused) asm volatile("bar.sync 1, 256;" ::: "memory");
+    if (D == 128 && p.fused) {  // (head_dim 64 plans have no fused tail)
       // ---------------------------------------------------------- fused a4 + a5
       // Publish this split's rows (every softmax thread's partial stores are ordered
       // before the counter by the barrier and the fence), then run this CTA's (event,
@@ -715,7 +741,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int task = plan_tasks(p)[blockIdx.x];
         if (task >= 0) {
           const int te = task / p.h_kv, th = task - (task / p.h_kv) * p.h_kv;
-          bm::run_task<kD, ROPE, 2>(p, q, kpool, vpool, out, lse, te, th, (int)threadIdx.x - 128, smem, p.tail_chunk, sy,
+          bm::run_task<D, ROPE, 2>(p, q, kpool, vpool, out, lse, te, th, (int)threadIdx.x - 128, smem, p.tail_chunk, sy,
                            false, [&]() {
                              const PadEventDesc ev = plan_events(p)[te];
                              const PadVideoDesc vd = plan_videos(p)[ev.video];
@@ -728,10 +754,6 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   __syncwarp();
   fence_before();
-  // This grid may run alongside the append kernel before it (it reads nothing that
-  // kernel writes); waiting for it here makes the completion of this grid imply the
-  // completion of the append, which the branch/merge pass after it relies on.
-  if (threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
   if (warp == 2) {
     // The block barrier above is not relied on to order the softmax warps' last TMEM
@@ -757,13 +779,13 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
   return fn;
 }
 
-// Token-major [T, h_kv, 128] bf16 prefix as a 3-D tensor (d, head, token); one box is
+// Token-major [T, h_kv, D] bf16 prefix as a 3-D tensor (d, head, token); one box is
 // 64 head-dim columns x 1 head x 128 tokens with the 128-byte swizzle.
-bool make_map(CUtensorMap* map, const void* base, int h_kv, int64_t tokens) {
+bool make_map(CUtensorMap* map, const void* base, int D, int h_kv, int64_t tokens) {
   auto enc = get_encode();
   if (!enc) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)kD, (cuuint64_t)h_kv, (cuuint64_t)tokens};
-  cuuint64_t strides[2] = {(cuuint64_t)kD * 2, (cuuint64_t)h_kv * kD * 2};
+  cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)h_kv, (cuuint64_t)tokens};
+  cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)h_kv * D * 2};
   cuuint32_t box[3] = {64, 1, (cuuint32_t)kBN};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides,
@@ -778,7 +800,7 @@ bool make_map(CUtensorMap* map, const void* base, int h_kv, int64_t tokens) {
 struct MapCacheEntry {
   const void* k;
   const void* v;
-  int h_kv;
+  int D, h_kv;
   int64_t tokens;
   int dev;
   CUtensorMap mk, mv;
@@ -789,12 +811,12 @@ int g_maps_n = 0, g_maps_next = 0;
 
 }  // namespace
 
-bool prefix_tensor_maps(const void* kp, const void* vp, int h_kv, int64_t tokens, int dev, CUtensorMap* mk,
+bool prefix_tensor_maps(const void* kp, const void* vp, int D, int h_kv, int64_t tokens, int dev, CUtensorMap* mk,
                         CUtensorMap* mv) {
   std::lock_guard<std::mutex> lk(g_map_mu);
   for (int i = 0; i < g_maps_n; ++i) {
     const MapCacheEntry& e = g_maps[i];
-    if (e.k == kp && e.v == vp && e.h_kv == h_kv && e.tokens == tokens && e.dev == dev) {
+    if (e.k == kp && e.v == vp && e.D == D && e.h_kv == h_kv && e.tokens == tokens && e.dev == dev) {
       std::memcpy(mk, &e.mk, sizeof(CUtensorMap));
       std::memcpy(mv, &e.mv, sizeof(CUtensorMap));
       return true;
@@ -803,10 +825,11 @@ bool prefix_tensor_maps(const void* kp, const void* vp, int h_kv, int64_t tokens
   MapCacheEntry ne;
   ne.k = kp;
   ne.v = vp;
+  ne.D = D;
   ne.h_kv = h_kv;
   ne.tokens = tokens;
   ne.dev = dev;
-  if (!make_map(&ne.mk, kp, h_kv, tokens) || !make_map(&ne.mv, vp, h_kv, tokens)) return false;
+  if (!make_map(&ne.mk, kp, D, h_kv, tokens) || !make_map(&ne.mv, vp, D, h_kv, tokens)) return false;
   g_maps[g_maps_next] = ne;
   g_maps_next = (g_maps_next + 1) % 8;
   if (g_maps_n < 8) ++g_maps_n;
@@ -817,25 +840,20 @@ bool prefix_tensor_maps(const void* kp, const void* vp, int h_kv, int64_t tokens
 
 int prefix_tc_tail_chunk(int branch_rows, int group, int max_splits) {
   int sch = std::min(bm::kMaxChunk, std::max(1, max_splits));
-  while (sch > 1 && bm::smem_bytes<kD>(branch_rows, group, sch) > kOffBar) --sch;
+  while (sch > 1 && bm::smem_bytes<128>(branch_rows, group, sch) > Cfg<128>::kOffBar) --sch;
   return sch;
 }
 
-cudaError_t launch_prefix_tc(const KParams& p, int max_rows, const void* q, const void* kp,
-                             const void* vp, int64_t total_prefix_tokens, const void* k_pool,
-                             const void* v_pool, void* out, float* lse, bool pdl, cudaStream_t s) {
-  if (p.n_items == 0) return cudaSuccess;
-  if (p.head_dim != kD || total_prefix_tokens <= 0 || total_prefix_tokens > (int64_t)INT32_MAX)
-    return cudaErrorInvalidValue;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  CUtensorMap mk, mv;
-  if (!prefix_tensor_maps(kp, vp, p.h_kv, total_prefix_tokens, dev, &mk, &mv)) return cudaErrorInvalidValue;
+template <int D>
+static cudaError_t launch_d(const KParams& p, int max_rows, const void* q, const CUtensorMap& mk, const CUtensorMap& mv,
+                            const void* k_pool, const void* v_pool, void* out, float* lse, bool pdl, int dev,
+                            cudaStream_t s) {
+  constexpr uint32_t smem = Cfg<D>::kSmemBytes;
   static bool configured[64] = {};
   if (dev >= 0 && dev < 64 && !configured[dev]) {
-    for (auto fn : {prefix_tc_kernel<false, false>, prefix_tc_kernel<true, false>,
-                    prefix_tc_kernel<false, true>, prefix_tc_kernel<true, true>}) {
-      cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    for (auto fn : {prefix_tc_kernel<D, false, false>, prefix_tc_kernel<D, true, false>,
+                    prefix_tc_kernel<D, false, true>, prefix_tc_kernel<D, true, true>}) {
+      cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
     }
     configured[dev] = true;
@@ -844,20 +862,34 @@ cudaError_t launch_prefix_tc(const KParams& p, int max_rows, const void* q, cons
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.cta_map ? p.n_ctas : p.n_items * n_groups);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (p.fused && bm::smem_bytes<kD>(p.branch_rows, p.group, p.tail_chunk) > kOffBar) return cudaErrorInvalidValue;
-  auto fn = p.rope_cs != nullptr
-                ? (p.g_self ? prefix_tc_kernel<true, true> : prefix_tc_kernel<true, false>)
-                : (p.g_self ? prefix_tc_kernel<false, true> : prefix_tc_kernel<false, false>);
+  if (p.fused && (D != 128 || bm::smem_bytes<D>(p.branch_rows, p.group, p.tail_chunk) > Cfg<D>::kOffBar))
+    return cudaErrorInvalidValue;
+  auto fn = p.rope_cs != nullptr ? (p.g_self ? prefix_tc_kernel<D, true, true> : prefix_tc_kernel<D, true, false>)
+                                 : (p.g_self ? prefix_tc_kernel<D, false, true> : prefix_tc_kernel<D, false, false>);
   return cudaLaunchKernelEx(&cfg, fn, p, static_cast<const __nv_bfloat16*>(q), n_groups, mk, mv,
                             static_cast<const __nv_bfloat16*>(k_pool), static_cast<const __nv_bfloat16*>(v_pool),
                             out, lse);
+}
+
+cudaError_t launch_prefix_tc(const KParams& p, int max_rows, const void* q, const void* kp,
+                             const void* vp, int64_t total_prefix_tokens, const void* k_pool,
+                             const void* v_pool, void* out, float* lse, bool pdl, cudaStream_t s) {
+  if (p.n_items == 0) return cudaSuccess;
+  if ((p.head_dim != 128 && p.head_dim != 64) || total_prefix_tokens <= 0 || total_prefix_tokens > (int64_t)INT32_MAX)
+    return cudaErrorInvalidValue;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  CUtensorMap mk, mv;
+  if (!prefix_tensor_maps(kp, vp, p.head_dim, p.h_kv, total_prefix_tokens, dev, &mk, &mv)) return cudaErrorInvalidValue;
+  return p.head_dim == 128 ? launch_d<128>(p, max_rows, q, mk, mv, k_pool, v_pool, out, lse, pdl, dev, s)
+                           : launch_d<64>(p, max_rows, q, mk, mv, k_pool, v_pool, out, lse, pdl, dev, s);
 }
 
 }  // namespace pad

@@ -340,10 +340,12 @@ __device__ __forceinline__ void prefetch_l2(const void* a) {
 // table, whose entries for those keys no kernel of this step writes), its Q rows and, in the
 // one-call step, its new K/V row.  Those tasks then start on warm lines instead of waiting
 // on HBM behind their page-table reads.  Page ids outside the pool are skipped.
+template <int D>
 __device__ __forceinline__ void prefetch_branch_tasks(const KParams& p, const __nv_bfloat16* q,
                                                    const __nv_bfloat16* kpool, const __nv_bfloat16* vpool,
                                                    int lane) {
   const int n_tasks = p.n_events * p.h_kv, G = p.group, ps = p.page_size;
+  constexpr int lines = D / 64;  // 128-byte lines of a row
   // one task per CTA at most: a warp that walked many tasks here would hold the CTA (and
   // the grid the branch/merge kernel waits for) open longer than the prefetch saves.  With
   // the fused tail, the task this CTA will run itself.
@@ -355,25 +357,26 @@ __device__ __forceinline__ void prefetch_branch_tasks(const KParams& p, const __
     for (int k = lane; k < len; k += 32) {
       const int pg = ptab[k / ps];
       if (pg < 0 || pg >= p.n_pages) continue;
-      const size_t off = (((size_t)pg * p.h_kv + h) * ps + (k % ps)) * 128;
-      prefetch_l2(kpool + off);
-      prefetch_l2(kpool + off + 64);
-      prefetch_l2(vpool + off);
-      prefetch_l2(vpool + off + 64);
+      const size_t off = (((size_t)pg * p.h_kv + h) * ps + (k % ps)) * D;
+#pragma unroll
+      for (int l = 0; l < lines; ++l) {
+        prefetch_l2(kpool + off + 64 * l);
+        prefetch_l2(vpool + off + 64 * l);
+      }
     }
-    if (lane < 2 * G) prefetch_l2(q + ((size_t)e * p.h_q + h * G + (lane >> 1)) * 128 + 64 * (lane & 1));
-    if (p.k_new != nullptr && lane < 4) {
-      const __nv_bfloat16* src = static_cast<const __nv_bfloat16*>(lane < 2 ? p.k_new : p.v_new);
-      prefetch_l2(src + ((size_t)e * p.h_kv + h) * 128 + 64 * (lane & 1));
+    if (lane < lines * G) prefetch_l2(q + ((size_t)e * p.h_q + h * G) * D + 64 * lane);
+    if (p.k_new != nullptr && lane < 2 * lines) {
+      const __nv_bfloat16* src = static_cast<const __nv_bfloat16*>(lane < lines ? p.k_new : p.v_new);
+      prefetch_l2(src + ((size_t)e * p.h_kv + h) * D + 64 * (lane % lines));
     }
   }
 }
 
 }  // namespace tc
 
-// Tensor maps of a token-major [tokens, h_kv, 128] bf16 K and V prefix (boxes of 64 head-dim
+// Tensor maps of a token-major [tokens, h_kv, D] bf16 K and V prefix (boxes of 64 head-dim
 // columns x 1 head x 128 tokens, 128-byte swizzle), cached per (buffers, shape, device).
-bool prefix_tensor_maps(const void* kp, const void* vp, int h_kv, int64_t tokens, int dev, CUtensorMap* mk,
+bool prefix_tensor_maps(const void* kp, const void* vp, int D, int h_kv, int64_t tokens, int dev, CUtensorMap* mk,
                         CUtensorMap* mv);
 
 }  // namespace pad

@@ -697,3 +697,65 @@ def test_prefix_score_outgrows_running_maximum(at):
         B.pad_device_status(plan)
         assert plan.info()["max_split_tiles"] > 1
         check_outputs(db.out.cpu().numpy(), db.lse.cpu().numpy(), ref_o, ref_lse, f"key {at}, {num_sms} SMs")
+
+
+# head_dim 64 on the tensor-core kernel: row-group, tile and page edges, several videos, every
+# option of the step
+_D64_TC_CASES = {
+    "one_row": dict(prefix=[130], epv=[1], lens=[0], h_q=1, h_kv=1),
+    "rows_17": dict(prefix=[512], epv=[17], lens=[0] * 17, h_q=1, h_kv=1),
+    "rows_127_129": dict(prefix=[700, 129], epv=[127, 129], lens=[1] * 256, h_q=2, h_kv=2),
+    "g7_tiles": dict(prefix=[3000], epv=[19], lens=list(range(19)), h_q=14, h_kv=2),
+    "ragged_videos": dict(prefix=[1, 128, 2, 1500], epv=[3, 5, 2, 20], lens=[16, 0, 31] * 10, h_q=16, h_kv=1),
+    "empty_video": dict(prefix=[400, 300], epv=[0, 6], lens=[15, 16, 17, 63, 64, 65], h_q=16, h_kv=4, page_size=32),
+}
+
+
+@pytest.mark.parametrize("one_call", [True, False])
+@pytest.mark.parametrize("option", ["plain", "rope", "self_g", "causal", "bf16"])
+@pytest.mark.parametrize("case", sorted(_D64_TC_CASES))
+def test_head_dim_64_on_tensor_cores(case, option, one_call):
+    c = dict(_D64_TC_CASES[case])
+    w = _w(c.pop("prefix"), c.pop("epv"), c.pop("lens"), D=64, seed=64, **c)
+    db = DeviceBatch(w, out_dtype=1 if option == "bf16" else 0)
+    ref, kw = w, {}
+    if option == "rope":
+        pos = synth.step_positions(w)
+        table = synth.rope_table(int(pos.max()) + 1, 64)
+        db.set_rope(pos, table)
+        ref = oracle.rotated_workload(w, pos, table)
+    elif option == "self_g":
+        db.self_g = _self_g_spec(w)
+        kw = dict(self_g=db.self_g)
+    elif option == "causal":
+        db.causal = True
+        kw = dict(causal=True)
+    plan = db.run_step(one_call=one_call)
+    torch.cuda.synchronize()
+    B.pad_device_status(plan)
+    assert plan.info()["prefix_kernel"] == B.FLAG_PREFIX_TC
+    check_bookkeeping(db, ref, plan)
+    ref_o, ref_lse = oracle.decode_step(ref, **kw)
+    got = db.out.float().cpu().numpy()
+    if option == "bf16":                 # the rounding alone contributes up to 2^-9
+        assert np.linalg.norm(got - ref_o) / np.linalg.norm(ref_o) <= REL_L2 + 2.0 ** -9
+    else:
+        check_outputs(got, db.lse.cpu().numpy(), ref_o, ref_lse, f"{case} {option}")
+
+
+def test_head_dim_64_forced_kernels_and_host_only_plans():
+    """Forced, with the fused tail's flag and without a workspace: the warp-level kernels."""
+    w = _w([900], [20], [3] * 20, h_q=4, h_kv=1, D=64)
+    for flags in (B.FLAG_PREFIX_MMA, B.FLAG_FUSED_MERGE):
+        _, plan = run_full(w, flags=flags)
+        assert plan.info()["prefix_kernel"] == B.FLAG_PREFIX_MMA
+    db = DeviceBatch(w)
+    plan = B.pad_plan(db.problem, db.cache, w.prefix_len, w.event_video, w.event_len, page_table=db.page_table,
+                      max_pages=w.max_pages, prefix_offset=w.prefix_offset)
+    assert plan.info()["prefix_kernel"] == B.FLAG_PREFIX_MMA
+    B.pad_kv_append(plan, db.k_new, db.v_new, db.k_pool, db.v_pool)
+    B.pad_event_decode_attn_static(plan, db.q, db.k_prefix, db.v_prefix, db.k_pool, db.v_pool, db.out, db.lse)
+    torch.cuda.synchronize()
+    B.pad_device_status(plan)
+    ref_o, ref_lse = oracle_step(w)
+    check_outputs(db.out.cpu().numpy(), db.lse.cpu().numpy(), ref_o, ref_lse, "static, head_dim 64")
