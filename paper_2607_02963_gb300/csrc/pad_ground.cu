@@ -8,7 +8,7 @@
 //
 // The segment score is linear in the token features, so sum_t <g, f_t> = <g, sum_t f_t>:
 // the prefix is read once, pooling each segment's projected features (ground_pool_kernel,
-// HBM-bound; loads are issued four at a time per thread, since a latency-bound stream of
+// HBM-bound; loads are issued eight at a time per thread, since a latency-bound stream of
 // single loads ran at a twentieth of the bandwidth), and scoring every event against the pooled rows is a small contraction over
 // L2-resident data (ground_score_kernel).  The aggregation reads the hidden states once,
 // pooling them per segment with the attention weights, and sums each event's segments
@@ -19,10 +19,19 @@
 
 #include "pad_internal.h"
 
+// The kernels here run for 2 to 25 us each, so the gaps between them count: all are launched
+// with programmatic dependent launch.  Each waits for the grid ahead before it reads or writes
+// anything that grid may touch, and releases its dependents only after that wait, so that a
+// kernel that has started knows every grid but the one right ahead of it to have completed.
+// What the grid ahead may still write while a kernel here runs is read past L1 (not through
+// the read-only path, which assumes that nobody writes).
 namespace pad {
 namespace {
 
 constexpr int kThreads = 256;
+
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 constexpr int kMaxSegments = 1024;
 
 struct Offsets {
@@ -34,7 +43,7 @@ struct Offsets {
 // of their first use, so that they are in flight together).
 __device__ __forceinline__ uint4 ld_stream(const void* p) {
   uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "l"(p));
   return v;
@@ -44,10 +53,10 @@ __device__ __forceinline__ uint4 ld_stream(const void* p) {
 __device__ __forceinline__ void ld_stream4(uint4 (&v)[4], const void* p0, const void* p1, const void* p2,
                                            const void* p3) {
   asm volatile(
-      "ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%16];\n"
-      "ld.global.nc.L1::no_allocate.v4.u32 {%4, %5, %6, %7}, [%17];\n"
-      "ld.global.nc.L1::no_allocate.v4.u32 {%8, %9, %10, %11}, [%18];\n"
-      "ld.global.nc.L1::no_allocate.v4.u32 {%12, %13, %14, %15}, [%19];"
+      "ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%16];\n"
+      "ld.global.L1::no_allocate.v4.u32 {%4, %5, %6, %7}, [%17];\n"
+      "ld.global.L1::no_allocate.v4.u32 {%8, %9, %10, %11}, [%18];\n"
+      "ld.global.L1::no_allocate.v4.u32 {%12, %13, %14, %15}, [%19];"
       : "=r"(v[0].x), "=r"(v[0].y), "=r"(v[0].z), "=r"(v[0].w), "=r"(v[1].x), "=r"(v[1].y), "=r"(v[1].z),
         "=r"(v[1].w), "=r"(v[2].x), "=r"(v[2].y), "=r"(v[2].z), "=r"(v[2].w), "=r"(v[3].x), "=r"(v[3].y),
         "=r"(v[3].z), "=r"(v[3].w)
@@ -64,95 +73,120 @@ __device__ __forceinline__ void unpack8(const uint4 v, float* f) {
   }
 }
 
-// Grid (segment, slice of 4 * RP rows): the 256 threads cover the row's 16-byte chunks
-// (CH = d / 8 of them) and RP = 256 / CH rows at a time, four rows per thread loaded
-// together; the RP partial sums are added in shared memory and then into seg_sum (zeroed
-// by the launcher) with atomics, so the slices of a segment add up in no fixed order.
+// Zeroes the sums ahead of the pooling kernel.
+__global__ void __launch_bounds__(kThreads) ground_zero_kernel(float4* __restrict__ out, int n4) {
+  grid_wait();
+  grid_release();
+  for (int i = blockIdx.x * kThreads + threadIdx.x; i < n4; i += gridDim.x * kThreads)
+    out[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// One CTA per chunk of kPoolRowsPerThread * RP tokens, whatever segments they belong to: the 256
+// threads cover the row's 16-byte chunks (CH = d / 8 of them) and RP = 256 / CH rows at a
+// time.  For each segment that overlaps the chunk a thread adds up its rows, the RP partial
+// sums are added in shared memory and then into seg_sum (zeroed by the kernel ahead) with
+// atomics, so the chunks of a segment add up in no fixed order.  It starts while that kernel
+// runs (which has seen everything before it complete) and waits for it before the first
+// atomic.  Chunks instead of slices of each segment keep the CTAs equal: a grid of segments x
+// (longest segment / slice) is mostly CTAs with nothing to do.
 constexpr int kPoolRowsPerThread = 16;
 __global__ void __launch_bounds__(kThreads) ground_pool_kernel(const __grid_constant__ Offsets so,
                                                                const __nv_bfloat16* __restrict__ f, int d,
                                                                float* __restrict__ seg_sum) {
   extern __shared__ float red[];  // [RP][d]
-  const int s = blockIdx.x;
   const int CH = d / 8, RP = kThreads / CH;
   const int c = threadIdx.x % CH, rg = threadIdx.x / CH;
-  const int lo = so.off[s] + blockIdx.y * kPoolRowsPerThread * RP, hi = so.off[s + 1];
-  if (lo >= hi) return;  // uniform over the CTA
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  if (rg < RP) {
-    const int t = lo + rg;
-    if (t + (kPoolRowsPerThread - 1) * RP < hi) {
-      // sixteen rows per thread, issued in groups of four
-      uint4 v[4][4];
+  const int chunk = kPoolRowsPerThread * RP;
+  const int t_lo = so.off[0] + (int)blockIdx.x * chunk, t_hi = t_lo + min(so.off[so.n] - t_lo, chunk);
+  int s = 0, sh = so.n - 1;  // the segment of token t_lo: the last s with off[s] <= t_lo
+  while (s < sh) {
+    const int mid = (s + sh + 1) >> 1;
+    if (so.off[mid] <= t_lo)
+      s = mid;
+    else
+      sh = mid - 1;
+  }
+  bool waited = false;
+  for (int t0 = t_lo; t0 < t_hi; ++s) {
+    const int t1 = min(t_hi, so.off[s + 1]);
+    if (t1 <= t0) continue;  // an empty segment
+    const int n = t1 - t0;
+    const __nv_bfloat16* row0 = f + (size_t)t0 * d;
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (rg < RP) {
+      for (int t = rg; t < n; t += 8 * RP) {
+        uint4 v[8];
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        const int tg = t + 4 * g * RP;
-        ld_stream4(v[g], reinterpret_cast<const uint4*>(f + (size_t)tg * d) + c,
-                   reinterpret_cast<const uint4*>(f + (size_t)(tg + RP) * d) + c,
-                   reinterpret_cast<const uint4*>(f + (size_t)(tg + 2 * RP) * d) + c,
-                   reinterpret_cast<const uint4*>(f + (size_t)(tg + 3 * RP) * d) + c);
-      }
+        for (int u = 0; u < 8; ++u) {
+          v[u] = make_uint4(0u, 0u, 0u, 0u);
+          if (t + u * RP < n) v[u] = ld_stream(reinterpret_cast<const uint4*>(row0 + (size_t)(t + u * RP) * d) + c);
+        }
 #pragma unroll
-      for (int g = 0; g < 4; ++g)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 8; ++u) {
           float x[8];
-          unpack8(v[g][u], x);
+          unpack8(v[u], x);
 #pragma unroll
           for (int j = 0; j < 8; ++j) acc[j] += x[j];
         }
-    } else {
-      for (int u = 0; u < kPoolRowsPerThread && t + u * RP < hi; ++u) {
-        float x[8];
-        unpack8(__ldg(reinterpret_cast<const uint4*>(f + (size_t)(t + u * RP) * d) + c), x);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[j] += x[j];
       }
-    }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) red[rg * d + c * 8 + j] = acc[j];
+      for (int j = 0; j < 8; ++j) red[rg * d + c * 8 + j] = acc[j];
+    }
+    if (!waited) {
+      grid_wait();
+      grid_release();
+      waited = true;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < d; i += kThreads) {
+      float tot = 0.f;
+      for (int r = 0; r < RP; ++r) tot += red[r * d + i];
+      atomicAdd(seg_sum + (size_t)s * d + i, tot);
+    }
+    __syncthreads();
+    t0 = t1;
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < d; i += kThreads) {
-    float tot = 0.f;
-    for (int r = 0; r < RP; ++r) tot += red[r * d + i];
-    atomicAdd(seg_sum + (size_t)s * d + i, tot);
-  }
+  if (!waited) grid_wait();
 }
 
 // One CTA per event: scores against every pooled segment row, the best score, the salient
 // set (score >= fraction * best when best > 0, else the first best segment alone) and the
 // first and last salient segments.
-__global__ void __launch_bounds__(kThreads) ground_score_kernel(const __nv_bfloat16* __restrict__ g, int S, int d,
+constexpr int kScoreThreads = 1024;  // 32 warps: a hundred segments are one round of loads
+constexpr int kScoreWarps = kScoreThreads / 32;
+__global__ void __launch_bounds__(kScoreThreads) ground_score_kernel(const __nv_bfloat16* __restrict__ g, int S, int d,
                                                                 const float* __restrict__ seg_sum, float frac,
                                                                 float* __restrict__ scores,
                                                                 uint8_t* __restrict__ salient,
                                                                 int32_t* __restrict__ interval) {
   extern __shared__ float gs[];  // [d] the event's projected token, then [S] scores
   float* sc = gs + d;
-  __shared__ float wbest[kThreads / 32];
-  __shared__ int wlo[kThreads / 32], whi[kThreads / 32], warg[kThreads / 32];
+  __shared__ float wbest[kScoreWarps];
+  __shared__ int wlo[kScoreWarps], whi[kScoreWarps], warg[kScoreWarps];
   const int i = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int c = threadIdx.x; c < d; c += kThreads) gs[c] = __bfloat162float(g[(size_t)i * d + c]);
+  grid_wait();
+  grid_release();
+  for (int c = threadIdx.x; c < d; c += kScoreThreads) gs[c] = __bfloat162float(__ldcg(g + (size_t)i * d + c));
   __syncthreads();
-  // a warp per segment row (lanes over its float4 columns), eight rows in flight per warp
+  // a warp per segment row (lanes over its float4 columns), four rows in flight per warp
   float best = -__builtin_huge_valf();
   const int d4 = d / 4;
-  for (int s0 = warp * 8; s0 < S; s0 += 8 * (kThreads / 32)) {
-    float part[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  for (int s0 = warp * 4; s0 < S; s0 += 4 * kScoreWarps) {
+    float part[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
     for (int c = lane; c < d4; c += 32) {
-      float4 v[8];
+      float4 v[4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
-        v[u] = s0 + u < S ? __ldg(reinterpret_cast<const float4*>(seg_sum + (size_t)(s0 + u) * d) + c)
+      for (int u = 0; u < 4; ++u)
+        v[u] = s0 + u < S ? __ldcg(reinterpret_cast<const float4*>(seg_sum + (size_t)(s0 + u) * d) + c)
                           : make_float4(0.f, 0.f, 0.f, 0.f);
       const float g0 = gs[4 * c], g1 = gs[4 * c + 1], g2 = gs[4 * c + 2], g3 = gs[4 * c + 3];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) part[u] += (g0 * v[u].x + g1 * v[u].y) + (g2 * v[u].z + g3 * v[u].w);
+      for (int u = 0; u < 4; ++u) part[u] += (g0 * v[u].x + g1 * v[u].y) + (g2 * v[u].z + g3 * v[u].w);
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < 4; ++u) {
       float v = part[u];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -171,20 +205,20 @@ __global__ void __launch_bounds__(kThreads) ground_score_kernel(const __nv_bfloa
   if (lane == 0) wbest[warp] = best;
   __syncthreads();
   best = wbest[0];
-  for (int w = 1; w < kThreads / 32; ++w) best = fmaxf(best, wbest[w]);
+  for (int w = 1; w < kScoreWarps; ++w) best = fmaxf(best, wbest[w]);
   // the first best segment (used alone when no score is positive)
   int arg = S;
-  for (int s = threadIdx.x; s < S; s += kThreads)
+  for (int s = threadIdx.x; s < S; s += kScoreThreads)
     if (sc[s] == best) arg = min(arg, s);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) arg = min(arg, __shfl_xor_sync(0xffffffffu, arg, o));
   if (lane == 0) warg[warp] = arg;
   __syncthreads();
   arg = warg[0];
-  for (int w = 1; w < kThreads / 32; ++w) arg = min(arg, warg[w]);
+  for (int w = 1; w < kScoreWarps; ++w) arg = min(arg, warg[w]);
   const float cut = frac * best;
   int lo = S, hi = -1;
-  for (int s = threadIdx.x; s < S; s += kThreads) {
+  for (int s = threadIdx.x; s < S; s += kScoreThreads) {
     const bool on = best > 0.f ? sc[s] >= cut : s == arg;
     salient[(size_t)i * S + s] = on ? 1 : 0;
     if (on) {
@@ -203,7 +237,7 @@ __global__ void __launch_bounds__(kThreads) ground_score_kernel(const __nv_bfloa
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < kThreads / 32; ++w) {
+    for (int w = 1; w < kScoreWarps; ++w) {
       lo = min(lo, wlo[w]);
       hi = max(hi, whi[w]);
     }
@@ -242,6 +276,8 @@ __global__ void __launch_bounds__(kThreads) attn_seg_pool_kernel(const __grid_co
                                                                  float* __restrict__ wsum, float* __restrict__ asum) {
   __shared__ float red[kAggGroups][kAggCols];
   __shared__ float ared[kAggGroups];
+  grid_wait();
+  grid_release();
   const int pc = blockIdx.x;
   int sl = 0, sh = pm.n - 1;  // the segment owning piece pc: the last s with pbeg[s] <= pc
   while (sl < sh) {
@@ -268,7 +304,7 @@ __global__ void __launch_bounds__(kThreads) attn_seg_pool_kernel(const __grid_co
                xc + (size_t)(t + 6 * kAggGroups) * rs, xc + (size_t)(t + 7 * kAggGroups) * rs);
     float w[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) w[u] = __ldg(attn + t + u * kAggGroups);
+    for (int u = 0; u < 8; ++u) w[u] = __ldcg(attn + t + u * kAggGroups);
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       float f[8];
@@ -279,9 +315,9 @@ __global__ void __launch_bounds__(kThreads) attn_seg_pool_kernel(const __grid_co
     }
   }
   for (; t < hi; t += kAggGroups) {
-    const float w0 = __ldg(attn + t);
+    const float w0 = __ldcg(attn + t);
     float f[8];
-    unpack8(__ldg(xc + (size_t)t * rs), f);
+    unpack8(ld_stream(xc + (size_t)t * rs), f);
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[j] = fmaf(w0, f[j], acc[j]);
     wacc += w0;
@@ -310,32 +346,47 @@ __global__ void __launch_bounds__(kThreads) attn_seg_pool_kernel(const __grid_co
 // shared memory, in order, and out = g_emb + sum W / sum A (g_emb alone when sum A is 0).
 __global__ void __launch_bounds__(kThreads) attn_event_kernel(const __grid_constant__ Pieces pm, int d,
                                                               const int32_t* __restrict__ interval,
-                                                              const float* __restrict__ wsum,
-                                                              const float* __restrict__ asum,
+                                                              const float* wsum, const float* asum,
                                                               const __nv_bfloat16* __restrict__ g_emb,
                                                               float* __restrict__ out) {
   __shared__ float red[kAggGroups][kAggCols];
   __shared__ float ared[kAggGroups];
   const int i = blockIdx.x, S = pm.n;
-  const int s_lo = min(max(interval[2 * i], 0), S - 1), s_hi = min(max(interval[2 * i + 1], s_lo), S - 1);
+  const int s_lo = min(max(__ldcg(interval + 2 * i), 0), S - 1);
+  const int s_hi = min(max(__ldcg(interval + 2 * i + 1), s_lo), S - 1);
   const int p0 = pm.pbeg[s_lo], p1 = pm.pbeg[s_hi + 1];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c8 = blockIdx.y * kAggCols + lane * 8;  // first of this lane's 8 columns
   float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   float a = 0.f;
+  grid_wait();  // (the interval was written before the pooling kernel started)
+  grid_release();
   if (c8 < d) {
-    for (int pc = p0 + w; pc < p1; pc += kAggGroups) {
-      const float4* src = reinterpret_cast<const float4*>(wsum + (size_t)pc * d + c8);
-      const float4 u0 = __ldg(src), u1 = __ldg(src + 1);
-      acc[0] += u0.x;
-      acc[1] += u0.y;
-      acc[2] += u0.z;
-      acc[3] += u0.w;
-      acc[4] += u1.x;
-      acc[5] += u1.y;
-      acc[6] += u1.z;
-      acc[7] += u1.w;
-      a += __ldg(asum + pc);
+    // four pieces' loads in flight
+    for (int pc = p0 + w; pc < p1; pc += 4 * kAggGroups) {
+      float4 u0[4], u1[4];
+      float av[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int q = pc + k * kAggGroups;
+        const float4* src = reinterpret_cast<const float4*>(wsum + (size_t)(q < p1 ? q : pc) * d + c8);
+        u0[k] = __ldcg(src);
+        u1[k] = __ldcg(src + 1);
+        av[k] = __ldcg(asum + (q < p1 ? q : pc));
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (pc + k * kAggGroups >= p1) break;
+        acc[0] += u0[k].x;
+        acc[1] += u0[k].y;
+        acc[2] += u0[k].z;
+        acc[3] += u0[k].w;
+        acc[4] += u1[k].x;
+        acc[5] += u1[k].y;
+        acc[6] += u1[k].z;
+        acc[7] += u1[k].w;
+        a += av[k];
+      }
     }
   }
 #pragma unroll
@@ -355,6 +406,22 @@ __global__ void __launch_bounds__(kThreads) attn_event_kernel(const __grid_const
   }
 }
 
+// A launch that may start while the grid ahead of it runs.
+template <class... KArgs, class... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 bool fill_offsets(Offsets& so, const int32_t* offsets, int32_t n_segments, int64_t n_tokens) {
   if (n_segments < 1 || n_segments > kMaxSegments || !offsets) return false;
   so.n = n_segments;
@@ -372,15 +439,18 @@ cudaError_t launch_ground_pool(const void* f_proj, int64_t n_tokens, int32_t d, 
   Offsets so;
   if (!fill_offsets(so, offsets, n_segments, n_tokens)) return cudaErrorInvalidValue;
   const int CH = d / 8, RP = kThreads / CH;
+  // (a segment of more than 65535 x 16 RP tokens has always been refused)
   int longest = 0;
   for (int i = 0; i < n_segments; ++i) longest = std::max(longest, so.off[i + 1] - so.off[i]);
-  const int slices = std::max(1, (longest + kPoolRowsPerThread * RP - 1) / (kPoolRowsPerThread * RP));
-  if (slices > 65535) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(seg_sum, 0, (size_t)n_segments * d * sizeof(float), s);
+  if (longest > (int64_t)65535 * kPoolRowsPerThread * RP) return cudaErrorInvalidValue;
+  const int n4 = n_segments * (d / 4);
+  cudaError_t e = launch_pdl(ground_zero_kernel, dim3(std::min(64, (n4 + kThreads - 1) / kThreads)), kThreads, 0, s,
+                             reinterpret_cast<float4*>(seg_sum), n4);
   if (e != cudaSuccess) return e;
-  ground_pool_kernel<<<dim3(n_segments, slices), kThreads, (size_t)RP * d * sizeof(float), s>>>(
-      so, static_cast<const __nv_bfloat16*>(f_proj), d, seg_sum);
-  return cudaGetLastError();
+  const int64_t tokens = (int64_t)so.off[n_segments] - so.off[0], chunk = (int64_t)kPoolRowsPerThread * RP;
+  if (tokens == 0) return cudaSuccess;
+  return launch_pdl(ground_pool_kernel, dim3((unsigned)((tokens + chunk - 1) / chunk)), kThreads,
+                    (size_t)RP * d * sizeof(float), s, so, static_cast<const __nv_bfloat16*>(f_proj), d, seg_sum);
 }
 
 cudaError_t launch_ground_score(const void* g_proj, int32_t n_events, const float* seg_sum, int32_t n_segments,
@@ -388,9 +458,8 @@ cudaError_t launch_ground_score(const void* g_proj, int32_t n_events, const floa
                                 cudaStream_t s) {
   if (n_events == 0) return cudaSuccess;
   const size_t smem = (size_t)(d + n_segments) * sizeof(float);
-  ground_score_kernel<<<n_events, kThreads, smem, s>>>(static_cast<const __nv_bfloat16*>(g_proj), n_segments, d,
-                                                       seg_sum, frac, scores, salient, interval);
-  return cudaGetLastError();
+  return launch_pdl(ground_score_kernel, dim3(n_events), kScoreThreads, smem, s,
+                    static_cast<const __nv_bfloat16*>(g_proj), n_segments, d, seg_sum, frac, scores, salient, interval);
 }
 
 size_t attn_aggregate_ws_floats(int64_t n_tokens, int32_t n_segments, int32_t d) {
@@ -418,14 +487,12 @@ cudaError_t launch_attn_aggregate(const void* x, int64_t n_tokens, int32_t d, co
   float* wsum = seg_ws;
   float* asum = seg_ws + (size_t)std::max(pieces, 1) * d;
   if (pieces > 0) {
-    attn_seg_pool_kernel<<<dim3(pieces, slices), kThreads, 0, s>>>(pm, static_cast<const __nv_bfloat16*>(x), d, attn,
-                                                                   wsum, asum);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(attn_seg_pool_kernel, dim3(pieces, slices), kThreads, 0, s, pm,
+                               static_cast<const __nv_bfloat16*>(x), d, attn, wsum, asum);
     if (e != cudaSuccess) return e;
   }
-  attn_event_kernel<<<dim3(n_events, slices), kThreads, 0, s>>>(pm, d, interval, wsum, asum,
-                                                                 static_cast<const __nv_bfloat16*>(g_emb), out);
-  return cudaGetLastError();
+  return launch_pdl(attn_event_kernel, dim3(n_events, slices), kThreads, 0, s, pm, d, interval, wsum, asum,
+                    static_cast<const __nv_bfloat16*>(g_emb), out);
 }
 
 }  // namespace pad
