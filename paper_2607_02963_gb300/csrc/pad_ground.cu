@@ -34,8 +34,24 @@ __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 constexpr int kMaxSegments = 1024;
 
+// A kernel's parameters are cold in the constant cache at every launch, and each step of a
+// binary search over a thousand of them is a dependent miss (the searches of the pooling
+// kernels cost 3 us).  So the host also passes, for each 64th of a grid, the segment its first
+// block falls into; the search then runs between two of these.
+constexpr int kHints = 64;
+struct Hints {
+  uint16_t seg[kHints + 1];
+  // range [lo, hi] of the segment of block b of nb
+  __device__ void range(unsigned b, unsigned nb, int& lo, int& hi) const {
+    const int g = (int)((unsigned long long)b * kHints / nb);
+    lo = seg[g];
+    hi = seg[g + 1];
+  }
+};
+
 struct Offsets {
   int32_t n;                       // segments
+  Hints hint;                      // by chunk of the pooling kernel
   int32_t off[kMaxSegments + 1];   // token ranges [off[s], off[s + 1])
 };
 
@@ -81,24 +97,28 @@ __global__ void __launch_bounds__(kThreads) ground_zero_kernel(float4* __restric
     out[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// One CTA per chunk of kPoolRowsPerThread * RP tokens, whatever segments they belong to: the 256
-// threads cover the row's 16-byte chunks (CH = d / 8 of them) and RP = 256 / CH rows at a
+// One CTA per chunk of pool_chunk tokens, whatever segments they belong to: the 256 threads
+// cover the row's 16-byte chunks (CH = d / 8 of them) and RP = 256 / CH rows at a
 // time.  For each segment that overlaps the chunk a thread adds up its rows, the RP partial
 // sums are added in shared memory and then into seg_sum (zeroed by the kernel ahead) with
 // atomics, so the chunks of a segment add up in no fixed order.  It starts while that kernel
 // runs (which has seen everything before it complete) and waits for it before the first
 // atomic.  Chunks instead of slices of each segment keep the CTAs equal: a grid of segments x
 // (longest segment / slice) is mostly CTAs with nothing to do.
-constexpr int kPoolRowsPerThread = 16;
+// Tokens of a chunk: 16 KB of them, so that the grid is several CTAs per SM (four or two times as
+// much: 6 or 0.9 us more per readout at d = 256), but at least 32, since every chunk adds a
+// row of d floats per segment to the sums.
+__host__ __device__ constexpr int pool_chunk(int RP) { return 4 * RP > 32 ? 4 * RP : 32; }
 __global__ void __launch_bounds__(kThreads) ground_pool_kernel(const __grid_constant__ Offsets so,
                                                                const __nv_bfloat16* __restrict__ f, int d,
                                                                float* __restrict__ seg_sum) {
-  extern __shared__ float red[];  // [RP][d]
+  extern __shared__ __align__(16) float red[];  // [RP][d]
   const int CH = d / 8, RP = kThreads / CH;
   const int c = threadIdx.x % CH, rg = threadIdx.x / CH;
-  const int chunk = kPoolRowsPerThread * RP;
+  const int chunk = pool_chunk(RP);
   const int t_lo = so.off[0] + (int)blockIdx.x * chunk, t_hi = t_lo + min(so.off[so.n] - t_lo, chunk);
-  int s = 0, sh = so.n - 1;  // the segment of token t_lo: the last s with off[s] <= t_lo
+  int s, sh;  // the segment of token t_lo: the last s with off[s] <= t_lo
+  so.hint.range(blockIdx.x, gridDim.x, s, sh);
   while (s < sh) {
     const int mid = (s + sh + 1) >> 1;
     if (so.off[mid] <= t_lo)
@@ -129,8 +149,9 @@ __global__ void __launch_bounds__(kThreads) ground_pool_kernel(const __grid_cons
           for (int j = 0; j < 8; ++j) acc[j] += x[j];
         }
       }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) red[rg * d + c * 8 + j] = acc[j];
+      float4* dst = reinterpret_cast<float4*>(red + rg * d + c * 8);
+      dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+      dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
     }
     if (!waited) {
       grid_wait();
@@ -138,10 +159,16 @@ __global__ void __launch_bounds__(kThreads) ground_pool_kernel(const __grid_cons
       waited = true;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < d; i += kThreads) {
-      float tot = 0.f;
-      for (int r = 0; r < RP; ++r) tot += red[r * d + i];
-      atomicAdd(seg_sum + (size_t)s * d + i, tot);
+    for (int i = threadIdx.x; i < d / 4; i += kThreads) {
+      float4 tot = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int r = 0; r < RP; ++r) {
+        const float4 v = *reinterpret_cast<const float4*>(red + r * d + 4 * i);
+        tot.x += v.x;
+        tot.y += v.y;
+        tot.z += v.z;
+        tot.w += v.w;
+      }
+      atomicAdd(reinterpret_cast<float4*>(seg_sum + (size_t)s * d) + i, tot);
     }
     __syncthreads();
     t0 = t1;
@@ -263,14 +290,17 @@ constexpr int kAggGroups = kThreads / 32;
 
 struct Pieces {
   int32_t n;                          // segments
+  Hints hint;                         // by piece
   int32_t off[kMaxSegments + 1];      // token ranges of the segments
   int32_t pbeg[kMaxSegments + 1];     // first piece of each segment; pbeg[n] = pieces
 };
 
 // attn_seg_pool_kernel: grid (piece, slice of kAggCols columns).  Eight row groups of 32
 // threads; a thread owns one 16-byte piece (8 columns) of every eighth row and keeps eight
-// rows' loads in flight; the row groups' sums are added in shared memory, in order.
-__global__ void __launch_bounds__(kThreads) attn_seg_pool_kernel(const __grid_constant__ Pieces pm,
+// rows' loads in flight; the row groups' sums are added in shared memory, in order.  HBM-bound:
+// about 25 us for 134 MB with five CTAs per SM (four: 1.5 us more).  Slices of 128 or 512 columns,
+// or a last batch of predicated loads (more registers, so fewer CTAs), were 4 to 10 us slower.
+__global__ void __launch_bounds__(kThreads, 5) attn_seg_pool_kernel(const __grid_constant__ Pieces pm,
                                                                  const __nv_bfloat16* __restrict__ x, int d,
                                                                  const float* __restrict__ attn,
                                                                  float* __restrict__ wsum, float* __restrict__ asum) {
@@ -279,7 +309,8 @@ __global__ void __launch_bounds__(kThreads) attn_seg_pool_kernel(const __grid_co
   grid_wait();
   grid_release();
   const int pc = blockIdx.x;
-  int sl = 0, sh = pm.n - 1;  // the segment owning piece pc: the last s with pbeg[s] <= pc
+  int sl, sh;  // the segment owning piece pc: the last s with pbeg[s] <= pc
+  pm.hint.range(blockIdx.x, gridDim.x, sl, sh);
   while (sl < sh) {
     const int mid = (sl + sh + 1) >> 1;
     if (pm.pbeg[mid] <= pc)
@@ -341,16 +372,17 @@ __global__ void __launch_bounds__(kThreads) attn_seg_pool_kernel(const __grid_co
 }
 
 // attn_event_kernel: grid (event, slice of kAggCols columns).  The pieces of the event's
-// interval (lo, hi), clamped to the segments, are spread over the eight warps (warp w takes
-// every eighth piece from the first); a lane adds 8 columns; the warps' sums are added in
+// interval (lo, hi), clamped to the segments, are spread over 16 warps (warp w takes every
+// 16th piece from the first, four in flight; eight or 32 warps were 1.4 us slower per readout); a lane adds 8 columns; the warps' sums are added in
 // shared memory, in order, and out = g_emb + sum W / sum A (g_emb alone when sum A is 0).
-__global__ void __launch_bounds__(kThreads) attn_event_kernel(const __grid_constant__ Pieces pm, int d,
+constexpr int kEventWarps = 16;
+__global__ void __launch_bounds__(32 * kEventWarps) attn_event_kernel(const __grid_constant__ Pieces pm, int d,
                                                               const int32_t* __restrict__ interval,
                                                               const float* wsum, const float* asum,
                                                               const __nv_bfloat16* __restrict__ g_emb,
                                                               float* __restrict__ out) {
-  __shared__ float red[kAggGroups][kAggCols];
-  __shared__ float ared[kAggGroups];
+  __shared__ float red[kEventWarps][kAggCols];
+  __shared__ float ared[kEventWarps];
   const int i = blockIdx.x, S = pm.n;
   const int s_lo = min(max(__ldcg(interval + 2 * i), 0), S - 1);
   const int s_hi = min(max(__ldcg(interval + 2 * i + 1), s_lo), S - 1);
@@ -363,12 +395,12 @@ __global__ void __launch_bounds__(kThreads) attn_event_kernel(const __grid_const
   grid_release();
   if (c8 < d) {
     // four pieces' loads in flight
-    for (int pc = p0 + w; pc < p1; pc += 4 * kAggGroups) {
+    for (int pc = p0 + w; pc < p1; pc += 4 * kEventWarps) {
       float4 u0[4], u1[4];
       float av[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const int q = pc + k * kAggGroups;
+        const int q = pc + k * kEventWarps;
         const float4* src = reinterpret_cast<const float4*>(wsum + (size_t)(q < p1 ? q : pc) * d + c8);
         u0[k] = __ldcg(src);
         u1[k] = __ldcg(src + 1);
@@ -376,7 +408,7 @@ __global__ void __launch_bounds__(kThreads) attn_event_kernel(const __grid_const
       }
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        if (pc + k * kAggGroups >= p1) break;
+        if (pc + k * kEventWarps >= p1) break;
         acc[0] += u0[k].x;
         acc[1] += u0[k].y;
         acc[2] += u0[k].z;
@@ -394,10 +426,10 @@ __global__ void __launch_bounds__(kThreads) attn_event_kernel(const __grid_const
   if (lane == 0) ared[w] = a;
   __syncthreads();
   const int col = blockIdx.y * kAggCols + threadIdx.x;
-  if (col < d) {
+  if (threadIdx.x < kAggCols && col < d) {
     float num = 0.f, den = 0.f;
 #pragma unroll
-    for (int r = 0; r < kAggGroups; ++r) {
+    for (int r = 0; r < kEventWarps; ++r) {
       num += red[r][threadIdx.x];
       den += ared[r];
     }
@@ -422,6 +454,24 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t 
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// hint.seg[g]: the last segment whose `first` entry is at most that of the first block of the
+// g-th 64th of `blocks` (Hints::range's split); the entry after the last is the last segment.
+template <class Of>
+void fill_hints(Hints& h, const int32_t* first, int n, int64_t blocks, Of value_of) {
+  int s = 0;
+  for (int g = 0; g < kHints; ++g) {
+    const int64_t b = (blocks * g + kHints - 1) / kHints;  // the first block b with b * kHints / blocks >= g
+    if (b >= blocks) {
+      h.seg[g] = (uint16_t)(n - 1);
+      continue;
+    }
+    const int64_t v = value_of(b);
+    while (s + 1 < n && first[s + 1] <= v) ++s;
+    h.seg[g] = (uint16_t)s;
+  }
+  h.seg[kHints] = (uint16_t)(n - 1);
+}
+
 bool fill_offsets(Offsets& so, const int32_t* offsets, int32_t n_segments, int64_t n_tokens) {
   if (n_segments < 1 || n_segments > kMaxSegments || !offsets) return false;
   so.n = n_segments;
@@ -442,14 +492,16 @@ cudaError_t launch_ground_pool(const void* f_proj, int64_t n_tokens, int32_t d, 
   // (a segment of more than 65535 x 16 RP tokens has always been refused)
   int longest = 0;
   for (int i = 0; i < n_segments; ++i) longest = std::max(longest, so.off[i + 1] - so.off[i]);
-  if (longest > (int64_t)65535 * kPoolRowsPerThread * RP) return cudaErrorInvalidValue;
+  if (longest > (int64_t)65535 * 16 * RP) return cudaErrorInvalidValue;
   const int n4 = n_segments * (d / 4);
   cudaError_t e = launch_pdl(ground_zero_kernel, dim3(std::min(64, (n4 + kThreads - 1) / kThreads)), kThreads, 0, s,
                              reinterpret_cast<float4*>(seg_sum), n4);
   if (e != cudaSuccess) return e;
-  const int64_t tokens = (int64_t)so.off[n_segments] - so.off[0], chunk = (int64_t)kPoolRowsPerThread * RP;
+  const int64_t tokens = (int64_t)so.off[n_segments] - so.off[0], chunk = pool_chunk(RP);
   if (tokens == 0) return cudaSuccess;
-  return launch_pdl(ground_pool_kernel, dim3((unsigned)((tokens + chunk - 1) / chunk)), kThreads,
+  const int64_t blocks = (tokens + chunk - 1) / chunk;
+  fill_hints(so.hint, so.off, n_segments, blocks, [&](int64_t b) { return so.off[0] + b * chunk; });
+  return launch_pdl(ground_pool_kernel, dim3((unsigned)blocks), kThreads,
                     (size_t)RP * d * sizeof(float), s, so, static_cast<const __nv_bfloat16*>(f_proj), d, seg_sum);
 }
 
@@ -487,11 +539,12 @@ cudaError_t launch_attn_aggregate(const void* x, int64_t n_tokens, int32_t d, co
   float* wsum = seg_ws;
   float* asum = seg_ws + (size_t)std::max(pieces, 1) * d;
   if (pieces > 0) {
+    fill_hints(pm.hint, pm.pbeg, n_segments, pieces, [](int64_t b) { return b; });
     cudaError_t e = launch_pdl(attn_seg_pool_kernel, dim3(pieces, slices), kThreads, 0, s, pm,
                                static_cast<const __nv_bfloat16*>(x), d, attn, wsum, asum);
     if (e != cudaSuccess) return e;
   }
-  return launch_pdl(attn_event_kernel, dim3(n_events, slices), kThreads, 0, s, pm, d, interval, wsum, asum,
+  return launch_pdl(attn_event_kernel, dim3(n_events, slices), 32 * kEventWarps, 0, s, pm, d, interval, wsum, asum,
                     static_cast<const __nv_bfloat16*>(g_emb), out);
 }
 

@@ -131,3 +131,30 @@ def test_aggregate_long_segment_is_split():
                              torch.zeros((4, 2), dtype=torch.int32, device="cuda"), _dev_bf16(gi.g_emb),
                              torch.empty((4, 520), dtype=torch.float32, device="cuda"), ws[:-1])
     assert ei.value.status == 4
+
+
+@pytest.mark.parametrize("dims", [
+    (33, 1, 1, 2048, 256, 0),         # one chunk and a token over; one 16-byte column group per thread
+    (1024, 1024, 2, 8, 8, 0),         # every token its own segment; the narrowest rows
+    (4097, 1000, 17, 256, 264, 3),    # many short segments per chunk; a slice of eight columns
+    (2500, 65, 33, 296, 3592, 0),     # rows that do not divide the block; more segments than hints
+    (6000, 64, 64, 1024, 512, 7),
+])
+def test_grounding_chunk_and_segment_edges(dims):
+    T, S, K, dp, dm, text = dims
+    _check(synth.grounding_inputs(sum(dims), T, S, K, dp, dm, text_tokens=text), 0.5)
+
+
+def test_grounding_empty_segments_between_chunks():
+    """Runs of empty segments, also at both ends: their sums are zero and nothing else moves."""
+    gi = synth.grounding_inputs(12, 900, 12, 4, 64, 64)
+    o = gi.offsets
+    gi.offsets = np.concatenate([[o[0]] * 70, o, [o[-1]] * 80, ]).astype(np.int32)
+    gi.offsets = np.sort(np.concatenate([gi.offsets, [300] * 40])).astype(np.int32)
+    seg = torch.empty((len(gi.offsets) - 1, 64), dtype=torch.float32, device="cuda")
+    f = _dev_bf16(gi.f_proj)
+    B.pad_ground_pool(f, gi.offsets, seg)
+    f64 = oracle.bf16_to_f64(gi.f_proj)
+    for s in range(len(gi.offsets) - 1):
+        part = f64[gi.offsets[s]:gi.offsets[s + 1]]
+        assert np.all(np.abs(seg[s].cpu().numpy() - part.sum(axis=0)) <= 1e-4 * np.abs(part).sum(axis=0) + 1e-6)
