@@ -109,9 +109,10 @@ __device__ __forceinline__ int64_t part_row(const PadVideoDesc& vd, int kvh, int
 __global__ void append_kernel(const __grid_constant__ KParams p, const uint4* __restrict__ k_new,
                               const uint4* __restrict__ v_new, uint4* __restrict__ k_pool,
                               uint4* __restrict__ v_pool) {
-  // the shared-prefix pass launched after this kernel reads nothing it writes before its
-  // griddepcontrol.wait
+  // Launched so that it may start while the grid ahead runs, and releases the grid behind it
+  // at once; each waits for the other's completion before it touches memory.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int chunks = p.head_dim / 8;
   const int per_event = p.h_kv * chunks;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -612,10 +613,17 @@ cudaError_t launch_append(const KParams& p, const void* k_new, const void* v_new
   const int total = p.n_events * p.h_kv * (p.head_dim / 8);
   if (total == 0) return cudaSuccess;
   const int bs = 256;
-  append_kernel<<<(total + bs - 1) / bs, bs, 0, s>>>(
-      p, static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new),
-      static_cast<uint4*>(k_pool), static_cast<uint4*>(v_pool));
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((total + bs - 1) / bs);
+  cfg.blockDim = dim3(bs);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, append_kernel, p, static_cast<const uint4*>(k_new),
+                            static_cast<const uint4*>(v_new), static_cast<uint4*>(k_pool), static_cast<uint4*>(v_pool));
 }
 
 cudaError_t launch_prefix_simt(const KParams& p, int max_rows, const void* q, const void* kp,
