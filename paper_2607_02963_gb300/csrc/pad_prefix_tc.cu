@@ -323,20 +323,53 @@ __global__ void __launch_bounds__(kThreads, 1)
   // four i from 4 ((w-4)/4) on (head_dim 64).  Rows past R are zero.
   constexpr int kQi = 4 * C::kHalves;
   uint4 qv[kQi];
+  // RoPE: element d < D/2 pairs with d + D/2, i.e. 16-byte chunk cc with chunk cc + D/16 of the same
+  // row.  A thread takes whole pairs instead (pair (t + 64 i) % (D/16) of the row (t + 64 i) /
+  // (D/16) of the quarter, t over its two warps), with the table entries beside them, so that
+  // everything is one round of loads and the rotation stays in registers (rotating rows already in
+  // shared memory, with a barrier and a second round for the table: 2.1 us more per step).
+  constexpr int kPairs = D / 16, kRi = 32 * kPairs / 64;
+  float4 tbl[ROPE ? 4 * kRi : 1];
   if (warp >= 4) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int lane_base = 32 * (warp & 3), half = (warp - 4) >> 2;
+    auto q_row = [&](int qrow, int& el) {
+      el = qrow / p.group;
+      const int gh = qrow - el * p.group;
+      return q + ((size_t)(it.first_event + el) * p.h_q + kvh * p.group + gh) * D;
+    };
+    if constexpr (ROPE) {
 #pragma unroll
-    for (int i = 0; i < kQi; ++i) {
-      const int idx = lane + 32 * (D == 128 ? i : i + 4 * half);
-      const int qrow = row0 + lane_base + (idx >> 3);
-      qv[i] = make_uint4(0u, 0u, 0u, 0u);
-      if (qrow < R) {
-        const int el = qrow / p.group;
-        const int gh = qrow - el * p.group;
-        const __nv_bfloat16* qr = q + ((size_t)(it.first_event + el) * p.h_q + kvh * p.group + gh) * D;
-        const int d0 = (D == 128 ? half * 64 : 0) + (idx & 7) * 8;
-        qv[i] = __ldg(reinterpret_cast<const uint4*>(qr + d0));
+      for (int i = 0; i < kRi; ++i) {
+        const int k = half * 32 + lane + 64 * i, cc = k % kPairs;
+        const int qrow = row0 + lane_base + k / kPairs;
+        qv[2 * i] = qv[2 * i + 1] = make_uint4(0u, 0u, 0u, 0u);
+        tbl[4 * i] = tbl[4 * i + 1] = tbl[4 * i + 2] = tbl[4 * i + 3] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (qrow < R) {
+          int el;
+          const __nv_bfloat16* qr = q_row(qrow, el);
+          qv[2 * i] = __ldg(reinterpret_cast<const uint4*>(qr + 8 * cc));
+          qv[2 * i + 1] = __ldg(reinterpret_cast<const uint4*>(qr + D / 2 + 8 * cc));
+          const float4* cs = reinterpret_cast<const float4*>(
+              p.rope_cs + (size_t)plan_events(p)[it.first_event + el].pos * D + 8 * cc);
+          tbl[4 * i] = __ldg(cs);
+          tbl[4 * i + 1] = __ldg(cs + 1);
+          tbl[4 * i + 2] = __ldg(cs + D / 8);
+          tbl[4 * i + 3] = __ldg(cs + D / 8 + 1);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < kQi; ++i) {
+        const int idx = lane + 32 * (D == 128 ? i : i + 4 * half);
+        const int qrow = row0 + lane_base + (idx >> 3);
+        qv[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (qrow < R) {
+          int el;
+          const __nv_bfloat16* qr = q_row(qrow, el);
+          const int d0 = (D == 128 ? half * 64 : 0) + (idx & 7) * 8;
+          qv[i] = __ldg(reinterpret_cast<const uint4*>(qr + d0));
+        }
       }
     }
   }
@@ -517,43 +550,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int lane_base = 32 * quarter;
     // Q rows (loaded in the prologue) into the 128-byte-swizzled K-major layout the
     // MMA reads: row r, 16-byte chunk cc of half h at h*16K + r*128 + ((cc ^ (r & 7)) << 4).
-#pragma unroll
-    for (int i = 0; i < kQi; ++i) {
-      const int idx = lane + 32 * (D == 128 ? i : i + 4 * half);
-      const int r = lane_base + (idx >> 3), cc = idx & 7;
-      *reinterpret_cast<uint4*>(smem + C::kOffQ + (D == 128 ? half * kQHalfBytes : 0) + r * 128 + ((cc ^ (r & 7)) << 4)) =
-          qv[i];
-    }
-    if (ROPE) {
-      // Rotation in place: element d < D/2 pairs with d + D/2.  At head_dim 128 that is chunk
-      // cc of half 0 with chunk cc of half 1 of the same row, at 64 chunk cc with chunk cc + 4;
-      // either way the other warp of this lane quarter may have stored it.  The two warps meet
-      // (named barrier 2 + quarter) and split the quarter's 32 rows x D / 16 chunk pairs;
-      // every table row is fetched once all are addressed.
-      asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");
-      constexpr int kPairs = D / 16, kRi = 32 * kPairs / 64;
-      const int t = half * 32 + lane;
-      const float* cs[kRi];
+    auto q_slot = [&](int r, int chunk) {  // chunk of the whole row
+      return reinterpret_cast<uint4*>(smem + C::kOffQ + (chunk >> 3) * kQHalfBytes + r * 128 +
+                                      (((chunk & 7) ^ (r & 7)) << 4));
+    };
+    if constexpr (ROPE) {
 #pragma unroll
       for (int i = 0; i < kRi; ++i) {
-        const int r = lane_base + (t + 64 * i) / kPairs;
-        cs[i] = row0 + r < R
-                    ? p.rope_cs + (size_t)plan_events(p)[it.first_event + (row0 + r) / p.group].pos * D
-                    : nullptr;
-      }
-#pragma unroll
-      for (int i = 0; i < kRi; ++i) {
-        if (cs[i] == nullptr) continue;
-        const int k = t + 64 * i;
+        const int k = half * 32 + lane + 64 * i;
         const int r = lane_base + k / kPairs, cc = k % kPairs;
-        const uint32_t hi_off = D == 128 ? kQHalfBytes + ((cc ^ (r & 7)) << 4) : (((cc + 4) ^ (r & 7)) << 4);
-        uint4* lo = reinterpret_cast<uint4*>(smem + C::kOffQ + r * 128 + ((cc ^ (r & 7)) << 4));
-        uint4* hi = reinterpret_cast<uint4*>(smem + C::kOffQ + r * 128 + hi_off);
-        const uint4 a = *lo, b = *hi;
-        const float4 c0 = *reinterpret_cast<const float4*>(cs[i] + 8 * cc);
-        const float4 c1 = *reinterpret_cast<const float4*>(cs[i] + 8 * cc + 4);
-        const float4 s0 = *reinterpret_cast<const float4*>(cs[i] + D / 2 + 8 * cc);
-        const float4 s1 = *reinterpret_cast<const float4*>(cs[i] + D / 2 + 8 * cc + 4);
+        const uint4 a = qv[2 * i], b = qv[2 * i + 1];
+        const float4 c0 = tbl[4 * i], c1 = tbl[4 * i + 1], s0 = tbl[4 * i + 2], s1 = tbl[4 * i + 3];
         const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
         const float s[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
         const uint32_t av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
@@ -569,8 +576,14 @@ __global__ void __launch_bounds__(kThreads, 1)
           ol[j] = *reinterpret_cast<const uint32_t*>(&l2);
           oh[j] = *reinterpret_cast<const uint32_t*>(&h2);
         }
-        *lo = make_uint4(ol[0], ol[1], ol[2], ol[3]);
-        *hi = make_uint4(oh[0], oh[1], oh[2], oh[3]);
+        *q_slot(r, cc) = make_uint4(ol[0], ol[1], ol[2], ol[3]);
+        *q_slot(r, cc + kPairs) = make_uint4(oh[0], oh[1], oh[2], oh[3]);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < kQi; ++i) {
+        const int idx = lane + 32 * (D == 128 ? i : i + 4 * half);
+        *q_slot(lane_base + (idx >> 3), (D == 128 ? half * 8 : 0) + (idx & 7)) = qv[i];
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
