@@ -121,6 +121,7 @@ struct Layout {
   // The branch/merge CTAs of a one-call step wait for the prefix grid before their branch
   // pass (see KParams::merge_first).
   bool merge_first = false;
+  int col_splits = 1;           // CTAs per branch/merge task (see KParams::col_splits)
   std::vector<int32_t> cta_task, cnt_base;
   int64_t n_counters = 0;
   size_t off_videos = 0, off_events = 0, off_items = 0, off_tasks = 0, upload_bytes = 0;
@@ -436,7 +437,16 @@ pad_status layout_for(const pad_problem* prob, int32_t n_videos, const int32_t* 
   L->merge_first = false;
   if (kern == PAD_FLAG_PREFIX_TC && !L->fused && L->n_ctas > 0 && L->n_ctas <= n_sms) {
     const int64_t free_slots = 2 * ((int64_t)n_sms - L->n_ctas);
-    L->merge_first = (int64_t)n_events * prob->h_kv > free_slots;
+    const int64_t tasks = (int64_t)n_events * prob->h_kv;
+    L->merge_first = tasks > free_slots;
+    // Beside the prefix grid, tasks are shared by as many CTAs as there are SMs left for one each:
+    // what follows the grid wait (staging the split partials and merging them) is then spread
+    // over more SMs.  us per step with 1, 2 and 4 CTAs per task: prefix 16384, 1 event 11.6, 10.7,
+    // 10.4; 8192, 8 events 10.4, 9.8, 10.0 (4 no longer get an SM each); head_dim 64, 16384, 16
+    // events 10.2, 9.7, 9.7.  Tasks that run after the prefix grid find every SM free anyway
+    // (32768, 32 events: 23.8 with one, 24.7 with two).
+    const int64_t free_sms = L->merge_first ? 0 : (int64_t)n_sms - L->n_ctas;
+    L->col_splits = 4 * tasks <= free_sms ? 4 : (2 * tasks <= free_sms ? 2 : 1);
   }
 
   size_t off = sizeof(PadDevHeader);
@@ -1073,6 +1083,7 @@ static void make_params(const pad_plan_t* plan, KParams& p) {
   p.n_ctas = (int32_t)plan->lay.n_ctas;
   p.tail_chunk = p.fused ? prefix_tc_tail_chunk(p.branch_rows, p.group, p.max_splits) : 0;
   p.merge_first = plan->lay.merge_first ? 1 : 0;
+  p.col_splits = plan->lay.col_splits;
   p.counters = reinterpret_cast<unsigned int*>(ws + plan->lay.off_cnt);
   p.n_counters = p.fused ? (int32_t)plan->lay.n_counters : 0;
   if (p.img_n > 0) {
@@ -1743,6 +1754,7 @@ pad_status static_params(const pad_plan_t* plan, cudaStream_t s, KParams& p, uin
   p.n_ctas = (int32_t)plan->lay.n_ctas;
   p.tail_chunk = p.fused ? prefix_tc_tail_chunk(p.branch_rows, p.group, p.max_splits) : 0;
   p.merge_first = plan->lay.merge_first ? 1 : 0;
+  p.col_splits = plan->lay.col_splits;
   p.tasks = reinterpret_cast<const int32_t*>(ws + plan->lay.off_tasks);
   p.counters = reinterpret_cast<unsigned int*>(ws + plan->lay.off_cnt);
   p.n_counters = p.fused ? (int32_t)plan->lay.n_counters : 0;

@@ -49,10 +49,10 @@ __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) / 16 * 
 __host__ __device__ constexpr size_t max_sz(size_t a, size_t b) { return a > b ? a : b; }
 
 // Shared memory of a task: this head, then three regions sized per launch (16-byte aligned):
-//   kv   K rows [nkr][LD] and V rows [nkr][LD] of a round (nkr = KParams::branch_rows);
-//        after the branch pass the warps' O rows, fp32 [warp][G][D]
+//   kv   K rows [nkr][LD] and V rows [nkr][W + 8] of a round (nkr = KParams::branch_rows);
+//        after the branch pass the warps' O rows, fp32 [warp][G][W]
 //   ml   the splits' (m, l) pairs of a chunk, [G][sch]
-//   po   the splits' O rows of a chunk, fp32 [sch][G][D]
+//   po   the splits' O rows of a chunk, fp32 [sch][G][W]
 template <int D>
 struct Head {
   static constexpr int LD = D + 8;            // padded bf16 row: ldmatrix rows in distinct banks
@@ -68,14 +68,15 @@ struct Head {
 __host__ __device__ constexpr int round_keys(int branch_rows, int NW) {
   return branch_rows < 16 * NW ? branch_rows : 16 * NW;
 }
-template <int D, int NW = kWarps>
+// (W: the output columns of the task, see run_task)
+template <int D, int NW = kWarps, int W = D>
 __host__ __device__ constexpr size_t kv_bytes(int nkr, int G) {
-  return align16(max_sz((size_t)2 * nkr * Head<D>::LD * 2, (size_t)NW * G * D * 4));
+  return align16(max_sz((size_t)nkr * (Head<D>::LD + W + 8) * 2, (size_t)NW * G * W * 4));
 }
-template <int D, int NW = kWarps>
+template <int D, int NW = kWarps, int W = D>
 __host__ __device__ constexpr size_t smem_bytes(int branch_rows, int G, int sch) {
-  return align16(sizeof(Head<D>)) + kv_bytes<D, NW>(round_keys(branch_rows, NW), G) + align16((size_t)G * sch * 8) +
-         (size_t)sch * G * D * 4;
+  return align16(sizeof(Head<D>)) + kv_bytes<D, NW, W>(round_keys(branch_rows, NW), G) + align16((size_t)G * sch * 8) +
+         (size_t)sch * G * W * 4;
 }
 
 #ifdef __CUDACC__
@@ -163,28 +164,33 @@ struct SyncNamed {
 // partials cannot be read (then only the status word is written).
 // CAUSAL: 0 = the method's own-branch keys, 1 = the causal-attention key list, 2 = read
 // KParams::causal at run time (separate instantiations keep the common one lean).
-template <int D, bool ROPE, int CAUSAL, int NW = kWarps, class Sync, class Ready>
+// W < D: the task is shared by D / W CTAs, each with the output columns w0 .. w0 + W - 1: all of
+// them find the scores and the weights, but each stages and merges its own columns of V and of
+// the split partials, which is most of what a task moves.  The first also appends and writes
+// the LSE.
+template <int D, bool ROPE, int CAUSAL, int NW = kWarps, int W = D, class Sync, class Ready>
 __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* __restrict__ q,
                                          const __nv_bfloat16* __restrict__ kpool,
                                          const __nv_bfloat16* __restrict__ vpool, void* __restrict__ out,
                                          float* __restrict__ lse, int e, int kvh, int tid,
                                          unsigned char* smem, int sch, const Sync& sy, bool early,
-                                         Ready partials_ready) {
+                                         Ready partials_ready, int w0 = 0) {
   static_assert(NW >= 1 && NW <= kWarps, "warps per task");
   constexpr int NT = 32 * NW;
   constexpr int CH = D / 8;                   // 16-byte pieces of a bf16 row
   constexpr int KS = D / 16;                  // k-steps of S = Q K^T
-  constexpr int OT = D / 8;                   // n8 tiles of O
-  constexpr int D4 = D / 4;
+  constexpr int OT = W / 8;                   // n8 tiles of O
+  constexpr int W4 = W / 4;
+  constexpr int LDV = W + 8;                  // padded bf16 V row
   constexpr int LD = Head<D>::LD;
   Head<D>& S = *reinterpret_cast<Head<D>*>(smem);
   const int G = p.group;
   const int nkr = round_keys(p.branch_rows, NW);  // keys per round (multiple of 16, <= 16 NW)
   unsigned char* kv_raw = smem + align16(sizeof(Head<D>));
   __nv_bfloat16 (*sK)[LD] = reinterpret_cast<__nv_bfloat16 (*)[LD]>(kv_raw);
-  __nv_bfloat16 (*sV)[LD] = reinterpret_cast<__nv_bfloat16 (*)[LD]>(kv_raw + (size_t)nkr * LD * 2);
-  float* wo = reinterpret_cast<float*>(kv_raw);  // [warp][G][d] after the branch pass
-  float2* sml = reinterpret_cast<float2*>(kv_raw + kv_bytes<D, NW>(nkr, G));
+  __nv_bfloat16 (*sV)[LDV] = reinterpret_cast<__nv_bfloat16 (*)[LDV]>(kv_raw + (size_t)nkr * LD * 2);
+  float* wo = reinterpret_cast<float*>(kv_raw);  // [warp][G][W] after the branch pass
+  float2* sml = reinterpret_cast<float2*>(kv_raw + kv_bytes<D, NW, W>(nkr, G));
   float* spo = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sml) + align16((size_t)G * sch * 8));
 
   const int warp = tid >> 5, lane = tid & 31;
@@ -251,7 +257,7 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
     else
       cp_async16(&S.q[g][c * 8], qr + c * 8, in);
   }
-  for (int i = tid; i < G * D; i += NT) S.ob[i / D][i % D] = 0.f;
+  for (int i = tid; i < G * W; i += NT) S.ob[i / W][i % W] = 0.f;
   if (tid < 16) {
     S.M[tid] = kNegInf;
     S.L[tid] = 0.f;
@@ -271,15 +277,15 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
                                                         : make_uint4(0u, 0u, 0u, 0u);
         else
           cp_async16(&sK[k][c * 8], knew + new_row + c * 8, in);
-        cp_async16(&sV[k][c * 8], vnew + new_row + c * 8, in);
+        if (W == D || (unsigned)(c * 8 - w0) < (unsigned)W) cp_async16(&sV[k][c * 8 - w0], vnew + new_row + c * 8, in);
         continue;
       }
       const size_t off = (((size_t)(in ? pg : 0) * p.h_kv + kvh) * ps + (in ? S.slot[k] : 0)) * D + c * 8;
       cp_async16(&sK[k][c * 8], kpool + off, in);
-      cp_async16(&sV[k][c * 8], vpool + off, in);
+      if (W == D || (unsigned)(c * 8 - w0) < (unsigned)W) cp_async16(&sV[k][c * 8 - w0], vpool + off, in);
     }
   };
-  if (knew != nullptr) {
+  if (knew != nullptr && w0 == 0) {
     // a2: this task's row of the new token into the pools (16-byte pieces of K, then V);
     // its page was located with the first round's keys when it is among them
     if (tid < 2 * CH) {
@@ -321,17 +327,19 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
   }
   cp_async_commit();                          // this round's keys
 
-  // the splits' O rows and (m, l) pairs of chunk [s0, s0 + nch): per split, the task's G
-  // rows are one contiguous block of G * D floats, R * D floats after the previous split's
+  // the splits' O rows (the task's columns of them) and (m, l) pairs of chunk [s0, s0 + nch): per
+  // split, the task's G rows are one block of G * D floats, R * D floats after the previous split's
   // (the flat index is advanced by NT without a division)
   auto stage_chunk = [&](int s0, int nch) {
-    const int gd4 = G * D4;
-    const float* base = p.part_o + part_row(vd, kvh, s0, R, rbase) * D;
+    const int gd4 = G * W4;
+    const float* base = p.part_o + part_row(vd, kvh, s0, R, rbase) * D + w0;
     const size_t split_stride = (size_t)R * D;
     int sl = tid / gd4, r = tid - (tid / gd4) * gd4;
     const int adv_sl = NT / gd4, adv_r = NT - (NT / gd4) * gd4;
     for (; sl < nch;) {
-      cp_async16(spo + (size_t)sl * G * D + (size_t)r * 4, base + sl * split_stride + (size_t)r * 4, true);
+      // piece r of the G x W block: row r / W4, float4 r % W4 of the task's columns
+      const size_t src = W == D ? (size_t)r * 4 : (size_t)(r / W4) * D + (size_t)(r % W4) * 4;
+      cp_async16(spo + (size_t)sl * G * W + (size_t)r * 4, base + sl * split_stride + src, true);
       sl += adv_sl;
       r += adv_r;
       if (r >= gd4) {
@@ -456,12 +464,12 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
     S.wl[warp][gq + 8] = l_hi;
   }
   if (gq < G) {
-    float* dst = wo + ((size_t)warp * G + gq) * D;
+    float* dst = wo + ((size_t)warp * G + gq) * W;
 #pragma unroll
     for (int i = 0; i < OT; ++i) *reinterpret_cast<float2*>(dst + i * 8 + 2 * t4) = make_float2(o[i][0], o[i][1]);
   }
   if (gq + 8 < G) {
-    float* dst = wo + ((size_t)warp * G + gq + 8) * D;
+    float* dst = wo + ((size_t)warp * G + gq + 8) * W;
 #pragma unroll
     for (int i = 0; i < OT; ++i) *reinterpret_cast<float2*>(dst + i * 8 + 2 * t4) = make_float2(o[i][2], o[i][3]);
   }
@@ -481,13 +489,13 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
     }
   }
   sy.sync();
-  for (int i = tid; i < G * D4; i += NT) {
-    const int g = i / D4, d4 = i - g * D4;
+  for (int i = tid; i < G * W4; i += NT) {
+    const int g = i / W4, d4 = i - g * W4;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int w = 0; w < NW; ++w) {
       const float c = S.sc[g][w];
-      const float4 v = reinterpret_cast<const float4*>(wo)[(w * G + g) * D4 + d4];
+      const float4 v = reinterpret_cast<const float4*>(wo)[(w * G + g) * W4 + d4];
       acc.x = fmaf(c, v.x, acc.x);
       acc.y = fmaf(c, v.y, acc.y);
       acc.z = fmaf(c, v.z, acc.z);
@@ -539,10 +547,10 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
       }
     }
     sy.sync();
-    for (int i = tid; i < G * D4; i += NT) {
-      const int g = i / D4, d4 = i - g * D4;
-      const float4* src = reinterpret_cast<const float4*>(spo) + g * D4 + d4;
-      const int step = G * D4;
+    for (int i = tid; i < G * W4; i += NT) {
+      const int g = i / W4, d4 = i - g * W4;
+      const float4* src = reinterpret_cast<const float4*>(spo) + g * W4 + d4;
+      const int step = G * W4;
       const float al = S.a[g];
       float4 acc = reinterpret_cast<const float4*>(&S.ob[g][0])[d4];
       acc.x *= al;
@@ -565,21 +573,21 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
   sy.sync();
   if (!ok) return;
 
-  for (int i = tid; i < G * D4; i += NT) {
-    const int g = i / D4, d4 = i - g * D4;
+  for (int i = tid; i < G * W4; i += NT) {
+    const int g = i / W4, d4 = i - g * W4;
     const float inv = 1.0f / S.L[g];
     float4 v = reinterpret_cast<const float4*>(&S.ob[g][0])[d4];
     v.x *= inv;
     v.y *= inv;
     v.z *= inv;
     v.w *= inv;
-    const size_t oi = ((size_t)e * p.h_q + kvh * G + g) * D + 4 * d4;
+    const size_t oi = ((size_t)e * p.h_q + kvh * G + g) * D + w0 + 4 * d4;
     if (p.out_bf16)
       *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(out) + oi) =
           make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
     else
       *reinterpret_cast<float4*>(reinterpret_cast<float*>(out) + oi) = v;
-    if (lse != nullptr && d4 == 0)
+    if (lse != nullptr && d4 == 0 && w0 == 0)
       lse[(size_t)e * p.h_q + kvh * G + g] = (S.M[g] + log2f(S.L[g])) * 0.69314718055994531f;
   }
 }

@@ -108,6 +108,7 @@ struct KParams {
                                   // the branch/merge CTAs to run beside it: each of them
                                   // waits for it first, then stages the split partials
                                   // while its branch pass runs
+  int32_t col_splits;             // CTAs that share a branch/merge task, by output columns
   float scale_log2;               // scale * log2(e)
   uint64_t gen;                   // generation of the plan (tags errors in the status word)
   PadDevHeader* header;

@@ -519,7 +519,8 @@ __global__ void __launch_bounds__(128) prefix_mma_kernel(const __grid_constant__
 // ---------------------------------------------------------------------------
 // NW warps per task: 8 (two CTAs per SM) by default, 4 (three per SM) when the step has more
 // than two waves of tasks, so that more of its latency-bound tasks are in flight at once.
-template <int D, bool ROPE, int CAUSAL, int NW>
+// W output columns per CTA: D / W CTAs share a task (KParams::col_splits).
+template <int D, bool ROPE, int CAUSAL, int NW, int W>
 __global__ void __launch_bounds__(32 * NW, NW == bm::kWarps ? 2 : 3) branch_merge_kernel(const __grid_constant__ KParams p,
                                                                     const __nv_bfloat16* __restrict__ q,
                                                                     const __nv_bfloat16* __restrict__ kpool,
@@ -532,10 +533,13 @@ __global__ void __launch_bounds__(32 * NW, NW == bm::kWarps ? 2 : 3) branch_merg
   // prefix kernel, which waits for this grid before it touches anything (an append kernel
   // after it is launched without programmatic serialisation and waits in any case).
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int e = blockIdx.x / p.h_kv;
-  const int kvh = blockIdx.x - e * p.h_kv;
-  bm::run_task<D, ROPE, CAUSAL, NW>(p, q, kpool, vpool, out, lse, e, kvh, (int)threadIdx.x, bm_raw, sch,
-                                     bm::SyncCta{}, true, [] { return true; });
+  constexpr int kShare = D / W;
+  const int task = blockIdx.x / kShare;
+  const int e = task / p.h_kv;
+  const int kvh = task - e * p.h_kv;
+  bm::run_task<D, ROPE, CAUSAL, NW, W>(p, q, kpool, vpool, out, lse, e, kvh, (int)threadIdx.x, bm_raw, sch,
+                                       bm::SyncCta{}, true, [] { return true; },
+                                       (int)(blockIdx.x % kShare) * W);
 }
 
 // Step inputs from page-locked, device-mapped host memory into device memory (the
@@ -677,12 +681,12 @@ cudaError_t launch_prefix_mma(const KParams& p, int max_rows, const void* q, con
 
 // Split partials merged per staged chunk: as many as a shared-memory budget allows next to
 // the branch staging.
-template <int D, int NW = bm::kWarps>
+template <int D, int NW, int W>
 int bm_chunk(const KParams& p, size_t budget) {
   const int G = p.group;
   const size_t fixed =
-      bm::align16(sizeof(bm::Head<D>)) + bm::kv_bytes<D, NW>(bm::round_keys(p.branch_rows, NW), G) + 16;
-  const size_t per_split = (size_t)G * D * sizeof(float) + sizeof(float2);
+      bm::align16(sizeof(bm::Head<D>)) + bm::kv_bytes<D, NW, W>(bm::round_keys(p.branch_rows, NW), G) + 16;
+  const size_t per_split = (size_t)G * W * sizeof(float) + sizeof(float2);
   int sch = fixed + per_split <= budget ? (int)((budget - fixed) / per_split) : 1;
   if (p.max_splits > 0 && sch > p.max_splits) sch = p.max_splits;
   return sch < 1 ? 1 : (sch > bm::kMaxChunk ? bm::kMaxChunk : sch);
@@ -690,34 +694,34 @@ int bm_chunk(const KParams& p, size_t budget) {
 // The standalone kernel: a grid of more CTAs than SMs keeps two per SM (8 warps each), one
 // of more than two waves three (4 warps each).
 inline bool bm_narrow(const KParams& p) { return (int64_t)p.n_events * p.h_kv > 2 * (int64_t)p.n_sms; }
-inline size_t n_cta_budget(const KParams& p) {
+inline size_t n_cta_budget(const KParams& p, int share) {
   if (bm_narrow(p)) return 74 * 1024;
-  return p.n_events * p.h_kv > p.n_sms ? 110 * 1024 : 200 * 1024;
+  return share > 1 || p.n_events * p.h_kv > p.n_sms ? 110 * 1024 : 200 * 1024;
 }
 
-template <int D, int NW>
+template <int D, int NW, int W>
 static cudaError_t launch_bm_nw(const KParams& p, const void* q, const void* k_pool, const void* v_pool,
                                 void* out, float* lse, bool pdl, cudaStream_t s) {
   const int G = p.group;
   const int nkr = p.branch_rows;
   if (nkr <= 0 || nkr > bm::kKeys || nkr % 16 != 0) return cudaErrorInvalidValue;
-  const int sch = bm_chunk<D, NW>(p, n_cta_budget(p));
-  const size_t smem = bm::smem_bytes<D, NW>(nkr, G, sch);
+  const int sch = bm_chunk<D, NW, W>(p, n_cta_budget(p, D / W));
+  const size_t smem = bm::smem_bytes<D, NW, W>(nkr, G, sch);
   constexpr int kMaxSmem = 227 * 1024;
   if (smem > (size_t)kMaxSmem) return cudaErrorInvalidValue;
   static bool configured[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !configured[dev]) {
-    for (auto fn : {branch_merge_kernel<D, false, 0, NW>, branch_merge_kernel<D, true, 0, NW>,
-                    branch_merge_kernel<D, false, 1, NW>, branch_merge_kernel<D, true, 1, NW>}) {
+    for (auto fn : {branch_merge_kernel<D, false, 0, NW, W>, branch_merge_kernel<D, true, 0, NW, W>,
+                    branch_merge_kernel<D, false, 1, NW, W>, branch_merge_kernel<D, true, 1, NW, W>}) {
       cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
       if (e != cudaSuccess) return e;
     }
     configured[dev] = true;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.n_events * p.h_kv);
+  cfg.gridDim = dim3(p.n_events * p.h_kv * (D / W));
   cfg.blockDim = dim3(32 * NW);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -726,8 +730,10 @@ static cudaError_t launch_bm_nw(const KParams& p, const void* q, const void* k_p
   attr[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  auto fn = p.causal ? (p.rope_cs != nullptr ? branch_merge_kernel<D, true, 1, NW> : branch_merge_kernel<D, false, 1, NW>)
-                     : (p.rope_cs != nullptr ? branch_merge_kernel<D, true, 0, NW> : branch_merge_kernel<D, false, 0, NW>);
+  auto fn = p.causal ? (p.rope_cs != nullptr ? branch_merge_kernel<D, true, 1, NW, W>
+                                             : branch_merge_kernel<D, false, 1, NW, W>)
+                     : (p.rope_cs != nullptr ? branch_merge_kernel<D, true, 0, NW, W>
+                                             : branch_merge_kernel<D, false, 0, NW, W>);
   return cudaLaunchKernelEx(&cfg, fn, p, static_cast<const __nv_bfloat16*>(q),
                             static_cast<const __nv_bfloat16*>(k_pool), static_cast<const __nv_bfloat16*>(v_pool),
                             out, lse, sch);
@@ -735,8 +741,10 @@ static cudaError_t launch_bm_nw(const KParams& p, const void* q, const void* k_p
 template <int D>
 static cudaError_t launch_bm(const KParams& p, const void* q, const void* k_pool, const void* v_pool,
                              void* out, float* lse, bool pdl, cudaStream_t s) {
-  return bm_narrow(p) ? launch_bm_nw<D, 4>(p, q, k_pool, v_pool, out, lse, pdl, s)
-                      : launch_bm_nw<D, bm::kWarps>(p, q, k_pool, v_pool, out, lse, pdl, s);
+  if (bm_narrow(p)) return launch_bm_nw<D, 4, D>(p, q, k_pool, v_pool, out, lse, pdl, s);
+  if (p.col_splits >= 4 && D == 128) return launch_bm_nw<D, bm::kWarps, D / 4>(p, q, k_pool, v_pool, out, lse, pdl, s);
+  if (p.col_splits >= 2) return launch_bm_nw<D, bm::kWarps, D / 2>(p, q, k_pool, v_pool, out, lse, pdl, s);
+  return launch_bm_nw<D, bm::kWarps, D>(p, q, k_pool, v_pool, out, lse, pdl, s);
 }
 
 cudaError_t launch_branch_merge(const KParams& p, const void* q, const void* k_pool,

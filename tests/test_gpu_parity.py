@@ -759,3 +759,19 @@ def test_head_dim_64_forced_kernels_and_host_only_plans():
     B.pad_device_status(plan)
     ref_o, ref_lse = oracle_step(w)
     check_outputs(db.out.cpu().numpy(), db.lse.cpu().numpy(), ref_o, ref_lse, "static, head_dim 64")
+
+
+@pytest.mark.parametrize("one_call", [True, False])
+@pytest.mark.parametrize("D,h_q,h_kv", [(128, 28, 4), (128, 16, 1), (64, 14, 2), (64, 3, 3)])
+@pytest.mark.parametrize("lens", [[0], [130], [5, 0, 200], [3, 16, 17, 1, 63, 64, 2]])
+def test_shared_branch_tasks_match_oracle(lens, D, h_q, h_kv, one_call):
+    """Tasks shared by two or four CTAs, by output columns (few tasks beside a prefix grid that
+    leaves SMs free): branches of no, some and more than one round of keys, every column and the
+    appended row against the oracle, in fp32 and (rounded once) bf16."""
+    w = _w([1200], [len(lens)], lens, seed=len(lens), h_q=h_q, h_kv=h_kv, D=D)
+    db, plan = run_full(w, one_call=one_call)
+    assert not plan.info()["merge_first"]
+    b16 = DeviceBatch(w, out_dtype=1)
+    b16.run_step(one_call=one_call)
+    torch.cuda.synchronize()
+    assert torch.equal(b16.out, db.out.bfloat16()) and torch.equal(b16.lse, db.lse)
