@@ -1180,8 +1180,10 @@ static pad_status launch_attention(const pad_plan_t* plan, const void* q, const 
     g_timing.n++;
   }
   if (!plan->lay.fused) {
-    const bool pdl = !timed && (plan->lay.prefix_kernel == PAD_FLAG_PREFIX_TC ||
-                                plan->lay.prefix_kernel == PAD_FLAG_PREFIX_DUAL);
+    // (only behind a prefix grid, which waits for everything ahead before it releases this one: a
+    // branch task reads q and the keys of earlier steps before its own wait)
+    const bool pdl = !timed && plan->lay.n_items > 0 &&
+                     (plan->lay.prefix_kernel == PAD_FLAG_PREFIX_TC || plan->lay.prefix_kernel == PAD_FLAG_PREFIX_DUAL);
     e = launch_branch_merge(p, q, k_pool, v_pool, out, lse, pdl, s);
     if (e != cudaSuccess) return cuda_fail(e, "branch/merge launch");
   }

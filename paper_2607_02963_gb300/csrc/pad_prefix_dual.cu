@@ -195,10 +195,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   DualBars* bars = reinterpret_cast<DualBars*>(smem + kOffBar);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // One-call step (k_new set): this is the step's first kernel, launched so that it may
-  // start while the grid before it finishes; every thread that touches global memory
-  // waits for that grid first (the Q loads, the first TMA issue).
-  const bool one_call = p.k_new != nullptr;
+  // Launched so that it may start while the grid before it (the previous step, or this step's
+  // append, which itself may still be waiting for the grid ahead of it) finishes; every thread
+  // that touches global memory waits for that grid first (the Q loads, the first TMA issue).
 
   // the CTA's work item and 256-row group: from the plan's CTA list, or the dense grid
   int item, grp;
@@ -234,7 +233,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // output unused).
   uint4 qv[16];
   if (warp >= 4) {
-    if (one_call) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int wg = (warp - 4) >> 2, tq = (int)threadIdx.x - 128 - 128 * wg;
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -278,7 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmK)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
-    if (one_call) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (n_tiles > 0) {
       load_k(0);
       load_v(0);
@@ -679,10 +678,6 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   __syncwarp();
   fence_before();
-  // This grid may run alongside the append kernel before it (it reads nothing that kernel
-  // writes); waiting for it here makes the completion of this grid imply the completion
-  // of the append, which the branch/merge pass after it relies on.
-  if (threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
   if (warp == 2) {
     // the softmax warps' own arrivals order their last TMEM reads before the deallocation

@@ -775,3 +775,46 @@ def test_shared_branch_tasks_match_oracle(lens, D, h_q, h_kv, one_call):
     b16.run_step(one_call=one_call)
     torch.cuda.synchronize()
     assert torch.equal(b16.out, db.out.bfloat16()) and torch.equal(b16.lse, db.lse)
+
+
+@pytest.mark.parametrize("one_call", [True, False])
+@pytest.mark.parametrize("prefix,flags", [([0, 0], 0), ([700, 300], 0), ([700, 300], B.FLAG_PREFIX_DUAL)])
+def test_steps_back_to_back_equal_steps_run_apart(prefix, flags, one_call):
+    """A generation loop enqueued without any wait between its kernels (each step reads the keys
+    that the one before appended, and q written by a kernel right ahead of the attention) equals
+    the same loop with a wait after every call; also with nothing but branches, where no prefix
+    grid stands between two steps."""
+    w = _w(prefix, [3, 4], [14, 15, 31, 0, 63, 64, 1], seed=70)
+    qs = [torch.randn(w.q.shape, device="cuda").bfloat16() for _ in range(6)]
+    res = []
+    for apart in (True, False):
+        wait = torch.cuda.synchronize if apart else (lambda: None)
+        db = DeviceBatch(w, flags=flags, fill_nan=False)
+        db.page_table = torch.cat([db.page_table, torch.full_like(db.page_table, -1)], dim=1).contiguous()
+        lens, outs, plans = w.event_len.copy(), [], []
+        for step in range(6):
+            plan = B.pad_plan(db.problem, db.cache, w.prefix_len, w.event_video, lens, page_table=db.page_table,
+                              max_pages=int(db.page_table.shape[1]), workspace=db.workspace,
+                              prefix_offset=w.prefix_offset)
+            plans.append(plan)
+            out, lse = torch.empty_like(db.out), torch.empty_like(db.lse)
+            wait()
+            if not one_call:
+                B.pad_kv_append(plan, db.k_new, db.v_new, db.k_pool, db.v_pool)
+                wait()
+            db.q.copy_(qs[step])
+            wait()
+            if one_call:
+                B.pad_decode_step(plan, db.q, db.k_new, db.v_new, db.k_prefix, db.v_prefix, db.k_pool, db.v_pool,
+                                  out, lse)
+            else:
+                B.pad_event_decode_attn(plan, db.q, db.k_prefix, db.v_prefix, db.k_pool, db.v_pool, out, lse)
+            wait()
+            outs += [out, lse]
+            lens = lens + 1
+        torch.cuda.synchronize()
+        for plan in plans:
+            B.pad_device_status(plan)
+        res.append(outs + [db.k_pool, db.v_pool, db.page_table])
+    for a, b in zip(*res):
+        assert torch.equal(a, b)
