@@ -1084,6 +1084,7 @@ static void make_params(const pad_plan_t* plan, KParams& p) {
   p.tail_chunk = p.fused ? prefix_tc_tail_chunk(p.branch_rows, p.group, p.max_splits) : 0;
   p.merge_first = plan->lay.merge_first ? 1 : 0;
   p.col_splits = plan->lay.col_splits;
+  p.keys_ready = 0;
   p.counters = reinterpret_cast<unsigned int*>(ws + plan->lay.off_cnt);
   p.n_counters = p.fused ? (int32_t)plan->lay.n_counters : 0;
   if (p.img_n > 0) {
@@ -1153,6 +1154,8 @@ static pad_status launch_attention(const pad_plan_t* plan, const void* q, const 
   make_params(plan, p);
   p.k_new = k_new;
   p.v_new = v_new;
+  p.keys_ready = plan->lay.n_items > 0 && !plan->lay.fused &&
+                 (plan->lay.prefix_kernel == PAD_FLAG_PREFIX_TC || plan->lay.prefix_kernel == PAD_FLAG_PREFIX_DUAL);
   const bool timed = g_timing.on && g_timing.n < g_timing.max;
   if (timed) cudaEventRecord(g_timing.ev[2 * g_timing.n], s);
   cudaError_t e = cudaSuccess;
@@ -1757,6 +1760,7 @@ pad_status static_params(const pad_plan_t* plan, cudaStream_t s, KParams& p, uin
   p.tail_chunk = p.fused ? prefix_tc_tail_chunk(p.branch_rows, p.group, p.max_splits) : 0;
   p.merge_first = plan->lay.merge_first ? 1 : 0;
   p.col_splits = plan->lay.col_splits;
+  p.keys_ready = 0;
   p.tasks = reinterpret_cast<const int32_t*>(ws + plan->lay.off_tasks);
   p.counters = reinterpret_cast<unsigned int*>(ws + plan->lay.off_cnt);
   p.n_counters = p.fused ? (int32_t)plan->lay.n_counters : 0;

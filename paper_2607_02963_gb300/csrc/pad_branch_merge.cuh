@@ -22,10 +22,11 @@
 // Staging before griddepcontrol.wait reads nothing the grids ahead write: Q rows, the
 // branch's page ids (key `len`'s page is the one this step took, else the table's entry
 // of an earlier step) and the K/V rows of keys 0..len-1, and key `len` itself when it
-// comes from k_new / v_new.  In a one-call step that is all the branch pass reads, so the
-// whole pass (and the merge of its warp states) runs before the wait.  After it: key `len`
-// when the append kernel wrote it (two-call step, the branch pass follows), and the
-// splits' (m, l) pairs and O rows once the caller says they are complete
+// comes from k_new / v_new, or when the append kernel wrote it and the prefix grid waited for
+// that kernel before it released this one (KParams::keys_ready; two-call step, prefix 8219, 13
+// events with RoPE: 16.0 -> 13.9 us).  That is all the branch pass reads, so the whole pass (and the
+// merge of its warp states) runs before the wait.  After it: key `len` in the other two-call
+// steps (the branch pass follows), and the splits' (m, l) pairs and O rows once the caller says they are complete
 // (`partials_ready`: at once for the standalone kernel, whose wait covers the prefix
 // grid; after the split counters for the tensor-core kernel).
 #pragma once
@@ -305,7 +306,7 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
   }
   const int nv0_16 = (nv0 + 15) & ~15;
   // this step's key waits for the grids ahead only when the append kernel wrote it
-  const bool len_in_first = own < nkr && knew == nullptr;
+  const bool len_in_first = own < nkr && knew == nullptr && !p.keys_ready;
   // rows 0..nv0_16-1 except that key (rows past nv0 are zero-filled)
   if (len_in_first) {
     stage_keys(0, nv0, 0, own);
@@ -314,11 +315,11 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
     stage_keys(0, nv0, 0, nv0_16);
   }
   cp_async_commit();
-  // One-call step: nothing the branch pass reads is written by the grids ahead, so the
-  // whole pass runs before the wait and only the merge of the splits' partials follows it;
+  // Where nothing the branch pass reads is written by a grid still running, the whole pass
+  // runs before the wait and only the merge of the splits' partials follows it;
   // unless the plan says this CTA cannot start before the prefix grid completes anyway
   // (merge_first), where waiting first lets the partials load during the branch pass.
-  const bool pre = knew != nullptr && !p.merge_first;
+  const bool pre = (knew != nullptr || p.keys_ready) && !p.merge_first;
 
   // ---------------- after the grids ahead (at least the append) completed
   if (!pre) {

@@ -108,6 +108,9 @@ struct KParams {
                                   // the branch/merge CTAs to run beside it: each of them
                                   // waits for it first, then stages the split partials
                                   // while its branch pass runs
+  int32_t keys_ready;             // two-call step behind the tensor-core prefix grid, which waits
+                                  // for the append before it releases the branch/merge grid:
+                                  // the appended keys may be read before that grid's own wait
   int32_t col_splits;             // CTAs that share a branch/merge task, by output columns
   float scale_log2;               // scale * log2(e)
   uint64_t gen;                   // generation of the plan (tags errors in the status word)
