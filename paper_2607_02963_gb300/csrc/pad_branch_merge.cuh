@@ -79,6 +79,13 @@ __host__ __device__ constexpr size_t smem_bytes(int branch_rows, int G, int sch)
   return align16(sizeof(Head<D>)) + kv_bytes<D, NW, W>(round_keys(branch_rows, NW), G) + align16((size_t)G * sch * 8) +
          (size_t)sch * G * W * 4;
 }
+// A task whose branch pass ends before its partials are staged (OVER) lays po over kv: ml first,
+// then one region for both.
+template <int D, int NW = kWarps, int W = D>
+__host__ __device__ constexpr size_t smem_bytes_over(int branch_rows, int G, int sch) {
+  return align16(sizeof(Head<D>)) + align16((size_t)G * sch * 8) +
+         max_sz(kv_bytes<D, NW, W>(round_keys(branch_rows, NW), G), (size_t)sch * G * W * 4);
+}
 
 #ifdef __CUDACC__
 __device__ __forceinline__ float ex2(float x) {
@@ -169,7 +176,9 @@ struct SyncNamed {
 // them find the scores and the weights, but each stages and merges its own columns of V and of
 // the split partials, which is most of what a task moves.  The first also appends and writes
 // the LSE.
-template <int D, bool ROPE, int CAUSAL, int NW = kWarps, int W = D, class Sync, class Ready>
+// OVER: the caller knows that the branch pass ends before the partials are staged (`pre` below),
+// so both use the same shared memory.
+template <int D, bool ROPE, int CAUSAL, int NW = kWarps, int W = D, bool OVER = false, class Sync, class Ready>
 __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* __restrict__ q,
                                          const __nv_bfloat16* __restrict__ kpool,
                                          const __nv_bfloat16* __restrict__ vpool, void* __restrict__ out,
@@ -187,12 +196,12 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
   Head<D>& S = *reinterpret_cast<Head<D>*>(smem);
   const int G = p.group;
   const int nkr = round_keys(p.branch_rows, NW);  // keys per round (multiple of 16, <= 16 NW)
-  unsigned char* kv_raw = smem + align16(sizeof(Head<D>));
+  unsigned char* kv_raw = smem + align16(sizeof(Head<D>)) + (OVER ? align16((size_t)G * sch * 8) : 0);
   __nv_bfloat16 (*sK)[LD] = reinterpret_cast<__nv_bfloat16 (*)[LD]>(kv_raw);
   __nv_bfloat16 (*sV)[LDV] = reinterpret_cast<__nv_bfloat16 (*)[LDV]>(kv_raw + (size_t)nkr * LD * 2);
   float* wo = reinterpret_cast<float*>(kv_raw);  // [warp][G][W] after the branch pass
-  float2* sml = reinterpret_cast<float2*>(kv_raw + kv_bytes<D, NW, W>(nkr, G));
-  float* spo = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sml) + align16((size_t)G * sch * 8));
+  float2* sml = reinterpret_cast<float2*>(OVER ? smem + align16(sizeof(Head<D>)) : kv_raw + kv_bytes<D, NW, W>(nkr, G));
+  float* spo = reinterpret_cast<float*>(OVER ? kv_raw : reinterpret_cast<unsigned char*>(sml) + align16((size_t)G * sch * 8));
 
   const int warp = tid >> 5, lane = tid & 31;
   const int gq = lane >> 2, t4 = lane & 3;
@@ -319,7 +328,7 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
   // runs before the wait and only the merge of the splits' partials follows it;
   // unless the plan says this CTA cannot start before the prefix grid completes anyway
   // (merge_first), where waiting first lets the partials load during the branch pass.
-  const bool pre = (knew != nullptr || p.keys_ready) && !p.merge_first;
+  const bool pre = OVER || ((knew != nullptr || p.keys_ready) && !p.merge_first);
 
   // ---------------- after the grids ahead (at least the append) completed
   if (!pre) {
@@ -508,6 +517,7 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
   if (early && pre) {
     // ---------------- after the grids ahead (the prefix pass) completed
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (OVER) sy.sync();                      // the warps' O rows have been read
     if (ns > 0) stage_chunk(0, min(sch, ns));
     cp_async_commit();
   }

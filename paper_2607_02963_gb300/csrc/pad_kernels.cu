@@ -520,8 +520,9 @@ __global__ void __launch_bounds__(128) prefix_mma_kernel(const __grid_constant__
 // NW warps per task: 8 (two CTAs per SM) by default, 4 (three per SM) when the step has more
 // than two waves of tasks, so that more of its latency-bound tasks are in flight at once.
 // W output columns per CTA: D / W CTAs share a task (KParams::col_splits).
-template <int D, bool ROPE, int CAUSAL, int NW, int W>
-__global__ void __launch_bounds__(32 * NW, NW == bm::kWarps ? 2 : 3) branch_merge_kernel(const __grid_constant__ KParams p,
+// OVER (4 warps): four CTAs per SM, the partials staged over the branch's keys.
+template <int D, bool ROPE, int CAUSAL, int NW, int W, bool OVER>
+__global__ void __launch_bounds__(32 * NW, NW == bm::kWarps ? 2 : (OVER ? 4 : 3)) branch_merge_kernel(const __grid_constant__ KParams p,
                                                                     const __nv_bfloat16* __restrict__ q,
                                                                     const __nv_bfloat16* __restrict__ kpool,
                                                                     const __nv_bfloat16* __restrict__ vpool,
@@ -537,7 +538,7 @@ __global__ void __launch_bounds__(32 * NW, NW == bm::kWarps ? 2 : 3) branch_merg
   const int task = blockIdx.x / kShare;
   const int e = task / p.h_kv;
   const int kvh = task - e * p.h_kv;
-  bm::run_task<D, ROPE, CAUSAL, NW, W>(p, q, kpool, vpool, out, lse, e, kvh, (int)threadIdx.x, bm_raw, sch,
+  bm::run_task<D, ROPE, CAUSAL, NW, W, OVER>(p, q, kpool, vpool, out, lse, e, kvh, (int)threadIdx.x, bm_raw, sch,
                                        bm::SyncCta{}, true, [] { return true; },
                                        (int)(blockIdx.x % kShare) * W);
 }
@@ -691,30 +692,40 @@ int bm_chunk(const KParams& p, size_t budget) {
   if (p.max_splits > 0 && sch > p.max_splits) sch = p.max_splits;
   return sch < 1 ? 1 : (sch > bm::kMaxChunk ? bm::kMaxChunk : sch);
 }
-// The standalone kernel: a grid of more CTAs than SMs keeps two per SM (8 warps each), one
-// of more than two waves three (4 warps each).
+// The standalone kernel: a grid of more CTAs than SMs keeps two per SM (8 warps each), one of
+// more than two waves three or four (4 warps each).  Its tasks are chains of latencies (page
+// ids, keys, partials), so more of them in flight is what helps: 16 ragged videos, 1032 tasks:
+// 93.5 us per step with three CTAs of 74 KB per SM, 88.9 with four, whose partials lie over the
+// branch's keys (OVER; possible where the branch pass precedes the grid wait).
 inline bool bm_narrow(const KParams& p) { return (int64_t)p.n_events * p.h_kv > 2 * (int64_t)p.n_sms; }
 inline size_t n_cta_budget(const KParams& p, int share) {
   if (bm_narrow(p)) return 74 * 1024;
   return share > 1 || p.n_events * p.h_kv > p.n_sms ? 110 * 1024 : 200 * 1024;
 }
 
-template <int D, int NW, int W>
+template <int D, int NW, int W, bool OVER = false>
 static cudaError_t launch_bm_nw(const KParams& p, const void* q, const void* k_pool, const void* v_pool,
                                 void* out, float* lse, bool pdl, cudaStream_t s) {
   const int G = p.group;
   const int nkr = p.branch_rows;
   if (nkr <= 0 || nkr > bm::kKeys || nkr % 16 != 0) return cudaErrorInvalidValue;
-  const int sch = bm_chunk<D, NW, W>(p, n_cta_budget(p, D / W));
-  const size_t smem = bm::smem_bytes<D, NW, W>(nkr, G, sch);
+  int sch = bm_chunk<D, NW, W>(p, n_cta_budget(p, D / W));
+  size_t smem = bm::smem_bytes<D, NW, W>(nkr, G, sch);
+  if (OVER) {
+    // four CTAs per SM: as many splits per chunk as fit 55 KB, at least what the branch's keys
+    // leave room for
+    sch = std::min(std::max(1, p.max_splits), bm::kMaxChunk);
+    while (sch > 1 && bm::smem_bytes_over<D, NW, W>(nkr, G, sch) > 55 * 1024) --sch;
+    smem = bm::smem_bytes_over<D, NW, W>(nkr, G, sch);
+  }
   constexpr int kMaxSmem = 227 * 1024;
   if (smem > (size_t)kMaxSmem) return cudaErrorInvalidValue;
   static bool configured[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !configured[dev]) {
-    for (auto fn : {branch_merge_kernel<D, false, 0, NW, W>, branch_merge_kernel<D, true, 0, NW, W>,
-                    branch_merge_kernel<D, false, 1, NW, W>, branch_merge_kernel<D, true, 1, NW, W>}) {
+    for (auto fn : {branch_merge_kernel<D, false, 0, NW, W, OVER>, branch_merge_kernel<D, true, 0, NW, W, OVER>,
+                    branch_merge_kernel<D, false, 1, NW, W, OVER>, branch_merge_kernel<D, true, 1, NW, W, OVER>}) {
       cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
       if (e != cudaSuccess) return e;
     }
@@ -730,10 +741,10 @@ static cudaError_t launch_bm_nw(const KParams& p, const void* q, const void* k_p
   attr[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  auto fn = p.causal ? (p.rope_cs != nullptr ? branch_merge_kernel<D, true, 1, NW, W>
-                                             : branch_merge_kernel<D, false, 1, NW, W>)
-                     : (p.rope_cs != nullptr ? branch_merge_kernel<D, true, 0, NW, W>
-                                             : branch_merge_kernel<D, false, 0, NW, W>);
+  auto fn = p.causal ? (p.rope_cs != nullptr ? branch_merge_kernel<D, true, 1, NW, W, OVER>
+                                             : branch_merge_kernel<D, false, 1, NW, W, OVER>)
+                     : (p.rope_cs != nullptr ? branch_merge_kernel<D, true, 0, NW, W, OVER>
+                                             : branch_merge_kernel<D, false, 0, NW, W, OVER>);
   return cudaLaunchKernelEx(&cfg, fn, p, static_cast<const __nv_bfloat16*>(q),
                             static_cast<const __nv_bfloat16*>(k_pool), static_cast<const __nv_bfloat16*>(v_pool),
                             out, lse, sch);
@@ -741,7 +752,11 @@ static cudaError_t launch_bm_nw(const KParams& p, const void* q, const void* k_p
 template <int D>
 static cudaError_t launch_bm(const KParams& p, const void* q, const void* k_pool, const void* v_pool,
                              void* out, float* lse, bool pdl, cudaStream_t s) {
-  if (bm_narrow(p)) return launch_bm_nw<D, 4, D>(p, q, k_pool, v_pool, out, lse, pdl, s);
+  if (bm_narrow(p)) {
+    const bool pre = (p.k_new != nullptr || p.keys_ready) && !p.merge_first;  // as in run_task
+    return pre ? launch_bm_nw<D, 4, D, true>(p, q, k_pool, v_pool, out, lse, pdl, s)
+               : launch_bm_nw<D, 4, D>(p, q, k_pool, v_pool, out, lse, pdl, s);
+  }
   if (p.col_splits >= 4 && D == 128) return launch_bm_nw<D, bm::kWarps, D / 4>(p, q, k_pool, v_pool, out, lse, pdl, s);
   if (p.col_splits >= 2) return launch_bm_nw<D, bm::kWarps, D / 2>(p, q, k_pool, v_pool, out, lse, pdl, s);
   return launch_bm_nw<D, bm::kWarps, D>(p, q, k_pool, v_pool, out, lse, pdl, s);

@@ -818,3 +818,26 @@ def test_steps_back_to_back_equal_steps_run_apart(prefix, flags, one_call):
         res.append(outs + [db.k_pool, db.v_pool, db.page_table])
     for a, b in zip(*res):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("one_call", [True, False])
+@pytest.mark.parametrize("D,h_q,h_kv", [(128, 28, 4), (128, 16, 1), (64, 14, 2)])
+def test_many_small_tasks_match_oracle(D, h_q, h_kv, one_call):
+    """More than two waves of branch tasks (few SMs) whose partials lie over the branch's keys:
+    none, part of, exactly and several rounds (64 keys) of keys; beside a tensor-core grid of
+    several waves, and with more splits (warp-level kernel) than a chunk of 55 KB holds."""
+    lens = [0, 63, 64, 62, 130, 5, 1, 128, 200, 16, 31, 2]
+    w = _w([3000, 700, 129, 1], [3, 4, 2, 3], lens, seed=12, h_q=h_q, h_kv=h_kv, D=D)
+    wide = _w([12000], [33], [0, 63, 64, 130, 7] + [3] * 28, seed=13, h_q=h_q, h_kv=h_kv, D=D)
+    for w, num_sms, flags in ((w, 2, 0), (w, 3, 0), (wide, 16, B.FLAG_PREFIX_MMA)):
+        ref_o, ref_lse = oracle_step(w)
+        db = DeviceBatch(w, num_sms=num_sms, flags=flags)
+        plan = db.run_step(one_call=one_call)
+        torch.cuda.synchronize()
+        B.pad_device_status(plan)
+        info = plan.info()
+        assert w.n_events * h_kv > 2 * num_sms and not info["merge_first"]
+        if flags and h_kv == 1:
+            assert info["partial_rows"] // (w.n_events * h_q) > 55 * 1024 // (h_q // h_kv * D * 4)
+        check_bookkeeping(db, w, plan)
+        check_outputs(db.out.cpu().numpy(), db.lse.cpu().numpy(), ref_o, ref_lse, f"{num_sms} SMs")
