@@ -686,7 +686,7 @@ template <int D, int NW, int W>
 int bm_chunk(const KParams& p, size_t budget) {
   const int G = p.group;
   const size_t fixed =
-      bm::align16(sizeof(bm::Head<D>)) + bm::kv_bytes<D, NW, W>(bm::round_keys(p.branch_rows, NW), G) + 16;
+      bm::align16(sizeof(bm::Head<D>)) + bm::kv_bytes<D, W>(bm::round_keys(p.branch_rows, NW)) + 16;
   const size_t per_split = (size_t)G * W * sizeof(float) + sizeof(float2);
   int sch = fixed + per_split <= budget ? (int)((budget - fixed) / per_split) : 1;
   if (p.max_splits > 0 && sch > p.max_splits) sch = p.max_splits;
