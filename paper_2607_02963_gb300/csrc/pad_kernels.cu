@@ -110,23 +110,35 @@ __global__ void append_kernel(const __grid_constant__ KParams p, const uint4* __
                               const uint4* __restrict__ v_new, uint4* __restrict__ k_pool,
                               uint4* __restrict__ v_pool) {
   // Launched so that it may start while the grid ahead runs, and releases the grid behind it
-  // at once; each waits for the other's completion before it touches memory.
+  // at once; each waits for the other's completion before it touches memory (the plan's
+  // descriptors apart).  A two-call step waits for all of this kernel, a chain of latencies: the
+  // index arithmetic runs ahead of the wait and the new rows are read beside the page id (prefix
+  // 8219, 13 events with RoPE: 13.2 us per step, now 12.7).
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int chunks = p.head_dim / 8;
   const int per_event = p.h_kv * chunks;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool mine = idx < p.n_events * per_event;
+  const int e = mine ? idx / per_event : 0;
+  int rem = idx - e * per_event;
+  int h = rem / chunks;
+  int c = rem - h * chunks;
+  PadEventDesc ev = {};
+  if (mine) ev = plan_events(p)[e];
+  int pidx = ev.len / p.page_size;
+  int slot = ev.len - pidx * p.page_size;
+  asm volatile("" : "+r"(rem), "+r"(h), "+r"(c), "+r"(pidx), "+r"(slot));  // (not sunk behind it)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   // the split counters of the fused tail start the step at zero (there are fewer of them
   // than threads here: at most h_kv per event)
   if (idx < p.n_counters) p.counters[idx] = 0u;
-  if (idx >= p.n_events * per_event) return;
-  const int e = idx / per_event;
-  const int rem = idx - e * per_event;
-  const int h = rem / chunks;
-  const int c = rem - h * chunks;
-  const PadEventDesc ev = plan_events(p)[e];
-  const int pidx = ev.len / p.page_size;
-  const int slot = ev.len - pidx * p.page_size;
+  if (!mine) return;
+  const size_t src = ((size_t)e * p.h_kv + h) * chunks + c;
+  const uint4 v = v_new[src];
+  const uint4 k = p.rope_cs != nullptr
+                      ? rope_chunk8(reinterpret_cast<const __nv_bfloat16*>(k_new + (src - c)), p.head_dim, 8 * c,
+                                    p.rope_cs + (size_t)ev.pos * p.head_dim)
+                      : k_new[src];
   int page;
   if (ev.new_page >= 0) {
     page = ev.new_page;
@@ -139,12 +151,8 @@ __global__ void append_kernel(const __grid_constant__ KParams p, const uint4* __
     return;
   }
   const size_t dst = (((size_t)page * p.h_kv + h) * p.page_size + slot) * chunks + c;
-  const size_t src = ((size_t)e * p.h_kv + h) * chunks + c;
-  k_pool[dst] = p.rope_cs != nullptr
-                    ? rope_chunk8(reinterpret_cast<const __nv_bfloat16*>(k_new + (src - c)), p.head_dim, 8 * c,
-                                  p.rope_cs + (size_t)ev.pos * p.head_dim)
-                    : k_new[src];
-  v_pool[dst] = v_new[src];
+  k_pool[dst] = k;
+  v_pool[dst] = v;
 }
 
 // ---------------------------------------------------------------------------
