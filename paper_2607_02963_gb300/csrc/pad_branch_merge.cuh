@@ -37,7 +37,7 @@
 // CTAs per SM (16 ragged videos, 1032 tasks), with keys staged by the whole CTA behind barriers,
 // unpadded O rows and rows weighted by single warps: 11800 / 2900 / 2500, now 10200 / 1500 / 1300.
 // us per step: 88.9 -> 84.3; prefix 32768, 32 events 23.8 -> 22.5; 16384, 64 events 24.1 -> 21.7;
-// 8192, 8 events 9.8 -> 9.4.
+// 8192, 8 events 9.8 -> 9.5.
 #pragma once
 
 #include <cuda_bf16.h>

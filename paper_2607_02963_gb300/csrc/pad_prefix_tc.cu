@@ -23,15 +23,17 @@
 //               tile, and again only when a row's sum shows that a score outgrew them by more
 //               than 2^8 (then O is rescaled and the tile redone).
 //
-// What bounds it: the chain S -> softmax -> P.V of each tile and the fixed cost per CTA (the
-// loop of a long split runs at 0.9 of the copy bandwidth).  Electing the issuing lane of a
+// What bounds it: on a long split the softmax's own instructions (about 1280 cycles per tile and
+// CTA at 32 and 64 events, 180 of them waits; 16 ragged videos, one row group each: 1760, a third
+// waits for K/V from HBM), on a short one the fixed cost per CTA.  Electing the issuing lane of a
 // uniform warp instead of branching to lane 0 (see elect_one) and skipping the maximum took,
-// per step: prefix 32768, 32 events 24.8 -> 23.7 us; 16384, 64 events 25.6 -> 23.9; 16384, 1
-// event 12.0 -> 11.4; 8192, 8 events 10.75 -> 10.6; 16 ragged videos 94.3 -> 93.0.
+// per step of that time: prefix 32768, 32 events 24.8 -> 23.7 us; 16384, 64 events 25.6 -> 23.9;
+// 16384, 1 event 12.0 -> 11.4; 8192, 8 events 10.75 -> 10.6; 16 ragged videos 94.3 -> 93.0.  With
+// what followed here and in the branch/merge pass: 22.5, 21.6, 9.3, 8.5 and 84.
 //
 // head_dim 64 (one 64-column box per tile, P.V with N = 64) takes the same pipeline: 14/2 heads,
-// prefix 16384, 16 events 24.0 us per step on the mma.sync kernel, 9.7 here; 4/1 heads, 512
-// tokens, 4 events 14.3 -> 6.2 (latency: programmatic dependent launch and the one-call order
+// prefix 16384, 16 events 24.0 us per step on the mma.sync kernel, 8.7 here; 4/1 heads, 512
+// tokens, 4 events 14.3 -> 6.3 (latency: programmatic dependent launch and the one-call order
 // come with this path).
 //
 // Every MMA has N = 128 (S: 128 tokens; P.V: 128 head-dim columns), the size at
