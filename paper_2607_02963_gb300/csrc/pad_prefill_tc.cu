@@ -10,6 +10,12 @@
 // branch to its last token) and masks per row only where a tile needs it.  Query tiles start
 // in descending order, so that the longest key ranges go first.
 //
+// A short sequence (SPLIT) has one slot of queries per CTA and shares out its key tiles instead:
+// the softmax warps 4-7 take the even ones, 8-11 the odd ones, each with an S buffer, a maximum
+// and an O of their own, merged at the end.  There a CTA's chain of tiles, one after the other, is
+// the whole time, and this halves it (512 + 160 tokens, 28/4 heads: 16.7 -> 14.5 us; 1100 + 160,
+// 16/1 heads: 24.8 -> 16.8).
+//
 //   warps 0, 3  TMA producers of K and V tiles (64-column boxes, 128-byte swizzle)
 //   warp 1      S issuer: S_g(k) = Q_g K(k)^T
 //   warp 2      TMEM allocation (512 columns) and deallocation, and P.V issuer: O_g += P_g(k)
@@ -51,6 +57,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -211,7 +218,7 @@ __device__ __forceinline__ void part_exp(const uint32_t (&s)[4][32], uint64_t sc
   }
 }
 
-template <int D>
+template <int D, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
     prefill_tc_kernel(const __grid_constant__ PrefillTcParams p, const __grid_constant__ CUtensorMap tmQ,
                       const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
@@ -226,7 +233,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
   const int N = p.n_tokens, S = p.prefix_len, G = p.group;
-  const int tpc = 2 * p.tps;                              // query tokens per CTA
+  const int tpc = (SPLIT ? 1 : 2) * p.tps;                              // query tokens per CTA
   const int n_qt = (N + tpc - 1) / tpc;
   const int qt = n_qt - 1 - (int)blockIdx.x / p.h_kv;
   const int kvh = (int)blockIdx.x % p.h_kv;
@@ -271,7 +278,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Q of both slots (box: 64 columns x G heads x tps tokens, so that smem row = token * G +
     // head; tokens past N are zero-filled) and the first K tile go out from here
     const uint32_t q_bytes = (uint32_t)C::kHalves * 128u * (uint32_t)(G * p.tps);
-    for (int g = 0; g < 2; ++g) {
+    for (int g = 0; g < (SPLIT ? 1 : 2); ++g) {
       mbar_expect_tx(&bars->qfull[g], q_bytes);
 #pragma unroll
       for (int h = 0; h < C::kHalves; ++h)
@@ -330,16 +337,18 @@ __global__ void __launch_bounds__(kThreads, 1)
       int s = 0, ph = 0;
       for (int t = 0; t < n_tiles && ok; ++t) {
         ok = pwait_warp(&bars->kfull[s], (uint32_t)ph, bars, p, 3);
+        const int j = SPLIT ? t >> 1 : t;      // the slot's how-manieth tile
 #pragma unroll
-        for (int g = 0; g < 2; ++g) {
+        for (int i = 0; i < (SPLIT ? 1 : 2); ++i) {
+          const int g = SPLIT ? t & 1 : i;
           if (!ok) break;
-          if (t == 0)
-            ok = pwait_warp(&bars->qfull[g], 0u, bars, p, 11);
-          else  // S_g holds P of tile t - 1 until its P.V has completed
-            ok = pwait_warp(&bars->pvdone[g], (uint32_t)((t - 1) & 1), bars, p, 6);
+          if (j == 0)
+            ok = pwait_warp(&bars->qfull[SPLIT ? 0 : g], 0u, bars, p, 11);
+          else  // S_g holds P of the slot's previous tile until its P.V has completed
+            ok = pwait_warp(&bars->pvdone[g], (uint32_t)((j - 1) & 1), bars, p, 6);
           if (!ok) break;
           fence_after();
-          const uint64_t qd = sdesc(sbase + (uint32_t)g * C::kTileBytes, 16, 1024);
+          const uint64_t qd = sdesc(sbase + (SPLIT ? 0u : (uint32_t)g * C::kTileBytes), 16, 1024);
           const uint64_t kd = dK + ((uint32_t)s * C::kTileBytes >> 4);
           if (el) {
 #pragma unroll
@@ -348,7 +357,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               mma_ss(tmem + 128u * g, qd + (off >> 4), kd + (off >> 4), C::kIdescS, kk > 0 ? 1u : 0u);
             }
             mma_commit(&bars->sfull[g]);
-            if (g == 1) mma_commit(&bars->kfree[s]);
+            if (SPLIT || g == 1) mma_commit(&bars->kfree[s]);
           }
           __syncwarp();
         }
@@ -370,19 +379,21 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int t = 0; t < n_tiles && ok; ++t) {
         ok = pwait_warp(&bars->vfull[s], (uint32_t)ph, bars, p, 4);
         const uint64_t vd = dV + ((uint32_t)s * C::kTileBytes >> 4);
+        const int j = SPLIT ? t >> 1 : t;
 #pragma unroll
-        for (int g = 0; g < 2; ++g) {
+        for (int i = 0; i < (SPLIT ? 1 : 2); ++i) {
+          const int g = SPLIT ? t & 1 : i;
           const uint32_t a = tmem + 128u * g;
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            if (ok) ok = pwait_warp(h ? &bars->phi[g] : &bars->plo[g], (uint32_t)(t & 1), bars, p, 5);
+            if (ok) ok = pwait_warp(h ? &bars->phi[g] : &bars->plo[g], (uint32_t)(j & 1), bars, p, 5);
             if (!ok) break;
             fence_after();
             if (el) {
 #pragma unroll
               for (int kk = h ? 2 * kLoGroups : 0; kk < (h ? 8 : 2 * kLoGroups); ++kk)
                 mma_ts(tmem + C::kColO + (uint32_t)D * g, a + kk * 8, vd + ((uint32_t)kk * 2048 >> 4), C::kIdescPV,
-                       (t > 0 || kk > 0) ? 1u : 0u);
+                       (j > 0 || kk > 0) ? 1u : 0u);
               if (C::kSplitP) {
 #pragma unroll
                 for (int kk = h ? 2 * kLoGroups : 0; kk < (h ? 8 : 2 * kLoGroups); ++kk)
@@ -392,7 +403,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               if (h == 0) mma_commit(&bars->pvlo[g]);
               if (h == 1) {
                 mma_commit(&bars->pvdone[g]);
-                if (g == 1) mma_commit(&bars->vfree[s]);
+                if (SPLIT || g == 1) mma_commit(&bars->vfree[s]);
               }
             }
             __syncwarp();
@@ -422,7 +433,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int wrow = 32 * (warp & 3);          // TMEM lanes wrow .. wrow + 31
     const int row = wrow + lane;               // row of the slot: token row / G, head row % G
     const int tl = row / G;
-    const int tok = tok0 + g * p.tps + tl;
+    const int tok = tok0 + (SPLIT ? 0 : g * p.tps) + tl;
     const bool active = tl < p.tps && tok < N;
     const int bs = active && tok >= S ? branch_start(p, tok) : -1;
     const uint32_t tb = tmem + ((uint32_t)wrow << 16);
@@ -440,7 +451,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // 2^8 means that every P is.  Only a part that exceeds it (and the first of all, which has
     // no m yet) finds the row's maximum, rescales O and l to it and is redone.
     auto tile = [&](int t, auto masked) -> bool {
-      if (!__all_sync(0xffffffffu, pwait(&bars->sfull[g], (uint32_t)(t & 1), bars, p, 8))) return false;
+      const int j = SPLIT ? t >> 1 : t;        // the slot's how-manieth tile
+      if (!__all_sync(0xffffffffu, pwait(&bars->sfull[g], (uint32_t)(j & 1), bars, p, 8))) return false;
       fence_after();
       uint32_t s[4][32];
 #pragma unroll
@@ -475,17 +487,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint64_t s2 = fadd2(fadd2(sum[0], sum[1]), fadd2(sum[2], sum[3]));
         const bool grow = active && (m_run == kNegInf || f2lo(s2) + f2hi(s2) > kRescaleSum);
         if (__any_sync(0xffffffffu, grow)) {
-          if (t > 0 || h == 1) {
+          if (j > 0 || h == 1) {
             // every P.V issued on O so far has completed: O may be rescaled
-            if (!__all_sync(0xffffffffu, h == 1 ? pwait(&bars->pvlo[g], (uint32_t)(t & 1), bars, p, 9)
-                                                : pwait(&bars->pvdone[g], (uint32_t)((t - 1) & 1), bars, p, 9)))
+            if (!__all_sync(0xffffffffu, h == 1 ? pwait(&bars->pvlo[g], (uint32_t)(j & 1), bars, p, 9)
+                                                : pwait(&bars->pvdone[g], (uint32_t)((j - 1) & 1), bars, p, 9)))
               return false;
             fence_after();
           }
           const float m_new = fmaxf(m_run, row_max(s) * sl2);
           const bool need = grow && m_new > m_run;
           const float alpha = need ? ex2(m_run - m_new) : 1.f;
-          if (t > 0 || h == 1) {
+          if (j > 0 || h == 1) {
 #pragma unroll 1
             for (int c = 0; c < D / 32; ++c) {
               uint32_t r[32];
@@ -518,19 +530,76 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) lim = min(lim, __shfl_xor_sync(0xffffffffu, lim, o));
     const int n_full = min(a_tiles, lim / kBN);
-    int t = 0;
-    for (; t < n_full && ok; ++t) ok = tile(t, std::false_type{});
-    for (; t < n_tiles && ok; ++t) ok = tile(t, std::true_type{});
+    constexpr int kStep = SPLIT ? 2 : 1;
+    int t = SPLIT ? g : 0;
+    for (; t < n_full && ok; t += kStep) ok = tile(t, std::false_type{});
+    for (; t < n_tiles && ok; t += kStep) ok = tile(t, std::true_type{});
     // O is final once the last P.V has completed; the slot's Q is idle by then too (its last S
     // completed before that P could be written)
-    if (ok) ok = pwait(&bars->pvdone[g], (uint32_t)((n_tiles - 1) & 1), bars, p, 10);
+    const int mine = SPLIT ? (n_tiles + 1 - g) >> 1 : n_tiles;  // tiles of this slot
+    if (ok && mine > 0) ok = pwait(&bars->pvdone[g], (uint32_t)((mine - 1) & 1), bars, p, 10);
     ok = __all_sync(0xffffffffu, ok);
+    const uint64_t a2 = fadd2(fadd2(acc[0], acc[1]), fadd2(acc[2], acc[3]));
+    float l = f2lo(a2) + f2hi(a2);
+    float wgt = 1.f;                           // of this slot's O in the result
+    // SPLIT: slot g writes the columns from D/2 g on, and takes the other's share of them.  (m, l)
+    // of both go through the second Q stage, which holds nothing here; then the O rows on the
+    // common maximum through the K stages, idle once both slots' last P.V has completed: fp32,
+    // row r's 16-byte chunk c at chunk c ^ (r % 16 or 8), so that both sides touch distinct banks.
+    constexpr int kCo = D / 4;                 // 16-byte chunks of an fp32 row
+    static_assert(128u * 4 * D <= C::kKS * C::kTileBytes, "the slots' O rows fit the K stages");
+    float2* sml = reinterpret_cast<float2*>(smem + C::kTileBytes);
+    uint8_t* so = smem + C::kOffK + (uint32_t)row * (4 * D);
+    if (SPLIT) {
+      sml[g * 128 + row] = make_float2(m_run, l);
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      const float2 other = sml[(g ^ 1) * 128 + row];
+      const float m = fmaxf(m_run, other.x);
+      wgt = mine > 0 && m_run > kNegInf ? ex2(m_run - m) : 0.f;
+      l = fmaf(l, wgt, other.x > kNegInf ? other.y * ex2(other.x - m) : 0.f);
+      m_run = m;
+      if (ok) {
+        fence_after();
+#pragma unroll 1
+        for (int c = (1 - g) * (D / 64); c < (2 - g) * (D / 64); ++c) {
+          uint32_t r[32];
+          if (mine > 0) {
+            tmem_ld32(tO + 32 * c, r);
+            tmem_wait_ld_dep(r);
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (mine > 0)
+              w = make_float4(__uint_as_float(r[4 * j]) * wgt, __uint_as_float(r[4 * j + 1]) * wgt,
+                              __uint_as_float(r[4 * j + 2]) * wgt, __uint_as_float(r[4 * j + 3]) * wgt);
+            *reinterpret_cast<float4*>(so + (((8 * c + j) ^ (lane & (kCo / 2 - 1))) << 4)) = w;
+          }
+        }
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+    }
+    // O of 32 columns of the row, from c0 on
+    auto load_o = [&](int c0, uint32_t* r) {
+      if (!SPLIT || mine > 0) {
+        tmem_ld32(tO + c0, r);
+        tmem_wait_ld_dep(r);
+      }
+      if (SPLIT) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float4 w = *reinterpret_cast<const float4*>(so + (((c0 / 4 + j) ^ (lane & (kCo / 2 - 1))) << 4));
+          const float a[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            r[4 * j + u] = __float_as_uint(mine > 0 ? fmaf(__uint_as_float(r[4 * j + u]), wgt, a[u]) : a[u]);
+        }
+      }
+    };
     if (ok) {
       fence_after();
-      const uint64_t a2 = fadd2(fadd2(acc[0], acc[1]), fadd2(acc[2], acc[3]));
-      const float l = f2lo(a2) + f2hi(a2);
       const float inv = 1.0f / l;
-      if (active && p.lse != nullptr)
+      if (active && (!SPLIT || g == 0) && p.lse != nullptr)
         p.lse[(int64_t)tok * p.h_q + kvh * G + row % G] = (m_run + log2f(l)) * 0.69314718055994531f;
       // Rows out through this warp's 32 rows of the slot's Q stage (2 D bytes per row: all
       // columns in bf16, half of them in fp32): row r's 16-byte chunk c at chunk position
@@ -540,13 +609,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int passes = p.out_bf16 ? 1 : 2;
       const int esz = p.out_bf16 ? 2 : 4;
 #pragma unroll 1
-      for (int ps = 0; ps < passes; ++ps) {
+      for (int ps = SPLIT && passes == 2 ? g : 0; ps < (SPLIT && passes == 2 ? g + 1 : passes); ++ps) {
         if (p.out_bf16) {
 #pragma unroll 1
-          for (int c = 0; c < D / 32; ++c) {
+          for (int c = SPLIT ? g * (D / 64) : 0; c < (SPLIT ? g + 1 : 2) * (D / 64); ++c) {
             uint32_t r[32];
-            tmem_ld32(tO + 32 * c, r);
-            tmem_wait_ld_dep(r);
+            load_o(32 * c, r);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               uint32_t w[4];
@@ -561,8 +629,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 1
           for (int c = 0; c < D / 64; ++c) {
             uint32_t r[32];
-            tmem_ld32(tO + (D / 2) * ps + 32 * c, r);
-            tmem_wait_ld_dep(r);
+            load_o((D / 2) * ps + 32 * c, r);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
               uint32_t w[4];
@@ -575,9 +642,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         __syncwarp();
 #pragma unroll 1
-        for (int i = lane; i < 32 * kCh; i += 32) {
-          const int r = i / kCh, c = i % kCh;
-          const int rr = wrow + r, rt = rr / G, rtok = tok0 + g * p.tps + rt;
+        for (int i = lane; i < 32 * kCh / (SPLIT && p.out_bf16 ? 2 : 1); i += 32) {
+          const int r = SPLIT && p.out_bf16 ? i / (kCh / 2) : i / kCh;
+          const int c = SPLIT && p.out_bf16 ? g * (kCh / 2) + i % (kCh / 2) : i % kCh;
+          const int rr = wrow + r, rt = rr / G, rtok = tok0 + (SPLIT ? 0 : g * p.tps) + rt;
           if (rt < p.tps && rtok < N) {
             const uint4 v = *reinterpret_cast<const uint4*>(stg + r * (2 * D) + ((c ^ (r & (kCh - 1))) << 4));
             const int64_t o = ((int64_t)rtok * p.h_q + kvh * G + (rr - rt * G)) * D * esz + (int64_t)ps * (2 * D) + 16 * c;
@@ -619,6 +687,37 @@ bool make_map(CUtensorMap* map, const void* base, int D, int heads, int64_t toke
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+constexpr double kSplitCtaUs = 8.5, kSplitRoundUs = 1.3, kPairCtaUs = 8.5, kPairTileUs = 1.54;
+
+template <int D, bool SPLIT>
+cudaError_t launch_slots(const PrefillTcParams& p, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
+                         int dev, cudaStream_t s) {
+  static bool configured[64] = {};
+  if (dev >= 0 && dev < 64 && !configured[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(prefill_tc_kernel<D, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)Cfg<D>::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    configured[dev] = true;
+  }
+  const int tpc = (SPLIT ? 1 : 2) * p.tps;
+  const int64_t n_qt = ((int64_t)p.n_tokens + tpc - 1) / tpc;
+  if (n_qt * p.h_kv > INT32_MAX) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n_qt * p.h_kv));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = Cfg<D>::kSmemBytes;
+  cfg.stream = s;
+  return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, SPLIT>, p, mq, mk, mv);
+}
+
+// SM count of a device (it does not change).
+int sm_count(int dev) {
+  static int n[64] = {};
+  if (dev < 0 || dev >= 64) return 148;
+  if (n[dev] == 0 && cudaDeviceGetAttribute(&n[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n[dev] = 148;
+  return n[dev];
+}
+
 template <int D>
 cudaError_t launch(const PrefillTcParams& p, const void* q, const void* k, const void* v, cudaStream_t s) {
   CUtensorMap mq, mk, mv;
@@ -627,21 +726,27 @@ cudaError_t launch(const PrefillTcParams& p, const void* q, const void* k, const
     return cudaErrorInvalidValue;
   int dev = 0;
   cudaGetDevice(&dev);
-  static bool configured[64] = {};
-  if (dev >= 0 && dev < 64 && !configured[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(prefill_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)Cfg<D>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    configured[dev] = true;
-  }
-  const int64_t n_qt = ((int64_t)p.n_tokens + 2 * p.tps - 1) / (2 * p.tps);
-  if (n_qt * p.h_kv > INT32_MAX) return cudaErrorInvalidValue;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(n_qt * p.h_kv));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = Cfg<D>::kSmemBytes;
-  cfg.stream = s;
-  return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D>, p, mq, mk, mv);
+  // Two slots of queries per CTA are the better use of a full GPU, one slot with its key tiles
+  // shared out of a short sequence: there a CTA's chain of tiles is the whole time.  Each is
+  // costed as its longest CTA and, where it needs a second wave, the first CTA of that behind
+  // the shortest of the first (CTAs start in descending order), with the costs measured on
+  // GB300: us per call for 512 + 160 tokens, 28/4 heads, 16.9 with two slots, 14.5 split; 1500 +
+  // 160, 16/1 heads, 29.0 and 22.8; but 1300 + 160, 28/4 heads, 29.0 and 32.7.
+  const int sms = sm_count(dev);
+  auto cost = [&](int tpc, int tiles_per_round, double cta_us, double round_us) {
+    const int64_t n_qt = ((int64_t)p.n_tokens + tpc - 1) / tpc, n = n_qt * p.h_kv;
+    auto rounds = [&](int64_t cta) {
+      const int64_t last = std::min<int64_t>((n_qt - cta / p.h_kv) * tpc, p.n_tokens) - 1;
+      const int64_t tiles = last < p.prefix_len ? last / kBN + 1 : (p.prefix_len + kBN - 1) / kBN + 1;
+      return (double)((tiles + tiles_per_round - 1) / tiles_per_round);
+    };
+    double t = cta_us + round_us * rounds(0);
+    // (the second of two CTAs finds its code and parameters cached)
+    if (n > sms) t = std::max(t, 1.8 * cta_us + round_us * (rounds(sms - 1) + rounds(sms)));
+    return n > 2 * (int64_t)sms + sms / 16 ? 1e30 : t;  // (a few over two waves, the shortest, are no third)
+  };
+  const bool split = cost(p.tps, 2, kSplitCtaUs, kSplitRoundUs) < cost(2 * p.tps, 1, kPairCtaUs, kPairTileUs);
+  return split ? launch_slots<D, true>(p, mq, mk, mv, dev, s) : launch_slots<D, false>(p, mq, mk, mv, dev, s);
 }
 
 }  // namespace

@@ -125,3 +125,23 @@ def test_prefill_growing_maximum(D, at):
     assert np.abs(go - ro).max() <= MAX_ABS
     assert np.linalg.norm(go - ro) / np.linalg.norm(ro) <= REL_L2
     assert np.abs(lse.cpu().numpy() - rl).max() <= LSE_ABS
+
+
+@pytest.mark.parametrize("D,h_q,h_kv,prefix,lens", [
+    # one slot of queries, its key tiles shared out: one tile, two, an odd and an even number of them
+    (128, 28, 4, 100, [3]), (128, 28, 4, 120, [40]), (128, 16, 1, 300, [5, 0, 130]), (64, 14, 2, 400, [1, 20]),
+    # enough kv-heads for two waves of those: two slots of queries, the last one empty or full
+    (128, 64, 32, 640, [30, 34]), (128, 64, 32, 690, [14, 0, 65]), (64, 64, 32, 700, [3]),
+])
+def test_prefill_slots(D, h_q, h_kv, prefix, lens):
+    """fp32 against the oracle; bf16 output is the same result rounded to nearest even."""
+    _run(prefix, lens, h_q, h_kv, D, seed=31)
+    q, k, v = (_dev(x) for x in synth.prefill_inputs(31, prefix, lens, h_q, h_kv, D))
+    outs = []
+    for dt in (torch.float32, torch.bfloat16):
+        out, lse = torch.empty(q.shape, dtype=dt, device="cuda"), torch.empty(q.shape[:2], device="cuda")
+        prob = B.make_problem(h_q, h_kv, D, 16, 1.0 / math.sqrt(D), out_dtype=int(dt == torch.bfloat16))
+        B.pad_prefill_attn(prob, prefix, lens, q, k, v, out, lse)
+        outs.append(out)
+    torch.cuda.synchronize()
+    assert torch.equal(outs[0].bfloat16(), outs[1])
