@@ -148,8 +148,12 @@ __device__ __forceinline__ bool mbar_wait_b(uint64_t* bar, uint32_t parity, int3
 }
 // Wait used while draining after an abort: bounded, reports nothing.
 __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
-  const unsigned long long t0 = globaltimer();
-  while (!mbar_try_wait(bar, parity) && globaltimer() - t0 < kWaitNs) {
+  unsigned long long t0 = 0;  // (read only in a wait that lasts)
+  for (uint32_t i = 1; !mbar_try_wait(bar, parity); ++i) {
+    if ((i & 63u) != 0) continue;
+    const unsigned long long now = globaltimer();
+    if (t0 == 0) t0 = now;
+    if (now - t0 > kWaitNs) return;
   }
 }
 
