@@ -471,13 +471,16 @@ pad_status layout_for(const pad_problem* prob, int32_t n_videos, const int32_t* 
 }
 
 // head_dim 64 without a forced kernel (or the fused tail, which that head size does not have):
-// a plan on a workspace takes the tensor-core kernel.  It is the faster one at every size
-// measured, from 4 rows over 512 tokens (6.3 us per step against 14 on mma.sync and 20 on warp
-// shuffles) to 128 rows over 16384 tokens x 8 kv-heads (14.9 against 44) and 16 ragged videos
-// (38 against 113).  A plan without a workspace runs in the static array, where the scratch of
-// up to three waves of splits could exceed what the warp-level kernels need: it keeps those.
-// So does a plan on a workspace that would no longer fit that array (its calls may go there
-// too), after one split length for all videos has been tried.
+// a plan on a workspace with more than 8 rows per (video, kv-head) takes the tensor-core kernel.
+// It is the faster one at every size measured, from 16 rows over 512 tokens (6.4 us per step
+// against 14 on mma.sync) to 128 rows over 16384 tokens x 8 kv-heads (14.9 against 44) and 16
+// ragged videos (38 against 113), and the more exact one (P as two bf16 numbers against one).
+// Up to 8 rows the warp-shuffle kernel stays: it holds P in 32 bits, and two bf16 numbers are less
+// (relative error of the output against 64 bits, one event whose branch is one key, 512 to 4096
+// tokens: 2e-7 against 2e-6).  A plan without a workspace runs in the static array, where the
+// scratch of up to three waves of splits could exceed what the warp-level kernels need: it keeps
+// those.  So does a plan on a workspace that would no longer fit that array (its calls may go
+// there too), after one split length for all videos has been tried.
 pad_status compute_layout(const pad_problem* prob, int32_t n_videos, const int32_t* prefix_len, int32_t n_events,
                           const int32_t* event_video, int n_sms, bool on_workspace, Layout* L) {
   auto attempt = [&](int kern, bool per_video) {
@@ -486,7 +489,7 @@ pad_status compute_layout(const pad_problem* prob, int32_t n_videos, const int32
   };
   pad_status st = attempt(0, true);
   if (st != PAD_OK || !on_workspace || prob->head_dim != 64 || (prob->flags & (kPrefixFlags | PAD_FLAG_FUSED_MERGE)) ||
-      L->max_rows > 64 * 128)  // (the CTA list holds a row group in six bits)
+      L->prefix_kernel != PAD_FLAG_PREFIX_MMA || L->max_rows > 64 * 128)  // (the CTA list holds a row group in six bits)
     return st;
   const bool fits = L->total_bytes <= kStaticScratchBytes;
   for (bool per_video : {true, false}) {

@@ -89,10 +89,11 @@ struct Cfg {
   static constexpr uint32_t kOffV = kOffK + kStages * kTileBytes;
   static constexpr uint32_t kOffBar = kOffV + kStages * kTileBytes;
   static constexpr uint32_t kSmemBytes = kOffBar + 256;
-  // head_dim 64: P as the sum of two bf16 numbers, each with its own P.V.  The warp-level
-  // kernels of this head size hold P in 32 bits (up to 8 rows) or in bf16 on maxima of 64 tokens;
-  // one bf16 on the lazily followed maxima here is less exact than either (relative error of
-  // the output 1.6e-3 against 4.5e-5 and 1.4e-3), two are as exact as the former.
+  // head_dim 64: P as the sum of two bf16 numbers, each with its own P.V.  The mma.sync kernel of
+  // this head size, whose place this one takes (above 8 rows), holds P in one bf16 on maxima of 64
+  // tokens; one bf16 on the lazily followed maxima here is less exact (relative error of the
+  // output 1.6e-3 against 1.4e-3), two are far more so (2e-6 where the branch is one key; longer
+  // branches add the branch pass's own rounding, up to 3e-4).
   static constexpr bool kSplitP = D == 64;
   static constexpr uint32_t kIdescS = make_idesc(128, kBN, false);  // S = Q K^T: B = K tile, K-major
   static constexpr uint32_t kIdescPV = make_idesc(128, D, true);    // O += P V: B = V tile, N(=d)-major

@@ -702,7 +702,7 @@ def test_prefix_score_outgrows_running_maximum(at):
 # head_dim 64 on the tensor-core kernel: row-group, tile and page edges, several videos, every
 # option of the step
 _D64_TC_CASES = {
-    "one_row": dict(prefix=[130], epv=[1], lens=[0], h_q=1, h_kv=1),
+    "rows_9": dict(prefix=[130], epv=[1], lens=[0], h_q=9, h_kv=1),
     "rows_17": dict(prefix=[512], epv=[17], lens=[0] * 17, h_q=1, h_kv=1),
     "rows_127_129": dict(prefix=[700, 129], epv=[127, 129], lens=[1] * 256, h_q=2, h_kv=2),
     "g7_tiles": dict(prefix=[3000], epv=[19], lens=list(range(19)), h_q=14, h_kv=2),
@@ -841,3 +841,16 @@ def test_many_small_tasks_match_oracle(D, h_q, h_kv, one_call):
             assert info["partial_rows"] // (w.n_events * h_q) > 55 * 1024 // (h_q // h_kv * D * 4)
         check_bookkeeping(db, w, plan)
         check_outputs(db.out.cpu().numpy(), db.lse.cpu().numpy(), ref_o, ref_lse, f"{num_sms} SMs")
+
+
+@pytest.mark.parametrize("one_call", [True, False])
+@pytest.mark.parametrize("h_q,h_kv,events", [(1, 1, 1), (14, 2, 1), (8, 8, 8), (32, 8, 2)])
+def test_head_dim_64_few_rows_hold_weights_in_32_bits(h_q, h_kv, events, one_call):
+    """Branches of one key (weight 1, exact in any format) leave only the prefix pass's error.  A weight's
+    relative error is that of its fp32 score: 64 products whose sum rounds at about 2^-25 per term on
+    scores of a few units, 2.4e-7; four times that is the bar.  (P in two bf16 numbers: 2e-6.)"""
+    w = _w([2100], [events], [0] * events, seed=5, h_q=h_q, h_kv=h_kv, D=64)
+    db, plan = run_full(w, one_call=one_call)
+    assert plan.info()["prefix_kernel"] == B.FLAG_PREFIX_SIMT
+    ref_o, _ = oracle_step(w)
+    assert np.linalg.norm(db.out.double().cpu().numpy() - ref_o) <= 1e-6 * np.linalg.norm(ref_o)

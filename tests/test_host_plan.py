@@ -495,3 +495,17 @@ def test_step_executor_setters_validate(padlib):
         assert L.pad_step_set_rope(h, None, None, 0) == 0                  # off again
     finally:
         L.pad_step_destroy(h)
+
+
+@pytest.mark.parametrize("h_q,h_kv,events", [(1, 1, 8), (4, 1, 2), (14, 2, 1), (16, 2, 1), (8, 8, 8), (32, 8, 2)])
+def test_head_dim_64_few_rows_keep_the_fp32_kernel(padlib, h_q, h_kv, events):
+    """Up to 8 rows per (video, kv-head) a plan on a workspace is the one a host-only plan gives: on the
+    warp-shuffle kernel, whose weights are in 32 bits."""
+    for prefix in ([512], [5000, 700]):
+        E = events * len(prefix)
+        video = np.repeat(np.arange(len(prefix)), events)
+        prob = B.make_problem(h_q, h_kv, 64, num_sms=152)
+        plan = _dry_plan(prob, B.CacheState(E), dict(prefix_len=prefix, event_video=video, event_len=[0] * E, max_pages=1))
+        info = plan.info()
+        assert info["prefix_kernel"] == B.FLAG_PREFIX_SIMT
+        assert B.pad_workspace_size(prob, prefix, video) == info["workspace_bytes"]
