@@ -223,7 +223,7 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
   const int key0 = (lane < 16 ? 0 : nkr - 16) + kb0 + lane;
   const int pi0 = key0 / ps;
   int page0 = -1;
-  if (!causal && kb0 < nkr && pi0 < p.max_pages) page0 = p.page_table[(size_t)e * p.max_pages + pi0];
+  if (!causal && kb0 < nkr && pi0 < p.max_pages) page0 = __ldcg(p.page_table + (size_t)e * p.max_pages + pi0);
   if (!ROPE) {
     for (int i = tid; i < 16 * CH; i += NT) {
       const int g = i / CH, c = i - (i / CH) * CH;
@@ -270,7 +270,7 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
       }
     }
     const int pi = t / ps;
-    return pool_row(row, pi, t - pi * ps, p.page_table[(size_t)row * p.max_pages + pi]);
+    return pool_row(row, pi, t - pi * ps, __ldcg(p.page_table + (size_t)row * p.max_pages + pi));
   };
   long long place = -1;                       // pool row of this lane's key (see above)
   if (kb0 < nkr && key0 < nk) place = causal ? row_of(key0) : pool_row(e, pi0, key0 - pi0 * ps, page0);
@@ -332,7 +332,7 @@ __device__ __forceinline__ void run_task(const KParams& p, const __nv_bfloat16* 
         const int c = lane % CH;
         const bool isv = lane >= CH;
         const uint4 v = (ROPE && !isv) ? rope_chunk8(knew + new_row, D, c * 8, cs)
-                                       : *reinterpret_cast<const uint4*>((isv ? vnew : knew) + new_row + c * 8);
+                                       : __ldcg(reinterpret_cast<const uint4*>((isv ? vnew : knew) + new_row + c * 8));
         *reinterpret_cast<uint4*>(const_cast<__nv_bfloat16*>(isv ? vpool : kpool) + (size_t)pl * D + c * 8) = v;
       }
     }

@@ -79,6 +79,11 @@ __device__ __forceinline__ void ld_stream4(uint4 (&v)[4], const void* p0, const 
       : "l"(p0), "l"(p1), "l"(p2), "l"(p3));
 }
 
+// One bf16 element past L1.  (The header's __ldcg of this type may be moved ahead of the wait.)
+__device__ __forceinline__ float ld_bf16(const __nv_bfloat16* p) {
+  return __bfloat162float(__ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(p))));
+}
+
 __device__ __forceinline__ void unpack8(const uint4 v, float* f) {
   const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -194,7 +199,7 @@ __global__ void __launch_bounds__(kScoreThreads) ground_score_kernel(const __nv_
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   grid_wait();
   grid_release();
-  for (int c = threadIdx.x; c < d; c += kScoreThreads) gs[c] = __bfloat162float(__ldcg(g + (size_t)i * d + c));
+  for (int c = threadIdx.x; c < d; c += kScoreThreads) gs[c] = ld_bf16(g + (size_t)i * d + c);
   __syncthreads();
   // a warp per segment row (lanes over its float4 columns), four rows in flight per warp
   float best = -__builtin_huge_valf();
@@ -433,7 +438,7 @@ __global__ void __launch_bounds__(32 * kEventWarps) attn_event_kernel(const __gr
       num += red[r][threadIdx.x];
       den += ared[r];
     }
-    const float base = __bfloat162float(g_emb[(size_t)i * d + col]);
+    const float base = ld_bf16(g_emb + (size_t)i * d + col);
     out[(size_t)i * d + col] = den > 0.f ? base + num / den : base;
   }
 }

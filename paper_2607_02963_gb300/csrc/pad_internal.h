@@ -201,15 +201,19 @@ __device__ __forceinline__ float rope_one(float own, float partner, float c, flo
              : __fadd_rn(__fmul_rn(own, c), __fmul_rn(partner, s));
 }
 // Elements d0 .. d0+7 (d0 a multiple of 8) of a bf16 row of length D, as packed bf16.
+// The row and the table are read past L1, and not through the read-only path, as everything is
+// that a grid ahead of a kernel with programmatic dependent launch may write: that path takes
+// the data to be constant while the kernel runs, and its loads were seen to be issued ahead of
+// the kernel's griddepcontrol.wait (q with RoPE in the prefix kernel).
 __device__ __forceinline__ uint4 rope_chunk8(const __nv_bfloat16* row, int D, int d0, const float* cs) {
   const int h = D >> 1;
   const bool low = d0 < h;
   const int i0 = low ? d0 : d0 - h;
-  const uint4 xa = *reinterpret_cast<const uint4*>(row + d0);
-  const uint4 xb = *reinterpret_cast<const uint4*>(row + (low ? d0 + h : i0));
-  const float4 c0 = *reinterpret_cast<const float4*>(cs + i0), c1 = *reinterpret_cast<const float4*>(cs + i0 + 4);
-  const float4 s0 = *reinterpret_cast<const float4*>(cs + h + i0),
-               s1 = *reinterpret_cast<const float4*>(cs + h + i0 + 4);
+  const uint4 xa = __ldcg(reinterpret_cast<const uint4*>(row + d0));
+  const uint4 xb = __ldcg(reinterpret_cast<const uint4*>(row + (low ? d0 + h : i0)));
+  const float4 c0 = __ldcg(reinterpret_cast<const float4*>(cs + i0)), c1 = __ldcg(reinterpret_cast<const float4*>(cs + i0 + 4));
+  const float4 s0 = __ldcg(reinterpret_cast<const float4*>(cs + h + i0)),
+               s1 = __ldcg(reinterpret_cast<const float4*>(cs + h + i0 + 4));
   const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
   const float s[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
   const uint32_t a[4] = {xa.x, xa.y, xa.z, xa.w}, b[4] = {xb.x, xb.y, xb.z, xb.w};

@@ -134,17 +134,17 @@ __global__ void append_kernel(const __grid_constant__ KParams p, const uint4* __
   if (idx < p.n_counters) p.counters[idx] = 0u;
   if (!mine) return;
   const size_t src = ((size_t)e * p.h_kv + h) * chunks + c;
-  const uint4 v = v_new[src];
+  const uint4 v = __ldcg(v_new + src);
   const uint4 k = p.rope_cs != nullptr
                       ? rope_chunk8(reinterpret_cast<const __nv_bfloat16*>(k_new + (src - c)), p.head_dim, 8 * c,
                                     p.rope_cs + (size_t)ev.pos * p.head_dim)
-                      : k_new[src];
+                      : __ldcg(k_new + src);
   int page;
   if (ev.new_page >= 0) {
     page = ev.new_page;
     if (rem == 0) p.page_table[(size_t)e * p.max_pages + pidx] = page;
   } else {
-    page = p.page_table[(size_t)e * p.max_pages + pidx];
+    page = __ldcg(p.page_table + (size_t)e * p.max_pages + pidx);
   }
   if (page < 0 || page >= p.n_pages) {
     pad_set_error(p.header, p.gen, PAD_ERR_DEVICE_BOUNDS, e, pidx, page);

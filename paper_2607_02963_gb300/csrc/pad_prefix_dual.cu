@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (qrow < R) {
         const int el = qrow / p.group;
         const int gh = qrow - el * p.group;
-        qv[i] = __ldg(reinterpret_cast<const uint4*>(
+        qv[i] = __ldcg(reinterpret_cast<const uint4*>(
             q + ((size_t)(it.first_event + el) * p.h_q + kvh * p.group + gh) * kD + 8 * c));
       }
     }

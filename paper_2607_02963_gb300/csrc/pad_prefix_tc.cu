@@ -354,22 +354,24 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
     for (int i = 0; i < kLd; ++i) asm volatile("" : "+l"(src[i]));  // (not sunk behind the wait)
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    // (past L1 and never through the read-only path, see rope_chunk8: the grid ahead may have
+    // been writing q while this one was resident)
 #pragma unroll
     for (int i = 0; i < kLd; ++i) {
       if constexpr (ROPE) {
         qv[2 * i] = qv[2 * i + 1] = make_uint4(0u, 0u, 0u, 0u);
         tbl[4 * i] = tbl[4 * i + 1] = tbl[4 * i + 2] = tbl[4 * i + 3] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (src[i] != nullptr) {
-          qv[2 * i] = __ldg(src[i]);
-          qv[2 * i + 1] = __ldg(src[i] + kPairs);
+          qv[2 * i] = __ldcg(src[i]);
+          qv[2 * i + 1] = __ldcg(src[i] + kPairs);
           const float4* cs = reinterpret_cast<const float4*>(p.rope_cs + (size_t)pos[i] * D + 8 * cc);
-          tbl[4 * i] = __ldg(cs);
-          tbl[4 * i + 1] = __ldg(cs + 1);
-          tbl[4 * i + 2] = __ldg(cs + D / 8);
-          tbl[4 * i + 3] = __ldg(cs + D / 8 + 1);
+          tbl[4 * i] = __ldcg(cs);
+          tbl[4 * i + 1] = __ldcg(cs + 1);
+          tbl[4 * i + 2] = __ldcg(cs + D / 8);
+          tbl[4 * i + 3] = __ldcg(cs + D / 8 + 1);
         }
       } else {
-        qv[i] = src[i] != nullptr ? __ldg(src[i]) : make_uint4(0u, 0u, 0u, 0u);
+        qv[i] = src[i] != nullptr ? __ldcg(src[i]) : make_uint4(0u, 0u, 0u, 0u);
       }
     }
   }
