@@ -263,14 +263,19 @@ pad_status pad_plan_destroy(pad_plan_t* plan);
  * One new token per branch per step (Eq. 3).  A plan built without a workspace (host-only)
  * is accepted too: its descriptors and status word then live in the library's static scratch
  * array (see pad_event_decode_attn_static, whose rules apply), so a caller with no device
- * scratch can run a whole step as pad_kv_append + pad_event_decode_attn_static. */
+ * scratch can run a whole step as pad_kv_append + pad_event_decode_attn_static.
+ * Its kernel uses programmatic dependent launch: it may start while the grid before it on the
+ * stream is still running, and waits for that grid's completion before it touches the tensors. */
 pad_status pad_kv_append(const pad_plan_t* plan, const void* k_new, const void* v_new,
                          void* k_pool, void* v_pool, pad_stream_t stream);
 
 /* a3-a5: decode attention of every active branch's query under the event-factorized
  * mask (Sec. 3.4): the shared prefix of its video plus its own event_len[e] + 1 private
  * keys (read through page_table, so pad_kv_append must precede this call on the stream).
- * All pointers device, 16-byte aligned; lse may be NULL. */
+ * All pointers device, 16-byte aligned; lse may be NULL.  Its first kernel uses programmatic
+ * dependent launch as pad_kv_append's does and reads none of these tensors before the grid
+ * ahead, and all that grid waited for, has completed: k_prefix and v_prefix too may be written
+ * by any grid ahead of this call. */
 pad_status pad_event_decode_attn(const pad_plan_t* plan, const void* q, const void* k_prefix,
                                  const void* v_prefix, const void* k_pool, const void* v_pool,
                                  void* out, float* lse, pad_stream_t stream);

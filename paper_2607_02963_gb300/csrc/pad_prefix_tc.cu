@@ -289,10 +289,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   TcBars* bars = reinterpret_cast<TcBars*>(smem + C::kOffBar);
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   // Launched so that it may start while the grid before it (the previous step, this step's
-  // append, or the caller's own kernel that wrote q) finishes.  Barrier set-up, TMEM
-  // allocation and the first K/V tile overlap that grid; every thread that touches other
-  // global memory waits for it first (the Q loads), and the block barrier after them orders
-  // everything else, including the release of the grid behind this one.
+  // append, or the caller's own kernel that wrote q) finishes.  Barrier set-up and TMEM
+  // allocation overlap that grid, and so does the first K/V tile of a one-call step; every
+  // thread that touches other global memory waits for it first (the Q loads), and the block
+  // barrier after them orders everything else, including the release of the grid behind this one.
 
   // the CTA's work item and 128-row group: from the plan's CTA list, or the dense grid
   int item, group;
@@ -380,15 +380,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     // The first K and V tile go out first (their barriers initialised, then the loads),
     // before the other barriers, TMEM allocation and the block barrier; the producer warps
     // issue the rest once that K tile has landed, so that every CTA's first tile is not
-    // queued in DRAM behind the later tiles of all the others.  The prefix K/V is written by
-    // no grid of the library's own that may run ahead of this one (and, by the call's
-    // contract, by no grid that releases its dependents before its writes), so that tile is
-    // requested even before the wait for the grid ahead; nothing else is.
+    // queued in DRAM behind the later tiles of all the others.  In a one-call step the prefix
+    // K/V is written by no grid that may run ahead of this one (none of the library's own, and by
+    // that call's contract none that releases its dependents before its writes), so that tile is
+    // requested even before the wait for the grid ahead; nothing else is.  The attention call of
+    // a two-call step has no such contract, and the append ahead of it releases this grid while
+    // it still waits itself, for a grid that may be writing the prefix: there the tile waits too
+    // (13 events over 8219 tokens with RoPE: 13.3 us per step, 12.7 without that wait).
     mbar_init(&bars->kfull[0], 1);
     mbar_init(&bars->vfull[0], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmK)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
+    if (p.k_new == nullptr) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (n_tiles > 0) {
       load_tile(&tmK, C::kOffK, 0, &bars->kfull[0]);
       load_tile(&tmV, C::kOffV, 0, &bars->vfull[0]);

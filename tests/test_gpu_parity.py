@@ -857,12 +857,13 @@ def test_head_dim_64_few_rows_hold_weights_in_32_bits(h_q, h_kv, events, one_cal
     assert np.linalg.norm(db.out.double().cpu().numpy() - ref_o) <= 1e-6 * np.linalg.norm(ref_o)
 
 
-@pytest.mark.parametrize("late", ["inputs_ahead_of_append", "q_ahead_of_attention", "inputs_ahead_of_one_call"])
+@pytest.mark.parametrize("late", ["all_ahead_of_append", "prefix_ahead_of_attention", "inputs_ahead_of_one_call"])
 @pytest.mark.parametrize("D,flags,rope", [(128, 0, False), (128, 0, True), (64, 0, False), (128, B.FLAG_PREFIX_DUAL, False),
                                           (128, B.FLAG_FUSED_MERGE, False), (128, B.FLAG_PREFIX_MMA, False)])
 def test_step_waits_for_a_grid_that_releases_early(late, D, flags, rope):
-    """q and the new rows that a grid ahead of the step stores long after it has released its dependents are
-    seen by the step: ahead of the two calls, between them, and ahead of the one call."""
+    """What a grid ahead of the step stores long after it has released its dependents is seen by the step:
+    everything ahead of the two calls, the prefix between them, q and the new rows ahead of the one call
+    (whose prefix must not be written so)."""
     w = _w([900, 130], [5, 6], [3, 0, 16, 5, 40, 1, 31, 2, 7, 15, 64], D=D, h_q=14, h_kv=2, seed=9)
     db = DeviceBatch(w, flags=flags, fill_nan=False)
     ref = w
@@ -871,8 +872,8 @@ def test_step_waits_for_a_grid_that_releases_early(late, D, flags, rope):
         table = synth.rope_table(int(pos.max()) + 1, D)
         db.set_rope(pos, table)
         ref = oracle.rotated_workload(w, pos, table)
-    names = {"inputs_ahead_of_append": ("q", "k_new", "v_new"),
-             "q_ahead_of_attention": ("q",),
+    names = {"all_ahead_of_append": ("q", "k_new", "v_new", "k_prefix", "v_prefix"),
+             "prefix_ahead_of_attention": ("q", "k_prefix", "v_prefix"),
              "inputs_ahead_of_one_call": ("q", "k_new", "v_new")}[late]
     true = {n: getattr(db, n).clone() for n in names}
     side = torch.cuda.Stream()
@@ -883,13 +884,13 @@ def test_step_waits_for_a_grid_that_releases_early(late, D, flags, rope):
         db.out.fill_(float("nan"))
         torch.cuda.synchronize()
         pairs = [(getattr(db, n), true[n]) for n in names]
-        if late == "q_ahead_of_attention":
+        if late == "prefix_ahead_of_attention":
             B.pad_kv_append(plan, db.k_new, db.v_new, db.k_pool, db.v_pool, side)
             late_store(pairs, side)
             B.pad_event_decode_attn(plan, db.q, db.k_prefix, db.v_prefix, db.k_pool, db.v_pool, db.out, db.lse, side)
         else:
             late_store(pairs, side)
-            if late == "inputs_ahead_of_append":
+            if late == "all_ahead_of_append":
                 B.pad_kv_append(plan, db.k_new, db.v_new, db.k_pool, db.v_pool, side)
                 B.pad_event_decode_attn(plan, db.q, db.k_prefix, db.v_prefix, db.k_pool, db.v_pool, db.out, db.lse, side)
             else:
