@@ -140,7 +140,10 @@ pad_status pad_cache_state_import(pad_cache_state* cache, const uint8_t* used, i
 typedef struct pad_plan_t pad_plan_t;
 
 /* Bytes of device workspace pad_plan needs for this batch (host arrays, same
- * meaning as in pad_plan).  Returns 0 on invalid arguments. */
+ * meaning as in pad_plan).  Returns 0 on invalid arguments.  At head_dim 128 a batch of fewer
+ * events may need more (fewer row groups leave room for more splits): a workspace for several
+ * batches takes the largest of their sizes.  At head_dim 64 a plan that finds less than its
+ * tensor-core kernel wants takes the warp-level kernel, whose need does not grow so. */
 size_t pad_workspace_size(const pad_problem* prob, int32_t n_videos, const int32_t* prefix_len,
                           int32_t n_events, const int32_t* event_video);
 

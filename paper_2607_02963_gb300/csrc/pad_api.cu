@@ -126,6 +126,7 @@ struct Layout {
   int64_t n_counters = 0;
   size_t off_videos = 0, off_events = 0, off_items = 0, off_tasks = 0, upload_bytes = 0;
   size_t off_ml = 0, off_o = 0, off_cnt = 0, total_bytes = 0;
+  size_t warp_level_bytes = 0;  // head_dim 64 on the tensor cores: total_bytes of the warp-level layout
 };
 
 // Device scratch inside the library for callers that have none to give (see
@@ -480,9 +481,12 @@ pad_status layout_for(const pad_problem* prob, int32_t n_videos, const int32_t* 
 // tokens: 2e-7 against 2e-6).  A plan without a workspace runs in the static array, where the
 // scratch of up to three waves of splits could exceed what the warp-level kernels need: it keeps
 // those.  So does a plan on a workspace that would no longer fit that array (its calls may go
-// there too), after one split length for all videos has been tried.
+// there too), after one split length for all videos has been tried, and one whose workspace has
+// only `room` bytes: the tensor-core scratch does not shrink with the batch (14/2 heads, 16384
+// tokens: 1.9 MB for 20 events in two row groups, 2.9 MB for 18 in one), so a workspace sized for
+// the first batch of a generation loop must still do as its events end.
 pad_status compute_layout(const pad_problem* prob, int32_t n_videos, const int32_t* prefix_len, int32_t n_events,
-                          const int32_t* event_video, int n_sms, bool on_workspace, Layout* L) {
+                          const int32_t* event_video, int n_sms, bool on_workspace, size_t room, Layout* L) {
   auto attempt = [&](int kern, bool per_video) {
     *L = Layout();
     return layout_for(prob, n_videos, prefix_len, n_events, event_video, n_sms, kern, per_video, L);
@@ -491,10 +495,14 @@ pad_status compute_layout(const pad_problem* prob, int32_t n_videos, const int32
   if (st != PAD_OK || !on_workspace || prob->head_dim != 64 || (prob->flags & (kPrefixFlags | PAD_FLAG_FUSED_MERGE)) ||
       L->prefix_kernel != PAD_FLAG_PREFIX_MMA || L->max_rows > 64 * 128)  // (the CTA list holds a row group in six bits)
     return st;
-  const bool fits = L->total_bytes <= kStaticScratchBytes;
+  const size_t warp_level_bytes = L->total_bytes;
+  const size_t most = std::min(room, warp_level_bytes <= kStaticScratchBytes ? kStaticScratchBytes : SIZE_MAX);
   for (bool per_video : {true, false}) {
     st = attempt(PAD_FLAG_PREFIX_TC, per_video);
-    if (st == PAD_OK && (!fits || L->total_bytes <= kStaticScratchBytes)) return st;
+    if (st == PAD_OK && L->total_bytes <= most) {
+      L->warp_level_bytes = warp_level_bytes;
+      return st;
+    }
   }
   return attempt(0, true);
 }
@@ -744,8 +752,9 @@ size_t pad_workspace_size(const pad_problem* prob, int32_t n_videos, const int32
   if (check_problem(prob) != PAD_OK) return 0;
   Layout L;
   const int sms = prob->num_sms > 0 ? prob->num_sms : query_num_sms();
-  if (compute_layout(prob, n_videos, prefix_len, n_events, event_video, sms, true, &L) != PAD_OK) return 0;
-  return L.total_bytes;
+  if (compute_layout(prob, n_videos, prefix_len, n_events, event_video, sms, true, SIZE_MAX, &L) != PAD_OK) return 0;
+  // (room for either kernel, so that a smaller batch, whose warp-level layout is no larger, fits)
+  return std::max(L.total_bytes, L.warp_level_bytes);
 }
 
 pad_status pad_plan(const pad_problem* prob, pad_cache_state* cache, int32_t n_videos,
@@ -769,7 +778,8 @@ pad_status pad_plan(const pad_problem* prob, pad_cache_state* cache, int32_t n_v
   const int sms = prob->num_sms > 0 ? prob->num_sms : (workspace ? query_num_sms() : kDefaultSms);
   auto* plan = new pad_plan_t();
   Layout& L = plan->lay;
-  st = compute_layout(prob, n_videos, prefix_len, n_events, event_video, sms, workspace != nullptr, &L);
+  st = compute_layout(prob, n_videos, prefix_len, n_events, event_video, sms, workspace != nullptr, workspace_bytes,
+                      &L);
   if (st != PAD_OK) {
     delete plan;
     return st;

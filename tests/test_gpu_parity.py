@@ -901,3 +901,28 @@ def test_step_waits_for_a_grid_that_releases_early(late, D, flags, rope):
         check_bookkeeping(db, ref, plan)
         ref_o, ref_lse = oracle_step(ref)
         check_outputs(db.out.cpu().numpy(), db.lse.cpu().numpy(), ref_o, ref_lse, f"{late}, turn {turn}")
+
+
+def test_head_dim_64_batch_shrinks_on_one_workspace():
+    """Events end and leave the list while the workspace stays the one sized for the first batch: every step
+    plans.  One that holds only what the warp-level kernel needs gets that kernel."""
+    first = None
+    for n in (20, 18, 12, 9, 5, 2, 1):
+        w = _w([16384], [n], [3] * n, h_q=14, h_kv=2, D=64, seed=n)
+        ref_o, ref_lse = oracle_step(w)
+        for tight in (False, True):
+            db = DeviceBatch(w)
+            first = db.workspace if first is None else first
+            db.workspace = first
+            if tight:
+                dry = B.pad_plan(db.problem, B.CacheState(w.n_pages), w.prefix_len, w.event_video, w.event_len,
+                                 max_pages=w.max_pages)
+                db.workspace = first[:dry.info()["workspace_bytes"]]
+            plan = db.run_step(one_call=True)
+            torch.cuda.synchronize()
+            B.pad_device_status(plan)
+            info = plan.info()
+            assert info["workspace_bytes"] <= db.workspace.numel()
+            assert info["prefix_kernel"] == (B.FLAG_PREFIX_SIMT if n == 1 else B.FLAG_PREFIX_TC) or tight
+            assert not (tight and n == 9) or info["prefix_kernel"] == B.FLAG_PREFIX_MMA
+            check_outputs(db.out.cpu().numpy(), db.lse.cpu().numpy(), ref_o, ref_lse, f"{n} events, {tight}")

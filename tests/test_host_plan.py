@@ -1,5 +1,6 @@
 """Host logic of the C ABI (no GPU): page bookkeeping of pad_plan against the oracle's
 simulation (bit-exact), the split-KV work list, and argument validation."""
+import ctypes
 import json
 import os
 
@@ -509,3 +510,31 @@ def test_head_dim_64_few_rows_keep_the_fp32_kernel(padlib, h_q, h_kv, events):
         info = plan.info()
         assert info["prefix_kernel"] == B.FLAG_PREFIX_SIMT
         assert B.pad_workspace_size(prob, prefix, video) == info["workspace_bytes"]
+
+
+@pytest.mark.parametrize("h_q,h_kv,prefix,events", [(14, 2, [16384], 20), (32, 8, [4096], 40), (4, 1, [9000, 700], 33)])
+def test_head_dim_64_workspace_serves_a_shrinking_batch(padlib, h_q, h_kv, prefix, events):
+    """A workspace sized for the first batch of a generation loop is enough for every smaller one.  (Without
+    a GPU the plan gets as far as its page-locked image, which comes after the check of the size.)"""
+    prob = B.make_problem(h_q, h_kv, 64, num_sms=152)
+
+    def batch(n):
+        return np.asarray(prefix, dtype=np.int32), np.repeat(np.arange(len(prefix), dtype=np.int32), n)
+
+    room = B.pad_workspace_size(prob, *batch(events))
+    host_only = B.pad_plan(prob, B.CacheState(events * len(prefix)), *batch(events), [0] * events * len(prefix),
+                           max_pages=1).info()
+    assert room >= host_only["workspace_bytes"]      # (what such a workspace held before, too)
+    lib, cache = B.lib(), B.CacheState(events * len(prefix))
+    for n in range(1, events + 1):
+        pl, ev = batch(n)
+        el, h = np.zeros(ev.size, dtype=np.int32), ctypes.c_void_p()
+        # (addresses are not looked at before the image exists)
+        for size, ok in ((room, True), (int(host_only["workspace_bytes"]), True), (256, False)):
+            st = lib.pad_plan(ctypes.byref(prob), cache.handle, pl.size, pl.ctypes.data_as(B._I32P), None, ev.size,
+                              ev.ctypes.data_as(B._I32P), el.ctypes.data_as(B._I32P), 4096, 1, 4096, size, None,
+                              ctypes.byref(h))
+            assert (st != 4) == ok, (n, size, st)
+            if st == 0:
+                lib.pad_plan_release_new_pages(h, cache.handle)
+                lib.pad_plan_destroy(h)
