@@ -393,7 +393,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           // half at +kHalfBytes (leading byte offset), 8-row groups 1024 apart.
           for (int i = 0; i < n_seq && ok; ++i) {
             const int g = i & 1, k = i >> 1, t = dual ? k : i, s = t % VS;
-            if (!dual || g == 0) ok = dwait(&bars->vfull[s], (uint32_t)((t / VS) & 1), bars, p.header, 4);
+            if (!dual || g == 0) {
+              ok = dwait(&bars->vfull[s], (uint32_t)((t / VS) & 1), bars, p.header, 4);
+              if (ok && (t + 1) * kBN > ntok) zero_v_rows<2>(smem + v_off(s), ntok - t * kBN, 0, 1);
+            }
             const uint64_t vb = sdesc(sbase + v_off(s), kHalfBytes, 1024);
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {

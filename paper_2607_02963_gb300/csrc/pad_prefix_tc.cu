@@ -15,7 +15,8 @@
 //               ahead of the softmax
 //   warp 2      TMEM allocator (512 columns) and deallocator, and issuer of O += P V with P
 //               read back from TMEM
-//   warp 3      TMA producer of V tiles (refilled once the P.V of the tile completed)
+//   warp 3      TMA producer of V tiles (refilled once the P.V of the tile completed); clears
+//               the rows of the last one that lie past the split's end
 //   warps 4-11  softmax: two warps per 32-row lane quarter, each with 16 of the quarter's rows
 //               and all 128 columns of a tile (two rows per thread, a row shared by a quad of
 //               lanes), so the warps never meet.  Online sum in base 2, P written as packed
@@ -113,6 +114,7 @@ struct TcBars {
   uint64_t drain_pv;          // every P.V MMA has completed (P.V issuer)
   uint64_t qready;            // Q staged in shared memory (8 warp arrivals)
   uint64_t tdone;             // the softmax warps are done with TMEM (8 warp arrivals)
+  uint64_t vpart;             // the last V tile, where the split ends inside it, has landed
   uint64_t gen;               // the plan's generation, for the status word
   uint32_t tmem_base;
   int32_t abort;
@@ -312,6 +314,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int n_tiles = (ntok + kBN - 1) / kBN;
   const int kvh = it.kvh;
   const int tok0 = (int)it.tok0;
+  // The split ends inside its last tile: that V tile is loaded to a barrier of its own, and becomes
+  // full (vfull) once the producer has cleared its rows past the end.
+  const bool part = ntok % kBN != 0;
   auto load_tile = [&](const CUtensorMap* map, uint32_t off, int t, uint64_t* full) {
     mbar_expect_tx(full, C::kTileBytes);
 #pragma unroll
@@ -389,13 +394,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     // (13 events over 8219 tokens with RoPE: 13.3 us per step, 12.7 without that wait).
     mbar_init(&bars->kfull[0], 1);
     mbar_init(&bars->vfull[0], 1);
+    mbar_init(&bars->vpart, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmK)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
     if (p.k_new == nullptr) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (n_tiles > 0) {
       load_tile(&tmK, C::kOffK, 0, &bars->kfull[0]);
-      load_tile(&tmV, C::kOffV, 0, &bars->vfull[0]);
+      load_tile(&tmV, C::kOffV, 0, part && n_tiles == 1 ? &bars->vpart : &bars->vfull[0]);
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int s = 0; s < kStages; ++s) {
@@ -441,12 +447,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0 || warp == 3) {
     // ------------------------------------------------------------ TMA producers
+    const bool isK = warp == 0;
+    bool ok = true;
     if (lane == 0) {
-      const bool isK = warp == 0;
       const CUtensorMap* map = isK ? &tmK : &tmV;
       int issued = min(1, n_tiles);  // tile 0 went out in the prologue
       // the other stages fill once the first K tile has landed
-      bool ok = n_tiles <= 1 || mbar_wait(&bars->kfull[0], 0u, bars, p.header, isK ? 1 : 2);
+      ok = n_tiles <= 1 || mbar_wait(&bars->kfull[0], 0u, bars, p.header, isK ? 1 : 2);
       for (int t = 1; t < n_tiles && ok; ++t) {
         const int s = t % kStages;
         if (t >= kStages) {
@@ -455,7 +462,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = mbar_wait(freed, (uint32_t)((t / kStages - 1) & 1), bars, p.header, isK ? 1 : 2);
           if (!ok) break;
         }
-        uint64_t* full = isK ? &bars->kfull[s] : &bars->vfull[s];
+        uint64_t* full = isK ? &bars->kfull[s] : (part && t == n_tiles - 1 ? &bars->vpart : &bars->vfull[s]);
         load_tile(map, (isK ? C::kOffK : C::kOffV) + s * C::kTileBytes, t, full);
         issued = t + 1;
       }
@@ -463,11 +470,24 @@ __global__ void __launch_bounds__(kThreads, 1)
         // the loads already issued must land before the CTA leaves
         for (int t = max(0, issued - kStages); t < issued; ++t) {
           uint64_t* full = isK ? &bars->kfull[t % kStages] : &bars->vfull[t % kStages];
-          drain_wait(full, (uint32_t)((t / kStages) & 1));
+          if (!isK && part && t == n_tiles - 1)
+            drain_wait(&bars->vpart, 0u);
+          else
+            drain_wait(full, (uint32_t)((t / kStages) & 1));
         }
       }
     }
     __syncwarp();
+    if (!isK && part && __shfl_sync(0xffffffffu, (int)ok, 0)) {
+      const int s = (n_tiles - 1) % kStages;
+      if (mbar_wait_warp(&bars->vpart, 0u, bars, p.header, 7)) {
+        zero_v_rows<C::kHalves>(smem + C::kOffV + s * C::kTileBytes, ntok % kBN, lane, 32);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->vfull[s]);
+      } else {
+        drain_wait(&bars->vpart, 0u);
+      }
+    }
     if (warp == 0 && !p.causal) prefetch_branch_tasks<D>(p, q, kpool, vpool, lane);
   } else if (warp == 1 || warp == 2) {
     // ------------------------------------------------------------ MMA issuers

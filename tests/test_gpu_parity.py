@@ -5,6 +5,7 @@ outputs within max-abs <= 1e-2 and relative-L2 <= 2e-3 (bf16 in, fp32
 accumulate); the natural-log LSE within 1e-3 absolute (a log of an fp32 sum of
 positive terms: its error is the relative error of that sum, ~1e-6 here).
 """
+import dataclasses
 import hashlib
 
 import numpy as np
@@ -926,3 +927,30 @@ def test_head_dim_64_batch_shrinks_on_one_workspace():
             assert info["prefix_kernel"] == (B.FLAG_PREFIX_SIMT if n == 1 else B.FLAG_PREFIX_TC) or tight
             assert not (tight and n == 9) or info["prefix_kernel"] == B.FLAG_PREFIX_MMA
             check_outputs(db.out.cpu().numpy(), db.lse.cpu().numpy(), ref_o, ref_lse, f"{n} events, {tight}")
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("one_call", [True, False])
+@pytest.mark.parametrize("D,flags", [(64, 0), (64, B.FLAG_PREFIX_MMA), (128, 0), (128, B.FLAG_PREFIX_DUAL),
+                                     (128, B.FLAG_FUSED_MERGE)])
+def test_tokens_outside_a_prefix_do_not_reach_its_result(D, flags, one_call, bad):
+    """Non-finite K and V in the gaps that prefix_offset leaves in the buffers, and all through the next video,
+    leave a video's own result as it is (prefixes that end inside a tile, at its edge and after one token)."""
+    w = _w([130, 256, 301, 1, 500], [3, 20, 4, 2, 5], [3] * 34, h_q=14, h_kv=2, D=D, seed=21)
+    ref_o, ref_lse = oracle_step(w)
+    for last_is_bad in (False, True):
+        db = DeviceBatch(w, flags=flags)
+        off = np.cumsum([37] + [int(n) + gap for n, gap in zip(w.prefix_len[:-1], (61, 0, 1, 300))]).astype(np.int64)
+        for name in ("k_prefix", "v_prefix"):
+            packed = getattr(db, name)
+            gaps = torch.full((int(off[-1]) + 500 + 90, *packed.shape[1:]), bad, dtype=torch.bfloat16, device="cuda")
+            for b, n in enumerate(w.prefix_len[:-1] if last_is_bad else w.prefix_len):
+                o = int(w.prefix_offset[b])
+                gaps[int(off[b]):int(off[b]) + int(n)] = packed[o:o + int(n)]
+            setattr(db, name, gaps)
+        db.w = dataclasses.replace(w, prefix_offset=off)
+        plan = db.run_step(one_call=one_call)
+        torch.cuda.synchronize()
+        B.pad_device_status(plan)
+        mine = slice(0, 29) if last_is_bad else slice(0, 34)
+        check_outputs(db.out.cpu().numpy()[mine], db.lse.cpu().numpy()[mine], ref_o[mine], ref_lse[mine], f"{bad}")
