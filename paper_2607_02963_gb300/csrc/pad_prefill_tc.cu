@@ -16,7 +16,8 @@
 // the whole time, and this halves it (512 + 160 tokens, 28/4 heads: 16.7 -> 14.5 us; 1100 + 160,
 // 16/1 heads: 24.8 -> 16.8).
 //
-//   warps 0, 3  TMA producers of K and V tiles (64-column boxes, 128-byte swizzle)
+//   warps 0, 3  TMA producers of K and V tiles (64-column boxes, 128-byte swizzle); warp 3 clears
+//               the rows of the last V tile that no row here sees
 //   warp 1      S issuer: S_g(k) = Q_g K(k)^T
 //   warp 2      TMEM allocation (512 columns) and deallocation, and P.V issuer: O_g += P_g(k)
 //               V(k), P read back from TMEM, 96 keys and then the last 32
@@ -120,6 +121,7 @@ struct Bars {
   uint64_t pvdone[2];         // its P.V has completed
   uint64_t drain_s, drain_pv; // every MMA of the S / P.V issuer has completed
   uint64_t tdone;             // the softmax warps are done with TMEM (8 warp arrivals)
+  uint64_t vpart;             // the last V tile, where it holds keys past the last visible one, has landed
   uint32_t tmem_base;
   int32_t abort;
 };
@@ -221,7 +223,8 @@ __device__ __forceinline__ void part_exp(const uint32_t (&s)[4][32], uint64_t sc
 template <int D, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
     prefill_tc_kernel(const __grid_constant__ PrefillTcParams p, const __grid_constant__ CUtensorMap tmQ,
-                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
+                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
+                      const __grid_constant__ CUtensorMap tmVp) {
   using C = Cfg<D>;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
@@ -248,6 +251,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   const int n_tiles = a_tiles + b_tiles;                  // >= 1
   auto tile_tok = [&](int t) { return t < a_tiles ? t * kBN : b_lo + (t - a_tiles) * kBN; };
+  // Keys that no row of the CTA sees stay out of its V tiles (see zero_v_rows).  The prefix tiles come
+  // through a map that ends with the prefix; the CTA's last tile, where it holds keys past `last`, is
+  // loaded to a barrier of its own, and becomes full (vfull) once the producer has cleared those rows.
+  const bool part = last + 1 - tile_tok(n_tiles - 1) < kBN;
+  auto v_map = [&](int t) { return t < a_tiles ? &tmVp : &tmV; };
   auto load_tile = [&](const CUtensorMap* map, uint32_t off, int t, uint64_t* full) {
     mbar_expect_tx(full, C::kTileBytes);
 #pragma unroll
@@ -273,6 +281,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(&bars->drain_s, 1);
     mbar_init(&bars->drain_pv, 1);
     mbar_init(&bars->tdone, 8);
+    mbar_init(&bars->vpart, 1);
     bars->abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     // Q of both slots (box: 64 columns x G heads x tps tokens, so that smem row = token * G +
@@ -286,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     &bars->qfull[g]);
       if (g == 0) load_tile(&tmK, C::kOffK, 0, &bars->kfull[0]);
     }
-    load_tile(&tmV, C::kOffV, 0, &bars->vfull[0]);
+    load_tile(v_map(0), C::kOffV, 0, part && n_tiles == 1 ? &bars->vpart : &bars->vfull[0]);
   }
   if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem_base)),
@@ -308,7 +317,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ------------------------------------------------------------ TMA producers
       if (lane == 0) {
         const bool isK = warp == 0;
-        const CUtensorMap* map = isK ? &tmK : &tmV;
         const int ns = isK ? C::kKS : C::kVS;
         uint64_t* full = isK ? bars->kfull : bars->vfull;
         uint64_t* freed = isK ? bars->kfree : bars->vfree;
@@ -321,13 +329,30 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           if (ph > 0) ok = pwait(&freed[s], (uint32_t)((ph - 1) & 1), bars, p, isK ? 1 : 2);
           if (!ok) break;
-          load_tile(map, base + (uint32_t)s * C::kTileBytes, t, &full[s]);
+          load_tile(isK ? &tmK : v_map(t), base + (uint32_t)s * C::kTileBytes, t,
+                    !isK && part && t == n_tiles - 1 ? &bars->vpart : &full[s]);
           issued = t + 1;
           ++s;
         }
         if (!ok) {
           // the loads already issued must land before the CTA leaves
-          for (int t = max(0, issued - ns); t < issued; ++t) drain_wait(&full[t % ns], (uint32_t)((t / ns) & 1));
+          for (int t = max(0, issued - ns); t < issued; ++t) {
+            if (!isK && part && t == n_tiles - 1)
+              drain_wait(&bars->vpart, 0u);
+            else
+              drain_wait(&full[t % ns], (uint32_t)((t / ns) & 1));
+          }
+        }
+      }
+      __syncwarp();
+      if (warp == 3 && part && __shfl_sync(0xffffffffu, (int)ok, 0)) {
+        const int s = (n_tiles - 1) % C::kVS;
+        if (pwait_warp(&bars->vpart, 0u, bars, p, 7)) {
+          zero_v_rows<C::kHalves>(smem + C::kOffV + (uint32_t)s * C::kTileBytes, last + 1 - tile_tok(n_tiles - 1), lane, 32);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bars->vfull[s]);
+        } else {
+          drain_wait(&bars->vpart, 0u);
         }
       }
     } else if (warp == 1) {
@@ -691,7 +716,7 @@ constexpr double kSplitCtaUs = 8.5, kSplitRoundUs = 1.3, kPairCtaUs = 8.5, kPair
 
 template <int D, bool SPLIT>
 cudaError_t launch_slots(const PrefillTcParams& p, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                         int dev, cudaStream_t s) {
+                         const CUtensorMap& mvp, int dev, cudaStream_t s) {
   static bool configured[64] = {};
   if (dev >= 0 && dev < 64 && !configured[dev]) {
     cudaError_t e = cudaFuncSetAttribute(prefill_tc_kernel<D, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -707,7 +732,7 @@ cudaError_t launch_slots(const PrefillTcParams& p, const CUtensorMap& mq, const 
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = Cfg<D>::kSmemBytes;
   cfg.stream = s;
-  return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, SPLIT>, p, mq, mk, mv);
+  return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, SPLIT>, p, mq, mk, mv, mvp);
 }
 
 // SM count of a device (it does not change).
@@ -720,9 +745,10 @@ int sm_count(int dev) {
 
 template <int D>
 cudaError_t launch(const PrefillTcParams& p, const void* q, const void* k, const void* v, cudaStream_t s) {
-  CUtensorMap mq, mk, mv;
+  CUtensorMap mq, mk, mv, mvp;                // (mvp: V up to the prefix's end)
   if (!make_map(&mq, q, D, p.h_q, p.n_tokens, p.group, p.tps) || !make_map(&mk, k, D, p.h_kv, p.n_tokens, 1, kBN) ||
-      !make_map(&mv, v, D, p.h_kv, p.n_tokens, 1, kBN))
+      !make_map(&mv, v, D, p.h_kv, p.n_tokens, 1, kBN) ||
+      !make_map(&mvp, v, D, p.h_kv, std::max(1, p.prefix_len), 1, kBN))
     return cudaErrorInvalidValue;
   int dev = 0;
   cudaGetDevice(&dev);
@@ -746,7 +772,7 @@ cudaError_t launch(const PrefillTcParams& p, const void* q, const void* k, const
     return n > 2 * (int64_t)sms + sms / 16 ? 1e30 : t;  // (a few over two waves, the shortest, are no third)
   };
   const bool split = cost(p.tps, 2, kSplitCtaUs, kSplitRoundUs) < cost(2 * p.tps, 1, kPairCtaUs, kPairTileUs);
-  return split ? launch_slots<D, true>(p, mq, mk, mv, dev, s) : launch_slots<D, false>(p, mq, mk, mv, dev, s);
+  return split ? launch_slots<D, true>(p, mq, mk, mv, mvp, dev, s) : launch_slots<D, false>(p, mq, mk, mv, mvp, dev, s);
 }
 
 }  // namespace

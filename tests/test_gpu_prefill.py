@@ -145,3 +145,36 @@ def test_prefill_slots(D, h_q, h_kv, prefix, lens):
         outs.append(out)
     torch.cuda.synchronize()
     assert torch.equal(outs[0].bfloat16(), outs[1])
+
+
+@pytest.mark.parametrize("D,h_q,h_kv,prefix,lens", [
+    (64, 14, 2, 300, [200, 90, 130]),     # key tiles shared out of one query group
+    (128, 28, 4, 300, [200, 90, 130]),
+    (64, 64, 32, 700, [140, 100, 200]),   # two query groups
+    (128, 64, 32, 700, [140, 100, 200]),
+])
+@pytest.mark.parametrize("flags", [0, B.FLAG_PREFIX_MMA])
+def test_prefill_branch_does_not_reach_the_others(D, h_q, h_kv, prefix, lens, flags):
+    """A branch of NaN and infinite K and V leaves the prefix and the other branches as they are, beside the
+    query tile that it shares with its neighbours (at most two groups of 128 / G tokens, or 64 on the
+    warp-level kernel)."""
+    q, k, v = (_dev(x) for x in synth.prefill_inputs(5, prefix, lens, h_q, h_kv, D))
+    prob = B.make_problem(h_q, h_kv, D, 16, 1.0 / math.sqrt(D), flags=flags)
+    lo = prefix
+    res = []
+    for bad in (False, True):
+        if bad:
+            k[lo:lo + lens[0]] = float("nan")
+            v[lo:lo + lens[0]] = float("inf")
+            v[lo:lo + lens[0]:2] = float("nan")
+        out, lse = torch.empty(q.shape, device="cuda"), torch.empty(q.shape[:2], device="cuda")
+        B.pad_prefill_attn(prob, prefix, lens, q, k, v, out, lse)
+        torch.cuda.synchronize()
+        B.pad_prefill_status()
+        res.append((out, lse))
+    share = 64 if flags else 2 * (128 // (h_q // h_kv))
+    keep = torch.ones(q.shape[0], dtype=torch.bool, device="cuda")
+    keep[max(0, lo - share):lo + lens[0] + share] = False
+    assert int(keep.sum()) > 100 and bool(keep[-1])
+    for a, b in zip(*res):
+        assert torch.equal(a[keep], b[keep])
