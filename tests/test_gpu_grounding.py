@@ -158,3 +158,23 @@ def test_grounding_empty_segments_between_chunks():
     for s in range(len(gi.offsets) - 1):
         part = f64[gi.offsets[s]:gi.offsets[s + 1]]
         assert np.all(np.abs(seg[s].cpu().numpy() - part.sum(axis=0)) <= 1e-4 * np.abs(part).sum(axis=0) + 1e-6)
+
+
+@pytest.mark.parametrize("d", [8, 40, 256, 680, 2048])
+@pytest.mark.parametrize("lens", [
+    [7, 7, 7, 7, 4] * 40,                    # a chunk of 32 tokens: five segments and more
+    [9, 9, 9, 9] * 40,                       # three or four
+    [1] * 37 + [0] * 300 + [1, 0, 2] * 30 + [0] * 9 + [400, 1, 1, 1, 1, 0, 1, 700, 3],   # runs of empty ones
+    [0, 0, 5, 1, 1, 1, 1],                   # one short chunk
+])
+def test_pool_chunks_of_many_segments(lens, d):
+    """Chunks that go by rows, by segments, and just on either side of the limit; every sum within fp32
+    rounding of its terms (each is at most 32 additions long before the sums of the row groups meet)."""
+    off = np.concatenate([[3], 3 + np.cumsum(lens)]).astype(np.int32)
+    f = torch.randn(int(off[-1]) + 5, d, device="cuda").bfloat16()
+    seg = torch.full((len(lens), d), float("nan"), device="cuda")
+    B.pad_ground_pool(f, off, seg)
+    f64, got = f.double().cpu().numpy(), seg.cpu().numpy()
+    for s in range(len(lens)):
+        part = f64[off[s]:off[s + 1]]
+        assert np.all(np.abs(got[s] - part.sum(axis=0)) <= 256 * 2.0 ** -24 * np.abs(part).sum(axis=0))
