@@ -79,6 +79,12 @@ __device__ __forceinline__ void ld_stream4(uint4 (&v)[4], const void* p0, const 
       : "l"(p0), "l"(p1), "l"(p2), "l"(p3));
 }
 
+// A row that a grid ahead wrote: through L1 where the kernel is launched in plain stream order only.
+template <bool L1>
+__device__ __forceinline__ float4 ld_row(const float4* p) {
+  return L1 ? __ldg(p) : __ldcg(p);
+}
+
 // One bf16 element past L1.  (The header's __ldcg of this type may be moved ahead of the wait.)
 __device__ __forceinline__ float ld_bf16(const __nv_bfloat16* p) {
   return __bfloat162float(__ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(p))));
@@ -246,41 +252,48 @@ __global__ void __launch_bounds__(kThreads) ground_pool_kernel(const __grid_cons
 // One CTA per event: scores against every pooled segment row, the best score, the salient
 // set (score >= fraction * best when best > 0, else the first best segment alone) and the
 // first and last salient segments.
-constexpr int kScoreThreads = 1024;  // 32 warps: a hundred segments are one round of loads
-constexpr int kScoreWarps = kScoreThreads / 32;
-__global__ void __launch_bounds__(kScoreThreads) ground_score_kernel(const __nv_bfloat16* __restrict__ g, int S, int d,
+// A warp takes ROWS segments at a time.  32 warps of four rows (a hundred segments are one round of
+// loads) are best while every CTA finds room, two per SM, and where an event's own work is long.
+// More events than that over few segments take eight warps of eight rows, eight CTAs per SM, and where
+// the rows of all events are more than 64 MB they come through L1, which the CTAs of an SM share (the
+// kernel is then launched in plain stream order).  us per call, 32 x 4, 8 x 8, 8 x 8 through L1: 1024 events, 8
+// segments, d = 64: 17.5, 6.1, -; 310, 128, 256: 10.5, 8.3, 10.4; 310, 1024, 256: 41.1, 48.2, 38.2; 1024,
+// 128, 256: 24.1, 13.9, 14.5; 620, 1024, 1024: 147.8, 168, 186.
+template <int WARPS, int ROWS, bool L1>
+__global__ void __launch_bounds__(32 * WARPS) ground_score_kernel(const __nv_bfloat16* __restrict__ g, int S, int d,
                                                                 const float* __restrict__ seg_sum, float frac,
                                                                 float* __restrict__ scores,
                                                                 uint8_t* __restrict__ salient,
                                                                 int32_t* __restrict__ interval) {
+  constexpr int kThr = 32 * WARPS;
   extern __shared__ float gs[];  // [d] the event's projected token, then [S] scores
   float* sc = gs + d;
-  __shared__ float wbest[kScoreWarps];
-  __shared__ int wlo[kScoreWarps], whi[kScoreWarps], warg[kScoreWarps];
+  __shared__ float wbest[WARPS];
+  __shared__ int wlo[WARPS], whi[WARPS], warg[WARPS];
   const int i = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   grid_wait();
   grid_release();
-  for (int c = threadIdx.x; c < d; c += kScoreThreads) gs[c] = ld_bf16(g + (size_t)i * d + c);
+  for (int c = threadIdx.x; c < d; c += kThr) gs[c] = L1 ? __bfloat162float(g[(size_t)i * d + c]) : ld_bf16(g + (size_t)i * d + c);
   __syncthreads();
-  // a warp per segment row (lanes over its float4 columns), four rows in flight per warp
+  // a warp per segment row (lanes over its float4 columns), ROWS rows in flight per warp
   float best = -__builtin_huge_valf();
   const int d4 = d / 4;
-  for (int s0 = warp * 4; s0 < S; s0 += 4 * kScoreWarps) {
-    float part[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 2
+  for (int s0 = warp * ROWS; s0 < S; s0 += ROWS * WARPS) {
+    float part[ROWS] = {};
+#pragma unroll 8 / ROWS
     for (int c = lane; c < d4; c += 32) {
-      float4 v[4];
+      float4 v[ROWS];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        v[u] = s0 + u < S ? __ldcg(reinterpret_cast<const float4*>(seg_sum + (size_t)(s0 + u) * d) + c)
+      for (int u = 0; u < ROWS; ++u)
+        v[u] = s0 + u < S ? ld_row<L1>(reinterpret_cast<const float4*>(seg_sum + (size_t)(s0 + u) * d) + c)
                           : make_float4(0.f, 0.f, 0.f, 0.f);
       const float g0 = gs[4 * c], g1 = gs[4 * c + 1], g2 = gs[4 * c + 2], g3 = gs[4 * c + 3];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) part[u] += (g0 * v[u].x + g1 * v[u].y) + (g2 * v[u].z + g3 * v[u].w);
+      for (int u = 0; u < ROWS; ++u) part[u] += (g0 * v[u].x + g1 * v[u].y) + (g2 * v[u].z + g3 * v[u].w);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < ROWS; ++u) {
       float v = part[u];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -299,20 +312,20 @@ __global__ void __launch_bounds__(kScoreThreads) ground_score_kernel(const __nv_
   if (lane == 0) wbest[warp] = best;
   __syncthreads();
   best = wbest[0];
-  for (int w = 1; w < kScoreWarps; ++w) best = fmaxf(best, wbest[w]);
+  for (int w = 1; w < WARPS; ++w) best = fmaxf(best, wbest[w]);
   // the first best segment (used alone when no score is positive)
   int arg = S;
-  for (int s = threadIdx.x; s < S; s += kScoreThreads)
+  for (int s = threadIdx.x; s < S; s += kThr)
     if (sc[s] == best) arg = min(arg, s);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) arg = min(arg, __shfl_xor_sync(0xffffffffu, arg, o));
   if (lane == 0) warg[warp] = arg;
   __syncthreads();
   arg = warg[0];
-  for (int w = 1; w < kScoreWarps; ++w) arg = min(arg, warg[w]);
+  for (int w = 1; w < WARPS; ++w) arg = min(arg, warg[w]);
   const float cut = frac * best;
   int lo = S, hi = -1;
-  for (int s = threadIdx.x; s < S; s += kScoreThreads) {
+  for (int s = threadIdx.x; s < S; s += kThr) {
     const bool on = best > 0.f ? sc[s] >= cut : s == arg;
     salient[(size_t)i * S + s] = on ? 1 : 0;
     if (on) {
@@ -331,7 +344,7 @@ __global__ void __launch_bounds__(kScoreThreads) ground_score_kernel(const __nv_
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < kScoreWarps; ++w) {
+    for (int w = 1; w < WARPS; ++w) {
       lo = min(lo, wlo[w]);
       hi = max(hi, whi[w]);
     }
@@ -440,16 +453,20 @@ __global__ void __launch_bounds__(kThreads, 5) attn_seg_pool_kernel(const __grid
 
 // attn_event_kernel: grid (event, slice of kAggCols columns).  The pieces of the event's
 // interval (lo, hi), clamped to the segments, are spread over 16 warps (warp w takes every
-// 16th piece from the first, four in flight; eight or 32 warps were 1.4 us slower per readout); a lane adds 8 columns; the warps' sums are added in
-// shared memory, in order, and out = g_emb + sum W / sum A (g_emb alone when sum A is 0).
-constexpr int kEventWarps = 16;
-__global__ void __launch_bounds__(32 * kEventWarps) attn_event_kernel(const __grid_constant__ Pieces pm, int d,
+// 16th piece from the first, four in flight; eight or 32 warps were 1.4 us slower per readout); a lane
+// adds 8 columns; the warps' sums are added in shared memory, in order, and out = g_emb + sum W / sum A
+// (g_emb alone when sum A is 0).  A grid of more than twelve CTAs per SM has eight warps with one piece at a
+// time, through L1, which the events share (in plain stream order, then): 1024 events, 32768 tokens,
+// d = 2048, 128 segments 65.4 us per call with 16 warps, 45.4 so; 400 events 38.2, 33.0; 200 (ten per
+// SM) 30.4, 31.0.
+template <int WARPS, bool L1>
+__global__ void __launch_bounds__(32 * WARPS) attn_event_kernel(const __grid_constant__ Pieces pm, int d,
                                                               const int32_t* __restrict__ interval,
                                                               const float* wsum, const float* asum,
                                                               const __nv_bfloat16* __restrict__ g_emb,
                                                               float* __restrict__ out) {
-  __shared__ float red[kEventWarps][kAggCols];
-  __shared__ float ared[kEventWarps];
+  __shared__ float red[WARPS][kAggCols];
+  __shared__ float ared[WARPS];
   const int i = blockIdx.x, S = pm.n;
   const int s_lo = min(max(__ldcg(interval + 2 * i), 0), S - 1);
   const int s_hi = min(max(__ldcg(interval + 2 * i + 1), s_lo), S - 1);
@@ -460,22 +477,39 @@ __global__ void __launch_bounds__(32 * kEventWarps) attn_event_kernel(const __gr
   float a = 0.f;
   grid_wait();  // (the interval was written before the pooling kernel started)
   grid_release();
-  if (c8 < d) {
+  if (L1 && c8 < d) {
+    for (int pc = p0 + w; pc < p1; pc += WARPS) {
+      const float4* src = reinterpret_cast<const float4*>(wsum + (size_t)pc * d + c8);
+      const float4 u0 = __ldg(src), u1 = __ldg(src + 1);
+      acc[0] += u0.x;
+      acc[1] += u0.y;
+      acc[2] += u0.z;
+      acc[3] += u0.w;
+      acc[4] += u1.x;
+      acc[5] += u1.y;
+      acc[6] += u1.z;
+      acc[7] += u1.w;
+      a += __ldg(asum + pc);
+    }
+  } else if (c8 < d) {
     // four pieces' loads in flight
-    for (int pc = p0 + w; pc < p1; pc += 4 * kEventWarps) {
+    for (int pc = p0 + w; pc < p1; pc += 4 * WARPS) {
       float4 u0[4], u1[4];
       float av[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const int q = pc + k * kEventWarps;
-        const float4* src = reinterpret_cast<const float4*>(wsum + (size_t)(q < p1 ? q : pc) * d + c8);
-        u0[k] = __ldcg(src);
-        u1[k] = __ldcg(src + 1);
-        av[k] = __ldcg(asum + (q < p1 ? q : pc));
+        const int q = pc + k * WARPS;
+        u0[k] = u1[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        av[k] = 0.f;
+        if (q < p1) {
+          const float4* src = reinterpret_cast<const float4*>(wsum + (size_t)q * d + c8);
+          u0[k] = __ldcg(src);
+          u1[k] = __ldcg(src + 1);
+          av[k] = __ldcg(asum + q);
+        }
       }
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        if (pc + k * kEventWarps >= p1) break;
         acc[0] += u0[k].x;
         acc[1] += u0[k].y;
         acc[2] += u0[k].z;
@@ -496,7 +530,7 @@ __global__ void __launch_bounds__(32 * kEventWarps) attn_event_kernel(const __gr
   if (threadIdx.x < kAggCols && col < d) {
     float num = 0.f, den = 0.f;
 #pragma unroll
-    for (int r = 0; r < kEventWarps; ++r) {
+    for (int r = 0; r < WARPS; ++r) {
       num += red[r][threadIdx.x];
       den += ared[r];
     }
@@ -505,9 +539,19 @@ __global__ void __launch_bounds__(32 * kEventWarps) attn_event_kernel(const __gr
   }
 }
 
-// A launch that may start while the grid ahead of it runs.
+// SM count of the current device (it does not change).
+int sm_count() {
+  static int n[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+  if (n[dev] == 0 && cudaDeviceGetAttribute(&n[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n[dev] = 152;
+  return n[dev];
+}
+
+// A launch that may start while the grid ahead of it runs (early), or in plain stream order.
 template <class... KArgs, class... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t s, Args... args) {
+cudaError_t launch_early(bool early, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                         Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
@@ -515,10 +559,14 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t 
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <class... KArgs, class... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t s, Args... args) {
+  return launch_early(true, kernel, grid, threads, smem, s, args...);
 }
 
 // hint.seg[g]: the last segment whose `first` entry is at most that of the first block of the
@@ -577,8 +625,11 @@ cudaError_t launch_ground_score(const void* g_proj, int32_t n_events, const floa
                                 cudaStream_t s) {
   if (n_events == 0) return cudaSuccess;
   const size_t smem = (size_t)(d + n_segments) * sizeof(float);
-  return launch_pdl(ground_score_kernel, dim3(n_events), kScoreThreads, smem, s,
-                    static_cast<const __nv_bfloat16*>(g_proj), n_segments, d, seg_sum, frac, scores, salient, interval);
+  const bool many = n_events > 2 * sm_count() && n_segments * d < (1 << 19);
+  const bool l1 = many && (int64_t)n_events * n_segments * d > (16 << 20);  // 64 MB of rows
+  auto* kernel = l1 ? ground_score_kernel<8, 8, true> : many ? ground_score_kernel<8, 8, false> : ground_score_kernel<32, 4, false>;
+  return launch_early(!l1, kernel, dim3(n_events), many ? 256 : 1024, smem, s, static_cast<const __nv_bfloat16*>(g_proj),
+                      n_segments, d, seg_sum, frac, scores, salient, interval);
 }
 
 size_t attn_aggregate_ws_floats(int64_t n_tokens, int32_t n_segments, int32_t d) {
@@ -611,8 +662,9 @@ cudaError_t launch_attn_aggregate(const void* x, int64_t n_tokens, int32_t d, co
                                static_cast<const __nv_bfloat16*>(x), d, attn, wsum, asum);
     if (e != cudaSuccess) return e;
   }
-  return launch_pdl(attn_event_kernel, dim3(n_events, slices), 32 * kEventWarps, 0, s, pm, d, interval, wsum, asum,
-                    static_cast<const __nv_bfloat16*>(g_emb), out);
+  const bool many = (int64_t)n_events * slices > 12 * sm_count();
+  return launch_early(!many, many ? attn_event_kernel<8, true> : attn_event_kernel<16, false>, dim3(n_events, slices),
+                      many ? 256 : 512, 0, s, pm, d, interval, wsum, asum, static_cast<const __nv_bfloat16*>(g_emb), out);
 }
 
 }  // namespace pad

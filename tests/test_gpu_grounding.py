@@ -178,3 +178,13 @@ def test_pool_chunks_of_many_segments(lens, d):
     for s in range(len(lens)):
         part = f64[off[s]:off[s + 1]]
         assert np.all(np.abs(got[s] - part.sum(axis=0)) <= 256 * 2.0 ** -24 * np.abs(part).sum(axis=0))
+
+
+@pytest.mark.parametrize("dims", [
+    (900, 40, 320, 64, 512, 0),       # many events: eight warps of eight rows
+    (2048, 1024, 320, 64, 2048, 0),   # and their rows through L1; many event CTAs
+    (600, 9, 1300, 8, 520, 0),
+])
+def test_grounding_many_events(dims):
+    T, S, K, dp, dm, text = dims
+    _check(synth.grounding_inputs(sum(dims), T, S, K, dp, dm, text_tokens=text), 0.5)
