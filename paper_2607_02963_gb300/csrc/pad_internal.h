@@ -111,6 +111,8 @@ struct KParams {
   int32_t keys_ready;             // two-call step behind the tensor-core prefix grid, which waits
                                   // for the append before it releases the branch/merge grid:
                                   // the appended keys may be read before that grid's own wait
+  int32_t wait_first;             // the branch/merge grid has no prefix grid ahead of it, which would
+                                  // have waited for what it reads: it waits before it reads
   int32_t col_splits;             // CTAs that share a branch/merge task, by output columns
   float scale_log2;               // scale * log2(e)
   uint64_t gen;                   // generation of the plan (tags errors in the status word)

@@ -780,7 +780,8 @@ def test_shared_branch_tasks_match_oracle(lens, D, h_q, h_kv, one_call):
 
 
 @pytest.mark.parametrize("one_call", [True, False])
-@pytest.mark.parametrize("prefix,flags", [([0, 0], 0), ([700, 300], 0), ([700, 300], B.FLAG_PREFIX_DUAL)])
+@pytest.mark.parametrize("prefix,flags", [([0, 0], 0), ([0, 0], B.FLAG_PREFIX_MMA), ([700, 300], 0),
+                                          ([700, 300], B.FLAG_PREFIX_DUAL)])
 def test_steps_back_to_back_equal_steps_run_apart(prefix, flags, one_call):
     """A generation loop enqueued without any wait between its kernels (each step reads the keys
     that the one before appended, and q written by a kernel right ahead of the attention) equals
@@ -859,13 +860,15 @@ def test_head_dim_64_few_rows_hold_weights_in_32_bits(h_q, h_kv, events, one_cal
 
 
 @pytest.mark.parametrize("late", ["all_ahead_of_append", "prefix_ahead_of_attention", "inputs_ahead_of_one_call"])
-@pytest.mark.parametrize("D,flags,rope", [(128, 0, False), (128, 0, True), (64, 0, False), (128, B.FLAG_PREFIX_DUAL, False),
-                                          (128, B.FLAG_FUSED_MERGE, False), (128, B.FLAG_PREFIX_MMA, False)])
-def test_step_waits_for_a_grid_that_releases_early(late, D, flags, rope):
+@pytest.mark.parametrize("D,flags,rope,prefix", [
+    (128, 0, False, [900, 130]), (128, 0, True, [900, 130]), (64, 0, False, [900, 130]),
+    (128, B.FLAG_PREFIX_DUAL, False, [900, 130]), (128, B.FLAG_FUSED_MERGE, False, [900, 130]),
+    (128, B.FLAG_PREFIX_MMA, False, [900, 130]), (128, 0, True, [0, 0]), (64, 0, False, [0, 0])])
+def test_step_waits_for_a_grid_that_releases_early(late, D, flags, rope, prefix):
     """What a grid ahead of the step stores long after it has released its dependents is seen by the step:
     everything ahead of the two calls, the prefix between them, q and the new rows ahead of the one call
     (whose prefix must not be written so)."""
-    w = _w([900, 130], [5, 6], [3, 0, 16, 5, 40, 1, 31, 2, 7, 15, 64], D=D, h_q=14, h_kv=2, seed=9)
+    w = _w(prefix, [5, 6], [3, 0, 16, 5, 40, 1, 31, 2, 7, 15, 64], D=D, h_q=14, h_kv=2, seed=9)
     db = DeviceBatch(w, flags=flags, fill_nan=False)
     ref = w
     if rope:
