@@ -1098,7 +1098,6 @@ static void make_params(const pad_plan_t* plan, KParams& p) {
   p.merge_first = plan->lay.merge_first ? 1 : 0;
   p.col_splits = plan->lay.col_splits;
   p.keys_ready = 0;
-  p.wait_first = 0;
   p.counters = reinterpret_cast<unsigned int*>(ws + plan->lay.off_cnt);
   p.n_counters = p.fused ? (int32_t)plan->lay.n_counters : 0;
   if (p.img_n > 0) {
@@ -1168,8 +1167,9 @@ static pad_status launch_attention(const pad_plan_t* plan, const void* q, const 
   make_params(plan, p);
   p.k_new = k_new;
   p.v_new = v_new;
-  p.keys_ready = plan->lay.n_items > 0 && !plan->lay.fused &&
-                 (plan->lay.prefix_kernel == PAD_FLAG_PREFIX_TC || plan->lay.prefix_kernel == PAD_FLAG_PREFIX_DUAL);
+  p.keys_ready = plan->lay.n_items == 0 ? 2
+                 : !plan->lay.fused && (plan->lay.prefix_kernel == PAD_FLAG_PREFIX_TC ||
+                                        plan->lay.prefix_kernel == PAD_FLAG_PREFIX_DUAL);
   const bool timed = g_timing.on && g_timing.n < g_timing.max;
   if (timed) cudaEventRecord(g_timing.ev[2 * g_timing.n], s);
   cudaError_t e = cudaSuccess;
@@ -1201,7 +1201,6 @@ static pad_status launch_attention(const pad_plan_t* plan, const void* q, const 
     // prefix grid, which waited for everything ahead before it released this one.  With no prefix at
     // all it starts early too, but waits before it reads anything (32 events: 4.3 us per step
     // against 6.2 in plain launch order).
-    p.wait_first = plan->lay.n_items == 0;
     const bool pdl = !timed && (plan->lay.n_items == 0 || plan->lay.prefix_kernel == PAD_FLAG_PREFIX_TC ||
                                 plan->lay.prefix_kernel == PAD_FLAG_PREFIX_DUAL);
     e = launch_branch_merge(p, q, k_pool, v_pool, out, lse, pdl, s);
@@ -1778,7 +1777,6 @@ pad_status static_params(const pad_plan_t* plan, cudaStream_t s, KParams& p, uin
   p.merge_first = plan->lay.merge_first ? 1 : 0;
   p.col_splits = plan->lay.col_splits;
   p.keys_ready = 0;
-  p.wait_first = 0;
   p.tasks = reinterpret_cast<const int32_t*>(ws + plan->lay.off_tasks);
   p.counters = reinterpret_cast<unsigned int*>(ws + plan->lay.off_cnt);
   p.n_counters = p.fused ? (int32_t)plan->lay.n_counters : 0;

@@ -110,9 +110,9 @@ struct KParams {
                                   // while its branch pass runs
   int32_t keys_ready;             // two-call step behind the tensor-core prefix grid, which waits
                                   // for the append before it releases the branch/merge grid:
-                                  // the appended keys may be read before that grid's own wait
-  int32_t wait_first;             // the branch/merge grid has no prefix grid ahead of it, which would
-                                  // have waited for what it reads: it waits before it reads
+                                  // the appended keys may be read before that grid's own wait;
+                                  // 2: no prefix grid is ahead of the branch/merge grid, which
+                                  // waits at its start instead, before it reads anything
   int32_t col_splits;             // CTAs that share a branch/merge task, by output columns
   float scale_log2;               // scale * log2(e)
   uint64_t gen;                   // generation of the plan (tags errors in the status word)

@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(32 * NW, NW == bm::kWarps ? 2 : (OVER ? 4 : 3)
   // The grid after this one may be scheduled now: in a one-call loop it is the next step's
   // prefix kernel, which waits for this grid before it touches anything (an append kernel
   // after it is launched without programmatic serialisation and waits in any case).
-  if (p.wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (p.keys_ready == 2) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   constexpr int kShare = D / W;
   const int task = blockIdx.x / kShare;
