@@ -17,7 +17,7 @@
 // 16/1 heads: 24.8 -> 16.8).
 //
 //   warps 0, 3  TMA producers of K and V tiles (64-column boxes, 128-byte swizzle); warp 3 clears
-//               the rows of the last V tile that no row here sees
+//               the rows of a branch's last V tile that no row here sees
 //   warp 1      S issuer: S_g(k) = Q_g K(k)^T
 //   warp 2      TMEM allocation (512 columns) and deallocation, and P.V issuer: O_g += P_g(k)
 //               V(k), P read back from TMEM, 96 keys and then the last 32
@@ -121,7 +121,7 @@ struct Bars {
   uint64_t pvdone[2];         // its P.V has completed
   uint64_t drain_s, drain_pv; // every MMA of the S / P.V issuer has completed
   uint64_t tdone;             // the softmax warps are done with TMEM (8 warp arrivals)
-  uint64_t vpart;             // the last V tile, where it holds keys past the last visible one, has landed
+  uint64_t vclear;            // the last V tile's rows past the last visible key are cleared
   uint32_t tmem_base;
   int32_t abort;
 };
@@ -223,8 +223,7 @@ __device__ __forceinline__ void part_exp(const uint32_t (&s)[4][32], uint64_t sc
 template <int D, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
     prefill_tc_kernel(const __grid_constant__ PrefillTcParams p, const __grid_constant__ CUtensorMap tmQ,
-                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                      const __grid_constant__ CUtensorMap tmVp) {
+                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
   using C = Cfg<D>;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
@@ -243,19 +242,20 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int tok0 = qt * tpc;
   const int last = min(tok0 + tpc, N) - 1;
   // key tiles: [0, a_end) of the prefix, then [b_lo, last] of the branches
-  const int a_tiles = (min(S, last + 1) + kBN - 1) / kBN;
+  const int a_end = min(S, last + 1);
+  const int a_tiles = (a_end + kBN - 1) / kBN;
   int b_lo = 0, b_tiles = 0;
   if (last >= S) {
     b_lo = branch_start(p, max(tok0, S));
     b_tiles = (last + 1 - b_lo + kBN - 1) / kBN;
   }
   const int n_tiles = a_tiles + b_tiles;                  // >= 1
-  auto tile_tok = [&](int t) { return t < a_tiles ? t * kBN : b_lo + (t - a_tiles) * kBN; };
-  // Keys that no row of the CTA sees stay out of its V tiles (see zero_v_rows).  The prefix tiles come
-  // through a map that ends with the prefix; the CTA's last tile, where it holds keys past `last`, is
-  // loaded to a barrier of its own, and becomes full (vfull) once the producer has cleared those rows.
-  const bool part = last + 1 - tile_tok(n_tiles - 1) < kBN;
-  auto v_map = [&](int t) { return t < a_tiles ? &tmVp : &tmV; };
+  auto tile_tok = [&](int t) { return t < a_tiles ? min(t * kBN, a_end - kBN) : b_lo + (t - a_tiles) * kBN; };
+  // Keys that no row of the CTA sees stay out of its V tiles (see zero_v_rows).  The last tile of the prefix
+  // ends where the visible prefix does: it starts that much earlier (rows before the first token are
+  // zero), and the columns that it shares with the tile before are masked.  The last tile of the branches
+  // would run into the branch before instead: the V producer clears its rows past `last` (vclear).
+  const bool part = b_tiles > 0 && (last + 1 - b_lo) % kBN != 0;
   auto load_tile = [&](const CUtensorMap* map, uint32_t off, int t, uint64_t* full) {
     mbar_expect_tx(full, C::kTileBytes);
 #pragma unroll
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(&bars->drain_s, 1);
     mbar_init(&bars->drain_pv, 1);
     mbar_init(&bars->tdone, 8);
-    mbar_init(&bars->vpart, 1);
+    mbar_init(&bars->vclear, 1);
     bars->abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     // Q of both slots (box: 64 columns x G heads x tps tokens, so that smem row = token * G +
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     &bars->qfull[g]);
       if (g == 0) load_tile(&tmK, C::kOffK, 0, &bars->kfull[0]);
     }
-    load_tile(v_map(0), C::kOffV, 0, part && n_tiles == 1 ? &bars->vpart : &bars->vfull[0]);
+    load_tile(&tmV, C::kOffV, 0, &bars->vfull[0]);
   }
   if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem_base)),
@@ -317,6 +317,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ------------------------------------------------------------ TMA producers
       if (lane == 0) {
         const bool isK = warp == 0;
+        const CUtensorMap* map = isK ? &tmK : &tmV;
         const int ns = isK ? C::kKS : C::kVS;
         uint64_t* full = isK ? bars->kfull : bars->vfull;
         uint64_t* freed = isK ? bars->kfree : bars->vfree;
@@ -329,30 +330,22 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           if (ph > 0) ok = pwait(&freed[s], (uint32_t)((ph - 1) & 1), bars, p, isK ? 1 : 2);
           if (!ok) break;
-          load_tile(isK ? &tmK : v_map(t), base + (uint32_t)s * C::kTileBytes, t,
-                    !isK && part && t == n_tiles - 1 ? &bars->vpart : &full[s]);
+          load_tile(map, base + (uint32_t)s * C::kTileBytes, t, &full[s]);
           issued = t + 1;
           ++s;
         }
         if (!ok) {
           // the loads already issued must land before the CTA leaves
-          for (int t = max(0, issued - ns); t < issued; ++t) {
-            if (!isK && part && t == n_tiles - 1)
-              drain_wait(&bars->vpart, 0u);
-            else
-              drain_wait(&full[t % ns], (uint32_t)((t / ns) & 1));
-          }
+          for (int t = max(0, issued - ns); t < issued; ++t) drain_wait(&full[t % ns], (uint32_t)((t / ns) & 1));
         }
       }
       __syncwarp();
       if (warp == 3 && part && __shfl_sync(0xffffffffu, (int)ok, 0)) {
         const int s = (n_tiles - 1) % C::kVS;
-        if (pwait_warp(&bars->vpart, 0u, bars, p, 7)) {
+        if (pwait_warp(&bars->vfull[s], (uint32_t)(((n_tiles - 1) / C::kVS) & 1), bars, p, 7)) {
           zero_v_rows<C::kHalves>(smem + C::kOffV + (uint32_t)s * C::kTileBytes, last + 1 - tile_tok(n_tiles - 1), lane, 32);
           __syncwarp();
-          if (lane == 0) mbar_arrive(&bars->vfull[s]);
-        } else {
-          drain_wait(&bars->vpart, 0u);
+          if (lane == 0) mbar_arrive(&bars->vclear);
         }
       }
     } else if (warp == 1) {
@@ -490,6 +483,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (active) {
           const int t0 = tile_tok(t);
           if (t < a_tiles) {
+            lo = t * kBN - t0;
             hi = (bs < 0 ? tok + 1 : S) - t0;
           } else {
             lo = bs < 0 ? kBN : bs - t0;
@@ -503,6 +497,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int col = 32 * c + i;
             if (col < lo || col >= hi) s[c][i] = 0xff800000u;  // -inf
           }
+        if (part && t == n_tiles - 1 && !__all_sync(0xffffffffu, pwait(&bars->vclear, 0u, bars, p, 12))) return false;
       }
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -716,7 +711,7 @@ constexpr double kSplitCtaUs = 8.5, kSplitRoundUs = 1.3, kPairCtaUs = 8.5, kPair
 
 template <int D, bool SPLIT>
 cudaError_t launch_slots(const PrefillTcParams& p, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                         const CUtensorMap& mvp, int dev, cudaStream_t s) {
+                         int dev, cudaStream_t s) {
   static bool configured[64] = {};
   if (dev >= 0 && dev < 64 && !configured[dev]) {
     cudaError_t e = cudaFuncSetAttribute(prefill_tc_kernel<D, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -732,7 +727,7 @@ cudaError_t launch_slots(const PrefillTcParams& p, const CUtensorMap& mq, const 
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = Cfg<D>::kSmemBytes;
   cfg.stream = s;
-  return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, SPLIT>, p, mq, mk, mv, mvp);
+  return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, SPLIT>, p, mq, mk, mv);
 }
 
 // SM count of a device (it does not change).
@@ -745,10 +740,9 @@ int sm_count(int dev) {
 
 template <int D>
 cudaError_t launch(const PrefillTcParams& p, const void* q, const void* k, const void* v, cudaStream_t s) {
-  CUtensorMap mq, mk, mv, mvp;                // (mvp: V up to the prefix's end)
+  CUtensorMap mq, mk, mv;
   if (!make_map(&mq, q, D, p.h_q, p.n_tokens, p.group, p.tps) || !make_map(&mk, k, D, p.h_kv, p.n_tokens, 1, kBN) ||
-      !make_map(&mv, v, D, p.h_kv, p.n_tokens, 1, kBN) ||
-      !make_map(&mvp, v, D, p.h_kv, std::max(1, p.prefix_len), 1, kBN))
+      !make_map(&mv, v, D, p.h_kv, p.n_tokens, 1, kBN))
     return cudaErrorInvalidValue;
   int dev = 0;
   cudaGetDevice(&dev);
@@ -772,7 +766,7 @@ cudaError_t launch(const PrefillTcParams& p, const void* q, const void* k, const
     return n > 2 * (int64_t)sms + sms / 16 ? 1e30 : t;  // (a few over two waves, the shortest, are no third)
   };
   const bool split = cost(p.tps, 2, kSplitCtaUs, kSplitRoundUs) < cost(2 * p.tps, 1, kPairCtaUs, kPairTileUs);
-  return split ? launch_slots<D, true>(p, mq, mk, mv, mvp, dev, s) : launch_slots<D, false>(p, mq, mk, mv, mvp, dev, s);
+  return split ? launch_slots<D, true>(p, mq, mk, mv, dev, s) : launch_slots<D, false>(p, mq, mk, mv, dev, s);
 }
 
 }  // namespace

@@ -195,6 +195,7 @@ __device__ __forceinline__ bool elect_one() {
 // a prefill, 1.4 % of a 32768-token step.)
 template <int HALVES>
 __device__ __forceinline__ void zero_v_rows(uint8_t* tile, int r0, int thread, int n) {
+#pragma unroll 8
   for (int i = 8 * r0 + thread; i < 128 * 8; i += n)
 #pragma unroll
     for (int h = 0; h < HALVES; ++h) *reinterpret_cast<uint4*>(tile + h * 16384 + i * 16) = make_uint4(0u, 0u, 0u, 0u);
