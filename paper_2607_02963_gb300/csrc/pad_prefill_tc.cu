@@ -102,6 +102,8 @@ struct Cfg {
 struct PrefillTcParams {
   int32_t n_tokens, prefix_len, n_branches;
   int32_t h_q, h_kv, group, tps;        // tps: query tokens per slot (128 / group)
+  int32_t tok_base, n_qt;               // the grid's query tiles: n_qt of them, from this token on
+  int32_t release, after;               // mixed launch: this grid releases the next / ends after the one ahead
   float scale_log2;
   int32_t out_bf16;
   uint64_t gen;
@@ -236,10 +238,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int N = p.n_tokens, S = p.prefix_len, G = p.group;
   const int tpc = (SPLIT ? 1 : 2) * p.tps;                              // query tokens per CTA
-  const int n_qt = (N + tpc - 1) / tpc;
-  const int qt = n_qt - 1 - (int)blockIdx.x / p.h_kv;
+  const int qt = p.n_qt - 1 - (int)blockIdx.x / p.h_kv;
   const int kvh = (int)blockIdx.x % p.h_kv;
-  const int tok0 = qt * tpc;
+  const int tok0 = p.tok_base + qt * tpc;
   const int last = min(tok0 + tpc, N) - 1;
   // key tiles: [0, a_end) of the prefix, then [b_lo, last] of the branches
   const int a_end = min(S, last + 1);
@@ -263,6 +264,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       tma_load_3d(sbase + off + h * C::kBoxBytes, map, 64 * h, kvh, tile_tok(t), full);
   };
 
+  if (SPLIT && p.release) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (threadIdx.x == 0) {
     for (int s = 0; s < 4; ++s) {
       mbar_init(&bars->kfull[s], 1);
@@ -444,6 +446,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       fence_after();
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
     }
+    // (a grid that ran beside the one ahead completes after it, as stream order has it)
+    if (!SPLIT && warp == 0 && p.after) asm volatile("griddepcontrol.wait;" ::: "memory");
   } else {
     // ------------------------------------------------------------ softmax
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::kRegsSoftmax));
@@ -707,7 +711,8 @@ bool make_map(CUtensorMap* map, const void* base, int D, int heads, int64_t toke
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-constexpr double kSplitCtaUs = 8.5, kSplitRoundUs = 1.3, kPairCtaUs = 8.5, kPairTileUs = 1.54;
+// (a CTA, and a round of two key tiles or a tile of its chain; the start and the end of a second grid)
+constexpr double kSplitCtaUs = 8.5, kSplitRoundUs = 1.3, kPairCtaUs = 8.5, kPairTileUs = 1.54, kLateUs = 1.5, kTwoGridsUs = 3.0;
 
 template <int D, bool SPLIT>
 cudaError_t launch_slots(const PrefillTcParams& p, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
@@ -719,14 +724,17 @@ cudaError_t launch_slots(const PrefillTcParams& p, const CUtensorMap& mq, const 
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
-  const int tpc = (SPLIT ? 1 : 2) * p.tps;
-  const int64_t n_qt = ((int64_t)p.n_tokens + tpc - 1) / tpc;
-  if (n_qt * p.h_kv > INT32_MAX) return cudaErrorInvalidValue;
+  if ((int64_t)p.n_qt * p.h_kv > INT32_MAX) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(n_qt * p.h_kv));
+  cfg.gridDim = dim3((unsigned)(p.n_qt * p.h_kv));
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = Cfg<D>::kSmemBytes;
   cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = p.after ? 1 : 0;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, SPLIT>, p, mq, mk, mv);
 }
 
@@ -751,22 +759,51 @@ cudaError_t launch(const PrefillTcParams& p, const void* q, const void* k, const
   // costed as its longest CTA and, where it needs a second wave, the first CTA of that behind
   // the shortest of the first (CTAs start in descending order), with the costs measured on
   // GB300: us per call for 512 + 160 tokens, 28/4 heads, 16.9 with two slots, 14.5 split; 1500 +
-  // 160, 16/1 heads, 29.0 and 22.8; but 1300 + 160, 28/4 heads, 29.0 and 32.7.
+  // 160, 16/1 heads, 29.0 and 22.8; but 1300 + 160, 28/4 heads, 29.0 and 32.7.  head_dim 64 is
+  // costed the same: what it has more of P.V it has less of loads (800 + 160, 32/8 heads, 24.4 with
+  // two slots, 22.7 split; 1200 + 160, 29.2 and 31.7; 512 + 160, 14/2 heads, 18.6 and 12.9).
   const int sms = sm_count(dev);
+  auto tiles_upto = [&](int64_t last) {        // key tiles of a query tile whose last token this is
+    return last < p.prefix_len ? last / kBN + 1 : (p.prefix_len + kBN - 1) / kBN + 1;
+  };
   auto cost = [&](int tpc, int tiles_per_round, double cta_us, double round_us) {
     const int64_t n_qt = ((int64_t)p.n_tokens + tpc - 1) / tpc, n = n_qt * p.h_kv;
     auto rounds = [&](int64_t cta) {
       const int64_t last = std::min<int64_t>((n_qt - cta / p.h_kv) * tpc, p.n_tokens) - 1;
-      const int64_t tiles = last < p.prefix_len ? last / kBN + 1 : (p.prefix_len + kBN - 1) / kBN + 1;
-      return (double)((tiles + tiles_per_round - 1) / tiles_per_round);
+      return (double)((tiles_upto(last) + tiles_per_round - 1) / tiles_per_round);
     };
     double t = cta_us + round_us * rounds(0);
     // (the second of two CTAs finds its code and parameters cached)
     if (n > sms) t = std::max(t, 1.8 * cta_us + round_us * (rounds(sms - 1) + rounds(sms)));
     return n > 2 * (int64_t)sms + sms / 16 ? 1e30 : t;  // (a few over two waves, the shortest, are no third)
   };
-  const bool split = cost(p.tps, 2, kSplitCtaUs, kSplitRoundUs) < cost(2 * p.tps, 1, kPairCtaUs, kPairTileUs);
-  return split ? launch_slots<D, true>(p, mq, mk, mv, dev, s) : launch_slots<D, false>(p, mq, mk, mv, dev, s);
+  const int64_t n_one = ((int64_t)p.n_tokens + p.tps - 1) / p.tps;  // query tiles of one slot
+  const double split_us = cost(p.tps, 2, kSplitCtaUs, kSplitRoundUs), pair_us = cost(2 * p.tps, 1, kPairCtaUs, kPairTileUs);
+  // Where the split form is some CTAs over one wave, the first tokens, whose key ranges are the
+  // shortest, go in pairs instead, just enough of them that everything runs at once: a second grid,
+  // which starts when the first one's CTAs have.  (us per call, split or pairs / two grids: 600 + 160 tokens,
+  // 28/4 heads 18.7 / 16.8; 500 + 160, 32/8 heads 18.6 / 16.5; 700 + 160, 32/8 heads 20.7 / 18.6.)
+  const int64_t pairs = n_one - sms / p.h_kv;
+  PrefillTcParams a = p;
+  if (pairs > 0 && 2 * pairs <= n_one) {
+    const double mixed_us = kTwoGridsUs + std::max(kSplitCtaUs + kSplitRoundUs * (double)((tiles_upto(p.n_tokens - 1) + 1) / 2),
+                                                   kLateUs + kPairCtaUs + kPairTileUs * (double)tiles_upto(2 * pairs * p.tps - 1));
+    if (mixed_us < split_us && mixed_us < pair_us) {
+      a.tok_base = (int32_t)(2 * pairs * p.tps);
+      a.n_qt = (int32_t)(n_one - 2 * pairs);
+      a.release = a.n_qt > 0;
+      cudaError_t e = a.n_qt > 0 ? launch_slots<D, true>(a, mq, mk, mv, dev, s) : cudaSuccess;
+      if (e != cudaSuccess) return e;
+      a.after = a.release;
+      a.release = 0;
+      a.tok_base = 0;
+      a.n_qt = (int32_t)pairs;
+      return launch_slots<D, false>(a, mq, mk, mv, dev, s);
+    }
+  }
+  const bool split = split_us < pair_us;
+  a.n_qt = (int32_t)((p.n_tokens + (int64_t)(split ? 1 : 2) * p.tps - 1) / ((split ? 1 : 2) * p.tps));
+  return split ? launch_slots<D, true>(a, mq, mk, mv, dev, s) : launch_slots<D, false>(a, mq, mk, mv, dev, s);
 }
 
 }  // namespace
@@ -806,6 +843,7 @@ cudaError_t launch_prefill_tc(int32_t n_tokens, int32_t prefix_len, int32_t n_br
   p.scale_log2 = (float)((double)scale * 1.4426950408889634);
   p.out_bf16 = out_bf16;
   p.gen = gen;
+  p.tok_base = p.n_qt = p.release = p.after = 0;
   cudaError_t e = prefill_header(&p.header);
   if (e != cudaSuccess) return e;
   p.out = out;

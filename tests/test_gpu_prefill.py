@@ -8,6 +8,7 @@ import pytest
 import torch
 
 import oracle
+from late_writer import late_store
 from paper_2607_02963_gb300 import binding as B
 from paper_2607_02963_gb300 import synth
 
@@ -178,3 +179,39 @@ def test_prefill_branch_does_not_reach_the_others(D, h_q, h_kv, prefix, lens, fl
     assert int(keep.sum()) > 100 and bool(keep[-1])
     for a, b in zip(*res):
         assert torch.equal(a[keep], b[keep])
+
+
+@pytest.mark.parametrize("D,h_q,h_kv,prefix,lens", [
+    # a few CTAs over one wave of 152 SMs: the first tokens in pairs beside the rest, from one token group
+    # in pairs to nearly half; all prefix, all branches and both among the pairs
+    (128, 32, 8, 600, [10]), (128, 32, 8, 500, [40, 0, 80, 40]), (128, 28, 4, 700, [40] * 4),
+    (128, 32, 8, 0, [200, 150, 300, 33]), (64, 32, 8, 560, [7] * 9), (128, 8, 8, 2300, [140, 1]),
+])
+@pytest.mark.parametrize("out_dtype", [0, 1])
+def test_prefill_two_grids(D, h_q, h_kv, prefix, lens, out_dtype):
+    """Behind a grid that stores the inputs long after it has released its dependents, and ahead of one that
+    reads the result at once: both grids of the call keep stream order.  (fp32 against the oracle; the bf16
+    output is that result rounded.)"""
+    if out_dtype == 0:
+        _run(prefix, lens, h_q, h_kv, D, seed=prefix + len(lens))
+    true = [_dev(x) for x in synth.prefill_inputs(prefix + len(lens), prefix, lens, h_q, h_kv, D)]
+    prob = B.make_problem(h_q, h_kv, D, 16, 1.0 / math.sqrt(D), out_dtype=out_dtype)
+    side, res = torch.cuda.Stream(), []
+    if out_dtype:
+        out32 = torch.empty(true[0].shape, device="cuda")
+        B.pad_prefill_attn(B.make_problem(h_q, h_kv, D, 16, 1.0 / math.sqrt(D)), prefix, lens, *true, out32)
+    for late in (False, True):
+        q, k, v = (torch.full_like(t, 2.0) if late else t.clone() for t in true)
+        out = torch.full(q.shape, float("nan"), dtype=torch.bfloat16 if out_dtype else torch.float32, device="cuda")
+        lse = torch.full(q.shape[:2], float("nan"), device="cuda")
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            if late:
+                late_store(list(zip((q, k, v), true)), side)
+            B.pad_prefill_attn(prob, prefix, lens, q, k, v, out, lse)
+            res.append((out.clone(), lse.clone()))
+        torch.cuda.synchronize()
+        B.pad_prefill_status(side)
+    for a, b in zip(*res):
+        assert torch.equal(a, b) and bool(torch.isfinite(a).all())
+    assert not out_dtype or torch.equal(res[0][0], out32.bfloat16())
