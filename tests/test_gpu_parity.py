@@ -780,9 +780,9 @@ def test_shared_branch_tasks_match_oracle(lens, D, h_q, h_kv, one_call):
 
 
 @pytest.mark.parametrize("one_call", [True, False])
-@pytest.mark.parametrize("prefix,flags", [([0, 0], 0), ([0, 0], B.FLAG_PREFIX_MMA), ([700, 300], 0),
-                                          ([700, 300], B.FLAG_PREFIX_DUAL)])
-def test_steps_back_to_back_equal_steps_run_apart(prefix, flags, one_call):
+@pytest.mark.parametrize("prefix,flags,rope", [([0, 0], 0, False), ([0, 0], B.FLAG_PREFIX_MMA, True), ([700, 300], 0, False),
+                                               ([700, 300], 0, True), ([700, 300], B.FLAG_PREFIX_DUAL, True)])
+def test_steps_back_to_back_equal_steps_run_apart(prefix, flags, rope, one_call):
     """A generation loop enqueued without any wait between its kernels (each step reads the keys
     that the one before appended, and q written by a kernel right ahead of the attention) equals
     the same loop with a wait after every call; also with nothing but branches, where no prefix
@@ -795,12 +795,18 @@ def test_steps_back_to_back_equal_steps_run_apart(prefix, flags, one_call):
         db = DeviceBatch(w, flags=flags, fill_nan=False)
         db.page_table = torch.cat([db.page_table, torch.full_like(db.page_table, -1)], dim=1).contiguous()
         lens, outs, plans = w.event_len.copy(), [], []
+        tables = [torch.from_numpy(synth.rope_table(2000, 128) * (1.0 + 0.125 * i)).cuda() for i in range(6)]
+        table = tables[0].clone()
         for step in range(6):
             plan = B.pad_plan(db.problem, db.cache, w.prefix_len, w.event_video, lens, page_table=db.page_table,
                               max_pages=int(db.page_table.shape[1]), workspace=db.workspace,
                               prefix_offset=w.prefix_offset)
             plans.append(plan)
+            if rope:
+                plan.set_rope(synth.step_positions(w) + step, table)
             out, lse = torch.empty_like(db.out), torch.empty_like(db.lse)
+            wait()
+            table.copy_(tables[step])    # (a model may keep the current rows of its table in one place)
             wait()
             if not one_call:
                 B.pad_kv_append(plan, db.k_new, db.v_new, db.k_pool, db.v_pool)
