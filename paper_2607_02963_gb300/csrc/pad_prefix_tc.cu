@@ -128,10 +128,10 @@ static_assert(sizeof(TcBars) <= 256, "barrier block fits its slot");
 // 2(t%4) + 1: s[x][4k..4k+3] = (a, c), (a, c+1), (a+8, c), (a+8, c+1) with
 // c = 64x + 8k + 2(t%4).  A row's maximum and sum are shared by the four threads of its
 // quad (lanes 4(t/4) .. +3).
-// Visible columns of one row: the first `valid`, or the set bits of a 128-column mask.
-struct ColsValid {
-  int valid;
-  __device__ bool vis(int c) const { return c < valid; }
+// Visible columns of one row: a range, or the set bits of a 128-column mask.
+struct ColsRange {
+  int lo, hi;
+  __device__ bool vis(int c) const { return c >= lo && c < hi; }
 };
 struct ColsBits {
   uint64_t lo, hi;  // columns 0-63, 64-127
@@ -314,14 +314,19 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int n_tiles = (ntok + kBN - 1) / kBN;
   const int kvh = it.kvh;
   const int tok0 = (int)it.tok0;
-  // The split ends inside its last tile: that V tile is loaded to a barrier of its own, and becomes
-  // full (vfull) once the producer has cleared its rows past the end.
-  const bool part = ntok % kBN != 0;
+  // Tokens past the split's end stay out of its V tiles (see zero_v_rows).  Where the prefix has 128
+  // tokens up to there, the last tile ends with the split: it starts that much earlier, and the columns
+  // that it shares with the tile before are masked.  A shorter prefix (one tile) would run into
+  // whatever lies ahead of it instead: its V tile is loaded to a barrier of its own, and becomes full
+  // (vfull) once the producer has cleared its rows past the end.  (Cleared so, 4000 tokens, 3 events
+  // took 8.5 us per step instead of 8.2.)
+  const bool whole = it.tok_end >= kBN, part = !whole && ntok % kBN != 0;
+  const int last_tok = whole ? ntok - kBN : 0;   // of the split: where its last tile starts
   auto load_tile = [&](const CUtensorMap* map, uint32_t off, int t, uint64_t* full) {
     mbar_expect_tx(full, C::kTileBytes);
 #pragma unroll
     for (int h = 0; h < C::kHalves; ++h)
-      tma_load_3d(sbase + off + h * kHalfBytes, map, 64 * h, kvh, tok0 + t * kBN, full);
+      tma_load_3d(sbase + off + h * kHalfBytes, map, 64 * h, kvh, tok0 + min(t * kBN, last_tok), full);
   };
 
   // The softmax warps load their Q rows now, so that the loads overlap barrier set-up
@@ -654,17 +659,20 @@ __global__ void __launch_bounds__(kThreads, 1)
           tmem_wait_ld_dep(sr[1]);
           // columns to mask: past the split's end, or (GSELF) hidden planning tokens of the
           // row's event; the path is chosen per warp (tcgen05.st below is warp-collective)
+          // (the last tile's columns: those from `lo` on, or the first `hi`, see `whole`)
+          const int lo = whole ? kBN - valid : 0, hi = whole ? kBN : valid;
           if (GSELF) {
             ColsBits ka{~0ull, ~0ull}, kb{~0ull, ~0ull};
-            const int t0 = it.tok_begin + j * kBN;
+            const int t0 = it.tok_begin + j * kBN - lo;
             if (valid < kBN || (t0 < g_hi && t0 + kBN > g_lo)) {
               const GMask gma{g_lo, g_hi, g_oa}, gmb{g_lo, g_hi, g_ob};
-              ka = ColsBits{keep_bits(valid, gma, t0), keep_bits(valid - 64, gma, t0 + 64)};
-              kb = ColsBits{keep_bits(valid, gmb, t0), keep_bits(valid - 64, gmb, t0 + 64)};
+              const uint64_t f0 = lo >= 64 ? 0ull : ~0ull << lo, f1 = lo > 64 ? ~0ull << (lo - 64) : ~0ull;
+              ka = ColsBits{keep_bits(hi, gma, t0) & f0, keep_bits(hi - 64, gma, t0 + 64) & f1};
+              kb = ColsBits{keep_bits(hi, gmb, t0) & f0, keep_bits(hi - 64, gmb, t0 + 64) & f1};
             }
             if (__any_sync(0xffffffffu, (ka.lo & ka.hi & kb.lo & kb.hi) != ~0ull)) mask_rows(sr, cq, ka, kb);
           } else if (valid < kBN) {
-            mask_rows(sr, cq, ColsValid{valid}, ColsValid{valid});
+            mask_rows(sr, cq, ColsRange{lo, hi}, ColsRange{lo, hi});
           }
           // P of the tile on the running maxima, over the first 64 columns of its S buffer, in
           // this warp's own rows.  The sums (ta, tb: this thread's share), which the row sums need

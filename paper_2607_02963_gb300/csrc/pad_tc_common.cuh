@@ -190,7 +190,8 @@ __device__ __forceinline__ bool elect_one() {
 // swizzle), by threads 0 .. n - 1 of those that do.  A tile is loaded whole, so past the keys that a
 // query may see it holds other tokens, another video's among them, or whatever lies in a gap of the
 // caller's buffer.  Their weights are 0, but 0 times a NaN or an infinity is not: they must not meet.
-// Call it once the tile has landed; what the MMAs wait for is arrived on after it.  (By the V producer,
+// Call it once the tile has landed; what the MMAs wait for is arrived on after it.  (Where it can, a
+// kernel has its last tile end with the visible keys instead, which costs nothing.  By the V producer,
 // which has time: in the loop of the P.V issuer, or in the softmax of such tiles, it cost 1 to 3 % of
 // a prefill, 1.4 % of a 32768-token step.)
 template <int HALVES>
