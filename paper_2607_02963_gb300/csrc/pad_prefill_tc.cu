@@ -56,7 +56,6 @@
 // PAD_ERR_DEVICE_TIMEOUT in the prefill status word, raises a CTA-wide abort flag, lets the
 // producers and issuers drain what they started, frees TMEM and returns.
 #include <cuda.h>
-#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <algorithm>
 #include <cstdint>
@@ -685,32 +684,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
-  static const PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000, cudaEnableDefault, &qres) != cudaSuccess ||
-        qres != cudaDriverEntryPointSuccess)
-      ptr = nullptr;
-    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
-  }();
-  return fn;
-}
-
-// Token-major [tokens, heads, D] bf16 as a 3-D tensor (d, head, token); one box is 64 columns
-// x box_heads x box_tokens with the 128-byte swizzle.
-bool make_map(CUtensorMap* map, const void* base, int D, int heads, int64_t tokens, int box_heads, int box_tokens) {
-  auto enc = get_encode();
-  if (!enc) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)heads, (cuuint64_t)tokens};
-  cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)heads * D * 2};
-  cuuint32_t box[3] = {64, (cuuint32_t)box_heads, (cuuint32_t)box_tokens};
-  cuuint32_t estr[3] = {1, 1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // (a CTA, and a round of two key tiles or a tile of its chain; the start and the end of a second grid)
 constexpr double kSplitCtaUs = 8.5, kSplitRoundUs = 1.3, kPairCtaUs = 8.5, kPairTileUs = 1.54, kLateUs = 1.5, kTwoGridsUs = 3.0;
 
@@ -749,8 +722,8 @@ int sm_count(int dev) {
 template <int D>
 cudaError_t launch(const PrefillTcParams& p, const void* q, const void* k, const void* v, cudaStream_t s) {
   CUtensorMap mq, mk, mv;
-  if (!make_map(&mq, q, D, p.h_q, p.n_tokens, p.group, p.tps) || !make_map(&mk, k, D, p.h_kv, p.n_tokens, 1, kBN) ||
-      !make_map(&mv, v, D, p.h_kv, p.n_tokens, 1, kBN))
+  if (!tma_map(&mq, q, D, p.h_q, p.n_tokens, p.group, p.tps) || !tma_map(&mk, k, D, p.h_kv, p.n_tokens, 1, kBN) ||
+      !tma_map(&mv, v, D, p.h_kv, p.n_tokens, 1, kBN))
     return cudaErrorInvalidValue;
   int dev = 0;
   cudaGetDevice(&dev);

@@ -702,7 +702,7 @@ cudaError_t launch_prefix_dual(const KParams& p, int max_rows, const void* q, co
   int dev = 0;
   cudaGetDevice(&dev);
   CUtensorMap mk, mv;
-  if (!prefix_tensor_maps(kp, vp, kD, p.h_kv, total_prefix_tokens, dev, &mk, &mv)) return cudaErrorInvalidValue;
+  if (!prefix_tensor_maps(kp, vp, kD, p.h_kv, total_prefix_tokens, &mk, &mv)) return cudaErrorInvalidValue;
   static bool configured[64] = {};
   if (dev >= 0 && dev < 64 && !configured[dev]) {
     for (auto fn : {prefix_dual_kernel<false, false>, prefix_dual_kernel<true, false>, prefix_dual_kernel<false, true>,

@@ -62,8 +62,6 @@
 #include <algorithm>
 #include <cstddef>
 #include <cstdint>
-#include <cstring>
-#include <mutex>
 
 #include "pad_branch_merge.cuh"
 #include "pad_internal.h"
@@ -814,75 +812,33 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  if (!fn) {
+  static const PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
     void* ptr = nullptr;
     cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000, cudaEnableDefault,
-                                         &qres) == cudaSuccess &&
-        qres == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
-  }
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000, cudaEnableDefault, &qres) != cudaSuccess ||
+        qres != cudaDriverEntryPointSuccess)
+      ptr = nullptr;
+    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
+  }();
   return fn;
 }
 
-// Token-major [T, h_kv, D] bf16 prefix as a 3-D tensor (d, head, token); one box is
-// 64 head-dim columns x 1 head x 128 tokens with the 128-byte swizzle.
-bool make_map(CUtensorMap* map, const void* base, int D, int h_kv, int64_t tokens) {
-  auto enc = get_encode();
-  if (!enc) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)h_kv, (cuuint64_t)tokens};
-  cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)h_kv * D * 2};
-  cuuint32_t box[3] = {64, 1, (cuuint32_t)kBN};
-  cuuint32_t estr[3] = {1, 1, 1};
-  CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides,
-                   box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
-// The tensor maps of the last few (K, V) prefix buffers, so a step does not re-encode
-// them (an encode costs microseconds of host time; the maps depend only on the base
-// address, the head count and the token extent).
-struct MapCacheEntry {
-  const void* k;
-  const void* v;
-  int D, h_kv;
-  int64_t tokens;
-  int dev;
-  CUtensorMap mk, mv;
-};
-std::mutex g_map_mu;
-MapCacheEntry g_maps[8];
-int g_maps_n = 0, g_maps_next = 0;
-
 }  // namespace
 
-bool prefix_tensor_maps(const void* kp, const void* vp, int D, int h_kv, int64_t tokens, int dev, CUtensorMap* mk,
-                        CUtensorMap* mv) {
-  std::lock_guard<std::mutex> lk(g_map_mu);
-  for (int i = 0; i < g_maps_n; ++i) {
-    const MapCacheEntry& e = g_maps[i];
-    if (e.k == kp && e.v == vp && e.D == D && e.h_kv == h_kv && e.tokens == tokens && e.dev == dev) {
-      std::memcpy(mk, &e.mk, sizeof(CUtensorMap));
-      std::memcpy(mv, &e.mv, sizeof(CUtensorMap));
-      return true;
-    }
-  }
-  MapCacheEntry ne;
-  ne.k = kp;
-  ne.v = vp;
-  ne.D = D;
-  ne.h_kv = h_kv;
-  ne.tokens = tokens;
-  ne.dev = dev;
-  if (!make_map(&ne.mk, kp, D, h_kv, tokens) || !make_map(&ne.mv, vp, D, h_kv, tokens)) return false;
-  g_maps[g_maps_next] = ne;
-  g_maps_next = (g_maps_next + 1) % 8;
-  if (g_maps_n < 8) ++g_maps_n;
-  std::memcpy(mk, &ne.mk, sizeof(CUtensorMap));
-  std::memcpy(mv, &ne.mv, sizeof(CUtensorMap));
-  return true;
+bool tma_map(CUtensorMap* map, const void* base, int D, int heads, int64_t tokens, int box_heads, int box_tokens) {
+  auto enc = get_encode();
+  if (!enc) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)heads, (cuuint64_t)tokens};
+  cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)heads * D * 2};
+  cuuint32_t box[3] = {64, (cuuint32_t)box_heads, (cuuint32_t)box_tokens};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool prefix_tensor_maps(const void* kp, const void* vp, int D, int h_kv, int64_t tokens, CUtensorMap* mk, CUtensorMap* mv) {
+  return tma_map(mk, kp, D, h_kv, tokens, 1, kBN) && tma_map(mv, vp, D, h_kv, tokens, 1, kBN);
 }
 
 int prefix_tc_tail_chunk(int branch_rows, int group, int max_splits) {
@@ -934,7 +890,7 @@ cudaError_t launch_prefix_tc(const KParams& p, int max_rows, const void* q, cons
   int dev = 0;
   cudaGetDevice(&dev);
   CUtensorMap mk, mv;
-  if (!prefix_tensor_maps(kp, vp, p.head_dim, p.h_kv, total_prefix_tokens, dev, &mk, &mv)) return cudaErrorInvalidValue;
+  if (!prefix_tensor_maps(kp, vp, p.head_dim, p.h_kv, total_prefix_tokens, &mk, &mv)) return cudaErrorInvalidValue;
   return p.head_dim == 128 ? launch_d<128>(p, max_rows, q, mk, mv, k_pool, v_pool, out, lse, pdl, dev, s)
                            : launch_d<64>(p, max_rows, q, mk, mv, k_pool, v_pool, out, lse, pdl, dev, s);
 }

@@ -395,9 +395,11 @@ __device__ __forceinline__ void prefetch_branch_tasks(const KParams& p, const __
 
 }  // namespace tc
 
-// Tensor maps of a token-major [tokens, h_kv, D] bf16 K and V prefix (boxes of 64 head-dim
-// columns x 1 head x 128 tokens, 128-byte swizzle), cached per (buffers, shape, device).
-bool prefix_tensor_maps(const void* kp, const void* vp, int D, int h_kv, int64_t tokens, int dev, CUtensorMap* mk,
-                        CUtensorMap* mv);
+// Token-major [tokens, heads, D] bf16 as a 3-D tensor (d, head, token); one box is 64 columns x
+// box_heads x box_tokens with the 128-byte swizzle.  Encoded for each launch: that takes 0.03 us a map on
+// the host, less than looking one up.
+bool tma_map(CUtensorMap* map, const void* base, int D, int heads, int64_t tokens, int box_heads, int box_tokens);
+// The maps of a K and V prefix (boxes of one head x 128 tokens).
+bool prefix_tensor_maps(const void* kp, const void* vp, int D, int h_kv, int64_t tokens, CUtensorMap* mk, CUtensorMap* mv);
 
 }  // namespace pad
