@@ -126,7 +126,6 @@ struct Layout {
   int64_t n_counters = 0;
   size_t off_videos = 0, off_events = 0, off_items = 0, off_tasks = 0, upload_bytes = 0;
   size_t off_ml = 0, off_o = 0, off_cnt = 0, total_bytes = 0;
-  size_t warp_level_bytes = 0;  // head_dim 64 on the tensor cores: total_bytes of the warp-level layout
 };
 
 // Device scratch inside the library for callers that have none to give (see
@@ -491,18 +490,18 @@ pad_status compute_layout(const pad_problem* prob, int32_t n_videos, const int32
     *L = Layout();
     return layout_for(prob, n_videos, prefix_len, n_events, event_video, n_sms, kern, per_video, L);
   };
-  pad_status st = attempt(0, true);
-  if (st != PAD_OK || !on_workspace || prob->head_dim != 64 || (prob->flags & (kPrefixFlags | PAD_FLAG_FUSED_MERGE)) ||
-      L->prefix_kernel != PAD_FLAG_PREFIX_MMA || L->max_rows > 64 * 128)  // (the CTA list holds a row group in six bits)
-    return st;
-  const size_t warp_level_bytes = L->total_bytes;
-  const size_t most = std::min(room, warp_level_bytes <= kStaticScratchBytes ? kStaticScratchBytes : SIZE_MAX);
+  if (!on_workspace || prob->head_dim != 64 || (prob->flags & (kPrefixFlags | PAD_FLAG_FUSED_MERGE))) return attempt(0, true);
+  // (the tensor-core layout first: where it fits, the warp-level one need not be built)
+  pad_status st = attempt(PAD_FLAG_PREFIX_TC, true);
+  if (st != PAD_OK || L->max_rows <= 8 || L->max_rows > 64 * 128)  // (the CTA list holds a row group in six bits)
+    return attempt(0, true);
+  if (L->total_bytes <= std::min(room, kStaticScratchBytes)) return st;
+  st = attempt(0, true);
+  if (st != PAD_OK) return st;
+  const size_t most = std::min(room, L->total_bytes <= kStaticScratchBytes ? kStaticScratchBytes : SIZE_MAX);
   for (bool per_video : {true, false}) {
     st = attempt(PAD_FLAG_PREFIX_TC, per_video);
-    if (st == PAD_OK && L->total_bytes <= most) {
-      L->warp_level_bytes = warp_level_bytes;
-      return st;
-    }
+    if (st == PAD_OK && L->total_bytes <= most) return st;
   }
   return attempt(0, true);
 }
@@ -753,8 +752,11 @@ size_t pad_workspace_size(const pad_problem* prob, int32_t n_videos, const int32
   Layout L;
   const int sms = prob->num_sms > 0 ? prob->num_sms : query_num_sms();
   if (compute_layout(prob, n_videos, prefix_len, n_events, event_video, sms, true, SIZE_MAX, &L) != PAD_OK) return 0;
-  // (room for either kernel, so that a smaller batch, whose warp-level layout is no larger, fits)
-  return std::max(L.total_bytes, L.warp_level_bytes);
+  const size_t bytes = L.total_bytes;
+  // (head_dim 64: room for either kernel, so that a smaller batch, whose warp-level layout is no larger, fits)
+  if (L.prefix_kernel != PAD_FLAG_PREFIX_TC || prob->head_dim != 64) return bytes;
+  if (compute_layout(prob, n_videos, prefix_len, n_events, event_video, sms, false, SIZE_MAX, &L) != PAD_OK) return 0;
+  return std::max(bytes, L.total_bytes);
 }
 
 pad_status pad_plan(const pad_problem* prob, pad_cache_state* cache, int32_t n_videos,
