@@ -249,9 +249,9 @@ typedef struct {
   uint64_t generation;      /* the number tagging this plan's device status word and counters */
   int32_t prefix_ctas;      /* CTAs of the prefix pass (a batch of videos may take several waves) */
   int32_t max_split_tiles;  /* 128-token tiles of the longest split */
-  int32_t merge_first;      /* 1: in a one-call step the branch tasks wait for the prefix pass
-                               before their branch pass (too few SMs are left beside it for
-                               them to run there), staging the split partials meanwhile */
+  int32_t merge_first;      /* 1: the branch tasks wait for the prefix pass before their branch
+                               pass (too few SMs are left beside it for them to run there),
+                               staging the split partials meanwhile */
 } pad_plan_info;
 pad_status pad_plan_get_info(const pad_plan_t* plan, pad_plan_info* info);
 pad_status pad_plan_destroy(pad_plan_t* plan);
@@ -472,7 +472,9 @@ pad_status pad_attn_aggregate(const void* x, int64_t n_tokens, int32_t d_model, 
  *               fp32 (natural log) or NULL; all device, 16-byte aligned (lse 4-byte)
  * One video per call; the work is asynchronous on `stream`.  It runs on the tensor-core
  * kernel (a CTA: two groups of 128 / G tokens x the G heads of one kv-head against their
- * visible key ranges, output normalised in place); with flags PAD_FLAG_PREFIX_MMA or
+ * visible key ranges, output normalised in place; a short sequence one group, whose key tiles
+ * two halves of the CTA share out, or both forms side by side).  A NaN or an infinity in one
+ * token's k or v can reach, besides the tokens that see it, those of its own group or pair; with flags PAD_FLAG_PREFIX_MMA or
  * PAD_FLAG_PREFIX_SIMT on the warp-level kernel (64 tokens x one head). */
 pad_status pad_prefill_attn(const pad_problem* prob, int32_t prefix_len, int32_t n_branches,
                             const int32_t* branch_len, const void* q, const void* k, const void* v, void* out,

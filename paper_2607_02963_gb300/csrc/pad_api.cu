@@ -1147,8 +1147,8 @@ pad_status pad_kv_append(const pad_plan_t* plan, const void* k_new, const void* 
 }
 
 // a3 (+ a4, a5 in the same kernel when the plan fuses them, else in the branch/merge
-// kernel after it).  k_new == NULL: the append kernel ran just before (the prefix kernel
-// overlaps it through programmatic dependent launch).  k_new set: no append kernel; each
+// kernel after it).  k_new == NULL: the append kernel ran just before (the prefix kernel's
+// set-up overlaps it through programmatic dependent launch).  k_new set: no append kernel; each
 // branch task appends its own row, and the prefix kernel is the step's first launch.
 static pad_status launch_attention(const pad_plan_t* plan, const void* q, const void* k_new,
                                    const void* v_new, const void* k_prefix, const void* v_prefix,
@@ -1179,11 +1179,10 @@ static pad_status launch_attention(const pad_plan_t* plan, const void* q, const 
     case PAD_FLAG_PREFIX_SIMT: e = launch_prefix_simt(p, plan->lay.max_rows, q, k_prefix, v_prefix, s); break;
     case PAD_FLAG_PREFIX_MMA: e = launch_prefix_mma(p, plan->lay.max_rows, q, k_prefix, v_prefix, s); break;
     case PAD_FLAG_PREFIX_TC:
-      // programmatic dependent launch: the prefix pass overlaps the append kernel and the
-      // branch/merge pass's prologue overlaps the prefix pass (not while timing events
-      // are recorded between the kernels).  As the first kernel of a one-call step it
-      // overlaps only the launch with the grid before it, and waits for that grid before
-      // it reads or writes anything.
+      // programmatic dependent launch: the prefix kernel's set-up overlaps the grid ahead (the append,
+      // or whatever precedes a one-call step, whose first K/V tile goes out then too), and
+      // the branch/merge pass's prologue overlaps the prefix pass (not while timing events
+      // are recorded between the kernels)
       e = launch_prefix_tc(p, plan->lay.max_rows, q, k_prefix, v_prefix, plan->total_prefix_tokens, k_pool,
                            v_pool, out, lse, !timed, s);
       break;

@@ -104,10 +104,10 @@ struct KParams {
   int32_t fused;                  // the tensor-core prefix kernel runs a4 + a5 itself (one
                                   // (event, kv-head) task per CTA after its split)
   int32_t tail_chunk;             // split partials merged per staged chunk in that tail
-  int32_t merge_first;            // one-call step whose prefix grid leaves too few SMs for
-                                  // the branch/merge CTAs to run beside it: each of them
-                                  // waits for it first, then stages the split partials
-                                  // while its branch pass runs
+  int32_t merge_first;            // the prefix grid leaves too few SMs for the branch/merge
+                                  // CTAs to run beside it (one call, or two with keys_ready):
+                                  // each of them waits for it first, then stages the split
+                                  // partials while its branch pass runs
   int32_t keys_ready;             // two-call step behind the tensor-core prefix grid, which waits
                                   // for the append before it releases the branch/merge grid:
                                   // the appended keys may be read before that grid's own wait;

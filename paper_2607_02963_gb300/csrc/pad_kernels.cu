@@ -110,8 +110,8 @@ __global__ void append_kernel(const __grid_constant__ KParams p, const uint4* __
                               const uint4* __restrict__ v_new, uint4* __restrict__ k_pool,
                               uint4* __restrict__ v_pool) {
   // Launched so that it may start while the grid ahead runs, and releases the grid behind it
-  // at once; each waits for the other's completion before it touches memory (the plan's
-  // descriptors apart).  A two-call step waits for all of this kernel, a chain of latencies: the
+  // at once; each waits for the completion of the one ahead of it before it touches memory (the
+  // plan's descriptors apart).  A two-call step waits for all of this kernel, a chain of latencies: the
   // index arithmetic runs ahead of the wait and the new rows are read beside the page id (prefix
   // 8219, 13 events with RoPE: 13.2 us per step, now 12.7).
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -525,8 +525,8 @@ __global__ void __launch_bounds__(128) prefix_mma_kernel(const __grid_constant__
 // programmatic dependent launch: its griddepcontrol.wait covers the prefix grid, so the
 // split partials are complete once it returns.
 // ---------------------------------------------------------------------------
-// NW warps per task: 8 (two CTAs per SM) by default, 4 (three per SM) when the step has more
-// than two waves of tasks, so that more of its latency-bound tasks are in flight at once.
+// NW warps per task: 8 (two CTAs per SM) by default, 4 (three per SM, four with OVER) when the step
+// has more than two waves of tasks, so that more of its latency-bound tasks are in flight at once.
 // W output columns per CTA: D / W CTAs share a task (KParams::col_splits).
 // OVER (4 warps): four CTAs per SM, the partials staged over the branch's keys.
 template <int D, bool ROPE, int CAUSAL, int NW, int W, bool OVER>
@@ -538,9 +538,9 @@ __global__ void __launch_bounds__(32 * NW, NW == bm::kWarps ? 2 : (OVER ? 4 : 3)
                                                                     float* __restrict__ lse,
                                                                     int sch) {
   extern __shared__ __align__(16) unsigned char bm_raw[];
-  // The grid after this one may be scheduled now: in a one-call loop it is the next step's
-  // prefix kernel, which waits for this grid before it touches anything (an append kernel
-  // after it is launched without programmatic serialisation and waits in any case).
+  // The grid after this one may be scheduled now: the next step's append, prefix or (no prefix)
+  // branch/merge kernel waits for this grid before it touches anything that this one reads or
+  // writes.  Without a prefix grid ahead, this one first waits itself.
   if (p.keys_ready == 2) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   constexpr int kShare = D / W;

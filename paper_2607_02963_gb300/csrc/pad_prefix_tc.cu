@@ -37,7 +37,7 @@
 // tokens, 4 events 14.3 -> 6.3 (latency: programmatic dependent launch and the one-call order
 // come with this path).
 //
-// Every MMA has N = 128 (S: 128 tokens; P.V: 128 head-dim columns), the size at
+// Every MMA has N = 128 (S: 128 tokens; P.V: 128 head-dim columns; 64 at head_dim 64), the size at
 // which one tcgen05.mma carries as much tensor work as it costs to issue.
 // TMEM columns: S[b] at 128*b (b = 0, 1, 2), O at 384.  Output: the partial
 // softmax state (m, l, O) of every row for this split, merged with the other
