@@ -5,13 +5,11 @@ issuer and eight softmax warps that hand 128-token tiles to each other through
 mbarriers waited on by phase parity: 3 K/V stages whose index is also the TMEM S buffer,
 per-stage barriers for "K tile loaded", "V tile loaded", "S done", "P written" and "P.V
 done".  A tcgen05.commit arrives when every MMA issued *by the committing thread* so far
-has completed, so each issuer has its own completion barriers.  In decode, each softmax
-warp owns 16 rows of the tile outright (all 128 columns), so it writes P over S columns
-that no other warp reads: the warps never meet inside the loop.  In whole-sequence
-prefill the two warps of a lane quarter split the columns and meet on a barrier of their
-own between the row maximum and the P store; that meeting is a step inside the softmax
-here (it involves no other role, and its parity alternates with the tile, like the S
-buffers').
+has completed, so each issuer has its own completion barriers.  Each softmax warp owns 16
+rows of the tile outright (all 128 columns), so it writes P over S columns that no other warp
+reads: the warps never meet inside the loop.  The last V tile of a prefix below 128 tokens lands on
+a barrier of its own and counts as loaded only once its producer has cleared the rows past the
+prefix (part).
 
 This model mirrors that schedule with asynchronous loads and MMAs that complete after
 random delays and in any order, and checks under many random interleavings that no stage
@@ -45,18 +43,16 @@ ST = 3  # K/V stages = S buffers
 
 
 MISTAKES = ("s_skips_pvfree", "k_refill_early", "v_refill_early", "rescale_without_wait",
-            "dealloc_without_tdone", "one_xchg_slot")
+            "dealloc_without_tdone", "part_lands_on_vfull")
 
 
-def run(n, seed, lazy_prob=0.3, single_barriers=False, n_softmax=8, prefetch=False, meet=False,
+def run(n, seed, lazy_prob=0.3, single_barriers=False, n_softmax=8, prefetch=False, part=False,
         mistake=None):
     """prefetch: the softmax warps load tile j + 1's S during tile j (after the row maximum,
     before P(j) is released), as a softmax that hides the load behind the exponentials would.
-    meet: the prefill softmax, where warps w and w + 4 (the two column halves of a lane
-    quarter) exchange their partial row maxima through two shared-memory slots (tile parity)
-    and a per-quarter barrier on every tile, and their row sums once more after the loop.
+    part: the last V tile holds rows that its producer clears before it arrives on "V tile loaded".
     mistake: one of MISTAKES, a plausible slip planted in the schedule (a wait left out, or
-    one exchange slot instead of two)."""
+    the tile to be cleared loaded to the shared barrier)."""
     assert mistake is None or mistake in MISTAKES
     rnd = random.Random(seed)
     kfull = [Bar(1) for _ in range(ST)]
@@ -66,8 +62,8 @@ def run(n, seed, lazy_prob=0.3, single_barriers=False, n_softmax=8, prefetch=Fal
     pvfree = [Bar(1) for _ in range(ST)]
     drain_s, drain_pv = Bar(1), Bar(1)
     tdone = Bar(n_softmax)
-    xbar = [Bar(2) for _ in range(n_softmax // 2)]
-    xslot = {}  # (slot, half, quarter) -> what the warp last wrote there
+    vpart = Bar(1)
+    cleared = set()
     tmem_users = [True] * n_softmax
     if single_barriers:
         pfull = [pfull[0]] * ST
@@ -122,6 +118,7 @@ def run(n, seed, lazy_prob=0.3, single_barriers=False, n_softmax=8, prefetch=Fal
         def chk():
             assert j in P_written, f"P.V({j}) before P({j})"
             assert vst[j % ST] == j, f"P.V({j}) reads a V stage not holding tile {j}"
+            assert not part or j < n - 1 or j in cleared, "P.V reads the last V tile before it is cleared"
             PV_issued.add(j)
         mma("PV", chk, lambda: PV_done.add(j))
 
@@ -148,10 +145,20 @@ def run(n, seed, lazy_prob=0.3, single_barriers=False, n_softmax=8, prefetch=Fal
                 assert (t - ST) in PV_done, f"V stage reused before P.V({t - ST}) done"
             vst[s] = None
 
-            def ld(t=t, s=s):
+            own = part and t == n - 1 and mistake != "part_lands_on_vfull"
+
+            def ld(t=t, s=s, own=own):
                 vst[s] = t
-                vfull[s].arrive()
+                (vpart if own else vfull[s]).arrive()
             async_op(ld)
+        if part:
+            s = (n - 1) % ST
+            yield (vpart, 0) if mistake != "part_lands_on_vfull" else (vfull[s], ((n - 1) // ST) & 1)
+            for _ in range(rnd.choice([0, 5, 80])):
+                yield None
+            cleared.add(n - 1)
+            if mistake != "part_lands_on_vfull":
+                vfull[s].arrive()
 
     def s_issuer():
         for t in range(n):
@@ -188,8 +195,6 @@ def run(n, seed, lazy_prob=0.3, single_barriers=False, n_softmax=8, prefetch=Fal
                 holding[w].add(j)
             for _ in range(rnd.randint(0, 2)):  # the row maximum
                 yield None
-            if meet:
-                yield from exchange(w, j, ("m", j))
             if prefetch and j + 1 < n:
                 yield (sfull[(j + 1) % ST], ((j + 1) // ST) & 1)
                 assert (j + 1) in S_done, f"softmax loads S({j + 1}) before it is done"
@@ -211,23 +216,8 @@ def run(n, seed, lazy_prob=0.3, single_barriers=False, n_softmax=8, prefetch=Fal
         assert len(PV_done) == n, "epilogue before every P.V completed"
         for _ in range(rnd.randint(0, 3)):  # reads O out of TMEM
             yield None
-        if meet:
-            yield from exchange(w, n, ("l", n))
         tmem_users[w] = False
         tdone.arrive()
-
-    def exchange(w, k, tag):
-        # write this half's value into slot k & 1, meet the other half (completion k of the
-        # quarter's barrier), read the other half's value of the same round
-        quarter, half = w % (n_softmax // 2), w // (n_softmax // 2)
-        slot = 0 if mistake == "one_xchg_slot" else k & 1
-        xslot[(slot, half, quarter)] = tag
-        xbar[quarter].arrive()
-        yield (xbar[quarter], k & 1)
-        for _ in range(rnd.randint(0, 2)):
-            yield None
-        assert xslot.get((slot, 1 - half, quarter)) == tag, \
-            f"warp {w} reads the other half's {xslot.get((slot, 1 - half, quarter))} for {tag}"
 
     def dealloc():
         # warp 2 frees TMEM once every softmax warp has arrived on tdone
@@ -297,23 +287,21 @@ def test_prefetching_softmax_keeps_the_protocol(n):
 
 
 @pytest.mark.parametrize("n", range(1, 13))
-def test_prefill_softmax_exchange_keeps_the_protocol(n):
-    """The prefill softmax's per-tile meeting of the two column halves (two slots by tile
-    parity, one barrier per lane quarter) reads the other half's value of the same tile,
-    and neither deadlocks nor disturbs the MMA schedule."""
+def test_cleared_last_tile_keeps_the_protocol(n):
+    """The last V tile cleared by its producer (one tile in the kernel, any number here)."""
     for seed in range(120):
-        assert run(n, seed * 191 + n, meet=True)
+        assert run(n, seed * 191 + n, part=True)
 
 
 @pytest.mark.parametrize("mistake", MISTAKES)
 def test_model_detects_planted_mistakes(mistake):
-    """Each plausible slip in the schedule (a wait dropped, or one exchange slot for both
-    tile parities) fails the model under some interleaving."""
+    """Each plausible slip in the schedule (a wait dropped, or the tile to be cleared on the shared
+    barrier) fails the model under some interleaving."""
     fails = 0
     for n in range(2, 10):
         for seed in range(40):
             try:
-                run(n, seed * 11 + n, lazy_prob=0.6, meet=True, mistake=mistake)
+                run(n, seed * 11 + n, lazy_prob=0.6, part=True, mistake=mistake)
             except AssertionError:
                 fails += 1
     assert fails > 0, mistake
