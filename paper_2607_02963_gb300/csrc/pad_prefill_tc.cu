@@ -28,8 +28,9 @@
 //               slot's (idle) Q stage.
 //
 // What bounds it, and why it looks like this (sequence of 34.7 k tokens, 28/4 heads, D 128: 7.08
-// ms with one 128-row group per CTA, 5.36 ms = 1.60 PFLOP/s of visible pairs, 0.86 of cuBLAS's
-// rate, as it is; 8.7 k tokens, 14/2 heads, D 64: 724 us on the mma.sync kernel, 203 us here):
+// ms with one 128-row group per CTA, as it is 5.1 to 5.5 ms over several GPUs = 1.56 to 1.68 PFLOP/s of
+// visible pairs, 0.83 to 0.89 of cuBLAS's rate; 8.7 k tokens, 14/2 heads, D 64: 724 us on the mma.sync
+// kernel, 198 us here):
 //   - Two slots share each K/V tile: with one 128-row group the MMAs' shared-memory operand
 //     reads (S: 8 KB per K = 16 step, P.V: 4 KB) and the 64 KB that a tile brings in exceed 128
 //     B per clock by a fifth; and one slot's softmax runs under the other's MMAs.

@@ -393,15 +393,26 @@ __global__ void __launch_bounds__(kThreads, 1)
     // that call's contract none that releases its dependents before its writes), so that tile is
     // requested even before the wait for the grid ahead; nothing else is.  The attention call of
     // a two-call step has no such contract, and the append ahead of it releases this grid while
-    // it still waits itself, for a grid that may be writing the prefix: there the tile waits too
-    // (13 events over 8219 tokens with RoPE: 13.3 us per step, 12.7 without that wait).
+    // it still waits itself, for a grid that may be writing the prefix: there the tile is only
+    // fetched into L2 ahead of the wait, and read after it.  (us per step, read ahead / fetched / neither:
+    // 16384 tokens, 1 event 10.4 / 10.5 / 10.7; head_dim 64, 8000 tokens, 9 events 10.6 / 10.4 / 10.8;
+    // 8219 tokens, 13 events with RoPE, which waits for q and its table anyway, 12.7 / 13.1 / 13.1.)
     mbar_init(&bars->kfull[0], 1);
     mbar_init(&bars->vfull[0], 1);
     mbar_init(&bars->vpart, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmK)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
-    if (p.k_new == nullptr) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (p.k_new == nullptr) {
+      if (n_tiles > 0) {
+#pragma unroll
+        for (int h = 0; h < C::kHalves; ++h) {
+          tma_prefetch_3d(&tmK, 64 * h, kvh, tok0 + min(0, last_tok));
+          tma_prefetch_3d(&tmV, 64 * h, kvh, tok0 + min(0, last_tok));
+        }
+      }
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
     if (n_tiles > 0) {
       load_tile(&tmK, C::kOffK, 0, &bars->kfull[0]);
       load_tile(&tmV, C::kOffV, 0, part && n_tiles == 1 ? &bars->vpart : &bars->vfull[0]);
